@@ -327,6 +327,9 @@ struct Phys32 {
   float g[3];
   float E[3];
   float zq[EK_MAX_SPECIES];  // z_k qs_k: charge of one unit of species k
+  float hp, hm;              // (1 + lambda_e)/2, (1 + lambda_o)/2
+  float gw, kw;              // 9/2 (2 + lambda_e) / 36, -9/2 lambda_e / 36
+  float lo12;                // -lambda_o / 12
 };
 Phys32 make_phys32(const Phys& ph);
 // one system's entry of the batched FP32 S2 / S3 launches
@@ -338,8 +341,10 @@ cudaError_t launch_lb_fused(const LBArgs& a, cudaStream_t s);
 cudaError_t launch_advection(const LBArgs& a, cudaStream_t s);
 // FP32-storage form
 cudaError_t lb32_prepare();  // once per process, before the first launch_lb32
-// z segments per tile column of the FP32 S2 grid, chosen from the occupancy
-int lb32_segments(const Grid& g, int K, bool pv);
+// planes per segment of the FP32 S2 grid for a number of tile columns (of one
+// box, or of all boxes of a batched launch), and a box's segments per column
+int lb32_planes(long long cols, int nz);
+int lb32_segments(const Grid& g);
 cudaError_t launch_lb32(const LBArgs& a, cudaStream_t s);
 cudaError_t launch_advection32(const LBArgs& a, cudaStream_t s);
 // z segments per tile column of the FP32 S3 grid: 32-plane segments on

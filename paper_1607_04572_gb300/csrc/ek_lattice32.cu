@@ -53,6 +53,11 @@ Phys32 make_phys32(const Phys& ph) {
     p.E[d] = (float)ph.E[d];
   }
   for (int k = 0; k < EK_MAX_SPECIES; ++k) p.zq[k] = (float)(ph.z[k] * ph.qscale[k]);
+  p.hp = (float)(0.5 * (1.0 + ph.lam_e));
+  p.hm = (float)(0.5 * (1.0 + ph.lam_o));
+  p.gw = (float)(4.5 * (2.0 + ph.lam_e) / 36.0);
+  p.kw = (float)(-4.5 * ph.lam_e / 36.0);
+  p.lo12 = (float)(-ph.lam_o / 12.0);
   return p;
 }
 
@@ -62,13 +67,19 @@ namespace {
 // plane offsets (periodic, 32-bit: N < 2^31): a neighbour's index is one
 // three-operand add.
 struct Off3 {
-  int X0, X1, X2, Y0, Y1, Y2, Z0, Z1, Z2;
+  unsigned X0, X1, X2, Y0, Y1, Y2, Z0, Z1, Z2;  // in bytes
 };
 __device__ __forceinline__ Off3 make_off3(const Nbr& b, int x, int y, int z, int nx, int ny) {
-  const int nxy = nx * ny;
-  return {b.xm, x, b.xp, nx * b.ym, nx * y, nx * b.yp, nxy * b.zm, nxy * z, nxy * b.zp};
+  const unsigned sy = 4u * (unsigned)nx, sz = sy * (unsigned)ny;
+  return {4u * b.xm, 4u * x, 4u * b.xp, sy * b.ym, sy * y, sy * b.yp, sz * b.zm, sz * z, sz * b.zp};
 }
-__device__ __forceinline__ int nbr32(int d, const Off3& o) {
+// 4-byte element at an unsigned byte offset of a field (edges at most 1024: a
+// field of 4-byte values spans at most 2^32 bytes)
+template <class T>
+__device__ __forceinline__ T& at32(T* f, unsigned bytes) {
+  return *(T*)((char*)f + bytes);
+}
+__device__ __forceinline__ unsigned nbr32(int d, const Off3& o) {
   return (dcx(d) > 0 ? o.X2 : (dcx(d) < 0 ? o.X0 : o.X1)) +
          (dcy(d) > 0 ? o.Y2 : (dcy(d) < 0 ? o.Y0 : o.Y1)) +
          (dcz(d) > 0 ? o.Z2 : (dcz(d) < 0 ? o.Z0 : o.Z1));
@@ -101,7 +112,7 @@ __device__ __forceinline__ void block_sum3(float (&v)[3], double* ipart, long lo
 // ---------------------------------------------------------------------------
 // 2.5D-tiled S2 (FP32 form) with asynchronous staging.  A 32 x 8 thread block
 // owns a (32 x 8) column of consecutive planes (the grid's z dimension splits
-// each column into nzb segments of about 8 planes).  The stencil fields of the planes
+// each column into nzb segments of consecutive planes).  The stencil fields of the planes
 // z - 1, z, z + 1 -- species (raw int units), Psi, Phi and the node class --
 // sit in a 4-slot shared-memory ring with a one-node halo, and the
 // populations of plane z in one of two shared buffers.  While plane z is
@@ -109,20 +120,51 @@ __device__ __forceinline__ void block_sum3(float (&v)[3], double* ipart, long lo
 // populations in, so the global-memory latency of the loads overlaps the
 // arithmetic instead of stalling it; every value is read from global memory
 // once per block.
+//
+// What bounds it (512^3, 1000 spheres, K = 2): the memory accesses.  With the
+// flux and collision arithmetic left out the same loads and stores took 5.22
+// of 5.82 ms (27 GB: 5.2 TB/s); stores without the one-node shift in x would
+// take 0.4 ms less (the ten shifted populations write five sectors per warp
+// for four).  Two species, or two pairs of populations, share one packed
+// f32x2 instruction: 1254 -> 1034 warp instructions per node.  6.96 -> 5.79
+// ms at 512^3, 0.936 -> 0.800 at 256^3 (K = 3), 0.110 -> 0.098 at 128^3, of
+// which the longer segments (lb32_planes) gave 0.69, 0.07 and 0.005.  Three
+// blocks per SM (80 registers) were slower: 7.11 ms at 4-plane segments
+// against 6.52.
 // ---------------------------------------------------------------------------
 constexpr int HX = TILE_X + 2, HY = TILE_Y + 2;  // tile with halo
 constexpr int HP = HX * HY;                    // nodes of one halo plane
 constexpr int TN = TILE_X * TILE_Y;            // nodes of one tile plane
 constexpr int RING = 4;
 
+// One halo plane of the stencil fields: node class, Phi, Psi (as copied; 1 - Psi
+// once landed), then the species (int units as copied; rho qscale as float
+// bits once landed), two species of a node side by side so that one 8-byte
+// load feeds the packed arithmetic, an odd last species on its own.
+template <int K>
+struct LBPlane {
+  static constexpr int NP = K / 2, NS = K & 1;
+  int own[HP];
+  float phi[HP];
+  float psi[HP];
+  float rho[K > 0 ? K * HP : 2];
+  __device__ __forceinline__ float* spc(int k, int e) {
+    return k < 2 * NP ? rho + 2 * (k / 2) * HP + 2 * e + (k & 1) : rho + 2 * NP * HP + e;
+  }
+};
+
 template <int K>
 struct LBRing {
-  int own[RING][HP];
-  float phi[RING][HP];
-  float psi[RING][HP];                // Psi as copied; 1 - Psi once landed
-  int rho[K > 0 ? K : 1][RING][HP];   // int units as copied; rho qscale (float bits) once landed
+  LBPlane<K> pl[RING];
   float pop[2][Q][TN];
 };
+
+// two floats in one register pair: each half rounds as the scalar operation
+__device__ __forceinline__ float2 two(float v) { return make_float2(v, v); }
+__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, two(-1.0f), a); }
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
 
 __device__ __forceinline__ void cp_async4(void* smem, const void* gmem) {
   const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
@@ -174,11 +216,12 @@ __device__ __forceinline__ void stage_plane(LBRing<K>& t, int slot, int zz, cons
     if (hoff[q] < 0) continue;
     const int e = tid + q * TN;
     const size_t m = (size_t)hoff[q] + pz;
-    cp_async4(&t.own[slot][e], a.owner + m);
-    cp_async4(&t.phi[slot][e], (const float*)a.phi + m);
-    if (PV) cp_async4(&t.psi[slot][e], (const float*)a.psi + m);
+    LBPlane<K>& p = t.pl[slot];
+    cp_async4(&p.own[e], a.owner + m);
+    cp_async4(&p.phi[e], (const float*)a.phi + m);
+    if (PV) cp_async4(&p.psi[e], (const float*)a.psi + m);
 #pragma unroll
-    for (int k = 0; k < K; ++k) cp_async4(&t.rho[k][slot][e], (const int*)a.rho_in + k * N + m);
+    for (int k = 0; k < K; ++k) cp_async4(p.spc(k, e), (const int*)a.rho_in + k * N + m);
   }
 }
 
@@ -218,14 +261,102 @@ __device__ __forceinline__ void stage_pops(LBRing<K>& t, int buf, int z, int x0,
 template <int K>
 constexpr size_t lb32_smem() { return sizeof(LBRing<K>); }
 
+// The collision of one node on the deviations g (Eqs. 8-9), TRT in pair form.
+// With s, d the sum and difference of an opposite pair and Ep, Em the even and
+// odd equilibrium and force parts, the two results are A + B and A - B,
+//   A = (1 + lambda_e)/2 s + Ep,   B = (1 + lambda_o)/2 d + Em.
+// Ep is quadratic: with h = w (9/2 (2 + lambda_e) F - 9/2 lambda_e rho u) the
+// edges x + y and x - y share b + u_x h_x + u_y h_y and differ in the sign of
+// u_x h_y + u_y h_x; a face takes twice the edge weight 1/36.  Two pairs ride
+// in one packed operation: (x, y), (x+y, x-y), (x+z, x-z), (y+z, y-z).
+struct LBPairs {
+  float2 a13, b13, a79, b79, aAC, bAC, aEG, bEG;  // populations (1,3) (2,4) (7,9) (8,10) (11,13) (12,14) (15,17) (16,18)
+  float a5, b5, g0;
+};
+__device__ __forceinline__ void lb32_collide(LBPairs& p, const Phys32& c, float Fx, float Fy, float Fz,
+                                             float& ux, float& uy, float& uz, float& rho, float& usq) {
+  const float2 s13 = add2(p.a13, p.b13), s79 = add2(p.a79, p.b79);
+  const float2 sAC = add2(p.aAC, p.bAC), sEG = add2(p.aEG, p.bEG);
+  const float2 d13 = sub2(p.a13, p.b13), d79 = sub2(p.a79, p.b79);
+  const float2 dAC = sub2(p.aAC, p.bAC), dEG = sub2(p.aEG, p.bEG);
+  const float s5 = p.a5 + p.b5, d5 = p.a5 - p.b5;
+  const float2 st = add2(add2(s13, s79), add2(sAC, sEG));
+  const float drho = (p.g0 + s5) + (st.x + st.y);
+  const float jx = d13.x + ((d79.x + d79.y) + (dAC.x + dAC.y));
+  const float jy = d13.y + ((d79.x - d79.y) + (dEG.x + dEG.y));
+  const float jz = d5 + ((dAC.x - dAC.y) + (dEG.x - dEG.y));
+  rho = c.rho0 + drho;
+  const float irho = 1.0f / rho;
+  ux = fmaf(0.5f, Fx, jx) * irho;
+  uy = fmaf(0.5f, Fy, jy) * irho;
+  uz = fmaf(0.5f, Fz, jz) * irho;
+  usq = fmaf(uz, uz, fmaf(uy, uy, ux * ux));
+  const float uF = fmaf(uz, Fz, fmaf(uy, Fy, ux * Fx));
+  const float base = fmaf(-1.5f * (2.0f + c.lam_e), uF, -c.lam_e * fmaf(-1.5f * rho, usq, drho));
+  const float bw = base * (1.0f / 36.0f), kw = c.kw * rho;
+  const float hx = fmaf(kw, ux, c.gw * Fx), hy = fmaf(kw, uy, c.gw * Fy), hz = fmaf(kw, uz, c.gw * Fz);
+  const float qx = fmaf(c.lo12, jx, (1.0f / 12.0f) * Fx);
+  const float qy = fmaf(c.lo12, jy, (1.0f / 12.0f) * Fy);
+  const float qz = fmaf(c.lo12, jz, (1.0f / 12.0f) * Fz);
+  const float bx = fmaf(ux, hx, bw), by = fmaf(uy, hy, bw), bz = fmaf(uz, hz, bw);
+  const float bxy = fmaf(uy, hy, bx), bxz = fmaf(uz, hz, bx), byz = fmaf(uz, hz, by);
+  const float mxy = fmaf(ux, hy, uy * hx), mxz = fmaf(ux, hz, uz * hx), myz = fmaf(uy, hz, uz * hy);
+  const float2 hp = two(c.hp), hm = two(c.hm);
+  p.g0 = fmaf(1.0f + c.lam_e, p.g0, 12.0f * bw);
+  float2 A = fma2(hp, s13, make_float2(bx + bx, by + by));
+  float2 B = fma2(hm, d13, make_float2(qx + qx, qy + qy));
+  p.a13 = add2(A, B);
+  p.b13 = sub2(A, B);
+  A = fma2(hp, s79, make_float2(bxy + mxy, bxy - mxy));
+  B = fma2(hm, d79, make_float2(qx + qy, qx - qy));
+  p.a79 = add2(A, B);
+  p.b79 = sub2(A, B);
+  A = fma2(hp, sAC, make_float2(bxz + mxz, bxz - mxz));
+  B = fma2(hm, dAC, make_float2(qx + qz, qx - qz));
+  p.aAC = add2(A, B);
+  p.bAC = sub2(A, B);
+  A = fma2(hp, sEG, make_float2(byz + myz, byz - myz));
+  B = fma2(hm, dEG, make_float2(qy + qz, qy - qz));
+  p.aEG = add2(A, B);
+  p.bEG = sub2(A, B);
+  const float A5 = fmaf(c.hp, s5, bz + bz), B5 = fmaf(c.hm, d5, qz + qz);
+  p.a5 = A5 + B5;
+  p.b5 = A5 - B5;
+}
+// population i of the pairs (i a constant after unrolling)
+__device__ __forceinline__ float lb32_pop(const LBPairs& p, int i) {
+  switch (i) {
+    case 1: return p.a13.x;
+    case 2: return p.b13.x;
+    case 3: return p.a13.y;
+    case 4: return p.b13.y;
+    case 5: return p.a5;
+    case 6: return p.b5;
+    case 7: return p.a79.x;
+    case 8: return p.b79.x;
+    case 9: return p.a79.y;
+    case 10: return p.b79.y;
+    case 11: return p.aAC.x;
+    case 12: return p.bAC.x;
+    case 13: return p.aAC.y;
+    case 14: return p.bAC.y;
+    case 15: return p.aEG.x;
+    case 16: return p.bEG.x;
+    case 17: return p.aEG.y;
+    case 18: return p.bEG.y;
+    default: return p.g0;
+  }
+}
+
 // One node of plane z.  SIMPLE: the block's stencil planes hold fluid nodes
 // only and Psi = 0 (no particle or wall near), so every link is a fluid link,
 // the partial-volume factors are 1 and nothing bounces back; the arithmetic is
 // the same as in the general path with those values.
 template <int K, bool PV, bool SIMPLE>
-__device__ __forceinline__ void lb32_node(const LBRing<K>& t, const LBArgs& a, const Phys32& c,
+__device__ __forceinline__ void lb32_node(LBRing<K>& t, const LBArgs& a, const Phys32& c,
                                           int x, int y, int z, int tid, int ex, int ey,
                                           float (&iv)[3]) {
+  constexpr int NP = LBPlane<K>::NP, NS = LBPlane<K>::NS;
   float* __restrict__ g_out = (float*)a.f_out;
   const int* __restrict__ n_in = (const int*)a.rho_in;
   int* __restrict__ n_out = (int*)a.rho_out;
@@ -233,55 +364,76 @@ __device__ __forceinline__ void lb32_node(const LBRing<K>& t, const LBArgs& a, c
   float* __restrict__ ifield = (float*)a.ifield;
   const size_t N = (size_t)a.g.N;
   const int nx = a.g.nx, ny = a.g.ny, nz = a.g.nz;
-  const int sl[3] = {(z + 3) & 3, z & 3, (z + 1) & 3};  // planes z - 1, z, z + 1
   const int e0 = ex + HX * ey;
-  const int n = x + nx * (y + ny * z);
+  const LBPlane<K>* const pl[3] = {&t.pl[(z + 3) & 3], &t.pl[z & 3], &t.pl[(z + 1) & 3]};  // planes z - 1, z, z + 1
   const Nbr b = make_nbr(x, y, z, a.g);
   const Off3 nb = make_off3(b, x, y, z, nx, ny);
-  if (!SIMPLE && t.own[sl[1]][e0] != FLUID) {
-    a.vsig[n] = 0;
+  const unsigned n = nb.X1 + nb.Y1 + nb.Z1;
+  if (!SIMPLE && pl[1]->own[e0] != FLUID) {
+    a.vsig[n >> 2] = 0;
 #pragma unroll
-    for (int k = 0; k < K; ++k) (n_out + k * N)[n] = (n_in + k * N)[n];
-    u[n] = 0.0f;
-    (u + N)[n] = 0.0f;
-    (u + 2 * N)[n] = 0.0f;
-    ifield[n] = 0.0f;
-    (ifield + N)[n] = 0.0f;
-    (ifield + 2 * N)[n] = 0.0f;
+    for (int k = 0; k < K; ++k) at32(n_out + k * N, n) = at32(n_in + k * N, n);
+    at32(u, n) = 0.0f;
+    at32(u + N, n) = 0.0f;
+    at32(u + 2 * N, n) = 0.0f;
+    at32(ifield, n) = 0.0f;
+    at32(ifield + N, n) = 0.0f;
+    at32(ifield + 2 * N, n) = 0.0f;
   } else {
     unsigned fluid = SIMPLE ? 0xFFFFFFFEu : 0u;
     if (!SIMPLE) {
 #pragma unroll
       for (int d = 1; d < Q; ++d)
-        if (t.own[sl[1 + dcz(d)]][e0 + dcx(d) + HX * dcy(d)] == FLUID) fluid |= 1u << d;
+        if (pl[1 + dcz(d)]->own[e0 + dcx(d) + HX * dcy(d)] == FLUID) fluid |= 1u << d;
     }
     // ---- S2a: quantised link fluxes (symmetric operands) and coupling force ----
+    // per link and species: A = rho_x (1 - Psi_y), B = rho_y (1 - Psi_x),
+    // J = D/(A_0 |c|) [(A - B) + z/2 (A + B) dPhi] in units, two species per
+    // packed operation
     float gx = 0.0f, gy = 0.0f, gz = 0.0f;
     int S[K > 0 ? K : 1];
-    float r0[K > 0 ? K : 1];
-    const float om0 = PV ? t.psi[sl[1]][e0] : 1.0f;
-    const float phi0 = t.phi[sl[1]][e0];
+    int nk[K > 0 ? K : 1];
+    float2 r0p[NP > 0 ? NP : 1];
+    float r0s = 0.0f;
+    const float om0 = PV ? pl[1]->psi[e0] : 1.0f;
+    const float phi0 = pl[1]->phi[e0];
 #pragma unroll
     for (int k = 0; k < K; ++k) {
       S[k] = 0;
-      r0[k] = __int_as_float(t.rho[k][sl[1]][e0]);
+      nk[k] = at32(n_in + k * N, n);
     }
+#pragma unroll
+    for (int p = 0; p < NP; ++p) r0p[p] = reinterpret_cast<const float2*>(pl[1]->rho)[p * HP + e0];
+    if (NS) r0s = pl[1]->rho[2 * NP * HP + e0];
 #pragma unroll
     for (int d = 1; d < Q; ++d) {
       if (K == 0 || !(fluid & (1u << d))) continue;
-      const int sd = sl[1 + dcz(d)], ed = e0 + dcx(d) + HX * dcy(d);
-      const float omj = PV ? t.psi[sd][ed] : 1.0f;
-      const float dphi = __fadd_rn(__fsub_rn(phi0, t.phi[sd][ed]), c.ec[d]);
+      const LBPlane<K>& q = *pl[1 + dcz(d)];
+      const int ed = e0 + dcx(d) + HX * dcy(d);
+      const float omj = PV ? q.psi[ed] : 1.0f;
+      const float dphi = __fadd_rn(__fsub_rn(phi0, q.phi[ed]), c.ec[d]);
       float tsum = 0.0f;
 #pragma unroll
-      for (int k = 0; k < K; ++k) {
-        const float rb = __int_as_float(t.rho[k][sd][ed]);
-        const float A = PV ? __fmul_rn(r0[k], omj) : r0[k];
+      for (int p = 0; p < NP; ++p) {
+        const float2 rb = reinterpret_cast<const float2*>(q.rho)[p * HP + ed];
+        const float2 A = PV ? mul2(r0p[p], two(omj)) : r0p[p];
+        const float2 B = PV ? mul2(rb, two(om0)) : rb;
+        const float2 hd = mul2(make_float2(c.hz[2 * p], c.hz[2 * p + 1]), two(dphi));
+        float2 br = fma2(add2(A, B), hd, sub2(A, B));
+        if (d >= 7) br = mul2(br, two(0.70710678f));
+        const float2 fl = mul2(br, make_float2(c.cq[2 * p], c.cq[2 * p + 1]));
+        S[2 * p] += __float2int_rn(fl.x);
+        S[2 * p + 1] += __float2int_rn(fl.y);
+        tsum = p == 0 ? br.x + br.y : (tsum + br.x) + br.y;
+      }
+      if (NS) {
+        const float rb = q.rho[2 * NP * HP + ed];
+        const float A = PV ? __fmul_rn(r0s, omj) : r0s;
         const float B = PV ? __fmul_rn(rb, om0) : rb;
-        float br = fmaf(__fadd_rn(A, B), __fmul_rn(c.hz[k], dphi), __fsub_rn(A, B));
+        float br = __fmaf_rn(__fadd_rn(A, B), __fmul_rn(c.hz[K - 1], dphi), __fsub_rn(A, B));
         if (d >= 7) br = __fmul_rn(br, 0.70710678f);
-        S[k] += __float2int_rn(__fmul_rn(br, c.cq[k]));
-        tsum += br;
+        S[K - 1] += __float2int_rn(__fmul_rn(br, c.cq[K - 1]));
+        tsum = NP == 0 ? br : tsum + br;
       }
       if (dcx(d)) gx += csgnf(dcx(d), tsum);
       if (dcy(d)) gy += csgnf(dcy(d), tsum);
@@ -290,95 +442,69 @@ __device__ __forceinline__ void lb32_node(const LBRing<K>& t, const LBArgs& a, c
     float qion = 0.0f;
 #pragma unroll
     for (int k = 0; k < K; ++k) {
-      const int nk = (n_in + k * N)[n];
-      (n_out + k * N)[n] = nk - S[k];
-      qion = fmaf(c.zq[k], (float)nk, qion);
+      at32(n_out + k * N, n) = nk[k] - S[k];
+      qion = fmaf(c.zq[k], (float)nk[k], qion);
     }
     constexpr float HALF_INV_A0 = 0.13060193748187072f;
     {
       const float ix = gx * HALF_INV_A0 - qion * c.E[0];
       const float iy = gy * HALF_INV_A0 - qion * c.E[1];
       const float iz = gz * HALF_INV_A0 - qion * c.E[2];
-      ifield[n] = ix;
-      (ifield + N)[n] = iy;
-      (ifield + 2 * N)[n] = iz;
+      at32(ifield, n) = ix;
+      at32(ifield + N, n) = iy;
+      at32(ifield + 2 * N, n) = iz;
       iv[0] += ix;
       iv[1] += iy;
       iv[2] += iz;
     }
-    // ---- S2b: TRT collision on the deviations (pair form) ----
-    float g[Q];
-#pragma unroll
-    for (int i = 0; i < Q; ++i) g[i] = t.pop[z & 1][i][tid];
-    float drho = g[0], jx = 0.0f, jy = 0.0f, jz = 0.0f;
-#pragma unroll
-    for (int i = 1; i < Q; i += 2) {
-      const float pd = g[i] - g[i + 1];
-      drho += g[i] + g[i + 1];
-      if (dcx(i)) jx += csgnf(dcx(i), pd);
-      if (dcy(i)) jy += csgnf(dcy(i), pd);
-      if (dcz(i)) jz += csgnf(dcz(i), pd);
-    }
-    const float rho = c.rho0 + drho;
-    const float Fx = fmaf(gx, HALF_INV_A0, c.g[0]);
-    const float Fy = fmaf(gy, HALF_INV_A0, c.g[1]);
-    const float Fz = fmaf(gz, HALF_INV_A0, c.g[2]);
-    const float irho = 1.0f / rho;
-    const float ux = (jx + 0.5f * Fx) * irho;
-    const float uy = (jy + 0.5f * Fy) * irho;
-    const float uz = (jz + 0.5f * Fz) * irho;
-    const float usq = ux * ux + uy * uy + uz * uz;
-    const float uF = ux * Fx + uy * Fy + uz * Fz;
-    const float le = c.lam_e, lo = c.lam_o;
-    const float gg = 2.0f + le;
-    const float qx = fmaf(-lo, jx, Fx), qy = fmaf(-lo, jy, Fy), qz = fmaf(-lo, jz, Fz);
-    const float base = fmaf(-1.5f * gg, uF, -le * fmaf(-1.5f * rho, usq, drho));
-    const float hle = 0.5f * le, hlo = 0.5f * lo;
-    const float k45 = -4.5f * le * rho;
+    // ---- S2b: collision and push stream (velocity bounce-back, Eq. 12) ----
+    const float* const gp = &t.pop[z & 1][0][tid];
+    LBPairs g;
+    g.g0 = gp[0];
+    g.a13 = make_float2(gp[1 * TN], gp[3 * TN]);
+    g.b13 = make_float2(gp[2 * TN], gp[4 * TN]);
+    g.a5 = gp[5 * TN];
+    g.b5 = gp[6 * TN];
+    g.a79 = make_float2(gp[7 * TN], gp[9 * TN]);
+    g.b79 = make_float2(gp[8 * TN], gp[10 * TN]);
+    g.aAC = make_float2(gp[11 * TN], gp[13 * TN]);
+    g.bAC = make_float2(gp[12 * TN], gp[14 * TN]);
+    g.aEG = make_float2(gp[15 * TN], gp[17 * TN]);
+    g.bEG = make_float2(gp[16 * TN], gp[18 * TN]);
+    float ux, uy, uz, rho, usq;
+    lb32_collide(g, c, fmaf(gx, HALF_INV_A0, c.g[0]), fmaf(gy, HALF_INV_A0, c.g[1]),
+                 fmaf(gz, HALF_INV_A0, c.g[2]), ux, uy, uz, rho, usq);
     if (!isfinite(rho) || !isfinite(usq)) atomicOr(a.status, ST_NONFINITE);
-    u[n] = ux;
-    (u + N)[n] = uy;
-    (u + 2 * N)[n] = uz;
-    a.vsig[n] = (unsigned char)(0x80u | sign_code(ux) | (sign_code(uy) << 2) | (sign_code(uz) << 4));
-    // ---- collide each pair and push-stream it (velocity bounce-back, Eq. 12) ----
-    g_out[n] = fmaf(1.0f + le, g[0], (float)wgt(0) * base);
+    at32(u, n) = ux;
+    at32(u + N, n) = uy;
+    at32(u + 2 * N, n) = uz;
+    a.vsig[n >> 2] = (unsigned char)(0x80u | sign_code(ux) | (sign_code(uy) << 2) | (sign_code(uz) << 4));
+    at32(g_out, n) = g.g0;
 #pragma unroll
-    for (int i = 1; i < Q; i += 2) {
-      const float w = (float)wgt(i);
-      const float cu = cdotf(i, ux, uy, uz);
-      const float cf = cdotf(i, Fx, Fy, Fz);
-      const float cqv = cdotf(i, qx, qy, qz);
-      const float Ep = w * fmaf(cu, fmaf(4.5f * gg, cf, k45 * cu), base);
-      const float Em = 3.0f * w * cqv;
-      const float X = fmaf(hle, g[i] + g[i + 1], Ep);
-      const float Y = fmaf(hlo, g[i] - g[i + 1], Em);
-      const float gsd[2] = {g[i] + (X + Y), g[i + 1] + (X - Y)};
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const int d = i + h;
-        if (fluid & (1u << d)) {
-          (g_out + d * N)[nbr32(d, nb)] = gsd[h];
-        } else {
-          float cvb = 0.0f;
-          const int om = t.own[sl[1 + dcz(d)]][e0 + dcx(d) + HX * dcy(d)];
-          if (om >= 0) {
-            const DevParticle& P = a.parts[om];
-            const int xb = dcx(d) > 0 ? b.xp : (dcx(d) < 0 ? b.xm : x);
-            const int yb = dcy(d) > 0 ? b.yp : (dcy(d) < 0 ? b.ym : y);
-            const int zb = dcz(d) > 0 ? b.zp : (dcz(d) < 0 ? b.zm : z);
-            // wall velocity at the boundary node in float (it enters the
-            // float population): the offset from the centre as integer part
-            // minus the centre's fraction, the velocities as float copies
-            const float dx = __fsub_rn((float)(P.lo[0] + wrapi(xb - P.lo[0], nx) - P.ipos[0]), P.fpos[0]);
-            const float dy = __fsub_rn((float)(P.lo[1] + wrapi(yb - P.lo[1], ny) - P.ipos[1]), P.fpos[1]);
-            const float dz = __fsub_rn((float)(P.lo[2] + wrapi(zb - P.lo[2], nz) - P.ipos[2]), P.fpos[2]);
-            const float vx = P.velf[0] + (P.omegaf[1] * dz - P.omegaf[2] * dy);
-            const float vy = P.velf[1] + (P.omegaf[2] * dx - P.omegaf[0] * dz);
-            const float vz = P.velf[2] + (P.omegaf[0] * dy - P.omegaf[1] * dx);
-            cvb = cdotf(d, vx, vy, vz);
-          }
-          (g_out + opp(d) * N)[n] = gsd[h] - 6.0f * (float)wgt(d) * c.rho0 * cvb;
+    for (int d = 1; d < Q; ++d) {
+      const float gs = lb32_pop(g, d);
+      if (fluid & (1u << d)) {
+        at32(g_out + d * N, nbr32(d, nb)) = gs;
+      } else {
+        float cvb = 0.0f;
+        const int om = pl[1 + dcz(d)]->own[e0 + dcx(d) + HX * dcy(d)];
+        if (om >= 0) {
+          const DevParticle& P = a.parts[om];
+          const int xb = dcx(d) > 0 ? b.xp : (dcx(d) < 0 ? b.xm : x);
+          const int yb = dcy(d) > 0 ? b.yp : (dcy(d) < 0 ? b.ym : y);
+          const int zb = dcz(d) > 0 ? b.zp : (dcz(d) < 0 ? b.zm : z);
+          // wall velocity at the boundary node in float (it enters the
+          // float population): the offset from the centre as integer part
+          // minus the centre's fraction, the velocities as float copies
+          const float dx = __fsub_rn((float)(P.lo[0] + wrapi(xb - P.lo[0], nx) - P.ipos[0]), P.fpos[0]);
+          const float dy = __fsub_rn((float)(P.lo[1] + wrapi(yb - P.lo[1], ny) - P.ipos[1]), P.fpos[1]);
+          const float dz = __fsub_rn((float)(P.lo[2] + wrapi(zb - P.lo[2], nz) - P.ipos[2]), P.fpos[2]);
+          const float vx = P.velf[0] + (P.omegaf[1] * dz - P.omegaf[2] * dy);
+          const float vy = P.velf[1] + (P.omegaf[2] * dx - P.omegaf[0] * dz);
+          const float vz = P.velf[2] + (P.omegaf[0] * dy - P.omegaf[1] * dx);
+          cvb = cdotf(d, vx, vy, vz);
         }
+        at32(g_out + opp(d) * N, n) = gs - 6.0f * (float)wgt(d) * c.rho0 * cvb;
       }
     }
   }
@@ -415,12 +541,12 @@ __device__ __forceinline__ void lb32_block(const LBArgs& a, const Phys32& c, int
   // (complete after its own wait); the barrier that follows publishes them.
   auto plane_flag = [&](int slot) -> int {
     bool f = false;
+    LBPlane<K>& p = t.pl[slot];
     for (int e = tid; e < HP; e += TN) {
-      f |= t.own[slot][e] != FLUID || (PV && t.psi[slot][e] != 0.0f);
-      if (PV) t.psi[slot][e] = __fsub_rn(1.0f, t.psi[slot][e]);
+      f |= p.own[e] != FLUID || (PV && p.psi[e] != 0.0f);
+      if (PV) p.psi[e] = __fsub_rn(1.0f, p.psi[e]);
 #pragma unroll
-      for (int k = 0; k < K; ++k)
-        t.rho[k][slot][e] = __float_as_int(__fmul_rn((float)t.rho[k][slot][e], c.qs[k]));
+      for (int k = 0; k < K; ++k) *p.spc(k, e) = __fmul_rn((float)__float_as_int(*p.spc(k, e)), c.qs[k]);
     }
     return f ? 1 : 0;
   };
@@ -833,16 +959,21 @@ cudaError_t lb32_prepare() {
   return e;
 }
 
-// Segments per tile column: about 4 planes each, with two blocks of 256
-// threads per SM (up to 128 registers, no spills).  Measured on GB300 at 128^3
-// (ms per launch): 4-plane segments 0.123, 3 planes 0.127, 2 planes 0.136,
-// 1 plane 0.173; with three blocks per SM (80 registers, spills) 8-plane
-// segments 0.185 and 16-plane 0.200.  Short segments let the block scheduler
-// balance the SMs; one-plane segments pay three halo planes per plane.
-int lb32_segments(const Grid& g, int K, bool pv) {
-  (void)K;
-  (void)pv;
-  return std::max(1, (g.nz + 3) / 4);
+// Planes per segment of S2 for `cols` tile columns of nz planes.  A segment
+// stages the plane on each side of it as well and starts with an empty
+// pipeline, so long segments waste less; short ones give the block scheduler
+// enough blocks (two resident per SM) to even out the SMs.  Measured on GB300
+// (ms per launch at 4 / 8 / 16 / 32 planes): 128^3 0.103, 0.098, 0.102,
+// 0.129; 256^3 (K = 3) 0.872, 0.816, 0.800, 0.830; 512^3 6.48, 6.01, 5.79,
+// 5.81.
+int lb32_planes(long long cols, int nz) {
+  auto blocks = [&](int p) { return cols * ((nz + p - 1) / p); };
+  return blocks(16) >= 4096 ? 16 : (blocks(8) >= 1024 ? 8 : 4);
+}
+int lb32_segments(const Grid& g) {
+  const long long cols = (long long)((g.nx + TILE_X - 1) / TILE_X) * ((g.ny + TILE_Y - 1) / TILE_Y);
+  const int planes = lb32_planes(cols, g.nz);
+  return std::max(1, (g.nz + planes - 1) / planes);
 }
 
 cudaError_t launch_lb32(const LBArgs& a, cudaStream_t s) {
