@@ -56,7 +56,7 @@ struct ek_ctx {
   double* ipart = nullptr;             // 3 doubles per lattice block: its sums
   int nipart = 0;
   int nipart_cap = 0;  // rows allocated for ipart (FP32: enough for 2-plane segments)
-  int nzb = 1;       // FP32 S2: z segments per tile column
+  int nzb = 1;       // S2: z segments per tile column
   int advseg = 1;    // FP32 S3: z segments per tile column
   int overlap = 1;   // particle chain on the auxiliary stream (1) or in line (0)
   unsigned long long version = 0;  // bumped whenever captured steps go stale
@@ -729,7 +729,7 @@ ek_status ek_create(const ek_params* p, ek_ctx** out) {
   }
   const size_t N = (size_t)g.N;
   const int K = std::max(p->nspecies, 1);
-  if (ctx->fp32 && lb32_prepare() != cudaSuccess) {
+  if ((ctx->fp32 ? lb32_prepare() : lb64_prepare()) != cudaSuccess) {
     delete ctx;
     return EK_ERR_CUDA;
   }
@@ -752,9 +752,9 @@ ek_status ek_create(const ek_params* p, ek_ctx** out) {
   alloc(&ctx->ifield, 3 * N * rsz);
   {
     // lattice-block partial sums of S2: one per block of its grid
-    if (ctx->fp32) ctx->nzb = lb32_segments(g);
+    ctx->nzb = ctx->fp32 ? lb32_segments(g) : lb64_segments(g);
     if (ctx->fp32) ctx->advseg = adv32_segments(g, false);
-    const dim3 lg = ctx->fp32 ? lattice_grid32(g, ctx->nzb) : lattice_grid(g);
+    const dim3 lg = lattice_grid32(g, ctx->nzb);
     ctx->nipart = (int)(lg.x * lg.y * lg.z);
     // the FP32 segment length may be retuned down to 2 planes (ek_batch_tune)
     ctx->nipart_cap = ctx->fp32 ? (int)(lg.x * lg.y) * std::max(1, (g.nz + 1) / 2) : ctx->nipart;

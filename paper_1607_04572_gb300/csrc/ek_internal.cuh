@@ -171,8 +171,8 @@ inline dim3 lattice_grid(const Grid& g) {
               (unsigned)g.nz);
 }
 inline dim3 lattice_block() { return dim3(TILE_X, TILE_Y, 1); }
-// the FP32 form's S2 kernel marches each (x, y) tile column through nzb
-// segments of consecutive planes
+// the S2 kernels march each (x, y) tile column through nzb segments of
+// consecutive planes
 inline dim3 lattice_grid32(const Grid& g, int nzb) {
   return dim3((unsigned)((g.nx + TILE_X - 1) / TILE_X), (unsigned)((g.ny + TILE_Y - 1) / TILE_Y),
               (unsigned)nzb);
@@ -314,7 +314,7 @@ struct LBArgs {
   double* ipart;   // per-block sums of ifield (3 per block of the lattice grid)
   const DevParticle* parts;
   int* status;
-  int nzb;         // FP32 S2: z segments per (x, y) tile column (lb32_segments)
+  int nzb;         // S2: z segments per (x, y) tile column (lb32_segments, lb64_segments)
   int advseg;      // FP32 S3: z segments per tile column (adv32_segments)
 };
 // Constants of the FP32 kernels, rounded once on the host.
@@ -338,6 +338,8 @@ struct LBBatchEntry {
   Phys32 c;
 };
 cudaError_t launch_lb_fused(const LBArgs& a, cudaStream_t s);
+cudaError_t lb64_prepare();           // before the first launch_lb_fused
+int lb64_segments(const Grid& g);     // z segments per tile column of the FP64 S2 grid
 cudaError_t launch_advection(const LBArgs& a, cudaStream_t s);
 // FP32-storage form
 cudaError_t lb32_prepare();  // once per process, before the first launch_lb32
