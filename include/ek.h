@@ -280,11 +280,12 @@ ek_status ek_poisson_solve_mg(const double* q, double* phi, int nx, int ny, int 
  * mean 0 (then with eps = 1 the result is ek_poisson_solve's).  Method:
  * preconditioned conjugate gradients in FP64 from Phi = 0 on the free nodes,
  * until ||r||_2 <= tol ||b||_2 over the free nodes or max_iter iterations.
- * The preconditioner is one multigrid V-cycle of the same operator (levels
- * halved while every edge is even and stays >= 4, coarse face permittivity
- * the halved sum of the 4 fine faces it covers, damped Jacobi smoothing,
- * the coarsest level of at most 8192 nodes by 40 sweeps) when the box has
- * at least two levels, else the diagonal (Jacobi); the residual is checked
+ * The preconditioner is one multigrid V-cycle of the same operator (edges of
+ * 8 or more halved per level, an odd one rounded up; coarse face permittivity
+ * the fine faces it covers, summed, over the halving along its axis; two
+ * red-black Gauss-Seidel sweeps before and after, damped Jacobi ones on levels
+ * with an odd edge; a few Jacobi sweeps on the coarsest level) when an edge can
+ * be halved, else the diagonal (Jacobi); the residual is checked
  * every 2 (multigrid) or 10 (Jacobi) iterations.  Every inner product is a
  * fixed-order sum, so a solve is bit-reproducible.
  *

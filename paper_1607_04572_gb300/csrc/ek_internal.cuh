@@ -275,7 +275,7 @@ cudaError_t poisson_solve_f32(const PoissonPlan& p, const int* rho, const float*
 cudaError_t charge_density(const Grid& g, const Phys& ph, const void* rho, const void* qwall,
                            const void* qpart, double* q, cudaStream_t s);
 // Poisson solve with an inhomogeneous permittivity and fixed-potential nodes
-// by Jacobi-preconditioned conjugate gradients (ek_krylov.cu); *bad_eps is set
+// by multigrid-preconditioned conjugate gradients (ek_krylov.cu); *bad_eps is set
 // (and nothing solved) when a permittivity is not positive and finite
 size_t poisson_cg_scratch_bytes(int nx, int ny, int nz);
 cudaError_t poisson_solve_cg(const double* q, const double* eps, const unsigned char* fixed,

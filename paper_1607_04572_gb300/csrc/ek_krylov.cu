@@ -15,28 +15,47 @@
 //
 // Every reduction (the CG inner products) is a fixed-order sum: each thread
 // of a fixed grid adds its grid-stride elements in order, the block adds its
-// threads in a fixed tree, one block adds the block sums in order; so a solve
-// is bit-reproducible.  The scalars alpha and beta stay on the device; the
-// host reads the residual every CG_CHECK (Jacobi) or PCG_CHECK (multigrid)
-// iterations.
+// threads in a fixed tree, and the last block to finish adds the block sums in
+// order and forms the scalar that needs them; so a solve is bit-reproducible.
+// The scalars alpha and beta stay on the device; the host reads the residual
+// every CG_CHECK (Jacobi) or PCG_CHECK (multigrid) iterations.
+//
+// What bounds it: the FP64 pipe (2 lanes per clock per SM) on the fine level,
+// launches on the coarse ones.  So the smoother gathers (b + sum c_f x_f) / D
+// with the stored diagonal D (7 FP64 instructions a node; differences
+// c_f (x - x_f) take 13), residuals are formed only where they are not zero,
+// and corrections are added only where they are read.  The outer operator keeps
+// the differences: its rounding is the solution's.  128^3, dielectric sphere
+// between electrodes, tol 1e-12 (GB300): 32 iterations of 0.60 ms (18.9 ms)
+// with damped Jacobi V(2,2) cycles and a launch per scalar, 18 of 0.41 ms (7.3
+// ms) with red-black Gauss-Seidel.  Of an iteration at 128^3 (launches one by
+// one, cold L2) the fine level's half sweeps take 0.138 ms, the operator 0.065
+// (FP64 pipe 43 us), the small levels 0.074, 64^3 0.054, the update 0.033,
+// the restriction 0.029.
 #include <math.h>
 
 #include <algorithm>
+
+#include <cooperative_groups.h>
 
 #include "ek_internal.cuh"
 
 namespace ek {
 
+namespace cg = cooperative_groups;
+
 namespace {
 
 constexpr int CG_T = 256;         // threads per block
-constexpr int CG_BLOCKS = 1216;   // blocks of the grid-stride kernels (8 per SM)
+constexpr int CG_BLOCKS = 608;    // blocks of the grid-stride kernels (4 per SM: a block's FP64 sum is
+                                  // spread over more nodes than with 8)
 constexpr int CG_CHECK = 10;      // iterations between residual reads (Jacobi)
 constexpr int PCG_CHECK = 2;      // with the multigrid V-cycle (an iteration costs several)
 
 // scalars on the device: [0] r.z, [1] p.Ap, [2] alpha, [3] beta, [4] r.r,
 // [5] b.b (then sum x), [6] sum q, [7] fixed-node count, [8] permittivities
-// that are not positive and finite, [9] sum of D^-1, [10] mean of r to remove
+// that are not positive and finite, [9] sum of D^-1, [10] mean of r to remove,
+// [12] the counter of finished blocks
 //
 // Without fixed nodes the operator is singular (constants): b has mean 0, and
 // so has r = b - A x in exact arithmetic, but rounding lets a constant
@@ -51,7 +70,7 @@ struct CGView {
   double* p;        // N: search direction
   double* ap;       // N: A p
   double* part;     // 4 * CG_BLOCKS block sums
-  double* sc;       // 12 scalars
+  double* sc;       // 16 scalars
 };
 
 size_t cg_layout(long long N, CGView* v, void* base) {
@@ -68,7 +87,7 @@ size_t cg_layout(long long N, CGView* v, void* base) {
   take(v ? &v->p : &dummy, (size_t)N);
   take(v ? &v->ap : &dummy, (size_t)N);
   take(v ? &v->part : &dummy, 4 * CG_BLOCKS);
-  take(v ? &v->sc : &dummy, 12);
+  take(v ? &v->sc : &dummy, 16);
   return off;
 }
 
@@ -77,7 +96,12 @@ struct Box {
   long long N;
 };
 
-__device__ __forceinline__ double harmonic(double a, double b) { return 2.0 * a * b / (a + b); }
+// harmonic mean; equal values (most faces of a piecewise constant medium) need
+// no division, which costs some 20 FP64 instructions
+__device__ __forceinline__ double harmonic(double a, double b) { return a == b ? a : 2.0 * a * b / (a + b); }
+
+// v is zero (a fixed node's D^-1), from its bits: no FP64 instruction
+__device__ __forceinline__ bool is_zero(double v) { return (__double_as_longlong(v) << 1) == 0; }
 
 // the block's sum of v (every thread), in a fixed tree; valid in thread 0
 __device__ __forceinline__ double block_total(double v) {
@@ -102,68 +126,100 @@ __device__ __forceinline__ double row_total(const double* part, int row, int nb)
   return block_total(t);
 }
 
-// sum of q, the number of fixed nodes and of permittivities that are not
-// positive and finite (block sums)
-__global__ void __launch_bounds__(CG_T) k_cg_stats(Box b, const double* q, const double* eps,
-                                                   const unsigned char* fixed, double* part) {
-  double sq = 0.0, nf = 0.0, ne = 0.0;
-  for (long long n = blockIdx.x * (long long)CG_T + threadIdx.x; n < b.N; n += (long long)gridDim.x * CG_T) {
+// true in every thread of the last block of the grid to get here, with the
+// other blocks' partial sums visible; the counter is left at zero
+__device__ __forceinline__ bool last_block(const CGView& v) {
+  __shared__ bool last;
+  if (threadIdx.x == 0) {
+    __threadfence();
+    unsigned* count = reinterpret_cast<unsigned*>(v.sc + 12);
+    const unsigned done = atomicAdd(count, 1u);
+    last = done == gridDim.x - 1;
+    if (last) {
+      *count = 0u;
+      __threadfence();
+    }
+  }
+  __syncthreads();
+  return last;
+}
+
+// the neighbours of node n = (x, y, z) across its +x, -x, +y, -y, +z, -z faces
+__device__ __forceinline__ void neighbours(int nx, int ny, int nz, int n, int x, int y, int z, int (&m)[6]) {
+  const int sy = nx, sz = nx * ny;
+  m[0] = n + (x + 1 < nx ? 1 : 1 - nx);
+  m[1] = n + (x > 0 ? -1 : nx - 1);
+  m[2] = n + (y + 1 < ny ? sy : sy - sz);
+  m[3] = n + (y > 0 ? -sy : sz - sy);
+  m[4] = n + (z + 1 < nz ? sz : sz - sz * nz);
+  m[5] = n + (z > 0 ? -sz : sz * nz - sz);
+}
+__device__ __forceinline__ void node_xyz(int nx, int ny, int n, int& x, int& y, int& z) {
+  const unsigned row = (unsigned)n / (unsigned)nx;
+  x = n - (int)row * nx;
+  z = (int)(row / (unsigned)ny);
+  y = (int)row - z * ny;
+}
+
+// face permittivities; the sum of q, the number of fixed nodes and of
+// permittivities that are not positive and finite
+__global__ void __launch_bounds__(CG_T) k_cg_faces(Box b, CGView v, const double* q, const double* eps,
+                                                   const unsigned char* fixed) {
+  double sq = 0.0;
+  int nf = 0, ne = 0;
+  for (long long i = blockIdx.x * (long long)CG_T + threadIdx.x; i < b.N; i += (long long)gridDim.x * CG_T) {
+    const int n = (int)i;
     sq += q[n];
-    if (fixed && fixed[n]) nf += 1.0;
-    if (eps && !(eps[n] > 0.0 && eps[n] < INFINITY)) ne += 1.0;
+    if (fixed && fixed[n]) ++nf;
+    double c0 = 1.0, c1 = 1.0, c2 = 1.0;
+    if (eps) {
+      int x, y, z, m[6];
+      node_xyz(b.nx, b.ny, n, x, y, z);
+      neighbours(b.nx, b.ny, b.nz, n, x, y, z, m);
+      const double e = eps[n];
+      if (!(e > 0.0 && e < INFINITY)) ++ne;
+      c0 = harmonic(e, eps[m[0]]);
+      c1 = harmonic(e, eps[m[2]]);
+      c2 = harmonic(e, eps[m[4]]);
+    }
+    v.cf[n] = c0;
+    v.cf[b.N + n] = c1;
+    v.cf[2 * b.N + n] = c2;
   }
   sq = block_total(sq);
-  nf = block_total(nf);
-  ne = block_total(ne);
+  const double df = block_total((double)nf), de = block_total((double)ne);
   if (threadIdx.x == 0) {
-    part[blockIdx.x] = sq;
-    part[CG_BLOCKS + blockIdx.x] = nf;
-    part[2 * CG_BLOCKS + blockIdx.x] = ne;
+    v.part[blockIdx.x] = sq;
+    v.part[CG_BLOCKS + blockIdx.x] = df;
+    v.part[2 * CG_BLOCKS + blockIdx.x] = de;
+  }
+  if (!last_block(v)) return;
+  const double a = row_total(v.part, 0, gridDim.x), c = row_total(v.part, 1, gridDim.x),
+               d = row_total(v.part, 2, gridDim.x);
+  if (threadIdx.x == 0) {
+    v.sc[6] = a;
+    v.sc[7] = c;
+    v.sc[8] = d;
   }
 }
 
-// the block sums of part's rows 0, 1, 2 (CG_BLOCKS apart), each added in
-// order, into sc[i0], sc[i1], sc[i2] (a negative index: that row is skipped)
-__global__ void __launch_bounds__(CG_T) k_cg_total(const double* part, int nb, double* sc, int i0, int i1,
-                                                   int i2) {
-  const double a = row_total(part, 0, nb);
-  const double c = i1 >= 0 ? row_total(part, 1, nb) : 0.0;
-  const double d = i2 >= 0 ? row_total(part, 2, nb) : 0.0;
-  if (threadIdx.x == 0) {
-    sc[i0] = a;
-    if (i1 >= 0) sc[i1] = c;
-    if (i2 >= 0) sc[i2] = d;
-  }
-}
-
-__device__ __forceinline__ void neighbours(const Box& b, long long n, long long (&m)[6]) {
-  const int x = (int)(n % b.nx), y = (int)((n / b.nx) % b.ny), z = (int)(n / ((long long)b.nx * b.ny));
-  const long long sy = b.nx, sz = (long long)b.nx * b.ny;
-  m[0] = n + (x + 1 < b.nx ? 1 : 1 - b.nx);   // +x
-  m[1] = n + (x > 0 ? -1 : b.nx - 1);         // -x
-  m[2] = n + (y + 1 < b.ny ? sy : sy - sz);   // +y
-  m[3] = n + (y > 0 ? -sy : sz - sy);         // -y
-  m[4] = n + (z + 1 < b.nz ? sz : sz - b.N);  // +z
-  m[5] = n + (z > 0 ? -sz : b.N - sz);        // -z
-}
-
-// faces, diagonal, right-hand side and the start x = 0 (free) / phi_fixed
-// (fixed); r = b, p = z = D^-1 r; block sums of r.z and b.b
-__global__ void __launch_bounds__(CG_T) k_cg_prep(Box b, CGView v, const double* q, const double* eps,
+// diagonal, right-hand side and the start x = 0 (free) / phi_fixed (fixed);
+// r = b, p = D^-1 r (Jacobi); r.p, b.b and the sum of D^-1.  Without fixed
+// nodes the mean charge is removed.
+__global__ void __launch_bounds__(CG_T) k_cg_prep(Box b, CGView v, double* D, const double* q,
                                                   const unsigned char* fixed, const double* phi_fixed,
-                                                  double* x, double scale, const double* sc, int neutral) {
-  const double qmean = neutral ? sc[6] / (double)b.N : 0.0;
+                                                  double* x, double scale) {
+  const double qmean = v.sc[7] == 0.0 ? v.sc[6] / (double)b.N : 0.0;
   double rz = 0.0, bb = 0.0, sd = 0.0;
-  for (long long n = blockIdx.x * (long long)CG_T + threadIdx.x; n < b.N; n += (long long)gridDim.x * CG_T) {
-    long long m[6];
-    neighbours(b, n, m);
-    const double en = eps ? eps[n] : 1.0;
-    double f[6];
-#pragma unroll
-    for (int k = 0; k < 6; ++k) f[k] = eps ? harmonic(en, eps[m[k]]) : 1.0;
-    v.cf[n] = f[0];
-    v.cf[b.N + n] = f[2];
-    v.cf[2 * b.N + n] = f[4];
+  for (long long i = blockIdx.x * (long long)CG_T + threadIdx.x; i < b.N; i += (long long)gridDim.x * CG_T) {
+    const int n = (int)i;
+    int xx, yy, zz, m[6];
+    node_xyz(b.nx, b.ny, n, xx, yy, zz);
+    neighbours(b.nx, b.ny, b.nz, n, xx, yy, zz, m);
+    const double f[6] = {v.cf[n],           v.cf[m[1]],           v.cf[b.N + n],
+                         v.cf[b.N + m[3]], v.cf[2 * b.N + n], v.cf[2 * b.N + m[5]]};
+    const double d = ((f[0] + f[1]) + (f[2] + f[3])) + (f[4] + f[5]);
+    D[n] = d;
     const bool fx = fixed && fixed[n];
     if (fx) {
       const double pv = phi_fixed ? phi_fixed[n] : 0.0;
@@ -174,11 +230,10 @@ __global__ void __launch_bounds__(CG_T) k_cg_prep(Box b, CGView v, const double*
       continue;
     }
     double rhs = scale * (q[n] - qmean);
-    double d = 0.0;
+    if (fixed) {
 #pragma unroll
-    for (int k = 0; k < 6; ++k) {
-      d += f[k];
-      if (fixed && fixed[m[k]]) rhs += f[k] * (phi_fixed ? phi_fixed[m[k]] : 0.0);
+      for (int k = 0; k < 6; ++k)
+        if (fixed[m[k]]) rhs += f[k] * (phi_fixed ? phi_fixed[m[k]] : 0.0);
     }
     const double di = 1.0 / d;
     x[n] = 0.0;
@@ -197,9 +252,17 @@ __global__ void __launch_bounds__(CG_T) k_cg_prep(Box b, CGView v, const double*
     v.part[CG_BLOCKS + blockIdx.x] = bb;
     v.part[2 * CG_BLOCKS + blockIdx.x] = sd;
   }
+  if (!last_block(v)) return;
+  const double a = row_total(v.part, 0, gridDim.x), c = row_total(v.part, 1, gridDim.x),
+               e = row_total(v.part, 2, gridDim.x);
+  if (threadIdx.x == 0) {
+    v.sc[0] = a;
+    v.sc[5] = c;
+    v.sc[9] = e;
+  }
 }
 
-// Ap on the free nodes (p is 0 on fixed nodes); block sums of p.Ap.  The
+// Ap on the free nodes (p is 0 on fixed nodes); alpha = r.z / p.Ap.  The
 // work items are the 32 x 8 tiles of every plane (tx x ty tiles per plane);
 // block b takes items b, b + gridDim.x, ...: node coordinates come from the
 // item, with no division per node.
@@ -215,7 +278,7 @@ __global__ void __launch_bounds__(CG_T) k_cg_apply(Box b, CGView v, int tx, int 
     const int x = bx * 32 + (threadIdx.x & 31), y = by * 8 + (threadIdx.x >> 5);
     if (x >= b.nx || y >= b.ny) continue;
     const int n = x + sy * y + sz * z;
-    if (v.dinv[n] == 0.0) {
+    if (is_zero(v.dinv[n])) {
       v.ap[n] = 0.0;
       continue;
     }
@@ -231,32 +294,32 @@ __global__ void __launch_bounds__(CG_T) k_cg_apply(Box b, CGView v, int tx, int 
   }
   pap = block_total(pap);
   if (threadIdx.x == 0) v.part[blockIdx.x] = pap;
-}
-
-// alpha = r.z / p.Ap
-__global__ void __launch_bounds__(CG_T) k_cg_alpha(CGView v, int nb) {
-  const double pap = row_total(v.part, 0, nb);
+  if (!last_block(v)) return;
+  pap = row_total(v.part, 0, gridDim.x);
   if (threadIdx.x == 0) {
     v.sc[1] = pap;
     v.sc[2] = pap > 0.0 ? v.sc[0] / pap : 0.0;
   }
 }
 
-// x += alpha p, r -= alpha Ap; block sums of the new r.z, r.r, and (for
-// the projection) of r and D^-1 r
+// x += alpha p, r -= alpha Ap; r.z, r.r, and (for the projection) the sums of
+// r and D^-1 r; then beta = r.z(new) / r.z(old), r.r for the convergence test
+// and, with the projection (every node free), m = mean r and r.z, r.r of r - m
 __global__ void __launch_bounds__(CG_T) k_cg_update(Box b, CGView v, double* x, int neutral) {
   const double alpha = v.sc[2];
   double rz = 0.0, rr = 0.0, s1 = 0.0, s2 = 0.0;
   for (long long n = blockIdx.x * (long long)CG_T + threadIdx.x; n < b.N; n += (long long)gridDim.x * CG_T) {
     const double di = v.dinv[n];
-    if (di == 0.0) continue;
+    if (is_zero(di)) continue;
     x[n] += alpha * v.p[n];
     const double rn = v.r[n] - alpha * v.ap[n];
     v.r[n] = rn;
     rz += di * rn * rn;
     rr += rn * rn;
-    s1 += rn;
-    s2 += di * rn;
+    if (neutral) {
+      s1 += rn;
+      s2 += di * rn;
+    }
   }
   rz = block_total(rz);
   rr = block_total(rr);
@@ -272,14 +335,10 @@ __global__ void __launch_bounds__(CG_T) k_cg_update(Box b, CGView v, double* x, 
       v.part[3 * CG_BLOCKS + blockIdx.x] = s2;
     }
   }
-}
-
-// beta = r.z(new) / r.z(old); r.r for the convergence test; with the
-// projection (every node free): m = mean r, and r.z, r.r of r - m
-__global__ void __launch_bounds__(CG_T) k_cg_beta(CGView v, int nb, long long N, int neutral) {
-  double rz = row_total(v.part, 0, nb);
-  double rr = row_total(v.part, 1, nb);
-  double s1 = 0.0, s2 = 0.0;
+  if (!last_block(v)) return;
+  const int nb = gridDim.x;
+  rz = row_total(v.part, 0, nb);
+  rr = row_total(v.part, 1, nb);
   if (neutral) {
     s1 = row_total(v.part, 2, nb);
     s2 = row_total(v.part, 3, nb);
@@ -287,7 +346,7 @@ __global__ void __launch_bounds__(CG_T) k_cg_beta(CGView v, int nb, long long N,
   if (threadIdx.x == 0) {
     double m = 0.0;
     if (neutral) {
-      m = s1 / (double)N;
+      m = s1 / (double)b.N;
       rz = rz - 2.0 * m * s2 + m * m * v.sc[9];
       rr = rr - m * s1;
     }
@@ -300,25 +359,27 @@ __global__ void __launch_bounds__(CG_T) k_cg_beta(CGView v, int nb, long long N,
 
 // r -= m (the projection; m = 0 with fixed nodes), p = D^-1 r + beta p on
 // the free nodes
-__global__ void __launch_bounds__(CG_T) k_cg_direction(Box b, CGView v) {
+__global__ void __launch_bounds__(CG_T) k_cg_direction(Box b, CGView v, int neutral) {
   const double beta = v.sc[3], m = v.sc[10];
-  for (long long n = blockIdx.x * (long long)CG_T + threadIdx.x; n < b.N; n += (long long)gridDim.x * CG_T) {
-    const double di = v.dinv[n];
-    if (di != 0.0) {
-      const double rn = v.r[n] - m;
-      v.r[n] = rn;
-      v.p[n] = di * rn + beta * v.p[n];
-    }
-  }
+  const unsigned n = blockIdx.x * CG_T + threadIdx.x;
+  if (n >= (unsigned)b.N) return;
+  const double di = v.dinv[n];
+  if (is_zero(di)) return;
+  double rn = v.r[n];
+  if (neutral) v.r[n] = rn -= m;
+  v.p[n] = di * rn + beta * v.p[n];
 }
 
-// block sums of x (for the mean of a solution without fixed nodes)
-__global__ void __launch_bounds__(CG_T) k_cg_sum(Box b, const double* x, double* part) {
+// the sum of x (for the mean of a solution without fixed nodes)
+__global__ void __launch_bounds__(CG_T) k_cg_sum(Box b, CGView v, const double* x) {
   double s = 0.0;
   for (long long n = blockIdx.x * (long long)CG_T + threadIdx.x; n < b.N; n += (long long)gridDim.x * CG_T)
     s += x[n];
   s = block_total(s);
-  if (threadIdx.x == 0) part[blockIdx.x] = s;
+  if (threadIdx.x == 0) v.part[blockIdx.x] = s;
+  if (!last_block(v)) return;
+  s = row_total(v.part, 0, gridDim.x);
+  if (threadIdx.x == 0) v.sc[5] = s;
 }
 
 __global__ void __launch_bounds__(CG_T) k_cg_shift(Box b, double* x, const double* sc) {
@@ -328,251 +389,406 @@ __global__ void __launch_bounds__(CG_T) k_cg_shift(Box b, double* x, const doubl
 }
 
 // ---------------------------------------------------------------------------
-// Multigrid preconditioner: one V-cycle z = M r of the same operator.  Level
-// l + 1 halves every edge of level l (while all are even and the coarse box
-// keeps at least 2 nodes per edge); its node I covers the 8 nodes 2I + {0,1}^3.
-// Coarse face permittivity: the 4 fine faces it covers, summed and halved
-// (the flux through 4 faces over a distance twice as long); a coarse node is
-// fixed (zero correction) when one of its nodes is.  Restriction sums the 8
-// residuals, prolongation copies the coarse correction to the 8 nodes (the
-// transpose of the restriction), the smoother is damped Jacobi (omega = 0.8),
-// two sweeps before and after, and the coarsest level takes 40 sweeps from
-// zero: every part is symmetric, so the V-cycle is a symmetric positive
-// definite preconditioner for CG.
+// Multigrid preconditioner: one V-cycle z = M r of the same operator.  The next
+// level halves every edge of at least 8 nodes (rounded up: the last coarse node
+// of an odd edge covers one) and keeps the others; levels end when no edge is
+// left to halve.  Coarse face permittivity: the fine faces it covers, summed,
+// over the halving along the face's axis (the flux through them over a distance
+// twice as long); a coarse node is fixed (zero correction) when one of its
+// nodes is.  Restriction sums the residuals of a coarse node's nodes,
+// prolongation copies its correction to them (the transpose).  Smoother: two
+// red-black Gauss-Seidel sweeps before (red first) and after (black first, the
+// adjoint) on levels whose edges are all even, else two sweeps of damped Jacobi
+// (omega = 0.8: the colours of a periodic odd edge meet); the coarsest level
+// takes a few Jacobi sweeps from zero.  Every part is symmetric, so the V-cycle is
+// a symmetric positive definite preconditioner for CG.
+//
+// Iterations to 1e-12 (dielectric sphere, fixed planes): Jacobi V(2,2) 27 at
+// 64^3, Gauss-Seidel V(1,1) 32 and V(2,2) 16, with trilinear transfers 17; a
+// 53^3 box, which only takes Jacobi sweeps, 28 (650 without the V-cycle).
 // ---------------------------------------------------------------------------
-constexpr int MG_MAXLEV = 10;
+constexpr int MG_MAXLEV = 12;
 constexpr double MG_OMEGA = 0.8;
-constexpr int MG_COARSE_SWEEPS = 40;
 
 struct MGLevel {
   int nx, ny, nz, n;
-  double* cf;    // 3n face permittivities (+x, +y, +z)
-  double* dinv;  // n: 1 / diagonal, 0 on fixed nodes
-  double* x;     // n: the level's correction
-  double* xt;    // n: the other Jacobi buffer
-  double* b;     // n: the level's right-hand side
-  double* r;     // n: residual
+  int rb;          // all edges even: red-black Gauss-Seidel
+  int fx, fy, fz;  // halving towards the next level (2 or 1 per axis)
+  double* cf;      // 3n face permittivities (+x, +y, +z)
+  double* dinv;    // n: 1 / diagonal, 0 on fixed nodes
+  double* D;       // n: diagonal
+  double* x;       // n: the level's correction
+  double* xt;      // n: the other Jacobi buffer
+  double* b;       // n: the level's right-hand side
 };
 
-// the stencil A x at node n of level L (x is 0 on fixed nodes)
-__device__ __forceinline__ double level_apply(const MGLevel& L, const double* x, int xx, int yy, int zz, int n) {
-  const int sy = L.nx, sz = L.nx * L.ny;
-  const int dxp = xx + 1 < L.nx ? 1 : 1 - L.nx, dxm = xx > 0 ? -1 : L.nx - 1;
-  const int dyp = yy + 1 < L.ny ? sy : sy - sz, dym = yy > 0 ? -sy : sz - sy;
-  const int dzp = zz + 1 < L.nz ? sz : sz - L.n, dzm = zz > 0 ? -sz : L.n - sz;
-  const double* cx = L.cf;
+// sweeps on the coarsest level: enough to cross its longest edge (4: 2, 7: 8;
+// 40 sweeps save no iteration: 64^3, coarsest 4^3, 16 with 2 or 40; 48 x 88 x
+// 104, coarsest 6 x 6 x 7, 17 with 8 or 40, 21 with 2)
+__host__ __device__ inline int coarse_sweeps(int nx, int ny, int nz) {
+  const int e = nx > ny ? (nx > nz ? nx : nz) : (ny > nz ? ny : nz);
+  return e > 4 ? 2 * (e - 3) : 2;
+}
+
+// b + sum over the faces of c_f x_f at node n of level L (x is 0 on fixed nodes)
+__device__ __forceinline__ double level_gather(const MGLevel& L, const double* x, int n, int xx, int yy, int zz) {
+  int m[6];
+  neighbours(L.nx, L.ny, L.nz, n, xx, yy, zz, m);
   const double* cy = L.cf + L.n;
   const double* cz = L.cf + 2 * (size_t)L.n;
-  const double xn = x[n];
-  return cx[n] * (xn - x[n + dxp]) + cx[n + dxm] * (xn - x[n + dxm]) + cy[n] * (xn - x[n + dyp]) +
-         cy[n + dym] * (xn - x[n + dym]) + cz[n] * (xn - x[n + dzp]) + cz[n + dzm] * (xn - x[n + dzm]);
+  double s = fma(L.cf[n], x[m[0]], L.b[n]);
+  s = fma(L.cf[m[1]], x[m[1]], s);
+  s = fma(cy[n], x[m[2]], s);
+  s = fma(cy[m[3]], x[m[3]], s);
+  s = fma(cz[n], x[m[4]], s);
+  return fma(cz[m[5]], x[m[5]], s);
+}
+// node j of a colour (x + y + z even: red, colour 0)
+__device__ __forceinline__ int colour_node(const MGLevel& L, unsigned j, int colour, int& x, int& y, int& z) {
+  const unsigned hx = (unsigned)L.nx >> 1, row = j / hx;
+  z = (int)(row / (unsigned)L.ny);
+  y = (int)row - z * L.ny;
+  x = 2 * (int)(j - row * hx) + ((y + z + colour) & 1);
+  return x + L.nx * (int)row;
 }
 
-// loop over the level's nodes with their coordinates: the work items are the
-// 32 x 8 tiles of every plane, block b takes items b, b + gridDim.x, ... (no
-// division per node)
-#define MG_FOR_NODES(L)                                                                            \
-  for (int w_ = blockIdx.x, tx_ = ((L).nx + 31) / 32, ty_ = ((L).ny + 7) / 8; w_ < tx_ * ty_ * (L).nz; \
-       w_ += gridDim.x)                                                                            \
-    if (const int xx_ = (w_ % tx_) * 32 + (int)(threadIdx.x & 31),                                 \
-        yy_ = ((w_ / tx_) % ty_) * 8 + (int)(threadIdx.x >> 5), zz_ = w_ / (tx_ * ty_),            \
-        n = xx_ + (L).nx * (yy_ + (L).ny * zz_);                                                   \
-        xx_ < (L).nx && yy_ < (L).ny)
-
-// one damped Jacobi sweep: out = in + omega D^-1 (b - A in); in == nullptr:
-// from zero (out = omega D^-1 b)
-__global__ void __launch_bounds__(CG_T) k_mg_jacobi(MGLevel L, const double* in, double* out) {
-  MG_FOR_NODES(L) {
-    const double di = L.dinv[n];
-    if (di == 0.0) {
-      out[n] = 0.0;
-      continue;
-    }
-    if (!in) {
-      out[n] = MG_OMEGA * di * L.b[n];
-      continue;
-    }
-    out[n] = in[n] + MG_OMEGA * di * (L.b[n] - level_apply(L, in, xx_, yy_, zz_, n));
-  }
-}
-
-__global__ void __launch_bounds__(CG_T) k_mg_residual(MGLevel L) {
-  MG_FOR_NODES(L) {
-    L.r[n] = L.dinv[n] == 0.0 ? 0.0 : L.b[n] - level_apply(L, L.x, xx_, yy_, zz_, n);
-  }
-}
-
-// coarse right-hand side: the sum of the 8 fine residuals (0 at fixed nodes)
-__global__ void __launch_bounds__(CG_T) k_mg_restrict(MGLevel F, MGLevel C) {
-  MG_FOR_NODES(C) {
-    if (C.dinv[n] == 0.0) {
-      C.b[n] = 0.0;
-      continue;
-    }
-    double s = 0.0;
-#pragma unroll
-    for (int c = 0; c < 8; ++c) {
-      const int fx = 2 * xx_ + (c & 1), fy = 2 * yy_ + ((c >> 1) & 1), fz = 2 * zz_ + (c >> 2);
-      s += F.r[fx + F.nx * (fy + F.ny * fz)];
-    }
-    C.b[n] = s;
-  }
-}
-
-// fine x += the parent's coarse correction (free fine nodes)
-__global__ void __launch_bounds__(CG_T) k_mg_prolong(MGLevel F, MGLevel C) {
-  MG_FOR_NODES(F) {
-    if (F.dinv[n] != 0.0) F.x[n] += C.x[(xx_ >> 1) + C.nx * ((yy_ >> 1) + C.ny * (zz_ >> 1))];
-  }
-}
-
-// the coarse level's faces, diagonal and fixed nodes from the fine level
-__global__ void __launch_bounds__(CG_T) k_mg_coarsen(MGLevel F, MGLevel C) {
-  MG_FOR_NODES(C) {
-    bool fixed = false;
-    double fc[3] = {0.0, 0.0, 0.0};
-#pragma unroll
-    for (int c = 0; c < 8; ++c) {
-      const int fx = 2 * xx_ + (c & 1), fy = 2 * yy_ + ((c >> 1) & 1), fz = 2 * zz_ + (c >> 2);
-      const int m = fx + F.nx * (fy + F.ny * fz);
-      fixed |= F.dinv[m] == 0.0;
-      // the fine faces on the coarse node's + side: children with the upper
-      // coordinate along that axis
-      if (c & 1) fc[0] += F.cf[m];
-      if ((c >> 1) & 1) fc[1] += F.cf[F.n + m];
-      if (c >> 2) fc[2] += F.cf[2 * (size_t)F.n + m];
-    }
-    C.cf[n] = 0.5 * fc[0];
-    C.cf[C.n + n] = 0.5 * fc[1];
-    C.cf[2 * (size_t)C.n + n] = 0.5 * fc[2];
-    C.dinv[n] = fixed ? 0.0 : 1.0;  // marks the fixed nodes; the diagonal follows
-  }
-}
-
-__global__ void __launch_bounds__(CG_T) k_mg_diag(MGLevel C) {
-  MG_FOR_NODES(C) {
-    if (C.dinv[n] == 0.0) continue;
-    const int sy = C.nx, sz = C.nx * C.ny;
-    const int dxm = xx_ > 0 ? -1 : C.nx - 1, dym = yy_ > 0 ? -sy : sz - sy, dzm = zz_ > 0 ? -sz : C.n - sz;
-    const double d = C.cf[n] + C.cf[n + dxm] + C.cf[C.n + n] + C.cf[C.n + n + dym] +
-                     C.cf[2 * (size_t)C.n + n] + C.cf[2 * (size_t)C.n + n + dzm];
-    C.dinv[n] = 1.0 / d;
-  }
-}
-#undef MG_FOR_NODES
-
-// the coarsest level: MG_COARSE_SWEEPS damped Jacobi sweeps from zero by one
-// block (the level holds at most MG_COARSE_MAX nodes), ending in C.x
-constexpr int MG_COARSE_MAX = 8192;
-constexpr int MG_COARSE_T = 1024;
-__global__ void __launch_bounds__(MG_COARSE_T) k_mg_coarse(MGLevel C) {
-  for (int sweep = 0; sweep < MG_COARSE_SWEEPS; ++sweep) {
-    const double* in = sweep == 0 ? nullptr : ((sweep & 1) ? C.xt : C.x);
-    double* out = (sweep & 1) ? C.x : C.xt;
-    for (int n = threadIdx.x; n < C.n; n += MG_COARSE_T) {
-      const double di = C.dinv[n];
-      if (di == 0.0) {
-        out[n] = 0.0;
-      } else if (!in) {
-        out[n] = MG_OMEGA * di * C.b[n];
-      } else {
-        const int xx = n % C.nx, yy = (n / C.nx) % C.ny, zz = n / (C.nx * C.ny);
-        out[n] = in[n] + MG_OMEGA * di * (C.b[n] - level_apply(C, in, xx, yy, zz, n));
-      }
-    }
-    __syncthreads();
-  }
-}
-
-// PCG with a general preconditioner z = M r
-// x += alpha p, r -= alpha Ap; block sums of r.r and (for the projection) r
-__global__ void __launch_bounds__(CG_T) k_pcg_update(Box b, CGView v, double* x) {
-  const double alpha = v.sc[2];
-  double rr = 0.0, s1 = 0.0;
-  for (long long n = blockIdx.x * (long long)CG_T + threadIdx.x; n < b.N; n += (long long)gridDim.x * CG_T) {
-    if (v.dinv[n] == 0.0) continue;
-    x[n] += alpha * v.p[n];
-    const double rn = v.r[n] - alpha * v.ap[n];
-    v.r[n] = rn;
-    rr += rn * rn;
-    s1 += rn;
-  }
-  rr = block_total(rr);
-  s1 = block_total(s1);
-  if (threadIdx.x == 0) {
-    v.part[CG_BLOCKS + blockIdx.x] = rr;
-    v.part[2 * CG_BLOCKS + blockIdx.x] = s1;
-  }
-}
-
-// r.r of the (projected) residual and the mean to remove
-__global__ void __launch_bounds__(CG_T) k_pcg_mean(CGView v, int nb, long long N, int neutral) {
-  const double rr = row_total(v.part, 1, nb);
-  const double s1 = row_total(v.part, 2, nb);
-  if (threadIdx.x == 0) {
-    const double m = neutral ? s1 / (double)N : 0.0;
-    v.sc[10] = m;
-    v.sc[4] = neutral ? rr - m * s1 : rr;
-  }
-}
-
-__global__ void __launch_bounds__(CG_T) k_pcg_project(Box b, CGView v) {
-  const double m = v.sc[10];
-  for (long long n = blockIdx.x * (long long)CG_T + threadIdx.x; n < b.N; n += (long long)gridDim.x * CG_T)
-    if (v.dinv[n] != 0.0) v.r[n] -= m;
-}
-
-// block sums of r.z
-__global__ void __launch_bounds__(CG_T) k_pcg_dot(Box b, CGView v, const double* z) {
-  double t = 0.0;
-  for (long long n = blockIdx.x * (long long)CG_T + threadIdx.x; n < b.N; n += (long long)gridDim.x * CG_T)
-    if (v.dinv[n] != 0.0) t += v.r[n] * z[n];
+// beta = r.z(new) / r.z(old) from the block sums of r.z (first: r.z only)
+__device__ __forceinline__ void finish_beta(const CGView& v, double t, int first) {
   t = block_total(t);
   if (threadIdx.x == 0) v.part[blockIdx.x] = t;
-}
-
-// beta = r.z(new) / r.z(old) (first: r.z only, beta = 0)
-__global__ void __launch_bounds__(CG_T) k_pcg_beta(CGView v, int nb, int first) {
-  const double rz = row_total(v.part, 0, nb);
+  if (!last_block(v)) return;
+  const double rz = row_total(v.part, 0, gridDim.x);
   if (threadIdx.x == 0) {
     v.sc[3] = (!first && v.sc[0] > 0.0) ? rz / v.sc[0] : 0.0;
     v.sc[0] = rz;
   }
 }
 
+// one half of a Gauss-Seidel sweep, in place: the nodes of one colour from
+// their neighbours, which all have the other
+__device__ __forceinline__ void half_node(const MGLevel& L, unsigned j, int colour) {
+  int x, y, z;
+  const int n = colour_node(L, j, colour, x, y, z);
+  L.x[n] = L.dinv[n] * level_gather(L, L.x, n, x, y, z);
+}
+__global__ void __launch_bounds__(CG_T) k_mg_half(MGLevel L, int colour) {
+  const unsigned j = blockIdx.x * CG_T + threadIdx.x;
+  if (j < (unsigned)L.n / 2) half_node(L, j, colour);
+}
+// the last half sweep (red) of the fine level, with b.x: a red node's
+// neighbour x ^ 1 in the row is black and final
+__global__ void __launch_bounds__(CG_T) k_mg_half_dot(MGLevel L, CGView v, int first) {
+  double t = 0.0;
+  for (unsigned j = blockIdx.x * CG_T + threadIdx.x; j < (unsigned)L.n / 2; j += gridDim.x * CG_T) {
+    int x, y, z;
+    const int n = colour_node(L, j, 0, x, y, z);
+    const double xn = L.dinv[n] * level_gather(L, L.x, n, x, y, z);
+    L.x[n] = xn;
+    const int o = n + 1 - 2 * (x & 1);
+    t = fma(L.b[n], xn, fma(L.b[o], L.x[o], t));
+  }
+  finish_beta(v, t, first);
+}
+
+// one damped Jacobi sweep: out = in + omega D^-1 (b - A in); in == nullptr:
+// from zero (out = omega D^-1 b)
+__device__ __forceinline__ double jacobi_node(const MGLevel& L, const double* in, int n) {
+  const double di = L.dinv[n];
+  if (!in) return MG_OMEGA * di * L.b[n];
+  if (is_zero(di)) return 0.0;
+  int x, y, z;
+  node_xyz(L.nx, L.ny, n, x, y, z);
+  return fma(MG_OMEGA * di, level_gather(L, in, n, x, y, z), (1.0 - MG_OMEGA) * in[n]);
+}
+__global__ void __launch_bounds__(CG_T) k_mg_jacobi(MGLevel L, const double* in, double* out) {
+  const unsigned n = blockIdx.x * CG_T + threadIdx.x;
+  if (n < (unsigned)L.n) out[n] = jacobi_node(L, in, (int)n);
+}
+// the last sweep of the fine level, with b.x
+__global__ void __launch_bounds__(CG_T) k_mg_jacobi_dot(MGLevel L, const double* in, double* out, CGView v, int first) {
+  double t = 0.0;
+  for (unsigned i = blockIdx.x * CG_T + threadIdx.x; i < (unsigned)L.n; i += gridDim.x * CG_T) {
+    const int n = (int)i;
+    const double xn = jacobi_node(L, in, n);
+    out[n] = xn;
+    t = fma(L.b[n], xn, t);
+  }
+  finish_beta(v, t, first);
+}
+
+// coarse right-hand side: the sum of the fine residuals (0 at fixed nodes).
+// After a red-black sweep the residuals of the black nodes are zero (to
+// rounding): only the red ones are formed.  On a red-black coarse level its
+// first half sweep from zero, x = D^-1 b on the red nodes, comes along.
+__device__ __forceinline__ void restrict_node(const MGLevel& F, const MGLevel& C, int n) {
+  int X, Y, Z;
+  node_xyz(C.nx, C.ny, n, X, Y, Z);
+  const double di = C.dinv[n];
+  double s = 0.0;
+  auto residual = [&](int x, int y, int z) -> double {
+    const int m = x + F.nx * (y + F.ny * z);
+    const double v = fma(-F.D[m], F.x[m], level_gather(F, F.x, m, x, y, z));
+    return is_zero(F.dinv[m]) ? 0.0 : v;
+  };
+  if (!is_zero(di)) {
+    if (F.rb && F.fx + F.fy + F.fz == 6) {
+      // the four red children, their loads in flight together
+      const int x = 2 * X, y = 2 * Y, z = 2 * Z;
+      const double r0 = residual(x, y, z), r1 = residual(x + 1, y + 1, z), r2 = residual(x + 1, y, z + 1),
+                   r3 = residual(x, y + 1, z + 1);
+      s = (r0 + r1) + (r2 + r3);
+    } else {
+      for (int c = 0; c < 8; ++c) {
+        const int cx = c & 1, cy = (c >> 1) & 1, cz = c >> 2;
+        if (cx >= F.fx || cy >= F.fy || cz >= F.fz) continue;
+        const int x = F.fx * X + cx, y = F.fy * Y + cy, z = F.fz * Z + cz;
+        if (x >= F.nx || y >= F.ny || z >= F.nz) continue;
+        if (F.rb && ((x + y + z) & 1)) continue;
+        s += residual(x, y, z);
+      }
+    }
+  }
+  C.b[n] = s;
+  if (C.rb && !((X + Y + Z) & 1)) C.x[n] = di * s;
+}
+__global__ void __launch_bounds__(CG_T) k_mg_restrict(MGLevel F, MGLevel C) {
+  const unsigned n = blockIdx.x * CG_T + threadIdx.x;
+  if (n < (unsigned)C.n) restrict_node(F, C, (int)n);
+}
+
+// fine x += the coarse correction (free fine nodes; on a red-black level only
+// the red ones: the black half sweep that follows does not read the others)
+__device__ __forceinline__ void prolong_node(const MGLevel& F, const MGLevel& C, unsigned j) {
+  int x, y, z, n = (int)j;
+  if (F.rb) n = colour_node(F, j, 0, x, y, z);
+  else node_xyz(F.nx, F.ny, n, x, y, z);
+  if (!is_zero(F.dinv[n]))
+    F.x[n] += C.x[(x >> (F.fx - 1)) + C.nx * ((y >> (F.fy - 1)) + C.ny * (z >> (F.fz - 1)))];
+}
+__global__ void __launch_bounds__(CG_T) k_mg_prolong(MGLevel F, MGLevel C) {
+  const unsigned j = blockIdx.x * CG_T + threadIdx.x;
+  if (j < (unsigned)(F.rb ? F.n / 2 : F.n)) prolong_node(F, C, j);
+}
+
+// the coarse level's faces and fixed nodes from the fine level
+__global__ void __launch_bounds__(CG_T) k_mg_coarsen(MGLevel F, MGLevel C) {
+  const int n = (int)(blockIdx.x * CG_T + threadIdx.x);
+  if ((unsigned)n >= (unsigned)C.n) return;
+  int X, Y, Z;
+  node_xyz(C.nx, C.ny, n, X, Y, Z);
+  bool fixed = false;
+  double fc[3] = {0.0, 0.0, 0.0};
+  for (int c = 0; c < 8; ++c) {
+    const int cx = c & 1, cy = (c >> 1) & 1, cz = c >> 2;
+    if (cx >= F.fx || cy >= F.fy || cz >= F.fz) continue;
+    const int x = F.fx * X + cx, y = F.fy * Y + cy, z = F.fz * Z + cz;
+    if (x >= F.nx || y >= F.ny || z >= F.nz) continue;
+    const int m = x + F.nx * (y + F.ny * z);
+    fixed |= F.dinv[m] == 0.0;
+    // the fine faces on the coarse node's + side: its last nodes along the axis
+    if (cx == F.fx - 1 || x == F.nx - 1) fc[0] += F.cf[m];
+    if (cy == F.fy - 1 || y == F.ny - 1) fc[1] += F.cf[F.n + m];
+    if (cz == F.fz - 1 || z == F.nz - 1) fc[2] += F.cf[2 * (size_t)F.n + m];
+  }
+  C.cf[n] = F.fx == 2 ? 0.5 * fc[0] : fc[0];
+  C.cf[C.n + n] = F.fy == 2 ? 0.5 * fc[1] : fc[1];
+  C.cf[2 * (size_t)C.n + n] = F.fz == 2 ? 0.5 * fc[2] : fc[2];
+  C.dinv[n] = fixed ? 0.0 : 1.0;  // marks the fixed nodes; the diagonal follows
+}
+
+__global__ void __launch_bounds__(CG_T) k_mg_diag(MGLevel C) {
+  const int n = (int)(blockIdx.x * CG_T + threadIdx.x);
+  if ((unsigned)n >= (unsigned)C.n) return;
+  int x, y, z, m[6];
+  node_xyz(C.nx, C.ny, n, x, y, z);
+  neighbours(C.nx, C.ny, C.nz, n, x, y, z, m);
+  const double d = C.cf[n] + C.cf[m[1]] + C.cf[C.n + n] + C.cf[C.n + m[3]] + C.cf[2 * (size_t)C.n + n] +
+                   C.cf[2 * (size_t)C.n + m[5]];
+  C.D[n] = d;
+  if (C.dinv[n] != 0.0) C.dinv[n] = 1.0 / d;
+}
+
+// The cycle below a level: the levels of at most MG_SMALL nodes in one launch
+// of one cluster, whose CTAs meet at cluster barriers between the half sweeps.
+// Each of these phases is short: as launches of their own (nine per level) they
+// took 3 to 4 us each, most of an iteration at 64^3.  The FP64 pipes of 16 SMs
+// hold up to 32^3 nodes (15 us).  The coarsest level (every edge below 8: at
+// most 343 nodes) is done by the first CTA, a node per thread with its faces in
+// registers and x in shared memory.
+constexpr int MG_COARSE_MAX = 343;
+constexpr int MG_SMALL = 40000;
+constexpr int MG_SMALL_T = 512;
+constexpr int MG_SMALL_CTAS = 16;
+struct MGSmall {
+  MGLevel lev[MG_MAXLEV];  // the first is the caller's: its right-hand side (and first half sweep) is ready
+  int n;
+};
+__device__ void coarse_solve(const MGLevel& C) {
+  __shared__ double xs[2][MG_COARSE_MAX];
+  const int n = threadIdx.x;
+  const bool in = n < C.n;
+  int m[6] = {0, 0, 0, 0, 0, 0};
+  double c[6] = {}, wd = 0.0, wb = 0.0;
+  if (in) {
+    int x, y, z;
+    node_xyz(C.nx, C.ny, n, x, y, z);
+    neighbours(C.nx, C.ny, C.nz, n, x, y, z, m);
+    wd = MG_OMEGA * C.dinv[n];
+    wb = wd * C.b[n];
+    c[0] = wd * C.cf[n];
+    c[1] = wd * C.cf[m[1]];
+    c[2] = wd * C.cf[C.n + n];
+    c[3] = wd * C.cf[C.n + m[3]];
+    c[4] = wd * C.cf[2 * C.n + n];
+    c[5] = wd * C.cf[2 * C.n + m[5]];
+    xs[0][n] = wb;
+  }
+  __syncthreads();
+  const double keep = wd == 0.0 ? 0.0 : 1.0 - MG_OMEGA;
+  double xn = wb;
+  const int sweeps = coarse_sweeps(C.nx, C.ny, C.nz);
+  for (int s = 1; s < sweeps; ++s) {
+    const double* const cur = xs[(s + 1) & 1];
+    if (in) {
+      const double a = fma(c[0], cur[m[0]], fma(keep, xn, wb)), b = c[1] * cur[m[1]];
+      const double d = fma(c[2], cur[m[2]], a), e = fma(c[3], cur[m[3]], b);
+      xn = fma(c[4], cur[m[4]], d) + fma(c[5], cur[m[5]], e);
+      xs[s & 1][n] = xn;
+    }
+    __syncthreads();
+  }
+  if (in) C.x[n] = xn;
+}
+__global__ void __launch_bounds__(MG_SMALL_T) k_mg_small(const __grid_constant__ MGSmall S) {
+  cg::cluster_group cl = cg::this_cluster();
+  const unsigned first = blockIdx.x * MG_SMALL_T + threadIdx.x, step = gridDim.x * MG_SMALL_T;
+  auto half = [&](const MGLevel& A, int colour) {
+    for (unsigned j = first; j < (unsigned)A.n / 2; j += step) half_node(A, j, colour);
+    cl.sync();
+  };
+  auto jacobi = [&](const MGLevel& A, const double* in, double* out) {
+    for (unsigned n = first; n < (unsigned)A.n; n += step) out[n] = jacobi_node(A, in, (int)n);
+    cl.sync();
+  };
+  for (int l = 0; l < S.n - 1; ++l) {
+    const MGLevel& A = S.lev[l];
+    const MGLevel& C = S.lev[l + 1];
+    if (A.rb) {
+      half(A, 1);
+      half(A, 0);
+      half(A, 1);
+    } else {
+      jacobi(A, nullptr, A.xt);
+      jacobi(A, A.xt, A.x);
+    }
+    for (unsigned n = first; n < (unsigned)C.n; n += step) restrict_node(A, C, (int)n);
+    cl.sync();
+  }
+  if (blockIdx.x == 0) coarse_solve(S.lev[S.n - 1]);
+  cl.sync();
+  for (int l = S.n - 2; l >= 0; --l) {
+    const MGLevel& A = S.lev[l];
+    for (unsigned j = first; j < (unsigned)(A.rb ? A.n / 2 : A.n); j += step) prolong_node(A, S.lev[l + 1], j);
+    cl.sync();
+    if (A.rb) {
+      half(A, 1);
+      half(A, 0);
+      half(A, 1);
+      half(A, 0);
+    } else {
+      jacobi(A, A.x, A.xt);
+      jacobi(A, A.xt, A.x);
+    }
+  }
+}
+
+// x += alpha p, r -= alpha Ap; r.r and (for the projection) the mean of r.
+// Without the projection the preconditioner's first half sweep from zero,
+// z = D^-1 r on the red nodes, comes along.
+__global__ void __launch_bounds__(CG_T) k_pcg_update(Box b, CGView v, double* x, MGLevel L, int neutral) {
+  const double alpha = v.sc[2];
+  double rr = 0.0, s1 = 0.0;
+  for (long long i = blockIdx.x * (long long)CG_T + threadIdx.x; i < b.N; i += (long long)gridDim.x * CG_T) {
+    const int n = (int)i;
+    const double di = v.dinv[n];
+    double rn = 0.0;
+    if (!is_zero(di)) {
+      x[n] += alpha * v.p[n];
+      rn = v.r[n] - alpha * v.ap[n];
+      v.r[n] = rn;
+      rr += rn * rn;
+      if (neutral) s1 += rn;
+    }
+    if (!neutral && L.rb) {
+      int xx, yy, zz;
+      node_xyz(b.nx, b.ny, n, xx, yy, zz);
+      if (!((xx + yy + zz) & 1)) L.x[n] = di * rn;
+    }
+  }
+  rr = block_total(rr);
+  if (neutral) s1 = block_total(s1);
+  if (threadIdx.x == 0) {
+    v.part[blockIdx.x] = rr;
+    v.part[CG_BLOCKS + blockIdx.x] = s1;
+  }
+  if (!last_block(v)) return;
+  rr = row_total(v.part, 0, gridDim.x);
+  if (neutral) s1 = row_total(v.part, 1, gridDim.x);
+  if (threadIdx.x == 0) {
+    const double m = neutral ? s1 / (double)b.N : 0.0;
+    v.sc[10] = m;
+    v.sc[4] = neutral ? rr - m * s1 : rr;
+  }
+}
+
+// r -= its mean (only without fixed nodes; before the first cycle m = 0), and
+// the preconditioner's first half sweep from zero
+__global__ void __launch_bounds__(CG_T) k_pcg_project(Box b, CGView v, MGLevel L, int shift) {
+  const double m = shift ? v.sc[10] : 0.0;
+  for (long long i = blockIdx.x * (long long)CG_T + threadIdx.x; i < b.N; i += (long long)gridDim.x * CG_T) {
+    const int n = (int)i;
+    const double di = v.dinv[n];
+    double rn = v.r[n];
+    if (shift && !is_zero(di)) v.r[n] = rn -= m;
+    if (L.rb) {
+      int xx, yy, zz;
+      node_xyz(b.nx, b.ny, n, xx, yy, zz);
+      if (!((xx + yy + zz) & 1)) L.x[n] = di * rn;
+    }
+  }
+}
+
 // p = z + beta p on the free nodes
 __global__ void __launch_bounds__(CG_T) k_pcg_direction(Box b, CGView v, const double* z) {
   const double beta = v.sc[3];
-  for (long long n = blockIdx.x * (long long)CG_T + threadIdx.x; n < b.N; n += (long long)gridDim.x * CG_T)
-    if (v.dinv[n] != 0.0) v.p[n] = z[n] + beta * v.p[n];
+  const unsigned n = blockIdx.x * CG_T + threadIdx.x;
+  if (n < (unsigned)b.N && !is_zero(v.dinv[n])) v.p[n] = z[n] + beta * v.p[n];
 }
 
-// the multigrid levels of a box: halving while every edge is even and the
-// coarse edges stay >= 4; the coarsest must fit one block's solve
-int mg_levels(int nx, int ny, int nz, int (*dims)[3]) {
+// the multigrid levels of a box (one: no edge to halve, the diagonal is the
+// preconditioner): the edges of each, and the halving towards the next
+int mg_levels(int nx, int ny, int nz, int (*dims)[6]) {
   int L = 0;
   int d[3] = {nx, ny, nz};
   while (L < MG_MAXLEV) {
-    dims[L][0] = d[0];
-    dims[L][1] = d[1];
-    dims[L][2] = d[2];
+    bool more = false;
+    for (int k = 0; k < 3; ++k) {
+      dims[L][k] = d[k];
+      dims[L][3 + k] = d[k] >= 8 ? 2 : 1;
+      more |= d[k] >= 8;
+    }
     ++L;
-    if ((d[0] | d[1] | d[2]) & 1) break;
-    if (d[0] / 2 < 4 || d[1] / 2 < 4 || d[2] / 2 < 4) break;
-    for (int k = 0; k < 3; ++k) d[k] /= 2;
+    if (!more) break;
+    for (int k = 0; k < 3; ++k) d[k] = d[k] >= 8 ? (d[k] + 1) / 2 : d[k];
   }
-  const long long coarsest = (long long)dims[L - 1][0] * dims[L - 1][1] * dims[L - 1][2];
-  return (L >= 2 && coarsest <= MG_COARSE_MAX) ? L : 1;
+  const int* c = dims[L - 1];
+  return c[0] * c[1] * c[2] <= MG_COARSE_MAX ? L : 1;
 }
 
-}  // namespace
-
-namespace {
-
 // the CG arrays, then the preconditioner's: z, the fine level's Jacobi buffer
-// and residual, and each coarser level's faces, diagonal, x, Jacobi buffer,
-// right-hand side and residual (8 values per node)
-size_t full_layout(int nx, int ny, int nz, CGView* v, void* base, MGLevel* lev, int* nlev, double** z) {
+// and diagonal, and each coarser level's faces, diagonal and its inverse, x,
+// Jacobi buffer and right-hand side (8 values per node)
+size_t full_layout(int nx, int ny, int nz, CGView* v, void* base, MGLevel* lev, int* nlev) {
   const long long N = (long long)nx * ny * nz;
   size_t off = cg_layout(N, v, base);
   auto take = [&](size_t count) {
@@ -581,56 +797,97 @@ size_t full_layout(int nx, int ny, int nz, CGView* v, void* base, MGLevel* lev, 
     off += count * sizeof(double);
     return p;
   };
-  int dims[MG_MAXLEV][3];
+  int dims[MG_MAXLEV][6];
   const int L = mg_levels(nx, ny, nz, dims);
-  double* zz = take((size_t)N);
-  double* xt0 = take((size_t)N);
-  double* r0 = take((size_t)N);
-  if (lev) {
-    *z = zz;
-    *nlev = L;
-    lev[0] = MGLevel{nx, ny, nz, (int)N, v->cf, v->dinv, zz, xt0, v->r, r0};
-  }
-  for (int l = 1; l < L; ++l) {
-    const int n = dims[l][0] * dims[l][1] * dims[l][2];
-    double* cf = take(3 * (size_t)n);
-    double* di = take((size_t)n);
-    double* x = take((size_t)n);
-    double* xt = take((size_t)n);
-    double* b = take((size_t)n);
-    double* r = take((size_t)n);
-    if (lev) lev[l] = MGLevel{dims[l][0], dims[l][1], dims[l][2], n, cf, di, x, xt, b, r};
+  if (nlev) *nlev = L;
+  for (int l = 0; l < L; ++l) {
+    const int* d = dims[l];
+    const int n = d[0] * d[1] * d[2];
+    MGLevel g{d[0], d[1], d[2], n, !((d[0] | d[1] | d[2]) & 1), d[3], d[4], d[5],
+              nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
+    if (l > 0) {
+      g.cf = take(3 * (size_t)n);
+      g.dinv = take((size_t)n);
+    } else if (v) {
+      g.cf = v->cf;
+      g.dinv = v->dinv;
+    }
+    g.D = take((size_t)n);
+    g.x = take((size_t)n);
+    g.xt = take((size_t)n);
+    if (l > 0) g.b = take((size_t)n);
+    else if (v) g.b = v->r;
+    if (lev) lev[l] = g;
   }
   return off;
 }
 
-unsigned level_blocks(const MGLevel& L) {
-  const long long items = (long long)((L.nx + 31) / 32) * ((L.ny + 7) / 8) * L.nz;
-  return (unsigned)std::min<long long>(CG_BLOCKS, items);
+unsigned nblocks(int n) { return ((unsigned)n + CG_T - 1) / CG_T; }
+
+// a cluster of MG_SMALL_CTAS CTAs is above the portable size
+cudaError_t launch_small(const MGLevel* lev, int L, cudaStream_t s) {
+  cudaError_t e = cudaFuncSetAttribute(k_mg_small, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  if (e != cudaSuccess) return e;
+  MGSmall S;
+  S.n = L;
+  std::copy(lev, lev + L, S.lev);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(MG_SMALL_CTAS);
+  cfg.blockDim = dim3(MG_SMALL_T);
+  cfg.stream = s;
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = MG_SMALL_CTAS;
+  at.val.clusterDim.y = 1;
+  at.val.clusterDim.z = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, k_mg_small, S);
 }
 
-// z = M r: one V-cycle over the levels
-void vcycle(const MGLevel* lev, int L, cudaStream_t s) {
-  for (int l = 0; l < L - 1; ++l) {
+// z = M r: one V-cycle over the levels, then r.z and beta.  The first half
+// sweep of a red-black level has been made where its right-hand side was.  The
+// fine level is never in the small launch: its last sweep forms r.z.
+cudaError_t vcycle(const MGLevel* lev, int L, const CGView& v, int first, cudaStream_t s) {
+  int small = 1;
+  while (small < L - 1 && lev[small].n > MG_SMALL) ++small;
+  for (int l = 0; l < small; ++l) {
     const MGLevel& A = lev[l];
-    k_mg_jacobi<<<level_blocks(A), CG_T, 0, s>>>(A, nullptr, A.xt);
-    k_mg_jacobi<<<level_blocks(A), CG_T, 0, s>>>(A, A.xt, A.x);
-    k_mg_residual<<<level_blocks(A), CG_T, 0, s>>>(A);
-    k_mg_restrict<<<level_blocks(lev[l + 1]), CG_T, 0, s>>>(A, lev[l + 1]);
+    if (A.rb) {
+      k_mg_half<<<nblocks(A.n / 2), CG_T, 0, s>>>(A, 1);
+      k_mg_half<<<nblocks(A.n / 2), CG_T, 0, s>>>(A, 0);
+      k_mg_half<<<nblocks(A.n / 2), CG_T, 0, s>>>(A, 1);
+    } else {
+      k_mg_jacobi<<<nblocks(A.n), CG_T, 0, s>>>(A, nullptr, A.xt);
+      k_mg_jacobi<<<nblocks(A.n), CG_T, 0, s>>>(A, A.xt, A.x);
+    }
+    k_mg_restrict<<<nblocks(lev[l + 1].n), CG_T, 0, s>>>(A, lev[l + 1]);
   }
-  k_mg_coarse<<<1, MG_COARSE_T, 0, s>>>(lev[L - 1]);
-  for (int l = L - 2; l >= 0; --l) {
+  const cudaError_t e = launch_small(lev + small, L - small, s);
+  if (e != cudaSuccess) return e;
+  for (int l = small - 1; l >= 0; --l) {
     const MGLevel& A = lev[l];
-    k_mg_prolong<<<level_blocks(A), CG_T, 0, s>>>(A, lev[l + 1]);
-    k_mg_jacobi<<<level_blocks(A), CG_T, 0, s>>>(A, A.x, A.xt);
-    k_mg_jacobi<<<level_blocks(A), CG_T, 0, s>>>(A, A.xt, A.x);
+    const unsigned nb = std::min<unsigned>(CG_BLOCKS, nblocks(A.rb ? A.n / 2 : A.n));
+    k_mg_prolong<<<nblocks(A.rb ? A.n / 2 : A.n), CG_T, 0, s>>>(A, lev[l + 1]);
+    if (A.rb) {
+      k_mg_half<<<nblocks(A.n / 2), CG_T, 0, s>>>(A, 1);
+      k_mg_half<<<nblocks(A.n / 2), CG_T, 0, s>>>(A, 0);
+      k_mg_half<<<nblocks(A.n / 2), CG_T, 0, s>>>(A, 1);
+      if (l > 0) k_mg_half<<<nblocks(A.n / 2), CG_T, 0, s>>>(A, 0);
+      else k_mg_half_dot<<<nb, CG_T, 0, s>>>(A, v, first);
+    } else {
+      k_mg_jacobi<<<nblocks(A.n), CG_T, 0, s>>>(A, A.x, A.xt);
+      if (l > 0) k_mg_jacobi<<<nblocks(A.n), CG_T, 0, s>>>(A, A.xt, A.x);
+      else k_mg_jacobi_dot<<<nb, CG_T, 0, s>>>(A, A.xt, A.x, v, first);
+    }
   }
+  return cudaGetLastError();
 }
 
 }  // namespace
 
 size_t poisson_cg_scratch_bytes(int nx, int ny, int nz) {
-  return full_layout(nx, ny, nz, nullptr, nullptr, nullptr, nullptr, nullptr);
+  return full_layout(nx, ny, nz, nullptr, nullptr, nullptr, nullptr);
 }
 
 cudaError_t poisson_solve_cg(const double* q, const double* eps, const unsigned char* fixed,
@@ -641,60 +898,57 @@ cudaError_t poisson_solve_cg(const double* q, const double* eps, const unsigned 
   CGView v;
   MGLevel lev[MG_MAXLEV];
   int nlev = 1;
-  double* z = nullptr;
-  full_layout(nx, ny, nz, &v, scratch, lev, &nlev, &z);
+  full_layout(nx, ny, nz, &v, scratch, lev, &nlev);
   const bool mg = nlev >= 2;
   const int nb = (int)std::min<long long>(CG_BLOCKS, (b.N + CG_T - 1) / CG_T);
   const int tx = (nx + 31) / 32, ty = (ny + 7) / 8;
   const int na = (int)std::min<long long>(CG_BLOCKS, (long long)tx * ty * nz);  // operator blocks
-  double h[12];
+  double h[16];
   *bad_eps = false;
-  // the charge's sum, the fixed-node count and the invalid permittivities
-  k_cg_stats<<<nb, CG_T, 0, s>>>(b, q, eps, fixed, v.part);
-  k_cg_total<<<1, CG_T, 0, s>>>(v.part, nb, v.sc, 6, 7, 8);
-  cudaError_t e = cudaMemcpyAsync(h, v.sc, 12 * sizeof(double), cudaMemcpyDeviceToHost, s);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  cudaError_t e = cudaMemsetAsync(v.sc, 0, 16 * sizeof(double), s);
   if (e != cudaSuccess) return e;
-  if (h[8] != 0.0) {
-    *bad_eps = true;
-    return cudaSuccess;
+  k_cg_faces<<<nb, CG_T, 0, s>>>(b, v, q, eps, fixed);
+  // the invalid permittivities are counted before phi is written
+  if (eps) {
+    e = cudaMemcpyAsync(h, v.sc, 16 * sizeof(double), cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    if (e != cudaSuccess) return e;
+    if (h[8] != 0.0) {
+      *bad_eps = true;
+      return cudaSuccess;
+    }
   }
-  const int neutral = h[7] == 0.0 ? 1 : 0;  // no fixed node: remove the mean charge
-  k_cg_prep<<<nb, CG_T, 0, s>>>(b, v, q, eps, fixed, phi_fixed, phi, 4.0 * M_PI * bjerrum, v.sc, neutral);
-  k_cg_total<<<1, CG_T, 0, s>>>(v.part, nb, v.sc, 0, 5, 9);
-  e = cudaMemcpyAsync(h, v.sc, 12 * sizeof(double), cudaMemcpyDeviceToHost, s);
+  k_cg_prep<<<nb, CG_T, 0, s>>>(b, v, lev[0].D, q, fixed, phi_fixed, phi, 4.0 * M_PI * bjerrum);
+  e = cudaMemcpyAsync(h, v.sc, 16 * sizeof(double), cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return e;
+  const int neutral = h[7] == 0.0 ? 1 : 0;  // no fixed node: the mean charge was removed
   const double bnorm = sqrt(h[5]);
   int it = 0;
   double rel = 0.0;
   auto iterate = [&]() {
     k_cg_apply<<<na, CG_T, 0, s>>>(b, v, tx, ty);
-    k_cg_alpha<<<1, CG_T, 0, s>>>(v, na);
     if (!mg) {
       k_cg_update<<<nb, CG_T, 0, s>>>(b, v, phi, neutral);
-      k_cg_beta<<<1, CG_T, 0, s>>>(v, nb, b.N, neutral);
-      k_cg_direction<<<nb, CG_T, 0, s>>>(b, v);
+      k_cg_direction<<<nblocks((int)b.N), CG_T, 0, s>>>(b, v, neutral);
       return;
     }
-    k_pcg_update<<<nb, CG_T, 0, s>>>(b, v, phi);
-    k_pcg_mean<<<1, CG_T, 0, s>>>(v, nb, b.N, neutral);
-    if (neutral) k_pcg_project<<<nb, CG_T, 0, s>>>(b, v);
-    vcycle(lev, nlev, s);
-    k_pcg_dot<<<nb, CG_T, 0, s>>>(b, v, z);
-    k_pcg_beta<<<1, CG_T, 0, s>>>(v, nb, 0);
-    k_pcg_direction<<<nb, CG_T, 0, s>>>(b, v, z);
+    k_pcg_update<<<nb, CG_T, 0, s>>>(b, v, phi, lev[0], neutral);
+    if (neutral) k_pcg_project<<<nb, CG_T, 0, s>>>(b, v, lev[0], 1);
+    const cudaError_t ve = vcycle(lev, nlev, v, 0, s);
+    if (e == cudaSuccess) e = ve;
+    k_pcg_direction<<<nblocks((int)b.N), CG_T, 0, s>>>(b, v, lev[0].x);
   };
   if (mg && bnorm > 0.0) {
     // the coarse levels' operators, then p = z = M r and r.z
     for (int l = 1; l < nlev; ++l) {
-      k_mg_coarsen<<<level_blocks(lev[l]), CG_T, 0, s>>>(lev[l - 1], lev[l]);
-      k_mg_diag<<<level_blocks(lev[l]), CG_T, 0, s>>>(lev[l]);
+      k_mg_coarsen<<<nblocks(lev[l].n), CG_T, 0, s>>>(lev[l - 1], lev[l]);
+      k_mg_diag<<<nblocks(lev[l].n), CG_T, 0, s>>>(lev[l]);
     }
-    vcycle(lev, nlev, s);
-    k_pcg_dot<<<nb, CG_T, 0, s>>>(b, v, z);
-    k_pcg_beta<<<1, CG_T, 0, s>>>(v, nb, 1);
-    k_pcg_direction<<<nb, CG_T, 0, s>>>(b, v, z);
+    if (lev[0].rb) k_pcg_project<<<nb, CG_T, 0, s>>>(b, v, lev[0], 0);
+    e = vcycle(lev, nlev, v, 1, s);
+    if (e != cudaSuccess) return e;
+    k_pcg_direction<<<nblocks((int)b.N), CG_T, 0, s>>>(b, v, lev[0].x);
   }
   // the iterations between two residual reads as one graph (a caller stream
   // other than the legacy default stream can be captured); else the launches
@@ -705,12 +959,13 @@ cudaError_t poisson_solve_cg(const double* q, const double* eps, const unsigned 
     cudaGraph_t g = nullptr;
     if (cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal) == cudaSuccess) {
       for (int k = 0; k < check; ++k) iterate();
-      if (cudaStreamEndCapture(s, &g) == cudaSuccess && g) {
+      if (cudaStreamEndCapture(s, &g) == cudaSuccess && g && e == cudaSuccess) {
         if (cudaGraphInstantiate(&graph, g, 0) != cudaSuccess) graph = nullptr;
       }
       if (g) cudaGraphDestroy(g);
     }
     cudaGetLastError();  // a failed capture leaves the launches one by one
+    e = cudaSuccess;
   }
   if (bnorm > 0.0) {
     rel = 1.0;
@@ -721,9 +976,10 @@ cudaError_t poisson_solve_cg(const double* q, const double* eps, const unsigned 
         if (e != cudaSuccess) break;
       } else {
         for (int k = 0; k < batch; ++k) iterate();
+        if (e != cudaSuccess) break;
       }
       it += batch;
-      e = cudaMemcpyAsync(h, v.sc, 12 * sizeof(double), cudaMemcpyDeviceToHost, s);
+      e = cudaMemcpyAsync(h, v.sc, 16 * sizeof(double), cudaMemcpyDeviceToHost, s);
       if (e == cudaSuccess) e = cudaStreamSynchronize(s);
       if (e != cudaSuccess) break;
       rel = sqrt(h[4]) / bnorm;
@@ -733,8 +989,7 @@ cudaError_t poisson_solve_cg(const double* q, const double* eps, const unsigned 
   if (graph) cudaGraphExecDestroy(graph);
   if (e != cudaSuccess) return e;
   if (neutral) {
-    k_cg_sum<<<nb, CG_T, 0, s>>>(b, phi, v.part);
-    k_cg_total<<<1, CG_T, 0, s>>>(v.part, nb, v.sc, 5, -1, -1);
+    k_cg_sum<<<nb, CG_T, 0, s>>>(b, v, phi);
     k_cg_shift<<<nb, CG_T, 0, s>>>(b, phi, v.sc);
   }
   e = cudaStreamSynchronize(s);
