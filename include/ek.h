@@ -246,8 +246,9 @@ ek_status ek_poisson_solve(const double* q, double* phi, int nx, int ny, int nz,
 
 /* The same periodic problem of Eq. 3 solved iteratively (the paper names
  * iterative solvers as the alternative to the FFT, Sec. III.C): geometric
- * multigrid V-cycles (two red-black Gauss-Seidel sweeps before and after,
- * full-weighting restriction, trilinear prolongation) on the box and its
+ * multigrid V-cycles (two red-black Gauss-Seidel sweeps before and after, on the
+ * box itself all four after; full-weighting restriction, trilinear prolongation)
+ * on the box and its
  * coarsenings by 2 (while every coarse edge stays even and >= 8, n_x / 2
  * even, and the level holds more than 4096 nodes), the coarsest level solved
  * exactly by the FFT; cycles until max|r| <= tol * max|b|, b = 4 pi l_B

@@ -3,13 +3,28 @@
 // (6 phi - sum of the 6 neighbours) = 4 pi l_B (q - mean q), mean phi = 0),
 // reached by V-cycles instead of a transform.  Levels: the box and its full
 // coarsenings by 2 while every coarse edge stays even and >= 8 (coarse n_x a
-// multiple of 2 for the real-to-complex transform) and the grid holds more
-// than 4096 nodes; on level l the operator is 4^-l (6 phi - sum nb) (the
-// same stencil on spacing 2^l).  Per V-cycle: two red-black Gauss-Seidel
-// sweeps, the residual, full-weighting restriction, the coarser cycle,
-// trilinear prolongation of the correction, two sweeps; the coarsest level is
-// solved exactly by the FFT solver.  Red-black sweeps need even edges, which
-// every level above the coarsest has.  All sums run in a fixed order.
+// multiple of 2 for the real-to-complex transform) and the grid holds
+// more than 4096 nodes; on level l the operator is 4^-l (6 phi - sum nb) (the
+// same stencil on spacing 2^l).  Per V-cycle and level: two red-black
+// Gauss-Seidel sweeps, the residual, full-weighting restriction, the coarser
+// cycle, trilinear prolongation of the correction, two sweeps; the coarsest
+// level is solved exactly by the FFT solver.  On the finest level the sweeps
+// before the next cycle's residual follow the prolongation, so that one
+// residual serves the convergence test and the restriction.  Red-black sweeps
+// need even edges, which every level above the coarsest has.  All sums run in a
+// fixed order.
+//
+// What bounds it: the FP64 pipe on the finest level, launches below.  So the
+// right-hand side is kept as b / (6 c) (a half sweep is 5 additions and one FMA
+// a node), residuals are formed on the red nodes only (those of the black ones,
+// updated last, are zero to rounding; the residual that is returned is taken
+// over all nodes), the restriction weighs the 13 red nodes of its 27, and the
+// correction goes to the black nodes only (the red half sweep that follows does
+// not read the others).  The coarse levels run while the host waits for the
+// residual.  128^3 to 1e-12 (GB300): 13 cycles of 0.51 ms -> 13 of 0.36 ms.  Of
+// a cycle (launches one by one, cold L2) the finest level's half sweeps take 8 x
+// 15 us (FP64 pipe: 10 us), its residual, restriction and prolongation 41 us,
+// 64^3 48 us, 32^3 35 us and the FFT of 16^3 50 us.
 #include <math.h>
 #include <string.h>
 
@@ -28,158 +43,204 @@ constexpr int MG_RED_BLOCKS = 512; // partial sums of a reduction
 struct Level {
   int nx, ny, nz;
   long long n;
-  double c;         // 4^-l
   double* phi;      // level 0: the caller's output
-  double* b;        // right-hand side
-  double* r;        // residual
+  double* b;        // right-hand side over 6 4^-l
+  double* r;        // residual over 4^-l, red nodes
 };
 
 __device__ __forceinline__ int wrap(int i, int n) { return i < 0 ? i + n : (i >= n ? i - n : i); }
 
-// b = s (q - qmean), qmean = sums[1] (written by k_sum_final)
-__global__ void k_mg_rhs(const double* q, double* b, long long n, double s, const double* sums) {
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  b[i] = s * (q[i] - sums[1]);
-}
+// scalars of a solve on the device
+struct Scalars {
+  double sum, mean;
+  unsigned long long max;  // bits of a maximum of absolute values
+  unsigned count;          // finished blocks of a sum
+};
 
-// block partial sums of x (fixed order: a grid-stride sum per thread, then a
-// tree over the block)
-__global__ void k_sum_partial(const double* x, long long n, double* part) {
+// sum of x and its mean over n values: block partial sums (a grid-stride sum
+// per thread, then a tree over the block), added in the same way by the last
+// block to finish
+__device__ __forceinline__ double block_sum(double s) {
   __shared__ double sh[MG_T];
-  double s = 0.0;
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += (long long)gridDim.x * blockDim.x)
-    s += x[i];
+  __syncthreads();
   sh[threadIdx.x] = s;
   __syncthreads();
   for (int w = MG_T / 2; w > 0; w >>= 1) {
     if ((int)threadIdx.x < w) sh[threadIdx.x] += sh[threadIdx.x + w];
     __syncthreads();
   }
-  if (threadIdx.x == 0) part[blockIdx.x] = sh[0];
+  return sh[0];
+}
+__global__ void k_mg_sum(const double* x, long long n, double* part, Scalars* out) {
+  __shared__ bool last;
+  double s = 0.0;
+  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
+       i += (long long)gridDim.x * blockDim.x)
+    s += x[i];
+  s = block_sum(s);
+  if (threadIdx.x == 0) {
+    part[blockIdx.x] = s;
+    __threadfence();
+    last = atomicAdd(&out->count, 1u) == gridDim.x - 1;
+    if (last) __threadfence();
+  }
+  __syncthreads();
+  if (!last) return;
+  s = 0.0;
+  for (int i = threadIdx.x; i < (int)gridDim.x; i += MG_T) s += part[i];
+  s = block_sum(s);
+  if (threadIdx.x == 0) {
+    out->sum = s;
+    out->mean = s / (double)n;
+    out->count = 0u;
+  }
 }
 
-// out[0] = sum of the nblk partial sums, in order (one thread); out[1] = the
-// mean over n values (one division, not one per node)
-__global__ void k_sum_final(const double* part, int nblk, long long n, double* out) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  double s = 0.0;
-  for (int i = 0; i < nblk; ++i) s += part[i];
-  out[0] = s;
-  out[1] = s / (double)n;
+// the bits of |v| (they order as the values do); 0 for a NaN
+__device__ __forceinline__ unsigned long long abs_bits(double v) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffULL;
+  return b > 0x7ff0000000000000ULL ? 0ULL : b;
+}
+// maximum over the grid (it does not depend on the order, and costs no FP64
+// instruction)
+__device__ __forceinline__ void grid_max(unsigned long long m, Scalars* out) {
+  __shared__ unsigned long long sh[MG_T / 32];
+  for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_down_sync(0xffffffffu, m, o));
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = m;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < MG_T / 32; ++w) m = max(m, sh[w]);
+    atomicMax(&out->max, m);
+  }
+}
+
+// node j of a colour (colour 0, red: x + y + z even; n_x even: half of every row)
+__device__ __forceinline__ int colour_node(unsigned j, int nx, int ny, int colour, int& x, int& y, int& z) {
+  const unsigned hx = (unsigned)nx / 2u, row = j / hx;
+  z = (int)(row / (unsigned)ny);
+  y = (int)row - z * ny;
+  x = 2 * (int)(j - row * hx) + ((y + z + colour) & 1);
+  return x + nx * (int)row;
 }
 
 // sum of the six neighbours of node i = (x, y, z) (32-bit indices: N < 2^31)
 __device__ __forceinline__ double nb_sum(const double* phi, int i, int x, int y, int z, int nx,
                                          int ny, int nz) {
   const int sy = nx, sz = nx * ny;
-  return phi[i - x + wrap(x - 1, nx)] + phi[i - x + wrap(x + 1, nx)] +
-         phi[i + (wrap(y - 1, ny) - y) * sy] + phi[i + (wrap(y + 1, ny) - y) * sy] +
-         phi[i + (wrap(z - 1, nz) - z) * sz] + phi[i + (wrap(z + 1, nz) - z) * sz];
+  return ((phi[i - x + wrap(x - 1, nx)] + phi[i - x + wrap(x + 1, nx)]) +
+          (phi[i + (wrap(y - 1, ny) - y) * sy] + phi[i + (wrap(y + 1, ny) - y) * sy])) +
+         (phi[i + (wrap(z - 1, nz) - z) * sz] + phi[i + (wrap(z + 1, nz) - z) * sz]);
 }
 
-// one colour of a red-black Gauss-Seidel sweep: the nodes with
-// (x + y + z) % 2 == colour take phi = (sum nb + b / c) / 6, as products
-// (inv_c = 1 / c = 4^l exactly; an FP64 division costs a long sequence on the
-// FP64 pipe, and the fixed point is set by the residual, which divides
-// nothing); thread j takes the j-th node of the colour (n_x even: half of
-// every row)
-__global__ void k_mg_rbgs(double* phi, const double* b, int nx, int ny, int nz, double inv_c,
-                          int colour) {
-  const unsigned j = blockIdx.x * blockDim.x + threadIdx.x;
-  const unsigned hx = (unsigned)nx / 2u;
-  if (j >= hx * (unsigned)ny * (unsigned)nz) return;
-  const unsigned row = j / hx;
-  const int y = (int)(row % (unsigned)ny), z = (int)(row / (unsigned)ny);
-  const int x = 2 * (int)(j - row * hx) + ((y + z + colour) & 1);
-  const int i = x + nx * (int)row;
+// b = s (q - mean q) / 6, and the first red half sweep from zero: phi = b on
+// the red nodes, 0 on the black ones; the maximum of |6 b|
+__global__ void __launch_bounds__(MG_T) k_mg_rhs(const double* q, double* phi, double* b, int nx, int ny, int nz,
+                                                 double s, Scalars* sc) {
+  const unsigned i = blockIdx.x * MG_T + threadIdx.x;
+  unsigned long long m = 0;
+  if (i < (unsigned)nx * (unsigned)ny * (unsigned)nz) {
+    const unsigned row = i / (unsigned)nx;
+    const int x = (int)(i - row * (unsigned)nx), y = (int)(row % (unsigned)ny), z = (int)(row / (unsigned)ny);
+    const double v = s * (q[i] - sc->mean);  // read before phi, which may alias q, is written
+    constexpr double SIXTH = 1.0 / 6.0;
+    b[i] = v * SIXTH;
+    phi[i] = ((x + y + z) & 1) ? 0.0 : v * SIXTH;
+    m = abs_bits(v);
+  }
+  grid_max(m, sc);
+}
+
+// one colour of a red-black Gauss-Seidel sweep: phi = sum nb / 6 + b
+__global__ void __launch_bounds__(MG_T) k_mg_half(double* phi, const double* b, int nx, int ny, int nz, int colour) {
+  const unsigned j = blockIdx.x * MG_T + threadIdx.x;
+  if (j >= (unsigned)nx / 2u * (unsigned)ny * (unsigned)nz) return;
+  int x, y, z;
+  const int i = colour_node(j, nx, ny, colour, x, y, z);
   constexpr double SIXTH = 1.0 / 6.0;
-  phi[i] = (nb_sum(phi, i, x, y, z, nx, ny, nz) + b[i] * inv_c) * SIXTH;
+  phi[i] = fma(nb_sum(phi, i, x, y, z, nx, ny, nz), SIXTH, b[i]);
 }
 
-// r = b - c (6 phi - sum nb)
-__global__ void k_mg_resid(const double* phi, const double* b, double* r, int nx, int ny, int nz,
-                           double c) {
-  const unsigned i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= (unsigned)nx * (unsigned)ny * (unsigned)nz) return;
-  const unsigned row = i / (unsigned)nx;
-  const int x = (int)(i - row * (unsigned)nx), y = (int)(row % (unsigned)ny), z = (int)(row / (unsigned)ny);
-  r[i] = b[i] - c * (6.0 * phi[i] - nb_sum(phi, (int)i, x, y, z, nx, ny, nz));
+// residual over 4^-l on the red nodes, r = sum nb - 6 (phi - b); with MAX the
+// maximum of |r|
+template <bool MAX>
+__global__ void __launch_bounds__(MG_T) k_mg_resid(const double* phi, const double* b, double* r, int nx, int ny,
+                                                   int nz, Scalars* sc) {
+  const unsigned j = blockIdx.x * MG_T + threadIdx.x;
+  unsigned long long m = 0;
+  if (j < (unsigned)nx / 2u * (unsigned)ny * (unsigned)nz) {
+    int x, y, z;
+    const int i = colour_node(j, nx, ny, 0, x, y, z);
+    const double v = fma(-6.0, phi[i] - b[i], nb_sum(phi, i, x, y, z, nx, ny, nz));
+    r[i] = v;
+    if (MAX) m = abs_bits(v);
+  }
+  if (MAX) grid_max(m, sc);
+}
+// the maximum of |r| over all nodes
+__global__ void __launch_bounds__(MG_T) k_mg_resid_max(const double* phi, const double* b, int nx, int ny, int nz,
+                                                       Scalars* sc) {
+  const unsigned i = blockIdx.x * MG_T + threadIdx.x;
+  unsigned long long m = 0;
+  if (i < (unsigned)nx * (unsigned)ny * (unsigned)nz) {
+    const unsigned row = i / (unsigned)nx;
+    const int x = (int)(i - row * (unsigned)nx), y = (int)(row % (unsigned)ny), z = (int)(row / (unsigned)ny);
+    m = abs_bits(fma(-6.0, phi[i] - b[i], nb_sum(phi, (int)i, x, y, z, nx, ny, nz)));
+  }
+  grid_max(m, sc);
 }
 
 // full weighting: coarse node (X, Y, Z) sits on fine node (2X, 2Y, 2Z) and
-// takes the weighted mean of the 27 fine residuals around it (weights
-// 1, 1/2, 1/4, 1/8 by the number of offset axes; every fine node gives a
-// total weight of 1, so the mean is kept); phi_c = 0 for the cycle below
-__global__ void k_mg_restrict(const double* rf, int nx, int ny, int nz, double* bc, double* phic) {
+// takes the weighted mean of the 27 fine residuals around it (weights 1, 1/2,
+// 1/4, 1/8 by the number of offset axes; every fine node gives a total weight
+// of 1, so the mean is kept), of which the 13 red ones (none or two offset
+// axes) are not zero; over 6 4^-(l+1) that is (r_0 + sum r / 4) / 12.  The
+// coarse level's first red half sweep from zero comes along.
+__global__ void __launch_bounds__(MG_T) k_mg_restrict(const double* rf, int nx, int ny, int nz, double* bc,
+                                                      double* phic) {
   const int cx = nx / 2, cy = ny / 2, cz = nz / 2;
-  const unsigned i = blockIdx.x * blockDim.x + threadIdx.x;
+  const unsigned i = blockIdx.x * MG_T + threadIdx.x;
   if (i >= (unsigned)cx * (unsigned)cy * (unsigned)cz) return;
   const unsigned row = i / (unsigned)cx;
   const int X = (int)(i - row * (unsigned)cx), Y = (int)(row % (unsigned)cy), Z = (int)(row / (unsigned)cy);
-  double s = 0.0;
-  for (int dz = -1; dz <= 1; ++dz) {
-    const int oz = wrap(2 * Z + dz, nz) * ny;
-    const double wz = dz ? 0.5 : 1.0;
-    for (int dy = -1; dy <= 1; ++dy) {
-      const int oy = (oz + wrap(2 * Y + dy, ny)) * nx;
-      const double wy = wz * (dy ? 0.5 : 1.0);
-      for (int dx = -1; dx <= 1; ++dx) s += wy * (dx ? 0.5 : 1.0) * rf[oy + wrap(2 * X + dx, nx)];
-    }
-  }
-  bc[i] = s / 8.0;
-  phic[i] = 0.0;
+  const int x[3] = {wrap(2 * X - 1, nx), 2 * X, 2 * X + 1};
+  const int y[3] = {nx * wrap(2 * Y - 1, ny), nx * (2 * Y), nx * (2 * Y + 1)};
+  const int sz = nx * ny, z[3] = {sz * wrap(2 * Z - 1, nz), sz * (2 * Z), sz * (2 * Z + 1)};
+  const double a = (rf[x[0] + y[0] + z[1]] + rf[x[2] + y[0] + z[1]]) + (rf[x[0] + y[2] + z[1]] + rf[x[2] + y[2] + z[1]]);
+  const double b = (rf[x[0] + y[1] + z[0]] + rf[x[2] + y[1] + z[0]]) + (rf[x[0] + y[1] + z[2]] + rf[x[2] + y[1] + z[2]]);
+  const double c = (rf[x[1] + y[0] + z[0]] + rf[x[1] + y[2] + z[0]]) + (rf[x[1] + y[0] + z[2]] + rf[x[1] + y[2] + z[2]]);
+  const double v = fma(0.25, (a + b) + c, rf[x[1] + y[1] + z[1]]) * (1.0 / 12.0);
+  bc[i] = v;
+  if (!((X + Y + Z) & 1)) phic[i] = v;
 }
 
-// trilinear prolongation of the coarse correction, added to the fine phi
-__global__ void k_mg_prolong_add(const double* phic, int nx, int ny, int nz, double* phif) {
+// trilinear prolongation of the coarse correction, added to the black nodes of
+// the fine phi: per axis an even fine index lies on coarse node x / 2, an odd
+// one half way between (x - 1) / 2 and (x + 1) / 2 (periodic); a black node has
+// one odd axis or three
+__global__ void __launch_bounds__(MG_T) k_mg_prolong(const double* phic, int nx, int ny, int nz, double* phif) {
   const int cx = nx / 2, cy = ny / 2, cz = nz / 2;
-  const unsigned i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= (unsigned)nx * (unsigned)ny * (unsigned)nz) return;
-  const unsigned row = i / (unsigned)nx;
-  const int x = (int)(i - row * (unsigned)nx), y = (int)(row % (unsigned)ny), z = (int)(row / (unsigned)ny);
-  // per axis: an even fine index lies on coarse node x / 2, an odd one half
-  // way between (x - 1) / 2 and (x + 1) / 2 (periodic); the weight of each
-  // of the (1, 2, 4 or 8) coarse nodes is 1/2 per odd axis
-  const int x0 = x >> 1, x1 = (x & 1) ? wrap(x0 + 1, cx) : x0;
-  const int y0 = (y >> 1) * cx, y1 = (y & 1) ? wrap((y >> 1) + 1, cy) * cx : y0;
-  const int z0 = (z >> 1) * cx * cy, z1 = (z & 1) ? wrap((z >> 1) + 1, cz) * cx * cy : z0;
-  // an even axis counts its one node twice and halves the sum: the same
-  // value as one node at weight 1
-  const double s = ((phic[z0 + y0 + x0] + phic[z0 + y0 + x1]) + (phic[z0 + y1 + x0] + phic[z0 + y1 + x1])) +
-                   ((phic[z1 + y0 + x0] + phic[z1 + y0 + x1]) + (phic[z1 + y1 + x0] + phic[z1 + y1 + x1]));
-  phif[i] += 0.125 * s;
-}
-
-// block maxima of |x| (a maximum does not depend on the order)
-__global__ void k_absmax_partial(const double* x, long long n, double* part) {
-  __shared__ double sh[MG_T];
-  double m = 0.0;
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += (long long)gridDim.x * blockDim.x)
-    m = fmax(m, fabs(x[i]));
-  sh[threadIdx.x] = m;
-  __syncthreads();
-  for (int w = MG_T / 2; w > 0; w >>= 1) {
-    if ((int)threadIdx.x < w) sh[threadIdx.x] = fmax(sh[threadIdx.x], sh[threadIdx.x + w]);
-    __syncthreads();
+  const unsigned j = blockIdx.x * MG_T + threadIdx.x;
+  if (j >= (unsigned)nx / 2u * (unsigned)ny * (unsigned)nz) return;
+  int x, y, z;
+  const int i = colour_node(j, nx, ny, 1, x, y, z);
+  const int x0 = x >> 1, y0 = (y >> 1) * cx, z0 = (z >> 1) * cx * cy;
+  const int x1 = wrap(x0 + 1, cx), y1 = wrap((y >> 1) + 1, cy) * cx, z1 = wrap((z >> 1) + 1, cz) * cx * cy;
+  const double a = phic[x0 + y0 + z0];
+  if (y & z & 1) {
+    const double s = ((a + phic[x1 + y0 + z0]) + (phic[x0 + y1 + z0] + phic[x1 + y1 + z0])) +
+                     ((phic[x0 + y0 + z1] + phic[x1 + y0 + z1]) + (phic[x0 + y1 + z1] + phic[x1 + y1 + z1]));
+    phif[i] = fma(0.125, s, phif[i]);
+  } else {
+    const double o = phic[(x & 1) ? x1 + y0 + z0 : (y & 1) ? x0 + y1 + z0 : x0 + y0 + z1];
+    phif[i] = fma(0.5, a + o, phif[i]);
   }
-  if (threadIdx.x == 0) part[blockIdx.x] = sh[0];
 }
 
-__global__ void k_max_final(const double* part, int nblk, double* out) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  double m = 0.0;
-  for (int i = 0; i < nblk; ++i) m = fmax(m, part[i]);
-  out[0] = m;
-}
-
-// phi -= mean phi (sums[1])
-__global__ void k_sub_mean(double* phi, long long n, const double* sums) {
+// phi -= its mean
+__global__ void __launch_bounds__(MG_T) k_sub_mean(double* phi, long long n, const Scalars* sc) {
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
-  phi[i] -= sums[1];
+  phi[i] -= sc->mean;
 }
 
 unsigned blocks(long long n) { return (unsigned)((n + MG_T - 1) / MG_T); }
@@ -191,7 +252,7 @@ size_t align256(size_t b) { return (b + 255) & ~(size_t)255; }
 // long as the level holds more than MG_COARSE nodes
 std::vector<Level> make_levels(int nx, int ny, int nz) {
   std::vector<Level> lv;
-  Level l{nx, ny, nz, (long long)nx * ny * nz, 1.0, nullptr, nullptr, nullptr};
+  Level l{nx, ny, nz, (long long)nx * ny * nz, nullptr, nullptr, nullptr};
   lv.push_back(l);
   while (l.n > MG_COARSE && l.nx % 4 == 0 && l.ny % 2 == 0 && l.nz % 2 == 0 && l.nx >= 16 &&
          l.ny >= 16 && l.nz >= 16) {
@@ -199,7 +260,6 @@ std::vector<Level> make_levels(int nx, int ny, int nz) {
     l.ny /= 2;
     l.nz /= 2;
     l.n = (long long)l.nx * l.ny * l.nz;
-    l.c /= 4.0;
     lv.push_back(l);
   }
   return lv;
@@ -233,56 +293,77 @@ struct Solver {
   std::vector<Level> lv;
   PoissonPlan coarse_plan;
   double2* spectrum;
-  double* part;   // MG_RED_BLOCKS partial results
-  double* out;    // [0] sum or maximum
+  double* part;   // MG_RED_BLOCKS partial sums
+  Scalars* sc;
   cudaStream_t s;
 };
 
-cudaError_t sum_of(const Solver& S, const double* x, long long n) {
+cudaError_t mean_of(const Solver& S, const double* x, long long n) {
   const int nb = (int)std::min<long long>(MG_RED_BLOCKS, (n + MG_T - 1) / MG_T);
-  k_sum_partial<<<nb, MG_T, 0, S.s>>>(x, n, S.part);
-  k_sum_final<<<1, 32, 0, S.s>>>(S.part, nb, n, S.out);
+  k_mg_sum<<<nb, MG_T, 0, S.s>>>(x, n, S.part, S.sc);
   return cudaGetLastError();
 }
 
-cudaError_t absmax_of(const Solver& S, const double* x, long long n, double& host) {
-  const int nb = (int)std::min<long long>(MG_RED_BLOCKS, (n + MG_T - 1) / MG_T);
-  k_absmax_partial<<<nb, MG_T, 0, S.s>>>(x, n, S.part);
-  k_max_final<<<1, 32, 0, S.s>>>(S.part, nb, S.out);
-  cudaError_t e = cudaMemcpyAsync(&host, S.out, sizeof(double), cudaMemcpyDeviceToHost, S.s);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(S.s);
-  return e;
+void half(const Solver& S, const Level& l, int colour) {
+  k_mg_half<<<blocks(l.n / 2), MG_T, 0, S.s>>>(l.phi, l.b, l.nx, l.ny, l.nz, colour);
+}
+void restrict_to(const Solver& S, const Level& l, const Level& c) {
+  k_mg_restrict<<<blocks(c.n), MG_T, 0, S.s>>>(l.r, l.nx, l.ny, l.nz, c.b, c.phi);
+}
+void prolong_to(const Solver& S, const Level& l, const Level& c) {
+  k_mg_prolong<<<blocks(l.n / 2), MG_T, 0, S.s>>>(c.phi, l.nx, l.ny, l.nz, l.phi);
 }
 
-cudaError_t smooth(const Solver& S, const Level& l) {
-  for (int sweep = 0; sweep < 2; ++sweep)
-    for (int colour = 0; colour < 2; ++colour)
-      k_mg_rbgs<<<blocks(l.n / 2), MG_T, 0, S.s>>>(l.phi, l.b, l.nx, l.ny, l.nz, 1.0 / l.c, colour);
-  return cudaGetLastError();
-}
-
-// one V-cycle from level k down
+// one V-cycle from level k >= 1 down, from zero; the red nodes have had their
+// first half sweep
 cudaError_t vcycle(const Solver& S, size_t k) {
   const Level& l = S.lv[k];
   if (k + 1 == S.lv.size()) {
-    // exact on the coarsest level: c (6 phi - sum nb) = b is the FFT
-    // solver's problem with 4 pi l_B = 1 / c
+    // exact on the coarsest level: 6 phi - sum nb = 6 b is the FFT solver's
+    // problem with 4 pi l_B = 6
     Phys ph;
     memset(&ph, 0, sizeof(ph));
-    ph.bjerrum = 1.0 / (4.0 * M_PI * l.c);
+    ph.bjerrum = 6.0 / (4.0 * M_PI);
     return poisson_solve(S.coarse_plan, l.b, nullptr, nullptr, nullptr, ph, l.phi, S.spectrum, S.s);
   }
-  const Level& c = S.lv[k + 1];
-  cudaError_t e = smooth(S, l);
+  half(S, l, 1);
+  half(S, l, 0);
+  half(S, l, 1);
+  k_mg_resid<false><<<blocks(l.n / 2), MG_T, 0, S.s>>>(l.phi, l.b, l.r, l.nx, l.ny, l.nz, S.sc);
+  restrict_to(S, l, S.lv[k + 1]);
+  cudaError_t e = vcycle(S, k + 1);
   if (e != cudaSuccess) return e;
-  k_mg_resid<<<blocks(l.n), MG_T, 0, S.s>>>(l.phi, l.b, l.r, l.nx, l.ny, l.nz, l.c);
-  k_mg_restrict<<<blocks(c.n), MG_T, 0, S.s>>>(l.r, l.nx, l.ny, l.nz, c.b, c.phi);
-  e = cudaGetLastError();
-  if (e == cudaSuccess) e = vcycle(S, k + 1);
-  if (e != cudaSuccess) return e;
-  k_mg_prolong_add<<<blocks(l.n), MG_T, 0, S.s>>>(c.phi, l.nx, l.ny, l.nz, l.phi);
-  return smooth(S, l);
+  prolong_to(S, l, S.lv[k + 1]);
+  for (int sweep = 0; sweep < 2; ++sweep) {
+    half(S, l, 0);
+    half(S, l, 1);
+  }
+  return cudaGetLastError();
 }
+
+// the device's maximum, read on a stream of its own once `ready` has passed,
+// while the solve's stream goes on
+struct Reader {
+  cudaStream_t s = nullptr;
+  cudaEvent_t ready = nullptr;
+  cudaError_t open() {
+    cudaError_t e = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking);
+    return e != cudaSuccess ? e : cudaEventCreateWithFlags(&ready, cudaEventDisableTiming);
+  }
+  ~Reader() {
+    if (ready) cudaEventDestroy(ready);
+    if (s) cudaStreamDestroy(s);
+  }
+  cudaError_t mark(cudaStream_t from) { return cudaEventRecord(ready, from); }
+  cudaError_t read(const Scalars* sc, double& v) {
+    unsigned long long bits = 0;
+    cudaError_t e = cudaStreamWaitEvent(s, ready, 0);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&bits, &sc->max, sizeof(bits), cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    memcpy(&v, &bits, sizeof(v));
+    return e;
+  }
+};
 
 }  // namespace
 
@@ -309,31 +390,85 @@ cudaError_t poisson_solve_mg(const PoissonPlan& coarse_plan, const double* q, do
   S.coarse_plan = coarse_plan;
   S.spectrum = reinterpret_cast<double2*>(base + L.spectrum);
   S.part = reinterpret_cast<double*>(base + L.red);
-  S.out = S.part + MG_RED_BLOCKS;
+  S.sc = reinterpret_cast<Scalars*>(S.part + MG_RED_BLOCKS);
   S.s = s;
-  const Level& f = S.lv[0];
-  // b = 4 pi l_B (q - mean q), read before phi (which may alias q) is written
-  cudaError_t e = sum_of(S, q, f.n);
+  Reader rd;
+  cudaError_t e = rd.open();
   if (e != cudaSuccess) return e;
-  k_mg_rhs<<<blocks(f.n), MG_T, 0, s>>>(q, f.b, f.n, 4.0 * M_PI * bjerrum, S.out);
-  e = cudaMemsetAsync(phi, 0, f.n * sizeof(double), s);
+  const Level& f = S.lv[0];
+  auto clear_max = [&]() { return cudaMemsetAsync(&S.sc->max, 0, sizeof(S.sc->max), s); };
+  // the maximum so far, as soon as the kernels launched until now have run
+  auto read_max = [&](double& v) -> cudaError_t {
+    cudaError_t r = cudaGetLastError();
+    if (r == cudaSuccess) r = rd.mark(s);
+    return r != cudaSuccess ? r : rd.read(S.sc, v);
+  };
+  e = cudaMemsetAsync(S.sc, 0, sizeof(Scalars), s);
+  // b = 4 pi l_B (q - mean q)
+  if (e == cudaSuccess) e = mean_of(S, q, f.n);
+  if (e != cudaSuccess) return e;
+  k_mg_rhs<<<blocks(f.n), MG_T, 0, s>>>(q, phi, f.b, f.nx, f.ny, f.nz, 4.0 * M_PI * bjerrum, S.sc);
   double bmax = 0.0, rmax = 0.0;
-  if (e == cudaSuccess) e = absmax_of(S, f.b, f.n, bmax);
+  e = read_max(bmax);
   if (e != cudaSuccess) return e;
   int done = 0;
-  while (bmax > 0.0 && done < max_cycles) {
-    e = vcycle(S, 0);
-    if (e != cudaSuccess) return e;
-    ++done;
-    k_mg_resid<<<blocks(f.n), MG_T, 0, s>>>(f.phi, f.b, f.r, f.nx, f.ny, f.nz, f.c);
-    e = absmax_of(S, f.r, f.n, rmax);
-    if (e != cudaSuccess) return e;
-    if (rmax <= tol * bmax) break;
+  if (S.lv.size() == 1 && bmax > 0.0) {
+    // a box that cannot be coarsened: the FFT, in as many cycles as the caller
+    // allows until its residual is below the tolerance (one)
+    while (done < max_cycles) {
+      Phys ph;
+      memset(&ph, 0, sizeof(ph));
+      ph.bjerrum = 6.0 / (4.0 * M_PI);
+      e = poisson_solve(S.coarse_plan, f.b, nullptr, nullptr, nullptr, ph, phi, S.spectrum, s);
+      if (e == cudaSuccess) e = clear_max();
+      if (e != cudaSuccess) return e;
+      ++done;
+      k_mg_resid_max<<<blocks(f.n), MG_T, 0, s>>>(f.phi, f.b, f.nx, f.ny, f.nz, S.sc);
+      e = read_max(rmax);
+      if (e != cudaSuccess) return e;
+      if (rmax <= tol * bmax) break;
+    }
+  } else if (bmax > 0.0) {
+    half(S, f, 1);  // the first sweep's black half
+    for (;;) {
+      e = clear_max();
+      if (e != cudaSuccess) return e;
+      k_mg_resid<true><<<blocks(f.n / 2), MG_T, 0, s>>>(f.phi, f.b, f.r, f.nx, f.ny, f.nz, S.sc);
+      e = rd.mark(s);
+      // the coarse correction does not touch phi: it runs while the host waits
+      // for the residual (and for nothing when that has converged)
+      const bool more = done < max_cycles;
+      if (e == cudaSuccess && more) {
+        restrict_to(S, f, S.lv[1]);
+        e = vcycle(S, 1);
+      }
+      if (e == cudaSuccess && done > 0) e = rd.read(S.sc, rmax);
+      if (e != cudaSuccess) return e;
+      if (done > 0 && (!more || rmax <= tol * bmax)) {
+        // the red nodes have converged (or no cycle is left): over all nodes
+        e = clear_max();
+        if (e != cudaSuccess) return e;
+        k_mg_resid_max<<<blocks(f.n), MG_T, 0, s>>>(f.phi, f.b, f.nx, f.ny, f.nz, S.sc);
+        e = read_max(rmax);
+        if (e != cudaSuccess) return e;
+        if (!more || rmax <= tol * bmax) break;
+      }
+      prolong_to(S, f, S.lv[1]);
+      for (int sweep = 0; sweep < 4; ++sweep) {
+        half(S, f, 0);
+        half(S, f, 1);
+      }
+      ++done;
+    }
   }
   // the zero-mean solution (the periodic problem fixes phi up to a constant)
-  e = sum_of(S, phi, f.n);
+  if (bmax == 0.0) {
+    e = cudaMemsetAsync(phi, 0, f.n * sizeof(double), s);
+    if (e != cudaSuccess) return e;
+  }
+  e = mean_of(S, phi, f.n);
   if (e != cudaSuccess) return e;
-  k_sub_mean<<<blocks(f.n), MG_T, 0, s>>>(phi, f.n, S.out);
+  k_sub_mean<<<blocks(f.n), MG_T, 0, s>>>(phi, f.n, S.sc);
   e = cudaGetLastError();
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (cycles) *cycles = done;
