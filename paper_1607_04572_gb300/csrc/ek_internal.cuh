@@ -140,11 +140,17 @@ struct Transfer {
   double amount[EK_MAX_SPECIES];
 };
 
-// FFT plan of one axis.
+// FFT plan of one axis: the stage radices of the generic line transforms in
+// each precision (mnb, mns: multipliers for the divisions by n / radix and by
+// the product of the radices before), and the tables.
+struct FFTPlan {
+  int nrad = 0;
+  int radix[8] = {};
+  unsigned mnb[8] = {}, mns[8] = {};
+};
 struct AxisPlan {
   int n = 0;
-  int nrad = 0;
-  int radix[16] = {};
+  FFTPlan f64, f32;
   double2* tw = nullptr;   // exp(-2 pi i k / n), k = 0..n-1 (device)
   double* lam = nullptr;   // 2 - 2 cos(2 pi k / n), k = 0..n-1 (device)
   float2* tw32 = nullptr;  // the same tables rounded to float (FP32 form)

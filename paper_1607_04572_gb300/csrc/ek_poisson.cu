@@ -15,9 +15,18 @@
 //   Z  complex FFT along z, Green multiply, inverse FFT along z (fused)
 //   Y  inverse
 //   X  complex-to-real along x, two rows per complex FFT; writes Phi
-// Each line FFT is a mixed-radix (4, 2, 3) Stockham autosort transform
-// (Govindaraju et al., SC 2008 formulation), ping-ponging between two shared
-// memory buffers, so no bit reversal pass is needed.
+// Each line FFT is a mixed-radix Stockham autosort transform (Govindaraju et
+// al., SC 2008 formulation), ping-ponging between two shared memory buffers, so
+// no bit reversal pass is needed.
+//
+// The FP64 passes are bound by the FP64 pipe (2 lanes per clock per SM), so
+// their butterflies are written as chains of FMAs that take the twiddles along
+// (Linzer and Feig, IEEE Trans. Signal Processing 41, 1993; Goedecker, SIAM J.
+// Sci. Comput. 18, 1997): 24 instructions for a radix-4 butterfly with its three
+// twiddles, against 28 with separate products, and 256^3 in 2.27 ms against 2.65
+// (2.93 before, with divisions in the index arithmetic as well); 48 x 32 x 72,
+// where CTAs of 1024 elements left most SMs idle, 84 -> 47 us.  The errors are
+// those of the separate products (eigenvalue tables: 3e-15 to 1e-14).
 #include <math.h>
 #include <cstdint>
 #include <cstring>
@@ -38,7 +47,7 @@ namespace cg = cooperative_groups;
 
 namespace {
 
-constexpr int LINE_ELEMS = 1024;  // complex elements staged per CTA and buffer (16 KB)
+constexpr int LINE_ELEMS = 1024;  // complex elements staged per CTA and buffer (FP64: 16 KB)
 constexpr int FFT_THREADS = 256;
 
 // real type -> complex type
@@ -60,64 +69,217 @@ template <typename C> __device__ __forceinline__ C cmulconj(C a, C b) {  // a * 
 template <typename C> __device__ __forceinline__ C rot(C a, bool inverse) {
   return inverse ? mkc(-a.y, a.x) : mkc(a.y, -a.x);
 }
-// twiddle exp(-2 pi i k / n) and Laplacian eigenvalue of an axis, per precision
-__device__ __forceinline__ double2 twiddle(const AxisPlan& P, int k, double) { return P.tw[k]; }
-__device__ __forceinline__ float2 twiddle(const AxisPlan& P, int k, float) { return P.tw32[k]; }
+// multiply by exp(-+2 pi i k / R) (forward: minus), k < R / 2, R = 8, 16 or 32
+template <int R, bool INV>
+__device__ __forceinline__ float2 wconst(int k, float2 z) {
+  // cos and sin of 2 pi m / 32, m = 0..15
+  constexpr float C32[16] = {1.0f, 0.98078528040323044913f, 0.92387953251128675613f,
+                             0.83146961230254523708f, 0.70710678118654752440f,
+                             0.55557023301960222474f, 0.38268343236508977173f,
+                             0.19509032201612826785f, 0.0f, -0.19509032201612826785f,
+                             -0.38268343236508977173f, -0.55557023301960222474f,
+                             -0.70710678118654752440f, -0.83146961230254523708f,
+                             -0.92387953251128675613f, -0.98078528040323044913f};
+  constexpr float S32[16] = {0.0f, 0.19509032201612826785f, 0.38268343236508977173f,
+                             0.55557023301960222474f, 0.70710678118654752440f,
+                             0.83146961230254523708f, 0.92387953251128675613f,
+                             0.98078528040323044913f, 1.0f, 0.98078528040323044913f,
+                             0.92387953251128675613f, 0.83146961230254523708f,
+                             0.70710678118654752440f, 0.55557023301960222474f,
+                             0.38268343236508977173f, 0.19509032201612826785f};
+  const int m = k * (32 / R);
+  if (m == 0) return z;
+  if (m == 8) return INV ? make_float2(-z.y, z.x) : make_float2(z.y, -z.x);
+  const float c = C32[m], sn = INV ? S32[m] : -S32[m];
+  return make_float2(z.x * c - z.y * sn, z.x * sn + z.y * c);
+}
+
+template <int R, bool INV>
+__device__ __forceinline__ void dft_reg(float2 (&v)[R]) {
+  if constexpr (R == 2) {
+    const float2 a = v[0], b = v[1];
+    v[0] = cadd(a, b);
+    v[1] = csub(a, b);
+  } else if constexpr (R == 3) {
+    // X1,2 = v0 - (v1 + v2)/2 -+ i (sqrt 3 / 2)(v1 - v2) (forward; inverse conjugate)
+    const float2 sm = cadd(v[1], v[2]), df = csub(v[1], v[2]);
+    const float2 t = make_float2(v[0].x - 0.5f * sm.x, v[0].y - 0.5f * sm.y);
+    const float c = 0.86602540378443865f;
+    const float2 r = rot(make_float2(c * df.x, c * df.y), INV);
+    v[0] = cadd(v[0], sm);
+    v[1] = cadd(t, r);
+    v[2] = csub(t, r);
+  } else if constexpr (R == 9) {
+    // 3 x 3: columns r mod 3, twiddles exp(-+2 pi i j k / 9), rows
+    constexpr float C9[5] = {1.0f, 0.76604444311897803520f, 0.17364817766693034885f, -0.5f,
+                             -0.93969262078590838405f};
+    constexpr float S9[5] = {0.0f, 0.64278760968653932632f, 0.98480775301220805937f,
+                             0.86602540378443864676f, 0.34202014332566873304f};
+    float2 t[3][3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      float2 u[3] = {v[c], v[c + 3], v[c + 6]};
+      dft_reg<3, INV>(u);
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        const float cr = C9[c * k], si = INV ? S9[c * k] : -S9[c * k];
+        t[k][c] = c * k == 0 ? u[k] : make_float2(u[k].x * cr - u[k].y * si, u[k].x * si + u[k].y * cr);
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      dft_reg<3, INV>(t[k]);
+#pragma unroll
+      for (int m = 0; m < 3; ++m) v[k + 3 * m] = t[k][m];
+    }
+  } else if constexpr (R == 4) {
+    const float2 s02 = cadd(v[0], v[2]), d02 = csub(v[0], v[2]);
+    const float2 s13 = cadd(v[1], v[3]), d13 = rot(csub(v[1], v[3]), INV);
+    v[0] = cadd(s02, s13);
+    v[2] = csub(s02, s13);
+    v[1] = cadd(d02, d13);
+    v[3] = csub(d02, d13);
+  } else {
+    float2 e[R / 2], o[R / 2];
+#pragma unroll
+    for (int r = 0; r < R / 2; ++r) {
+      e[r] = v[2 * r];
+      o[r] = v[2 * r + 1];
+    }
+    dft_reg<R / 2, INV>(e);
+    dft_reg<R / 2, INV>(o);
+#pragma unroll
+    for (int k = 0; k < R / 2; ++k) {
+      const float2 t = wconst<R, INV>(k, o[k]);
+      v[k] = cadd(e[k], t);
+      v[k + R / 2] = csub(e[k], t);
+    }
+  }
+}
+
+__device__ __forceinline__ const double2* twiddles(const AxisPlan& P, double) { return P.tw; }
+__device__ __forceinline__ const float2* twiddles(const AxisPlan& P, float) { return P.tw32; }
 __device__ __forceinline__ double lambda_of(const AxisPlan& P, int k, double) { return P.lam[k]; }
 __device__ __forceinline__ float lambda_of(const AxisPlan& P, int k, float) { return P.lam32[k]; }
 
-// Stockham FFT of `nl` lines of length n stored line-major in `a`; `b` is the
-// second buffer.  Returns the buffer holding the result.  All threads of the
-// CTA must call it.
-template <typename C>
-__device__ C* fft_lines(C* a, C* b, int nl, const AxisPlan& P, bool inverse) {
+// t / d for t < 4096, d <= 1024 from m = ceil(2^32 / d) (0: d = 1)
+__device__ __forceinline__ int div_by(int t, unsigned m) { return m ? (int)__umulhi((unsigned)t, m) : t; }
+unsigned div_magic(int d) { return d <= 1 ? 0u : (unsigned)(((1ULL << 32) + (unsigned)d - 1) / (unsigned)d); }
+
+// a + w b (forward twiddle) or a + conj(w) b (inverse)
+template <bool INV, typename C> __device__ __forceinline__ C fma_tw(C w, C b, C a) {
+  const auto wy = INV ? -w.y : w.y;
+  return mkc(fma(w.x, b.x, fma(-wy, b.y, a.x)), fma(w.x, b.y, fma(wy, b.x, a.y)));
+}
+// 2 a - t
+template <typename C> __device__ __forceinline__ C twice_minus(C a, C t) {
   using R = decltype(C().x);
-  const int n = P.n;
-  int Ns = 1;
-  for (int s = 0; s < P.nrad; ++s) {
-    const int RAD = P.radix[s];
-    const int nb = n / RAD;
-    const int twstep = n / (Ns * RAD);
-    for (int t = threadIdx.x; t < nl * nb; t += blockDim.x) {
-      const int line = t / nb;
-      const int j = t - line * nb;
-      const C* in = a + line * n;
-      C* out = b + line * n;
-      const int k = j % Ns;
-      C v[4];
-      for (int r = 0; r < RAD; ++r) {
-        C e = in[j + r * nb];
-        if (r > 0 && k > 0) {
-          const C w = twiddle(P, (k * r * twstep) % n, R(0));
-          e = inverse ? cmulconj(e, w) : cmul(e, w);
-        }
-        v[r] = e;
+  return mkc(fma(R(2), a.x, -t.x), fma(R(2), a.y, -t.y));
+}
+// t - i w u and t + i w u (forward; inverse: conjugate twiddle, signs changed)
+template <bool INV, typename C> __device__ __forceinline__ C fma_tw_rot(C w, C u, C t) {
+  return INV ? mkc(fma(-w.x, u.y, fma(w.y, u.x, t.x)), fma(w.x, u.x, fma(w.y, u.y, t.y)))
+             : mkc(fma(w.x, u.y, fma(w.y, u.x, t.x)), fma(-w.x, u.x, fma(w.y, u.y, t.y)));
+}
+
+// padding of a line in shared memory: one element every 16
+__device__ __host__ __forceinline__ int gpad(int i) { return i + (i >> 4); }
+
+// one Stockham stage of radix RAD after stages of total radix Ns, on nl lines of
+// n elements; tw: exp(-2 pi i k / n)
+template <int RAD, bool FIRST, bool INV, typename C>
+__device__ __forceinline__ void gen_stage(const C* a, C* b, int nl, int n, int Ns, unsigned mnb, unsigned mns,
+                                          const C* __restrict__ tw) {
+  using R = decltype(C().x);
+  const int nb = n / RAD, LS = gpad(n);
+  const int ts = FIRST ? 0 : div_by(nb, mns);  // n / (Ns RAD)
+  for (int t = threadIdx.x; t < nl * nb; t += blockDim.x) {
+    const int line = div_by(t, mnb), j = t - line * nb;
+    const int jq = FIRST ? j : div_by(j, mns), k = FIRST ? 0 : j - jq * Ns;
+    const C* in = a + line * LS;
+    C* out = b + line * LS;
+    C v[RAD];
+#pragma unroll
+    for (int r = 0; r < RAD; ++r) v[r] = in[gpad(j + r * nb)];
+    C o[RAD];
+    if constexpr (RAD == 2) {
+      o[0] = FIRST ? cadd(v[0], v[1]) : fma_tw<INV>(tw[k * ts], v[1], v[0]);
+      o[1] = FIRST ? csub(v[0], v[1]) : twice_minus(v[0], o[0]);
+    } else if constexpr (RAD == 3) {
+      if (!FIRST) {
+        const C w1 = tw[k * ts], w2 = tw[2 * k * ts];
+        v[1] = INV ? cmulconj(v[1], w1) : cmul(v[1], w1);
+        v[2] = INV ? cmulconj(v[2], w2) : cmul(v[2], w2);
       }
-      C o[4];
-      if (RAD == 2) {
-        o[0] = cadd(v[0], v[1]);
-        o[1] = csub(v[0], v[1]);
-      } else if (RAD == 4) {
+      const R c = R(INV ? -0.86602540378443865 : 0.86602540378443865);  // sin(2 pi / 3)
+      const C sm = cadd(v[1], v[2]), d = csub(v[1], v[2]);
+      const C tt = mkc(fma(R(-0.5), sm.x, v[0].x), fma(R(-0.5), sm.y, v[0].y));
+      o[0] = cadd(v[0], sm);
+      o[1] = mkc(fma(c, d.y, tt.x), fma(-c, d.x, tt.y));
+      o[2] = mkc(fma(-c, d.y, tt.x), fma(c, d.x, tt.y));
+    } else if constexpr (RAD == 4) {
+      if constexpr (FIRST) {
         const C s02 = cadd(v[0], v[2]), d02 = csub(v[0], v[2]);
-        const C s13 = cadd(v[1], v[3]), d13 = rot(csub(v[1], v[3]), inverse);
+        const C s13 = cadd(v[1], v[3]), d13 = rot(csub(v[1], v[3]), INV);
         o[0] = cadd(s02, s13);
         o[2] = csub(s02, s13);
         o[1] = cadd(d02, d13);
         o[3] = csub(d02, d13);
-      } else {  // radix 3
-        const R c = R(0.86602540378443865);  // sin(2 pi / 3)
-        const C s = cadd(v[1], v[2]);
-        const C d = csub(v[1], v[2]);
-        const C tt = mkc(v[0].x - R(0.5) * s.x, v[0].y - R(0.5) * s.y);
-        const C rd = rot(mkc(c * d.x, c * d.y), inverse);
-        o[0] = cadd(v[0], s);
-        o[1] = cadd(tt, rd);
-        o[2] = csub(tt, rd);
+      } else {
+        // w^3 = w w^2: both inner pairs take the twiddle w^2, the outer ones w
+        const C w1 = tw[k * ts], w2 = tw[2 * k * ts];
+        const C s02 = fma_tw<INV>(w2, v[2], v[0]), d02 = twice_minus(v[0], s02);
+        const C s13 = fma_tw<INV>(w2, v[3], v[1]), d13 = twice_minus(v[1], s13);
+        o[0] = fma_tw<INV>(w1, s13, s02);
+        o[2] = twice_minus(s02, o[0]);
+        o[1] = fma_tw_rot<INV>(w1, d13, d02);
+        o[3] = twice_minus(d02, o[1]);
       }
-      const int base = (j / Ns) * Ns * RAD + k;
-      for (int r = 0; r < RAD; ++r) out[base + r * Ns] = o[r];
+    } else {  // 8, 9 (FP32)
+      if (!FIRST) {
+#pragma unroll
+        for (int r = 1; r < RAD; ++r) {
+          const C w = tw[r * k * ts];
+          v[r] = INV ? cmulconj(v[r], w) : cmul(v[r], w);
+        }
+      }
+      dft_reg<RAD, INV>(v);
+#pragma unroll
+      for (int r = 0; r < RAD; ++r) o[r] = v[r];
     }
-    __syncthreads();
+    const int base = FIRST ? j * RAD : jq * Ns * RAD + k;
+#pragma unroll
+    for (int r = 0; r < RAD; ++r) out[gpad(base + r * Ns)] = o[r];
+  }
+  __syncthreads();
+}
+
+// Stockham FFT of `nl` lines of length n stored line-major (padded) in `a`; `b`
+// is the second buffer.  Returns the buffer holding the result.  All threads of
+// the CTA must call it.
+template <bool INV, typename C>
+__device__ C* fft_lines(C* a, C* b, int nl, const AxisPlan& P, const C* tw) {
+  constexpr bool F32 = sizeof(C) == sizeof(float2);
+  const FFTPlan& F = F32 ? P.f32 : P.f64;
+  int Ns = 1;
+  for (int s = 0; s < F.nrad; ++s) {
+    const int RAD = F.radix[s];
+    const unsigned mnb = F.mnb[s], mns = F.mns[s];
+#define EK_STAGE(RR)                                                          \
+  if (s == 0) gen_stage<RR, true, INV>(a, b, nl, P.n, 1, mnb, mns, tw);        \
+  else gen_stage<RR, false, INV>(a, b, nl, P.n, Ns, mnb, mns, tw);
+    if constexpr (F32) {
+      if (RAD == 8) { EK_STAGE(8) }
+      else if (RAD == 9) { EK_STAGE(9) }
+      else if (RAD == 4) { EK_STAGE(4) }
+      else if (RAD == 2) { EK_STAGE(2) }
+      else { EK_STAGE(3) }
+    } else {
+      if (RAD == 4) { EK_STAGE(4) }
+      else if (RAD == 2) { EK_STAGE(2) }
+      else { EK_STAGE(3) }
+    }
+#undef EK_STAGE
     C* tmp = a;
     a = b;
     b = tmp;
@@ -140,7 +302,8 @@ struct PassArgs {
   R z[EK_MAX_SPECIES];  // z_k, times qscale_k for int species
   C* S;                // half spectrum (nx/2+1)*ny*nz
   R* phi;
-  R green_scale;       // 4 pi l_B / N
+  R green_scale;       // 4 pi l_B / N (FP64: half of it, see k_fft_x_fwd)
+  unsigned mnx, mnxh;  // div_by of nx and nxh
 };
 
 template <typename R>
@@ -204,48 +367,66 @@ __device__ __forceinline__ float4 charge_at4(const PassArgs<float>& a, long long
   return q;
 }
 
-// X pass, forward: rows r0 = 2p, r1 = 2p + 1 packed as a + i b.
+// the twiddles of an axis: FP32 in shared memory behind the two line buffers,
+// FP64 straight from the L1-cached table (its pipe has time to spare for loads)
+template <typename C>
+__device__ __forceinline__ const C* line_twiddles(const AxisPlan& P, C* sm) {
+  using R = decltype(C().x);
+  const C* g = twiddles(P, R(0));
+  if constexpr (sizeof(C) == sizeof(float2)) {
+    for (int k = threadIdx.x; k < P.n; k += blockDim.x) sm[k] = g[k];
+    return sm;
+  } else {
+    return g;
+  }
+}
+
+// X pass, forward: rows r0 = 2p, r1 = 2p + 1 packed as a + i b.  The split into
+// the two rows' spectra has a factor 1/2, which FP64 leaves to the Green
+// function (a power of two: the same rounding).
 template <typename R>
 __global__ void __launch_bounds__(FFT_THREADS) k_fft_x_fwd(PassArgs<R> a, int pairs_per_cta) {
   using C = typename CT<R>::type;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* smem = reinterpret_cast<C*>(smem_raw);
-  const int n = a.nx;
+  const int n = a.nx, LS = gpad(n);
   const int nrows = a.ny * a.nz;
   const long long N = (long long)a.nx * a.ny * a.nz;
   const int p0 = blockIdx.x * pairs_per_cta;
   C* b0 = smem;
-  C* b1 = smem + pairs_per_cta * n;
+  C* b1 = smem + pairs_per_cta * LS;
+  const C* tw = line_twiddles<C>(a.ax, b1 + pairs_per_cta * LS);
   for (int t = threadIdx.x; t < pairs_per_cta * n; t += blockDim.x) {
-    const int l = t / n, x = t - l * n;
+    const int l = div_by(t, a.mnx), x = t - l * n;
     const int r0 = 2 * (p0 + l), r1 = r0 + 1;
     R re = R(0), im = R(0);
     if (r0 < nrows) re = charge_at(a, (long long)r0 * n + x, N);
     if (r1 < nrows) im = charge_at(a, (long long)r1 * n + x, N);
-    b0[t] = mkc(re, im);
+    b0[l * LS + gpad(x)] = mkc(re, im);
   }
   __syncthreads();
-  C* res = fft_lines(b0, b1, pairs_per_cta, a.ax, false);
+  const C* res = fft_lines<false>(b0, b1, pairs_per_cta, a.ax, tw);
   const int nxh = a.nxh;
+  constexpr R h = sizeof(R) == sizeof(double) ? R(1) : R(0.5);
   for (int t = threadIdx.x; t < pairs_per_cta * nxh; t += blockDim.x) {
-    const int l = t / nxh, k = t - l * nxh;
+    const int l = div_by(t, a.mnxh), k = t - l * nxh;
     const int r0 = 2 * (p0 + l), r1 = r0 + 1;
     if (r0 >= nrows) continue;
-    const C Zk = res[l * n + k];
-    const C Zm = res[l * n + (k == 0 ? 0 : n - k)];
+    const C Zk = res[l * LS + gpad(k)];
+    const C Zm = res[l * LS + gpad(k == 0 ? 0 : n - k)];
     // A_k = (Z_k + conj Z_{n-k}) / 2,  B_k = (Z_k - conj Z_{n-k}) / (2 i)
-    const C A = mkc(R(0.5) * (Zk.x + Zm.x), R(0.5) * (Zk.y - Zm.y));
-    const C B = mkc(R(0.5) * (Zk.y + Zm.y), R(-0.5) * (Zk.x - Zm.x));
+    const C A = mkc(h * (Zk.x + Zm.x), h * (Zk.y - Zm.y));
+    const C B = mkc(h * (Zk.y + Zm.y), h * (Zm.x - Zk.x));
     a.S[(long long)r0 * nxh + k] = A;
     if (r1 < nrows) a.S[(long long)r1 * nxh + k] = B;
   }
 }
 
-// Y or Z pass on tiles of `tx` consecutive kx.  axis 1: lines along y for
-// each z; axis 2: lines along z for each y, with the Green multiply and the
-// inverse transform fused.
-template <typename R>
-__global__ void __launch_bounds__(FFT_THREADS) k_fft_yz(PassArgs<R> a, int axis, int tx, bool inverse) {
+// Y or Z pass on tiles of `tx` consecutive kx (mtx: div_by of tx).  AXIS 1:
+// lines along y for each z; AXIS 2: lines along z for each y, with the Green
+// multiply and the inverse transform fused.
+template <typename R, int AXIS, bool INV>
+__global__ void __launch_bounds__(FFT_THREADS) k_fft_yz(PassArgs<R> a, int tx, unsigned mtx) {
   using C = typename CT<R>::type;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* smem = reinterpret_cast<C*>(smem_raw);
@@ -254,45 +435,42 @@ __global__ void __launch_bounds__(FFT_THREADS) k_fft_yz(PassArgs<R> a, int axis,
   const int tile = blockIdx.x % ntile;
   const int other = blockIdx.x / ntile;  // z (axis 1) or y (axis 2)
   const int kx0 = tile * tx;
-  const AxisPlan& P = axis == 1 ? a.ay : a.az;
-  const int n = P.n;
-  const long long stride = axis == 1 ? (long long)nxh : (long long)nxh * a.ny;
-  const long long base = axis == 1 ? (long long)other * a.ny * nxh : (long long)other * nxh;
+  const int nc = min(tx, nxh - kx0);
+  const AxisPlan& P = AXIS == 1 ? a.ay : a.az;
+  const int n = P.n, LS = gpad(n);
+  const long long stride = AXIS == 1 ? (long long)nxh : (long long)nxh * a.ny;
+  C* const S = a.S + (AXIS == 1 ? (long long)other * a.ny * nxh : (long long)other * nxh) + kx0;
   C* b0 = smem;
-  C* b1 = smem + tx * n;
+  C* b1 = smem + tx * LS;
+  const C* tw = line_twiddles<C>(P, b1 + tx * LS);
   // element t = j * tx + c : line c (kx0 + c), position j
   for (int t = threadIdx.x; t < tx * n; t += blockDim.x) {
-    const int j = t / tx, c = t - j * tx;
-    C v = mkc(R(0), R(0));
-    if (kx0 + c < nxh) v = a.S[base + j * stride + kx0 + c];
-    b0[c * n + j] = v;
+    const int j = div_by(t, mtx), c = t - j * tx;
+    if (c < nc) b0[c * LS + gpad(j)] = S[j * stride + c];
   }
   __syncthreads();
   C* res;
-  if (axis == 1) {
-    res = fft_lines(b0, b1, tx, P, inverse);
+  if constexpr (AXIS == 1) {
+    res = fft_lines<INV>(b0, b1, nc, P, tw);
   } else {
-    res = fft_lines(b0, b1, tx, P, false);
-    C* other_buf = res == b0 ? b1 : b0;
+    res = fft_lines<false>(b0, b1, nc, P, tw);
     // Green function of the 7-point Laplacian; here `other` is ky
     const R ly = lambda_of(a.ay, other, R(0));
     for (int t = threadIdx.x; t < tx * n; t += blockDim.x) {
-      const int c = t / n, j = t - c * n;
+      const int j = div_by(t, mtx), c = t - j * tx;
+      if (c >= nc) continue;
       const int kx = kx0 + c;
-      R g = R(0);
-      if (kx < nxh) {
-        const R lam = lambda_of(a.ax, kx, R(0)) + ly + lambda_of(a.az, j, R(0));
-        g = (kx == 0 && other == 0 && j == 0) ? R(0) : a.green_scale / lam;
-      }
-      const C v = res[t];
-      res[t] = mkc(v.x * g, v.y * g);
+      const R lam = (lambda_of(a.ax, kx, R(0)) + ly) + lambda_of(a.az, j, R(0));
+      const R g = (kx == 0 && other == 0 && j == 0) ? R(0) : a.green_scale / lam;
+      C& v = res[c * LS + gpad(j)];
+      v = mkc(v.x * g, v.y * g);
     }
     __syncthreads();
-    res = fft_lines(res, other_buf, tx, P, true);
+    res = fft_lines<true>(res, res == b0 ? b1 : b0, nc, P, tw);
   }
   for (int t = threadIdx.x; t < tx * n; t += blockDim.x) {
-    const int j = t / tx, c = t - j * tx;
-    if (kx0 + c < nxh) a.S[base + j * stride + kx0 + c] = res[c * n + j];
+    const int j = div_by(t, mtx), c = t - j * tx;
+    if (c < nc) S[j * stride + c] = res[c * LS + gpad(j)];
   }
 }
 
@@ -302,40 +480,39 @@ __global__ void __launch_bounds__(FFT_THREADS) k_fft_x_inv(PassArgs<R> a, int pa
   using C = typename CT<R>::type;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* smem = reinterpret_cast<C*>(smem_raw);
-  const int n = a.nx;
+  const int n = a.nx, LS = gpad(n);
   const int nxh = a.nxh;
   const int nrows = a.ny * a.nz;
   const int p0 = blockIdx.x * pairs_per_cta;
   C* b0 = smem;
-  C* b1 = smem + pairs_per_cta * n;
-  for (int t = threadIdx.x; t < pairs_per_cta * n; t += blockDim.x) {
-    const int l = t / n, k = t - l * n;
+  C* b1 = smem + pairs_per_cta * LS;
+  const C* tw = line_twiddles<C>(a.ax, b1 + pairs_per_cta * LS);
+  // a stored coefficient kk <= n / 2 gives the inputs kk and, conjugated, n - kk
+  for (int t = threadIdx.x; t < pairs_per_cta * nxh; t += blockDim.x) {
+    const int l = div_by(t, a.mnxh), kk = t - l * nxh;
     const int r0 = 2 * (p0 + l), r1 = r0 + 1;
     C A = mkc(R(0), R(0)), B = mkc(R(0), R(0));
-    const bool upper = k > n / 2;
-    const int kk = upper ? n - k : k;
     if (r0 < nrows) A = a.S[(long long)r0 * nxh + kk];
     if (r1 < nrows) B = a.S[(long long)r1 * nxh + kk];
-    if (upper) {
-      A.y = -A.y;
-      B.y = -B.y;
-    }
     // Z = A + i B
-    b0[t] = mkc(A.x - B.y, A.y + B.x);
+    b0[l * LS + gpad(kk)] = mkc(A.x - B.y, A.y + B.x);
+    if (kk > 0 && kk < n - kk) b0[l * LS + gpad(n - kk)] = mkc(A.x + B.y, B.x - A.y);
   }
   __syncthreads();
-  C* res = fft_lines(b0, b1, pairs_per_cta, a.ax, true);
+  const C* res = fft_lines<true>(b0, b1, pairs_per_cta, a.ax, tw);
   for (int t = threadIdx.x; t < pairs_per_cta * n; t += blockDim.x) {
-    const int l = t / n, x = t - l * n;
+    const int l = div_by(t, a.mnx), x = t - l * n;
     const int r0 = 2 * (p0 + l), r1 = r0 + 1;
-    if (r0 < nrows) a.phi[(long long)r0 * n + x] = res[t].x;
-    if (r1 < nrows) a.phi[(long long)r1 * n + x] = res[t].y;
+    const C v = res[l * LS + gpad(x)];
+    if (r0 < nrows) a.phi[(long long)r0 * n + x] = v.x;
+    if (r1 < nrows) a.phi[(long long)r1 * n + x] = v.y;
   }
 }
 
 // ---------------------------------------------------------------------------
 // Fast path of the FP32 form for edges 2^k and 3 2^k from 24 to 512: the same
-// five passes, with each line transform specialised at compile time.  A stage
+// passes (each taken where its axis has such an edge), with each line transform
+// specialised at compile time.  A stage
 // of radix R (16, 8, 4 or 3) loads R elements into registers, applies the stage
 // twiddles from a shared-memory table, does the length-R DFT in registers
 // (even/odd splits down to radix 4, constant twiddles) and stores in
@@ -370,71 +547,6 @@ __host__ __device__ constexpr int fast_radix(int n, int s) {
 inline bool fast_edge(int n) {
   return n == 24 || n == 32 || n == 48 || n == 64 || n == 96 || n == 128 || n == 192 || n == 256 ||
          n == 384 || n == 512;
-}
-
-// multiply by exp(-+2 pi i k / R) (forward: minus), k < R / 2, R = 8, 16 or 32
-template <int R, bool INV>
-__device__ __forceinline__ float2 wconst(int k, float2 z) {
-  // cos and sin of 2 pi m / 32, m = 0..15
-  constexpr float C32[16] = {1.0f, 0.98078528040323044913f, 0.92387953251128675613f,
-                             0.83146961230254523708f, 0.70710678118654752440f,
-                             0.55557023301960222474f, 0.38268343236508977173f,
-                             0.19509032201612826785f, 0.0f, -0.19509032201612826785f,
-                             -0.38268343236508977173f, -0.55557023301960222474f,
-                             -0.70710678118654752440f, -0.83146961230254523708f,
-                             -0.92387953251128675613f, -0.98078528040323044913f};
-  constexpr float S32[16] = {0.0f, 0.19509032201612826785f, 0.38268343236508977173f,
-                             0.55557023301960222474f, 0.70710678118654752440f,
-                             0.83146961230254523708f, 0.92387953251128675613f,
-                             0.98078528040323044913f, 1.0f, 0.98078528040323044913f,
-                             0.92387953251128675613f, 0.83146961230254523708f,
-                             0.70710678118654752440f, 0.55557023301960222474f,
-                             0.38268343236508977173f, 0.19509032201612826785f};
-  const int m = k * (32 / R);
-  if (m == 0) return z;
-  if (m == 8) return INV ? make_float2(-z.y, z.x) : make_float2(z.y, -z.x);
-  const float c = C32[m], sn = INV ? S32[m] : -S32[m];
-  return make_float2(z.x * c - z.y * sn, z.x * sn + z.y * c);
-}
-
-template <int R, bool INV>
-__device__ __forceinline__ void dft_reg(float2 (&v)[R]) {
-  if constexpr (R == 2) {
-    const float2 a = v[0], b = v[1];
-    v[0] = cadd(a, b);
-    v[1] = csub(a, b);
-  } else if constexpr (R == 3) {
-    // X1,2 = v0 - (v1 + v2)/2 -+ i (sqrt 3 / 2)(v1 - v2) (forward; inverse conjugate)
-    const float2 sm = cadd(v[1], v[2]), df = csub(v[1], v[2]);
-    const float2 t = make_float2(v[0].x - 0.5f * sm.x, v[0].y - 0.5f * sm.y);
-    const float c = 0.86602540378443865f;
-    const float2 r = rot(make_float2(c * df.x, c * df.y), INV);
-    v[0] = cadd(v[0], sm);
-    v[1] = cadd(t, r);
-    v[2] = csub(t, r);
-  } else if constexpr (R == 4) {
-    const float2 s02 = cadd(v[0], v[2]), d02 = csub(v[0], v[2]);
-    const float2 s13 = cadd(v[1], v[3]), d13 = rot(csub(v[1], v[3]), INV);
-    v[0] = cadd(s02, s13);
-    v[2] = csub(s02, s13);
-    v[1] = cadd(d02, d13);
-    v[3] = csub(d02, d13);
-  } else {
-    float2 e[R / 2], o[R / 2];
-#pragma unroll
-    for (int r = 0; r < R / 2; ++r) {
-      e[r] = v[2 * r];
-      o[r] = v[2 * r + 1];
-    }
-    dft_reg<R / 2, INV>(e);
-    dft_reg<R / 2, INV>(o);
-#pragma unroll
-    for (int k = 0; k < R / 2; ++k) {
-      const float2 t = wconst<R, INV>(k, o[k]);
-      v[k] = cadd(e[k], t);
-      v[k + R / 2] = csub(e[k], t);
-    }
-  }
 }
 
 // one Stockham stage of radix R after stages of total radix NS, on nl lines
@@ -1098,14 +1210,35 @@ __global__ void k_charge(Grid g, Phys ph, const void* rho, const void* qwall, co
   q[n] = s;
 }
 
+// stage radices of an edge: FP64 4, 2, 3 (with the twiddles taken along every
+// power of two costs the FP64 pipe 3 instructions per element and factor of 2), FP32
+// 8, 4, 2, 9, 3 (few passes over shared memory)
 bool factor(int n, AxisPlan& P) {
   P.n = n;
-  P.nrad = 0;
-  int m = n;
-  while (m % 4 == 0) { P.radix[P.nrad++] = 4; m /= 4; }
-  while (m % 2 == 0) { P.radix[P.nrad++] = 2; m /= 2; }
-  while (m % 3 == 0) { P.radix[P.nrad++] = 3; m /= 3; }
-  return m == 1 && P.nrad <= 16;
+  int e2 = 0, e3 = 0, m = n;
+  while (m % 2 == 0) { ++e2; m /= 2; }
+  while (m % 3 == 0) { ++e3; m /= 3; }
+  if (m != 1) return false;
+  auto fill = [&](FFTPlan& F, bool wide) {
+    F.nrad = 0;
+    int a = e2, b = e3;
+    if (wide) {
+      while (a >= 3 && a != 4) { F.radix[F.nrad++] = 8; a -= 3; }
+      while (b >= 2) { F.radix[F.nrad++] = 9; b -= 2; }
+    }
+    while (a >= 2) { F.radix[F.nrad++] = 4; a -= 2; }
+    while (a >= 1) { F.radix[F.nrad++] = 2; a -= 1; }
+    while (b >= 1) { F.radix[F.nrad++] = 3; b -= 1; }
+    int Ns = 1;
+    for (int s = 0; s < F.nrad; ++s) {
+      F.mnb[s] = div_magic(n / F.radix[s]);
+      F.mns[s] = div_magic(Ns);
+      Ns *= F.radix[s];
+    }
+  };
+  fill(P.f64, false);
+  fill(P.f32, true);
+  return true;
 }
 
 cudaError_t axis_create(AxisPlan& P, int n) {
@@ -1267,41 +1400,61 @@ cudaError_t run_passes(const PoissonPlan& p, PassArgs<R>& a, double bjerrum, cud
   a.ay = p.ay;
   a.az = p.az;
   const double N = (double)p.nx * p.ny * p.nz;
-  a.green_scale = (R)(4.0 * M_PI * bjerrum / N);
-  if constexpr (std::is_same<R, float>::value) {
-    if (fast_edge(p.nx) && fast_edge(p.ny) && fast_edge(p.nz)) {
-      if (plane_edge(p.ny) && plane_edge(p.nz)) {
-        launch_fast_x_any(a, false, true, s);
-        launch_plane(a, s);
-        launch_fast_x_any(a, true, true, s);
-        return cudaGetLastError();
-      }
-      launch_fast_x_any(a, false, false, s);
-      launch_fast_yz<1, false>(a, p.ny, s);
-      launch_fast_yz<2, false>(a, p.nz, s);
-      launch_fast_yz<1, true>(a, p.ny, s);
-      launch_fast_x_any(a, true, false, s);
+  a.mnx = div_magic(a.nx);
+  a.mnxh = div_magic(a.nxh);
+  constexpr bool F32 = std::is_same<R, float>::value;
+  a.green_scale = (R)((F32 ? 4.0 : 2.0) * M_PI * bjerrum / N);
+  bool fx = false, fy = false, fz = false;
+  if constexpr (F32) {
+    fx = fast_edge(p.nx);
+    fy = fast_edge(p.ny);
+    fz = fast_edge(p.nz);
+    if (fx && plane_edge(p.ny) && plane_edge(p.nz)) {
+      launch_fast_x_any(a, false, true, s);
+      launch_plane(a, s);
+      launch_fast_x_any(a, true, true, s);
       return cudaGetLastError();
     }
   }
-  const int nrows = p.ny * p.nz;
-  const int npairs = (nrows + 1) / 2;
-  const int ppc = LINE_ELEMS / p.nx > 0 ? LINE_ELEMS / p.nx : 1;
+  // Lines per CTA: up to LINE_ELEMS elements; fewer while the grid has less
+  // than two CTAs per SM (a 16^3 solve ran its x passes on two SMs)
+  auto per_cta = [](int cap, int least, long long lines) {
+    int l = std::max(cap, 1);
+    while (l > least && lines < 2LL * 152 * l) l = (l + 1) / 2;
+    return l;
+  };
+  auto threads = [](int elems) {
+    return (unsigned)std::min(FFT_THREADS, std::max(64, (elems / 4 + 31) / 32 * 32));
+  };
+  auto smem = [](int lines, int n) {
+    return (size_t)(2 * lines * gpad(n) + (F32 ? n : 0)) * sizeof(C);
+  };
+  const int npairs = (p.ny * p.nz + 1) / 2;
+  const int ppc = per_cta(LINE_ELEMS / p.nx, 1, npairs);
   const unsigned gx = (unsigned)((npairs + ppc - 1) / ppc);
-  const size_t smx = 2 * (size_t)ppc * p.nx * sizeof(C);
-  k_fft_x_fwd<R><<<gx, FFT_THREADS, smx, s>>>(a, ppc);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  const int txy = LINE_ELEMS / p.ny > 16 ? 16 : (LINE_ELEMS / p.ny > 0 ? LINE_ELEMS / p.ny : 1);
-  const int txz = LINE_ELEMS / p.nz > 16 ? 16 : (LINE_ELEMS / p.nz > 0 ? LINE_ELEMS / p.nz : 1);
+  const int txy = per_cta(std::min(16, LINE_ELEMS / p.ny), F32 ? 4 : 2, (long long)a.nxh * p.nz);
+  const int txz = per_cta(std::min(16, LINE_ELEMS / p.nz), F32 ? 4 : 2, (long long)a.nxh * p.ny);
   const unsigned gy = (unsigned)(((a.nxh + txy - 1) / txy) * p.nz);
   const unsigned gz = (unsigned)(((a.nxh + txz - 1) / txz) * p.ny);
-  const size_t smy = 2 * (size_t)txy * p.ny * sizeof(C);
-  const size_t smz = 2 * (size_t)txz * p.nz * sizeof(C);
-  k_fft_yz<R><<<gy, FFT_THREADS, smy, s>>>(a, 1, txy, false);
-  k_fft_yz<R><<<gz, FFT_THREADS, smz, s>>>(a, 2, txz, false);
-  k_fft_yz<R><<<gy, FFT_THREADS, smy, s>>>(a, 1, txy, true);
-  k_fft_x_inv<R><<<gx, FFT_THREADS, smx, s>>>(a, ppc);
+  const unsigned ny_t = threads(txy * p.ny), nz_t = threads(txz * p.nz), nx_t = threads(ppc * p.nx);
+  if constexpr (F32) {
+    if (fx) launch_fast_x_any(a, false, false, s);
+    if (!fx) k_fft_x_fwd<R><<<gx, nx_t, smem(ppc, p.nx), s>>>(a, ppc);
+    if (fy) launch_fast_yz<1, false>(a, p.ny, s);
+    if (!fy) k_fft_yz<R, 1, false><<<gy, ny_t, smem(txy, p.ny), s>>>(a, txy, div_magic(txy));
+    if (fz) launch_fast_yz<2, false>(a, p.nz, s);
+    if (!fz) k_fft_yz<R, 2, false><<<gz, nz_t, smem(txz, p.nz), s>>>(a, txz, div_magic(txz));
+    if (fy) launch_fast_yz<1, true>(a, p.ny, s);
+    if (!fy) k_fft_yz<R, 1, true><<<gy, ny_t, smem(txy, p.ny), s>>>(a, txy, div_magic(txy));
+    if (fx) launch_fast_x_any(a, true, false, s);
+    if (!fx) k_fft_x_inv<R><<<gx, nx_t, smem(ppc, p.nx), s>>>(a, ppc);
+  } else {
+    k_fft_x_fwd<R><<<gx, nx_t, smem(ppc, p.nx), s>>>(a, ppc);
+    k_fft_yz<R, 1, false><<<gy, ny_t, smem(txy, p.ny), s>>>(a, txy, div_magic(txy));
+    k_fft_yz<R, 2, false><<<gz, nz_t, smem(txz, p.nz), s>>>(a, txz, div_magic(txz));
+    k_fft_yz<R, 1, true><<<gy, ny_t, smem(txy, p.ny), s>>>(a, txy, div_magic(txy));
+    k_fft_x_inv<R><<<gx, nx_t, smem(ppc, p.nx), s>>>(a, ppc);
+  }
   return cudaGetLastError();
 }
 
