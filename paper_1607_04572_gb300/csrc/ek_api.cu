@@ -320,10 +320,12 @@ ek_status run_setup(ek_ctx* ctx) {
     const double dmax = sqrt(3.0) * (rmax + ceil(rmax) + FORCE_MARGIN + 2.0) + 1.0;
     ctx->tie_thr = (float)(2.0 * ldexp(dmax + rmax + 1.0, -21) + ldexp(dmax + rmax, -22));
   }
-  // cells per S4 force CTA: FORCE_CHUNK, doubled while the particles still
-  // fill eight waves of 912 CTAs (152 SMs x 6) with the larger chunks
+  // cells per S4 force CTA: FORCE_CHUNK for a few particles; twice that when
+  // those chunks fill two waves of 760 CTAs (152 SMs x 5), and doubled on while
+  // the particles still fill eight waves of 912
   int fcells = FORCE_CHUNK;
-  while (fcells < 8 * FORCE_CHUNK &&
+  if ((long long)ctx->P * ((emax + 2 * fcells - 1) / (2 * fcells)) >= 2LL * 152 * 5) fcells *= 2;
+  while (fcells < 16 * FORCE_CHUNK &&
          (long long)ctx->P * ((emax + 2 * fcells - 1) / (2 * fcells)) >= 8LL * 152 * 6)
     fcells *= 2;
   const int fchunks = (emax + fcells - 1) / fcells;
@@ -465,7 +467,7 @@ ek_status enqueue_stage(ek_ctx* ctx, int stage, cudaEvent_t mid = nullptr) {
     case 4: {
       PartArgs a = part_args(ctx);
       EK_CUDA(launch_particle_forces(a, s));
-      ctx->launches += ctx->P > 0 ? 3 : 0;
+      ctx->launches += ctx->P > 0 ? 1 + assign_kernels(ctx->P) : 0;
       return EK_OK;
     }
     case 5: {
@@ -500,7 +502,7 @@ ek_status enqueue_step(ek_ctx* ctx) {
     EK_CUDA(launch_reflag(pa, true, s, 1));
     EK_CUDA(ctx->fp32 ? launch_advection32(la, s) : launch_advection(la, s));
     EK_CUDA(launch_reflag(pa, true, s, 2));
-    ctx->launches += (ctx->p.nspecies > 0 ? 2 : 1) + 10;
+    ctx->launches += (ctx->p.nspecies > 0 ? 2 : 1) + 8 + assign_kernels(ctx->P);
     return EK_OK;
   }
   if (ctx->P) {
@@ -530,7 +532,7 @@ ek_status enqueue_step(ek_ctx* ctx) {
     EK_CUDA(cudaStreamWaitEvent(s, ctx->ev_part, 0));
     EK_CUDA(launch_reflag(pa, true, s, 2));
     EK_CUDA(cudaStreamWaitEvent(s, ctx->ev_join, 0));
-    ctx->launches += 10;
+    ctx->launches += 8 + assign_kernels(ctx->P);
   }
   return EK_OK;
 }

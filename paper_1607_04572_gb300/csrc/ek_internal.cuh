@@ -431,9 +431,12 @@ struct PartArgs {
 // cells per CTA of the S4 force kernel: FORCE_T threads, each over `fcells /
 // FORCE_T` rows of FORCE_T cells, fcells a multiple of FORCE_CHUNK chosen at
 // set-up (larger when many particles give enough CTAs anyway, so fewer block
-// sums are made); fpart holds P * fchunks * FPART doubles
+// sums are made); fpart holds P * fchunks * FPART doubles.  Few particles leave
+// most SMs idle and wait for the rows of a thread one after another: chunks of
+// 128 / 256 / 512 cells, S4 in us: one sphere R = 8 44.8, 42.3, 45.4; R = 4 31.8,
+// 32.6, 34.2; eight R = 4 48.8, 43.0, 44.8; 64 of R = 5 (256^3) 256 / 512: 167, 130.
 constexpr int FORCE_T = 128;
-constexpr int FORCE_CHUNK = 512;
+constexpr int FORCE_CHUNK = 256;
 // per particle: [0..5] Fh Th (momentum exchange), [6..11] Fs Ts (reaction of
 // the solute force), [12] sum q and [13..15] sum q (r - r_p) of the particle's
 // own charge (the field's force and torque are E and M x E times these),
@@ -445,6 +448,9 @@ constexpr int FPART = 24;
 // integration (after S2), which also clear the assignment keys
 constexpr int S4_ASSIGN = 1, S4_FORCES = 2, S4_ALL = 3;
 cudaError_t launch_particle_forces(const PartArgs& a, cudaStream_t s, int parts = S4_ALL);
+// kernels of the assignment (a single particle owns every node of its widened
+// box: none)
+inline int assign_kernels(int P) { return P > 1 ? 2 : 0; }
 // CTAs per particle that cover its union box (previous and current box)
 int union_chunks(int boxmax);
 // S5; parts: 1 = re-flag, Psi and charge (no species access), 2 = transitions

@@ -85,27 +85,54 @@ __device__ __forceinline__ unsigned nbr32(int d, const Off3& o) {
          (dcz(d) > 0 ? o.Z2 : (dcz(d) < 0 ? o.Z0 : o.Z1));
 }
 
-// block total of the per-thread sums: warps in float (32 threads, each over
-// its segment's nodes), the warp sums in FP64; the GPU's FP64 rate is a small
-// fraction of its FP32 rate, so the per-node accumulation stays in float
-__device__ __forceinline__ void block_sum3(float (&v)[3], double* ipart, long long blk) {
+// The lattice total of the internal force: every thread adds its nodes in float
+// pairs (hi + lo, the rounding errors of the float additions kept: Knuth's
+// two-sum), the lanes of a warp are added as pairs, the warps in FP64, so that
+// the total does not depend on how the planes are cut into segments beyond some
+// 1e-14 (plain float sums differed by 1e-7).  In FP64 from the threads on, the
+// conversions and additions on its narrow pipe cost S2 10% at 128^3.
+struct Sum3 {
+  float2 hxy, lxy;
+  float hz, lz;
+};
+__device__ __forceinline__ void sum3_add(Sum3& s, float2 v, float z, float2 vl, float zl) {
+  const float2 m = make_float2(-1.0f, -1.0f);
+  const float2 t = __fadd2_rn(s.hxy, v);
+  const float2 bb = __ffma2_rn(s.hxy, m, t);
+  const float2 e = __fadd2_rn(__ffma2_rn(__ffma2_rn(bb, m, t), m, s.hxy), __ffma2_rn(bb, m, v));
+  s.hxy = t;
+  s.lxy = __fadd2_rn(s.lxy, __fadd2_rn(e, vl));
+  const float tz = __fadd_rn(s.hz, z), bz = __fsub_rn(tz, s.hz);
+  const float ez = __fadd_rn(__fsub_rn(s.hz, __fsub_rn(tz, bz)), __fsub_rn(z, bz));
+  s.lz = __fadd_rn(s.lz, __fadd_rn(ez, zl));
+  s.hz = tz;
+}
+__device__ __forceinline__ void sum3_add(Sum3& s, float x, float y, float z) {
+  sum3_add(s, make_float2(x, y), z, make_float2(0.0f, 0.0f), 0.0f);
+}
+// the block's sums, in a fixed order, into ipart[3 blk ..]
+__device__ __forceinline__ void block_sum3(Sum3 s, double* ipart, long long blk) {
   __shared__ double red[TILE_X * TILE_Y / 32][3];
   const int t = threadIdx.x + TILE_X * threadIdx.y;
   const int lane = t & 31, warp = t >> 5;
 #pragma unroll
-  for (int cc = 0; cc < 3; ++cc) {
-    float s = v[cc];
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-    if (lane == 0) red[warp][cc] = (double)s;
+  for (int o = 16; o > 0; o >>= 1) {
+    const float hx = __shfl_down_sync(0xffffffffu, s.hxy.x, o), hy = __shfl_down_sync(0xffffffffu, s.hxy.y, o);
+    const float lx = __shfl_down_sync(0xffffffffu, s.lxy.x, o), ly = __shfl_down_sync(0xffffffffu, s.lxy.y, o);
+    const float hz = __shfl_down_sync(0xffffffffu, s.hz, o), lz = __shfl_down_sync(0xffffffffu, s.lz, o);
+    sum3_add(s, make_float2(hx, hy), hz, make_float2(lx, ly), lz);
+  }
+  if (lane == 0) {
+    red[warp][0] = (double)s.hxy.x + (double)s.lxy.x;
+    red[warp][1] = (double)s.hxy.y + (double)s.lxy.y;
+    red[warp][2] = (double)s.hz + (double)s.lz;
   }
   __syncthreads();
-  if (t == 0) {
+  if (t < 3) {
+    double v = 0.0;
 #pragma unroll
-    for (int cc = 0; cc < 3; ++cc) {
-      double s = 0.0;
-      for (int w = 0; w < TILE_X * TILE_Y / 32; ++w) s += red[w][cc];
-      ipart[3 * blk + cc] = s;
-    }
+    for (int w = 0; w < TILE_X * TILE_Y / 32; ++w) v += red[w][t];
+    ipart[3 * blk + t] = v;
   }
 }
 
@@ -355,7 +382,7 @@ __device__ __forceinline__ float lb32_pop(const LBPairs& p, int i) {
 template <int K, bool PV, bool SIMPLE>
 __device__ __forceinline__ void lb32_node(LBRing<K>& t, const LBArgs& a, const Phys32& c,
                                           int x, int y, int z, int tid, int ex, int ey,
-                                          float (&iv)[3]) {
+                                          Sum3& iv) {
   constexpr int NP = LBPlane<K>::NP, NS = LBPlane<K>::NS;
   float* __restrict__ g_out = (float*)a.f_out;
   const int* __restrict__ n_in = (const int*)a.rho_in;
@@ -453,9 +480,7 @@ __device__ __forceinline__ void lb32_node(LBRing<K>& t, const LBArgs& a, const P
       at32(ifield, n) = ix;
       at32(ifield + N, n) = iy;
       at32(ifield + 2 * N, n) = iz;
-      iv[0] += ix;
-      iv[1] += iy;
-      iv[2] += iz;
+      sum3_add(iv, ix, iy, iz);
     }
     // ---- S2b: collision and push stream (velocity bounce-back, Eq. 12) ----
     const float* const gp = &t.pop[z & 1][0][tid];
@@ -525,7 +550,7 @@ __device__ __forceinline__ void lb32_block(const LBArgs& a, const Phys32& c, int
   const int tid = threadIdx.x + TILE_X * threadIdx.y;
   const bool in_xy = x < nx && y < ny;
   const int ex = threadIdx.x + 1, ey = threadIdx.y + 1;
-  float iv[3] = {0.0f, 0.0f, 0.0f};
+  Sum3 iv = {};
   int hoff[2];
   halo_offsets(hoff, x0, y0, a);
   // ring slot of plane zz: zz mod 4 (zz >= -1)
@@ -962,13 +987,20 @@ cudaError_t lb32_prepare() {
 // Planes per segment of S2 for `cols` tile columns of nz planes.  A segment
 // stages the plane on each side of it as well and starts with an empty
 // pipeline, so long segments waste less; short ones give the block scheduler
-// enough blocks (two resident per SM) to even out the SMs.  Measured on GB300
-// (ms per launch at 4 / 8 / 16 / 32 planes): 128^3 0.103, 0.098, 0.102,
-// 0.129; 256^3 (K = 3) 0.872, 0.816, 0.800, 0.830; 512^3 6.48, 6.01, 5.79,
-// 5.81.
+// enough blocks (two resident per SM) to even out the SMs, and a small box
+// enough to fill them at all.  Measured on GB300 (ms per launch at 1 / 2 / 4 / 8
+// planes): 32^3 0.0142, 0.0187, 0.0290, 0.0492; 48 x 64 x 32 0.0167, 0.0212,
+// 0.0294, 0.0492; 64^3 0.0264, 0.0235, 0.0344, 0.0474; 96^3 0.0738, 0.0614,
+// 0.0634, 0.0751; 192 x 108 x 72 0.116, 0.0863, 0.0777, 0.0787; at 4 / 8 / 16 /
+// 32 planes: 128^3 0.103, 0.098, 0.102, 0.129; 256^3 (K = 3) 0.872, 0.816,
+// 0.800, 0.830; 512^3 6.48, 6.01, 5.79, 5.81.
 int lb32_planes(long long cols, int nz) {
   auto blocks = [&](int p) { return cols * ((nz + p - 1) / p); };
-  return blocks(16) >= 4096 ? 16 : (blocks(8) >= 1024 ? 8 : 4);
+  return blocks(16) >= 4096 ? 16
+       : blocks(8) >= 1024 ? 8
+       : blocks(4) >= 1024 ? 4
+       : blocks(2) >= 512  ? 2
+                           : 1;
 }
 int lb32_segments(const Grid& g) {
   const long long cols = (long long)((g.nx + TILE_X - 1) / TILE_X) * ((g.ny + TILE_Y - 1) / TILE_Y);

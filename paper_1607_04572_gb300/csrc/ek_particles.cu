@@ -295,7 +295,8 @@ __device__ void block_sum(double (&v)[NV]) {
 // S4: forces and integration.
 //   k_force_assign   every fluid node of a particle's widened box records the
 //                    particle with the nearest surface (minimum image): an
-//                    atomicMin on the key (quantised surface distance, index)
+//                    atomicMin on the key (quantised surface distance, index);
+//                    not with a single particle, which claims them all
 //   k_particle_forces  grid (particle, chunk of fcells widened-box cells):
 //                    momentum exchange (Eq. 11), the solute force on the
 //                    particle (reaction of the internal solute force on the
@@ -483,7 +484,10 @@ __device__ void block_sum_t(Get v, const bool (&group_on)[NV / 6], double* out) 
 // Block (p, b) takes the rows b, b + nb, b + 2 nb, ... of FORCE_T cells of the
 // widened box (nb blocks for this particle), so the cells next to the sphere
 // are spread over all blocks.
-template <class FM>
+// ONE: a single particle, which claims every node of its widened box without
+// keys (1), several (0), or either (2: the batched launch; tested per cell it
+// costs 8% at 1000 particles).
+template <class FM, int ONE>
 __device__ __forceinline__ void particle_forces_body(const PartArgs& a, const Blk bk) {
   const int p = bk.x;
   const DevParticle& P = a.parts[p];
@@ -576,9 +580,10 @@ __device__ __forceinline__ void particle_forces_body(const PartArgs& a, const Bl
   // widened box are the particle's own), so no load waits on the key
   float nif[3] = {0.0f, 0.0f, 0.0f};
   const float* const ifl = (const float*)a.ifield;
+  const bool only = ONE == 2 ? a.P == 1 : ONE == 1;
   auto fetch = [&]() {
     nown = a.owner[nn];
-    nkey = a.fkey[nn];
+    if (!only) nkey = a.fkey[nn];
     if (FM::fp32) {
       nif[0] = ifl[nn];
       nif[1] = ifl[N + nn];
@@ -737,8 +742,8 @@ __device__ __forceinline__ void particle_forces_body(const PartArgs& a, const Bl
     // the key of a node is cleared by the particle it names, right after
     // reading it: any other particle reading it meanwhile finds either that
     // key or an empty one, and neither names it
-    bool mine = false;
-    if (first && (int)(key & 0xFFFFFull) == p) {
+    bool mine = only && first;
+    if (!only && first && (int)(key & 0xFFFFFull) == p) {
       a.fkey[n] = ~0ULL;
       mine = true;
     }
@@ -876,9 +881,12 @@ __device__ __forceinline__ void particle_forces_body(const PartArgs& a, const Bl
   }
 }
 
-template <class FM>
+template <class FM, int ONE>
 __global__ void __launch_bounds__(FORCE_T, FM::fp32 ? 5 : 4) k_particle_forces(PartArgs a) {
-  particle_forces_body<FM>(a, grid_blk());
+  particle_forces_body<FM, ONE>(a, grid_blk());
+}
+__device__ __forceinline__ void particle_forces_any(const PartArgs& a, const Blk bk) {
+  particle_forces_body<FormF32, 2>(a, bk);
 }
 
 // New box of a particle at `pos`: the cells within R (+1 below, +2 above),
@@ -1693,11 +1701,14 @@ __global__ void k_apply_transfers(PartArgs a) { apply_transfers_body<FM>(a, grid
 template <class FM>
 cudaError_t particle_forces_t(const PartArgs& a, cudaStream_t s, int parts) {
   const unsigned echunks = (unsigned)((a.emax + PT - 1) / PT);
-  if (parts & S4_ASSIGN) {
+  if ((parts & S4_ASSIGN) && assign_kernels(a.P)) {
     k_force_assign<<<dim3(a.P, echunks), PT, 0, s>>>(a);
     k_tie_resolve<<<8, 256, 0, s>>>(a);
   }
-  if (parts & S4_FORCES) k_particle_forces<FM><<<dim3(a.P, a.fchunks), FORCE_T, 0, s>>>(a);
+  if (parts & S4_FORCES) {
+    if (a.P == 1) k_particle_forces<FM, 1><<<dim3(1, a.fchunks), FORCE_T, 0, s>>>(a);
+    else k_particle_forces<FM, 0><<<dim3(a.P, a.fchunks), FORCE_T, 0, s>>>(a);
+  }
   return cudaGetLastError();
 }
 
@@ -1747,7 +1758,7 @@ cudaError_t reflag_t(const PartArgs& a, bool transitions, cudaStream_t s, int pa
   }
 EK_PART_BATCH(k_force_assign_batch, force_assign_body, __launch_bounds__(PT))
 EK_PART_BATCH(k_tie_resolve_batch, tie_resolve_body, __launch_bounds__(256))
-EK_PART_BATCH(k_particle_forces_batch, particle_forces_body<FormF32>, __launch_bounds__(FORCE_T, 4))
+EK_PART_BATCH(k_particle_forces_batch, particle_forces_any, __launch_bounds__(FORCE_T, 4))
 EK_PART_BATCH(k_save_prev_batch, save_prev_body, __launch_bounds__(PT))
 EK_PART_BATCH(k_clear_batch, clear_body<FormF32>, __launch_bounds__(PT))
 EK_PART_BATCH(k_claim_batch, claim_body<FormF32>, __launch_bounds__(PT))
@@ -1872,7 +1883,10 @@ void particle_batch_grid(int k, const PartArgs& a, int& gx, int& gy) {
   const int uchunks = union_chunks(a.boxmax);
   const int bchunks = (a.boxmax + PT - 1) / PT;
   switch (k) {
-    case PK_ASSIGN: gy = (a.emax + PT - 1) / PT; break;
+    case PK_ASSIGN:
+      gy = (a.emax + PT - 1) / PT;
+      if (!assign_kernels(a.P)) gx = 0;
+      break;
     case PK_FORCES: gy = a.fchunks; break;
     case PK_SAVE_PREV:
     case PK_CLEAR:
@@ -1882,7 +1896,7 @@ void particle_batch_grid(int k, const PartArgs& a, int& gx, int& gy) {
     // grid-stride kernels: their lists are short for a few particles (a CTA
     // per system), Psi's surface cells some hundreds per particle (eight
     // warps per CTA, eight CTAs per particle)
-    case PK_TIE:
+    case PK_TIE: gx = assign_kernels(a.P) ? 1 : 0; break;
     case PK_APPLY: gx = 1; break;
     case PK_PSI: gx = std::min(8 * 152, 8 * a.P); break;
     default: gx = 0;
