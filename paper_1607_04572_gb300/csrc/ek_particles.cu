@@ -445,33 +445,44 @@ __device__ __forceinline__ void tie_resolve_body(const PartArgs& a, const Blk bk
 __global__ void k_tie_resolve(PartArgs a) { tie_resolve_body(a, grid_blk()); }
 
 // Sum of FORCE_T values per component, fixed order: the block's values are
-// transposed through shared memory and each of 4 threads per component adds a
-// strided quarter, then one thread adds the quarters.  Components of a group
-// no thread touched are skipped (they stay 0).  Result in out[j] for
-// threadIdx.x == j < NV.  Few FP64 instructions: a warp-shuffle tree would
-// spend 5 * NV double adds per thread.
+// transposed through shared memory; of every group of six components that some
+// thread touched (bit j / 6 of `on`; the others stay 0) 16 threads per component
+// add a strided sixteenth, then one thread adds the sixteenths.  Few FP64
+// instructions and a short chain of them: a warp-shuffle tree would spend 5 * NV
+// double adds per thread, quarters 32 adds one after another.
 template <int NC>
 __device__ void column_sums(const double* tab, int nrow, int stride, int col0, double* out);
 __device__ void integrate_all(const PartArgs& a);
 
 template <int NV, class Get>
-__device__ void block_sum_t(Get v, const bool (&group_on)[NV / 6], double* out) {
+__device__ void block_sum_t(Get v, unsigned on, double* out) {
+  constexpr int S = 16;
   __shared__ double tr[NV][FORCE_T + 1];
-  __shared__ double quarter[NV][4];
   const int t = threadIdx.x;
 #pragma unroll
   for (int j = 0; j < NV; ++j)
-    if (group_on[j / 6]) tr[j][t] = v(j);
+    if (on >> (j / 6) & 1u) tr[j][t] = v(j);
   __syncthreads();
-  if (t < 4 * NV) {
-    const int j = t >> 2, w = t & 3;
-    double s = 0.0;
-    if (group_on[j / 6])
-      for (int i = w; i < FORCE_T; i += 4) s += tr[j][i];
-    quarter[j][w] = s;
+  for (int g = 0; g < NV / 6; ++g) {
+    if (!(on >> g & 1u)) continue;
+    if (t < 6 * S) {
+      const int j = 6 * g + t / S, w = t % S;
+      double s = 0.0;
+#pragma unroll
+      for (int i = 0; i < FORCE_T / S; ++i) s += tr[j][w + i * S];
+      tr[j][w] = s;  // read by this thread alone
+    }
   }
   __syncthreads();
-  if (t < NV) out[t] = ((quarter[t][0] + quarter[t][1]) + quarter[t][2]) + quarter[t][3];
+  if (t < NV) {
+    double s = 0.0;
+    if (on >> (t / 6) & 1u) {
+#pragma unroll
+      for (int w = 0; w < S; w += 4)
+        s += (tr[t][w] + tr[t][w + 1]) + (tr[t][w + 2] + tr[t][w + 3]);
+    }
+    out[t] = s;
+  }
 }
 
 // Per fluid node x next to particle p, with d0 = x - r_p and
@@ -479,8 +490,9 @@ __device__ void block_sum_t(Get v, const bool (&group_on)[NV / 6], double* out) 
 // midpoint) has c_i . v_b = c_i . w, since c_i . (Omega x c_i) = 0, and the
 // link torque (x + c_i - r_p) x F_i sums to d0 x sum_i F_i, since
 // c_i x c_i = 0.  So the per-link work is one dot product and one add.
-// The field on the particle's own charge is kept as sum q and sum q (r - r_p)
-// (force E sum q, torque (sum q (r - r_p)) x E).
+// The field on the particle's own charge is kept as the sums of the weights w
+// (Psi_p, or 1 on the boundary nodes) and of w (r - r_p); the charge per unit
+// weight, a division, is applied once per particle (integrate_all).
 // Block (p, b) takes the rows b, b + nb, b + 2 nb, ... of FORCE_T cells of the
 // widened box (nb blocks for this particle), so the cells next to the sphere
 // are spread over all blocks.
@@ -497,33 +509,6 @@ __device__ __forceinline__ void particle_forces_body(const PartArgs& a, const Bl
   const int nb = (ncell + a.fcells - 1) / a.fcells;
   if ((int)bk.y >= nb) return;  // whole CTA beyond this particle's widened box
   const bool pv = a.ph.pv != 0;
-  // the charge per unit weight (FP64 form: every thread; FP32 form: one
-  // thread of the block, in float to the others, as the GPU's FP64 pipe is
-  // narrow)
-  auto charge_norm = [&]() {
-    if (pv)
-      return (a.ph.flags & EK_CHARGE_NORM_VP)
-                 ? P.charge / (4.0 / 3.0 * M_PI * P.radius * P.radius * P.radius)
-                 : (psi_sum(P) > 0.0 ? P.charge / psi_sum(P) : 0.0);
-    return P.nb > 0 ? P.charge / (double)P.nb : 0.0;
-  };
-  double qnorm = 0.0;
-  float qnormf = 0.0f;
-  bool qnz = false;  // qnorm != 0
-  if (FM::fp32) {
-    __shared__ float s_qn;
-    __shared__ int s_qnz;
-    if (threadIdx.x == 0) {
-      const double q = charge_norm();
-      s_qn = (float)q;
-      s_qnz = q != 0.0;
-    }
-    __syncthreads();
-    qnormf = s_qn;
-    qnz = s_qnz != 0;
-  } else {
-    qnorm = charge_norm();
-  }
   const double rho0 = a.ph.rho0;
   // the particle's velocities, rho0 and centre in float (FP32 form; the
   // particle record keeps float copies of the velocities and the centre's
@@ -542,7 +527,7 @@ __device__ __forceinline__ void particle_forces_body(const PartArgs& a, const Bl
   float macc[10] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
   const int cxi = P.ipos[0], cyi = P.ipos[1], czi = P.ipos[2];  // floor(pos)
   const float frx = P.fpos[0], fry = P.fpos[1], frz = P.fpos[2];  // pos - floor(pos), rounded
-  bool touched[4] = {false, false, false, false};
+  unsigned touched = 0;  // groups of six sums with an entry
   const int rows = a.fcells / FORCE_T;
   // FP32 form: a thread's cells are rows of FORCE_T apart in the widened
   // box's x-fastest order, nb rows per step, so their box-local coordinates
@@ -706,7 +691,7 @@ __device__ __forceinline__ void particle_forces_body(const PartArgs& a, const Bl
         fx += cst * (float)kx;
         fy += cst * (float)ky;
         fz += cst * (float)kz;
-        touched[0] = true;
+        touched |= 1u;
         macc[0] += fx;
         macc[1] += fy;
         macc[2] += fz;
@@ -729,7 +714,7 @@ __device__ __forceinline__ void particle_forces_body(const PartArgs& a, const Bl
           if (dcy(i)) fy = dcy(i) > 0 ? fy + mom : fy - mom;
           if (dcz(i)) fz = dcz(i) > 0 ? fz + mom : fz - mom;
         }
-        touched[0] = true;
+        touched |= 1u;
         acc[0] += fx;
         acc[1] += fy;
         acc[2] += fz;
@@ -748,7 +733,7 @@ __device__ __forceinline__ void particle_forces_body(const PartArgs& a, const Bl
       mine = true;
     }
     if (mine && own == FLUID) {
-      touched[1] = true;
+      touched |= 2u;
       if (FM::fp32) {
         const float ix = ifx, iy = ify, iz = ifz;
         // minimum-image offset of the wrapped node from the centre
@@ -777,39 +762,32 @@ __device__ __forceinline__ void particle_forces_body(const PartArgs& a, const Bl
     }
     // the particle's own charge in this cell
     if (in_box) {
-      double qq = 0.0;
+      double ps = 0.0;
       float psf = 0.0f;
       bool has_q = false;
       if (pv) {
         const int bx = P.hi[0] - P.lo[0], by = P.hi[1] - P.lo[1];
         const int cb = (X - P.lo[0]) + bx * ((Y - P.lo[1]) + by * (Z - P.lo[2]));
-        const double ps = a.psibox[(long long)p * a.boxmax + cb];
-        if (FM::fp32) {
-          // the weight itself is applied in float below
-          psf = psibox_float((unsigned long long)__double_as_longlong(ps));
-          has_q = psf != 0.0f;
-        } else {
-          qq = qnorm * ps;
-          has_q = qq != 0.0;
-        }
+        ps = a.psibox[(long long)p * a.boxmax + cb];
+        has_q = (__double_as_longlong(ps) << 1) != 0;
+        if (FM::fp32) psf = psibox_float((unsigned long long)__double_as_longlong(ps));
       } else if (own == p) {
-        qq = qnorm;
+        ps = 1.0;
         psf = 1.0f;
-        has_q = FM::fp32 ? qnz : qq != 0.0;
+        has_q = true;
       }
       if (has_q) {
-        touched[2] = true;
+        touched |= 4u;
         if (FM::fp32) {
-          const float qf = qnormf * psf;
-          macc[6] += qf;
-          macc[7] += qf * __fsub_rn((float)(X - P.ipos[0]), P.fpos[0]);
-          macc[8] += qf * __fsub_rn((float)(Y - P.ipos[1]), P.fpos[1]);
-          macc[9] += qf * __fsub_rn((float)(Z - P.ipos[2]), P.fpos[2]);
+          macc[6] += psf;
+          macc[7] += psf * __fsub_rn((float)(X - P.ipos[0]), P.fpos[0]);
+          macc[8] += psf * __fsub_rn((float)(Y - P.ipos[1]), P.fpos[1]);
+          macc[9] += psf * __fsub_rn((float)(Z - P.ipos[2]), P.fpos[2]);
         } else {
-          acc[12] += qq;
-          acc[13] += qq * ((double)X - P.pos[0]);
-          acc[14] += qq * ((double)Y - P.pos[1]);
-          acc[15] += qq * ((double)Z - P.pos[2]);
+          acc[12] += ps;
+          acc[13] += ps * ((double)X - P.pos[0]);
+          acc[14] += ps * ((double)Y - P.pos[1]);
+          acc[15] += ps * ((double)Z - P.pos[2]);
         }
       }
     }
@@ -835,18 +813,20 @@ __device__ __forceinline__ void particle_forces_body(const PartArgs& a, const Bl
     double lat = 0.0;  // component threadIdx.x % 3 (the stride 126 keeps it)
     for (int q = threadIdx.x; q < 3 * (r1 - r0) && threadIdx.x < 126; q += 126) {
       lat += __ldcg(a.ipart + 3LL * r0 + q);
-      touched[3] = true;
+      touched |= 8u;
     }
     const int j = threadIdx.x % 3;
     if (j == 0) acc[18] = lat;
     else if (j == 1) acc[19] = lat;
     else acc[20] = lat;
   }
-  bool on[4];
-  on[0] = __syncthreads_or(touched[0]);
-  on[1] = __syncthreads_or(touched[1]);
-  on[2] = __syncthreads_or(touched[2]);
-  on[3] = __syncthreads_or(touched[3]);
+  __shared__ unsigned warp_touched[FORCE_T / 32];
+  touched = __reduce_or_sync(0xffffffffu, touched);
+  if ((threadIdx.x & 31) == 0) warp_touched[threadIdx.x >> 5] = touched;
+  __syncthreads();
+  unsigned on = 0;
+#pragma unroll
+  for (int w = 0; w < FORCE_T / 32; ++w) on |= warp_touched[w];
   double* out = a.fpart + ((long long)p * a.fchunks + bk.y) * FPART;
   if (FM::fp32) {
     // each thread's float sums over its own few cells, widened to FP64 (the
@@ -881,8 +861,11 @@ __device__ __forceinline__ void particle_forces_body(const PartArgs& a, const Bl
   }
 }
 
+// four blocks per SM: with five (96 registers, spills in the cell loop) S4 takes
+// 1.50 ms instead of 1.35 at 512^3 with 1000 particles, 126 us instead of 121 at
+// 256^3 with 64, 33.4 instead of 29.5 with one at 128^3
 template <class FM, int ONE>
-__global__ void __launch_bounds__(FORCE_T, FM::fp32 ? 5 : 4) k_particle_forces(PartArgs a) {
+__global__ void __launch_bounds__(FORCE_T, 4) k_particle_forces(PartArgs a) {
   particle_forces_body<FM, ONE>(a, grid_blk());
 }
 __device__ __forceinline__ void particle_forces_any(const PartArgs& a, const Blk bk) {
@@ -973,6 +956,14 @@ __device__ void column_sums(const double* tab, int nrow, int stride, int col0, d
   __syncthreads();
 }
 
+// the particle's charge per unit weight (Psi_p, or a boundary node)
+__device__ double charge_norm(const PartArgs& a, const DevParticle& P) {
+  if (!a.ph.pv) return P.nb > 0 ? P.charge / (double)P.nb : 0.0;
+  if (a.ph.flags & EK_CHARGE_NORM_VP) return P.charge / (4.0 / 3.0 * M_PI * P.radius * P.radius * P.radius);
+  const double w = psi_sum(P);
+  return w > 0.0 ? P.charge / w : 0.0;
+}
+
 // Run by the block that finishes S4 last: the remainder of the solute force
 // on nodes no particle claims (lattice total of the internal force minus the
 // claimed sums) is split evenly; every particle then moves by symplectic
@@ -1004,9 +995,11 @@ __device__ void integrate_all(const PartArgs& a) {
       for (int d = d0; d < 3; d += dstep) {
         const int d1 = d == 2 ? 0 : d + 1, d2 = d == 0 ? 2 : d - 1;  // (d, d1, d2) cyclic
         const int nn = d == 0 ? a.g.nx : (d == 1 ? a.g.ny : a.g.nz);
-        // field on the own charge: E sum q, (sum q (r - r_p)) x E
-        const double Tq = __ldcg(acc + 13 + d1) * E[d2] - __ldcg(acc + 13 + d2) * E[d1];
-        const double F = __ldcg(acc + d) + __ldcg(acc + 6 + d) + __ldcg(acc + 12) * E[d] - rem[d] +
+        // field on the own charge: E sum q, (sum q (r - r_p)) x E, with q the
+        // summed weights times the charge per unit weight
+        const double qn = charge_norm(a, *Pp);
+        const double Tq = qn * (__ldcg(acc + 13 + d1) * E[d2] - __ldcg(acc + 13 + d2) * E[d1]);
+        const double F = __ldcg(acc + d) + __ldcg(acc + 6 + d) + qn * __ldcg(acc + 12) * E[d] - rem[d] +
                          Pp->ftrans[d];
         const double T = __ldcg(acc + 3 + d) + __ldcg(acc + 9 + d) + Tq;
         double pos = Pp->pos[d], vel = Pp->vel[d], omega = Pp->omega[d];
