@@ -4,6 +4,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <functional>
 #include <atomic>
 #include <map>
 #include <mutex>
@@ -997,14 +998,19 @@ ek_status ek_get_fields(ek_ctx* ctx, ek_field which, int component, double* dst,
   const Grid& g = ctx->g;
   cudaStream_t s = ctx->stream;
   const bool f32 = ctx->fp32 != 0;
+  // A converted field goes straight to a device destination (a copy of its own
+  // would move every value twice more), to a host one, or one that no double
+  // may be stored to, through tmp.
+  const bool direct = dst_on_device && ((uintptr_t)dst & (sizeof(double) - 1)) == 0;
+  double* const conv = direct ? dst : ctx->tmp;
   // copy one converted N-element block (tmp) to dst + offset
   auto out_block = [&](size_t offset) -> cudaError_t {
-    return cudaMemcpyAsync(dst + offset, ctx->tmp, N * sizeof(double), kind, s);
+    return direct ? cudaSuccess : cudaMemcpyAsync(dst + offset, ctx->tmp, N * sizeof(double), kind, s);
   };
   // a real field of the current form -> dst + offset
   auto out_real = [&](const void* src, size_t offset) -> cudaError_t {
     if (!f32) return cudaMemcpyAsync(dst + offset, src, N * sizeof(double), kind, s);
-    cudaError_t e = convert32(CONV_F32_TO_F64, g, 0, 0.0, src, ctx->tmp, ctx->status, s);
+    cudaError_t e = convert32(CONV_F32_TO_F64, g, 0, 0.0, src, direct ? dst + offset : ctx->tmp, ctx->status, s);
     return e != cudaSuccess ? e : out_block(offset);
   };
   switch (which) {
@@ -1012,7 +1018,7 @@ ek_status ek_get_fields(ek_ctx* ctx, ek_field which, int component, double* dst,
       if (component < 0 || component >= ctx->p.nspecies) return fail(ctx, EK_ERR_ARG, "bad species index");
       if (f32) {
         EK_CUDA(convert32(CONV_SPC_TO_F64, g, 0, ctx->ph.qscale[component],
-                          (const int*)ctx->rho[ctx->cur] + component * N, ctx->tmp, ctx->status, s));
+                          (const int*)ctx->rho[ctx->cur] + component * N, conv, ctx->status, s));
         EK_CUDA(out_block(0));
       } else {
         EK_CUDA(cudaMemcpyAsync(dst, (const double*)ctx->rho[ctx->cur] + component * N,
@@ -1020,7 +1026,9 @@ ek_status ek_get_fields(ek_ctx* ctx, ek_field which, int component, double* dst,
       }
       break;
     case EK_FIELD_POPULATIONS:
-      if (f32) {
+      if (f32 && direct) {
+        EK_CUDA(convert32(CONV_POPS_TO_F64, g, 0, ctx->ph.rho0, ctx->f[ctx->cur], dst, ctx->status, s));
+      } else if (f32) {
         for (int i = 0; i < Q; ++i) {
           EK_CUDA(convert32(CONV_POP_TO_F64, g, i, ctx->ph.rho0, ctx->f[ctx->cur], ctx->tmp, ctx->status, s));
           EK_CUDA(out_block(i * N));
@@ -1030,7 +1038,13 @@ ek_status ek_get_fields(ek_ctx* ctx, ek_field which, int component, double* dst,
       }
       break;
     case EK_FIELD_VELOCITY:
-      for (int d = 0; d < 3; ++d) EK_CUDA(out_real((const char*)ctx->u + d * N * ctx->rsz, d * N));
+      if (f32 && direct) {  // the three components lie one after another on both sides
+        Grid g3 = g;
+        g3.N = 3 * g.N;
+        EK_CUDA(convert32(CONV_F32_TO_F64, g3, 0, 0.0, ctx->u, dst, ctx->status, s));
+      } else {
+        for (int d = 0; d < 3; ++d) EK_CUDA(out_real((const char*)ctx->u + d * N * ctx->rsz, d * N));
+      }
       break;
     case EK_FIELD_E_EXT:
     case EK_FIELD_BODY_FORCE: {
@@ -1040,7 +1054,7 @@ ek_status ek_get_fields(ek_ctx* ctx, ek_field which, int component, double* dst,
       break;
     }
     case EK_FIELD_WALL:
-      k_u8_to_double<<<nblk(g.N), 256, 0, s>>>(g, ctx->wall, ctx->tmp);
+      k_u8_to_double<<<nblk(g.N), 256, 0, s>>>(g, ctx->wall, conv);
       EK_CUDA(cudaGetLastError());
       EK_CUDA(out_block(0));
       break;
@@ -1048,8 +1062,8 @@ ek_status ek_get_fields(ek_ctx* ctx, ek_field which, int component, double* dst,
       EK_CUDA(out_real(ctx->qwall, 0));
       break;
     case EK_FIELD_DENSITY:
-      if (f32) EK_CUDA(density32(g, (const float*)ctx->f[ctx->cur], ctx->ph.rho0, ctx->tmp, s));
-      else k_density<<<nblk(g.N), 256, 0, s>>>(g, (const double*)ctx->f[ctx->cur], ctx->tmp);
+      if (f32) EK_CUDA(density32(g, (const float*)ctx->f[ctx->cur], ctx->ph.rho0, conv, s));
+      else k_density<<<nblk(g.N), 256, 0, s>>>(g, (const double*)ctx->f[ctx->cur], conv);
       EK_CUDA(cudaGetLastError());
       EK_CUDA(out_block(0));
       break;
@@ -1060,19 +1074,19 @@ ek_status ek_get_fields(ek_ctx* ctx, ek_field which, int component, double* dst,
       if (f32) {
         EK_CUDA(out_real(ctx->psi, 0));  // clamped to 1 by S5
       } else {
-        k_psi_clamped<<<nblk(g.N), 256, 0, s>>>(g, (const double*)ctx->psi, ctx->tmp);
+        k_psi_clamped<<<nblk(g.N), 256, 0, s>>>(g, (const double*)ctx->psi, conv);
         EK_CUDA(cudaGetLastError());
         EK_CUDA(out_block(0));
       }
       break;
     case EK_FIELD_OWNER:
-      k_int_to_double<<<nblk(g.N), 256, 0, s>>>(g, ctx->owner, ctx->tmp);
+      k_int_to_double<<<nblk(g.N), 256, 0, s>>>(g, ctx->owner, conv);
       EK_CUDA(cudaGetLastError());
       EK_CUDA(out_block(0));
       break;
     case EK_FIELD_CHARGE:
       EK_CUDA(charge_density(g, ctx->ph, ctx->rho[ctx->cur], ctx->has_qwall ? ctx->qwall : nullptr,
-                             ctx->qpart, ctx->tmp, s));
+                             ctx->qpart, conv, s));
       EK_CUDA(out_block(0));
       break;
     default:
@@ -1662,19 +1676,35 @@ ek_status batch_capture_fused(ek_batch* b, int key) {
     ok(part(PK_ASSIGN, ps));
     ok(part(PK_TIE, ps));
   }
-  for (int pass = 0; pass < 3; ++pass) {
-    for (const ek_batch::Launch& L : F.fft[pass]) {
-      ok(launch_poisson_batch(pass, L.variant, base + F.o_pa, (const BatchSlot*)(base + L.slot), L.nslot,
-                              L.ctas, s));
-      ++count;
+  // S1: a pass has up to nine kernel variants, each with a few systems' CTAs (a
+  // part of the SMs): they run side by side on the branch streams, and so do the
+  // systems whose S1 is their own (64 boxes of edges 32-64: a batch step 1.05
+  // ms one after another, 0.96 side by side)
+  const size_t nbr = b->branch.size();
+  const auto side_by_side = [&](size_t items, const std::function<void(size_t, cudaStream_t)>& run) {
+    const size_t used = std::min(items > 0 ? items - 1 : 0, nbr);
+    if (used) ok(cudaEventRecord(b->ev_fork, s));
+    for (size_t w = 0; w < used; ++w) ok(cudaStreamWaitEvent(b->branch[w], b->ev_fork, 0));
+    for (size_t i = 0; i < items; ++i) run(i, i % (used + 1) == 0 ? s : b->branch[i % (used + 1) - 1]);
+    for (size_t w = 0; w < used; ++w) {
+      ok(cudaEventRecord(b->ev_join[w], b->branch[w]));
+      ok(cudaStreamWaitEvent(s, b->ev_join[w], 0));
     }
+  };
+  for (int pass = 0; pass < 3; ++pass) {
+    side_by_side(F.fft[pass].size(), [&](size_t i, cudaStream_t on) {
+      const ek_batch::Launch& L = F.fft[pass][i];
+      ok(launch_poisson_batch(pass, L.variant, base + F.o_pa, (const BatchSlot*)(base + L.slot), L.nslot,
+                              L.ctas, on));
+      ++count;
+    });
   }
-  for (int i : F.s1_alone) {
-    ek_ctx* c = b->sys[i];
+  side_by_side(F.s1_alone.size(), [&](size_t i, cudaStream_t on) {
+    ek_ctx* c = b->sys[F.s1_alone[i]];
     ok(poisson_solve_f32(c->plan, (const int*)c->rho[c->cur], c->has_qwall ? (const float*)c->qwall : nullptr,
-                         (const float*)c->qpart, c->ph, (float*)c->phi, (float2*)c->spectrum, s));
-    alone[i] += poisson_kernel_count(c->plan, true);
-  }
+                         (const float*)c->qpart, c->ph, (float*)c->phi, (float2*)c->spectrum, on));
+    alone[F.s1_alone[i]] += poisson_kernel_count(c->plan, true);
+  });
   ok(launch_lb32_batch(lbl(F.lb), K, pv, s));
   ++count;
   if (b->overlap) {

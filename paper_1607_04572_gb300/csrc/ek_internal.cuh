@@ -376,6 +376,7 @@ enum {
   CONV_SPC_FROM_F64 = 3,  // density -> int units (scale = qscale)
   CONV_F32_TO_F64 = 4,
   CONV_F64_TO_F32 = 5,
+  CONV_POPS_TO_F64 = 6,   // all 19 directions -> f (double), direction-major
 };
 // N-element conversion; `scale` is rho0 for populations, qscale for species
 cudaError_t convert32(int op, const Grid& g, int index, double scale, const void* in, void* out,
@@ -438,8 +439,9 @@ struct PartArgs {
 constexpr int FORCE_T = 128;
 constexpr int FORCE_CHUNK = 256;
 // per particle: [0..5] Fh Th (momentum exchange), [6..11] Fs Ts (reaction of
-// the solute force), [12] sum q and [13..15] sum q (r - r_p) of the particle's
-// own charge (the field's force and torque are E and M x E times these),
+// the solute force), [12] sum w and [13..15] sum w (r - r_p) of the weights of
+// the particle's own charge (times the charge per unit weight, the field's force
+// and torque are E and M x E times these),
 // [18..20] a slice of the lattice total of the internal force (first particle
 // only), [16..17] and [21..23] unused
 constexpr int FPART = 24;

@@ -891,6 +891,11 @@ __global__ void k_pop_to_f64(long long N, int i, float rho0, const float* g, dou
   const long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (n < N) out[n] = (double)g[i * N + n] + wgt(i) * (double)rho0;
 }
+__global__ void k_pops_to_f64(long long N, float rho0, const float* g, double* out) {
+  const long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  const int i = blockIdx.y;
+  if (n < N) out[i * N + n] = (double)g[i * N + n] + wgt(i) * (double)rho0;
+}
 __global__ void k_pop_from_f64(long long N, int i, float rho0, const double* in, float* g) {
   const long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (n < N) g[i * N + n] = (float)(in[n] - wgt(i) * (double)rho0);
@@ -1116,6 +1121,7 @@ cudaError_t convert32(int op, const Grid& g, int index, double scale, const void
   const unsigned nb = blocks_for(N, 256);
   switch (op) {
     case CONV_POP_TO_F64: k_pop_to_f64<<<nb, 256, 0, s>>>(N, index, (float)scale, (const float*)in, (double*)out); break;
+    case CONV_POPS_TO_F64: k_pops_to_f64<<<dim3(nb, Q), 256, 0, s>>>(N, (float)scale, (const float*)in, (double*)out); break;
     case CONV_POP_FROM_F64: k_pop_from_f64<<<nb, 256, 0, s>>>(N, index, (float)scale, (const double*)in, (float*)out); break;
     case CONV_SPC_TO_F64: k_spc_to_f64<<<nb, 256, 0, s>>>(N, scale, (const int*)in, (double*)out); break;
     case CONV_SPC_FROM_F64: k_spc_from_f64<<<nb, 256, 0, s>>>(N, scale, (const double*)in, (int*)out, status); break;
