@@ -58,7 +58,7 @@ struct ek_ctx {
   int nipart = 0;
   int nipart_cap = 0;  // rows allocated for ipart (FP32: enough for 2-plane segments)
   int nzb = 1;       // S2: z segments per tile column
-  int advseg = 1;    // FP32 S3: z segments per tile column
+  int advseg = 1;    // S3: z segments per tile column
   int overlap = 1;   // particle chain on the auxiliary stream (1) or in line (0)
   unsigned long long version = 0;  // bumped whenever captured steps go stale
   unsigned long long* fkey = nullptr;  // N: nearest-particle keys of S4
@@ -756,7 +756,7 @@ ek_status ek_create(const ek_params* p, ek_ctx** out) {
   {
     // lattice-block partial sums of S2: one per block of its grid
     ctx->nzb = ctx->fp32 ? lb32_segments(g) : lb64_segments(g);
-    if (ctx->fp32) ctx->advseg = adv32_segments(g, false);
+    ctx->advseg = ctx->fp32 ? adv32_segments(g, false) : adv64_segments(g);
     const dim3 lg = lattice_grid32(g, ctx->nzb);
     ctx->nipart = (int)(lg.x * lg.y * lg.z);
     // the FP32 segment length may be retuned down to 2 planes (ek_batch_tune)

@@ -168,14 +168,9 @@ __host__ __device__ inline int wrapi(int v, int n) {
   return r < 0 ? r + n : r;
 }
 
-// Lattice kernels run on a 3D grid of 32 x 8 thread tiles (x, y) per z plane:
-// no integer division to find a node's coordinates, and a warp covers 32
-// consecutive x (coalesced).
+// Lattice kernels run on 32 x 8 thread tiles (x, y): no integer division to
+// find a node's coordinates, and a warp covers 32 consecutive x (coalesced).
 constexpr int TILE_X = 32, TILE_Y = 8;
-inline dim3 lattice_grid(const Grid& g) {
-  return dim3((unsigned)((g.nx + TILE_X - 1) / TILE_X), (unsigned)((g.ny + TILE_Y - 1) / TILE_Y),
-              (unsigned)g.nz);
-}
 inline dim3 lattice_block() { return dim3(TILE_X, TILE_Y, 1); }
 // the S2 kernels march each (x, y) tile column through nzb segments of
 // consecutive planes
@@ -321,7 +316,7 @@ struct LBArgs {
   const DevParticle* parts;
   int* status;
   int nzb;         // S2: z segments per (x, y) tile column (lb32_segments, lb64_segments)
-  int advseg;      // FP32 S3: z segments per tile column (adv32_segments)
+  int advseg;      // S3: z segments per tile column (adv32_segments, adv64_segments)
 };
 // Constants of the FP32 kernels, rounded once on the host.
 struct Phys32 {
@@ -346,6 +341,7 @@ struct LBBatchEntry {
 cudaError_t launch_lb_fused(const LBArgs& a, cudaStream_t s);
 cudaError_t lb64_prepare();           // before the first launch_lb_fused
 int lb64_segments(const Grid& g);     // z segments per tile column of the FP64 S2 grid
+int adv64_segments(const Grid& g);    // and of the FP64 S3 grid
 cudaError_t launch_advection(const LBArgs& a, cudaStream_t s);
 // FP32-storage form
 cudaError_t lb32_prepare();  // once per process, before the first launch_lb32

@@ -7,6 +7,8 @@
 // a warp touches consecutive x: coalesced 8-byte accesses.
 #include <math.h>
 
+#include <algorithm>
+
 #include "ek_internal.cuh"
 
 namespace ek {
@@ -481,90 +483,149 @@ __global__ void __launch_bounds__(256, K <= 2 ? 2 : 1) k_lb_fused(LBArgs a, Coll
              blockIdx.x + (long long)gridDim.x * (blockIdx.y + (long long)gridDim.y * blockIdx.z));
 }
 
-// sign (-1, 0, +1) and magnitude of a double from its bits: integer work
-// only, so the advection's tests cost no FP64 instructions (-0 counts as 0)
-__device__ __forceinline__ int sgn_bits(double v) {
-  const long long b = __double_as_longlong(v);
-  if ((b << 1) == 0) return 0;
-  return b < 0 ? -1 : 1;
-}
-__device__ __forceinline__ double abs_bits(double v) {
-  return __longlong_as_double(__double_as_longlong(v) & 0x7fffffffffffffffLL);
-}
-
 // S3: rho' = (rho - div J) + volume-of-fluid advection.  rho_out holds
 // rho - div J (written by S2) and is updated in place; rho_in is the species
 // field at the start of the step (the advected one).  The cell displaced by
 // u overlaps the neighbours at offsets s with s_a in {0, sign(u_a)}; the share
 // of offset s is prod_a w_a, w_a = 1 - |u_a| (s_a = 0) or |u_a|.
+//
+// 32 x 8 tiles marching through a segment of planes.  The weights |u_a| and
+// 1 - |u_a|, the species and the sign bytes of three planes with a one-node
+// halo are in shared memory (a fourth slot takes the next plane), each weight
+// formed once.  A node first marks the neighbours of which it receives a share
+// (integer work on the sign bytes), then all lanes of the warp take their marked
+// neighbours one after another: a branch per neighbour would be issued by the
+// warp for every direction that any of its lanes receives from.  FP64
+// instructions per node (K = 2): 4 for the weights, 28 for the shares sent, 4
+// per share received (seven on average).  One thread per node with the
+// neighbours' velocities from global memory took 0.51 ms at 128^3, 0.097 at 64^3.
 template <int K>
-__global__ void __launch_bounds__(256) k_advect(LBArgs a) {
-  const double* rho_in = (const double*)a.rho_in;
-  double* rho_out = (double*)a.rho_out;
-  const double* u = (const double*)a.u;
+struct Adv64Plane {
+  double w[6][HP];    // |u_x|, |u_y|, |u_z|, then 1 - each
+  double rho[K][HP];
+  unsigned char sg[HP + 4];  // sign bytes of S2 (bit 7 fluid)
+};
+template <int K>
+struct Adv64Smem {
+  Adv64Plane<K> pl[4];  // plane p in slot p & 3
+};
+
+template <int K>
+__global__ void __launch_bounds__(256, 2) k_advect(LBArgs a) {
+  extern __shared__ __align__(16) unsigned char adv64_smem[];
+  Adv64Smem<K>& t = *reinterpret_cast<Adv64Smem<K>*>(adv64_smem);
+  const int nx = a.g.nx, ny = a.g.ny, nz = a.g.nz;
   const long long N = a.g.N;
-  const int x = blockIdx.x * TILE_X + threadIdx.x;
-  const int y = blockIdx.y * TILE_Y + threadIdx.y;
-  const int z = blockIdx.z;
-  if (x >= a.g.nx || y >= a.g.ny) return;
-  const long long n = node_index(a.g, x, y, z);
-  if (!(a.vsig[n] & 0x80u)) return;  // fluid bit of S2 (the flags may change meanwhile)
-  const Nbr b = make_nbr(x, y, z, a.g);
-  double acc[K];
-  double rs[K];
+  double* rho_out = (double*)a.rho_out;
+  const int x0 = blockIdx.x * TILE_X, y0 = blockIdx.y * TILE_Y;
+  const int z0 = (int)((long long)blockIdx.z * nz / a.advseg);
+  const int zend = (int)((long long)(blockIdx.z + 1) * nz / a.advseg);
+  const int x = x0 + threadIdx.x, y = y0 + threadIdx.y;
+  const int tid = threadIdx.x + TILE_X * threadIdx.y;
+  const bool in_xy = x < nx && y < ny;
+  const int e0 = threadIdx.x + 1 + HX * (threadIdx.y + 1);
+  int hoff[2];
 #pragma unroll
-  for (int k = 0; k < K; ++k) {
-    acc[k] = rho_out[k * N + n];
-    rs[k] = rho_in[k * N + n];
+  for (int q = 0; q < 2; ++q) {
+    const int e = tid + q * TN, ey = e / HX, ex = e - ey * HX;
+    hoff[q] = e < HP ? halo_wrap(x0 - 1 + ex, nx) + nx * halo_wrap(y0 - 1 + ey, ny) : -1;
   }
-  // outflow of this cell
-  const double ux = u[n], uy = u[N + n], uz = u[2 * N + n];
-  const int sx = sgn_bits(ux), sy = sgn_bits(uy), sz = sgn_bits(uz);
-  const double ax = abs_bits(ux), ay = abs_bits(uy), az = abs_bits(uz);
-  const double bx = 1.0 - ax, by = 1.0 - ay, bz = 1.0 - az;
-  for (int oz = 0; oz <= (sz != 0); ++oz) {
-    for (int oy = 0; oy <= (sy != 0); ++oy) {
-      for (int ox = 0; ox <= (sx != 0); ++ox) {
-        if (!ox && !oy && !oz) continue;
-        const long long m = node_index(a.g, nb_x(b, x, ox ? sx : 0), nb_y(b, y, oy ? sy : 0),
-                                       nb_z(b, z, oz ? sz : 0));
-        if (!(a.vsig[m] & 0x80u)) continue;  // share aimed at a boundary stays here
-        const double frac = (ox ? ax : bx) * (oy ? ay : by) * (oz ? az : bz);
+  auto stage = [&](int z) {
+    Adv64Plane<K>& p = t.pl[z & 3];
+    const size_t pz = (size_t)nx * ny * wrap_plane(z, nz);
 #pragma unroll
-        for (int k = 0; k < K; ++k) acc[k] -= rs[k] * frac;
+    for (int q = 0; q < 2; ++q) {
+      if (hoff[q] < 0) continue;
+      const int e = tid + q * TN;
+      const size_t m = hoff[q] + pz;
+#pragma unroll
+      for (int d = 0; d < 3; ++d) cp_async8(&p.w[d][e], (const double*)a.u + d * N + m);
+#pragma unroll
+      for (int k = 0; k < K; ++k) cp_async8(&p.rho[k][e], (const double*)a.rho_in + k * N + m);
+      p.sg[e] = a.vsig[m];
+    }
+  };
+  // a landed plane: the weights, each thread the elements that it copied
+  auto land = [&](int z) {
+    Adv64Plane<K>& p = t.pl[z & 3];
+    for (int e = tid; e < HP; e += TN) {
+#pragma unroll
+      for (int d = 0; d < 3; ++d) {
+        const double v = __longlong_as_double(__double_as_longlong(p.w[d][e]) & 0x7fffffffffffffffLL);
+        p.w[d][e] = v;
+        p.w[3 + d][e] = 1.0 - v;
       }
     }
-  }
-  // inflow from the 26 neighbours y = x - s: only those whose velocity points
-  // here along every nonzero component of s contribute
-  for (int qz = -1; qz <= 1; ++qz) {
-    for (int qy = -1; qy <= 1; ++qy) {
-      for (int qx = -1; qx <= 1; ++qx) {
-        if (!qx && !qy && !qz) continue;
-        const long long m = node_index(a.g, nb_x(b, x, -qx), nb_y(b, y, -qy), nb_z(b, z, -qz));
-        // the source must be fluid and move towards this node along every nonzero q
-        const unsigned mask = 0x80u | (qx ? 3u : 0u) | (qy ? 12u : 0u) | (qz ? 48u : 0u);
-        const unsigned want = 0x80u | (qx > 0 ? 1u : (qx < 0 ? 2u : 0u)) |
-                              (qy > 0 ? 4u : (qy < 0 ? 8u : 0u)) | (qz > 0 ? 16u : (qz < 0 ? 32u : 0u));
-        if ((a.vsig[m] & mask) != want) continue;
-        const double vx = u[m], vy = u[N + m], vz = u[2 * N + m];
-        if ((qx && sgn_bits(vx) != qx) || (qy && sgn_bits(vy) != qy) || (qz && sgn_bits(vz) != qz))
-          continue;
-        const double wx = qx ? abs_bits(vx) : 1.0 - abs_bits(vx);
-        const double wy = qy ? abs_bits(vy) : 1.0 - abs_bits(vy);
-        const double wz = qz ? abs_bits(vz) : 1.0 - abs_bits(vz);
-        const double frac = wx * wy * wz;
-#pragma unroll
-        for (int k = 0; k < K; ++k) acc[k] += rho_in[k * N + m] * frac;
-      }
-    }
-  }
+  };
+  stage(z0 - 1);
+  stage(z0);
+  stage(z0 + 1);
+  cp_async_wait_all();
+  land(z0 - 1);
+  land(z0);
   bool bad = false;
+  for (int z = z0; z < zend; ++z) {
+    const long long n = node_index(a.g, x, y, z);
+    double acc[K];
+    if (in_xy) {
 #pragma unroll
-  for (int k = 0; k < K; ++k) {
-    rho_out[k * N + n] = acc[k];
-    bad |= !isfinite(acc[k]);
+      for (int k = 0; k < K; ++k) acc[k] = rho_out[k * N + n];  // S2's result, issued early
+    }
+    cp_async_wait_all();
+    land(z + 1);
+    __syncthreads();  // planes z - 1, z, z + 1 ready; plane z - 2 no longer read
+    if (z + 1 < zend) stage(z + 2);
+    const Adv64Plane<K>& P0 = t.pl[z & 3];
+    const unsigned own = in_xy ? P0.sg[e0] : 0u;
+    if (!(own & 0x80u)) continue;  // fluid bit of S2 (the flags may change meanwhile)
+    // the neighbours that move here along every nonzero component of q
+    unsigned from = 0;
+#pragma unroll
+    for (int c = 0; c < 27; ++c) {
+      const int qx = c % 3 - 1, qy = c / 3 % 3 - 1, qz = c / 9 - 1;
+      if (!qx && !qy && !qz) continue;
+      const unsigned mask = 0x80u | (qx ? 3u : 0u) | (qy ? 12u : 0u) | (qz ? 48u : 0u);
+      const unsigned want = 0x80u | (qx > 0 ? 1u : (qx < 0 ? 2u : 0u)) | (qy > 0 ? 4u : (qy < 0 ? 8u : 0u)) |
+                            (qz > 0 ? 16u : (qz < 0 ? 32u : 0u));
+      const unsigned sg = t.pl[(z + 4 - qz) & 3].sg[e0 - qx - HX * qy];
+      if ((sg & mask) == want) from |= 1u << c;
+    }
+    // outflow: the shares that land on fluid nodes (one aimed at a boundary
+    // stays; one along a component of zero velocity is zero)
+    auto sign_of = [](unsigned v) { return v == 1u ? 1 : (v == 2u ? -1 : 0); };
+    const int sx = sign_of(own & 3u), sy = sign_of((own >> 2) & 3u), sz = sign_of((own >> 4) & 3u);
+    {
+      const double ax = P0.w[0][e0], ay = P0.w[1][e0], az = P0.w[2][e0];
+      const double bx = P0.w[3][e0], by = P0.w[4][e0], bz = P0.w[5][e0];
+      const double wxy[4] = {bx * by, ax * by, bx * ay, ax * ay};
+      const unsigned char* const f0 = P0.sg;
+      const unsigned char* const f1 = t.pl[(z + 4 + sz) & 3].sg;
+#pragma unroll
+      for (int o = 1; o < 8; ++o) {
+        const int e = e0 + ((o & 1) ? sx : 0) + ((o & 2) ? HX * sy : 0);
+        if (!(((o & 4) ? f1 : f0)[e] & 0x80u)) continue;
+        const double frac = wxy[o & 3] * ((o & 4) ? az : bz);
+#pragma unroll
+        for (int k = 0; k < K; ++k) acc[k] = fma(-P0.rho[k][e0], frac, acc[k]);
+      }
+    }
+    while (from) {
+      const int c = __ffs(from) - 1;
+      from &= from - 1u;
+      const int cz = c / 9, cy = (c - 9 * cz) / 3, cx = c - 9 * cz - 3 * cy;  // q + 1
+      const Adv64Plane<K>& P = t.pl[(z + 5 - cz) & 3];
+      const int e = e0 + 1 - cx + HX * (1 - cy);
+      const double frac = P.w[cx == 1 ? 3 : 0][e] * P.w[cy == 1 ? 4 : 1][e] * P.w[cz == 1 ? 5 : 2][e];
+#pragma unroll
+      for (int k = 0; k < K; ++k) acc[k] = fma(P.rho[k][e], frac, acc[k]);
+    }
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+      rho_out[k * N + n] = acc[k];
+      bad |= !finite_bits(acc[k]);
+    }
   }
+  cp_async_wait_all();
   if (bad) atomicOr(a.status, ST_NONFINITE);
 }
 
@@ -593,6 +654,11 @@ cudaError_t lb64_prepare() {
     e = cudaFuncSetAttribute(k_lb_fused<KK, PV>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(LB64Smem<KK>));
   EK_ATTR(0, true) EK_ATTR(1, true) EK_ATTR(2, true) EK_ATTR(3, true) EK_ATTR(4, true)
   EK_ATTR(0, false) EK_ATTR(1, false) EK_ATTR(2, false) EK_ATTR(3, false) EK_ATTR(4, false)
+#undef EK_ATTR
+#define EK_ATTR(KK)     \
+  if (e == cudaSuccess) \
+    e = cudaFuncSetAttribute(k_advect<KK>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Adv64Smem<KK>));
+  EK_ATTR(1) EK_ATTR(2) EK_ATTR(3) EK_ATTR(4)
 #undef EK_ATTR
   return e;
 }
@@ -644,13 +710,27 @@ cudaError_t launch_lb_fused(const LBArgs& a, cudaStream_t s) {
   return cudaGetLastError();
 }
 
+// Segments per tile column of S3: 8 planes each (a segment loads the plane on
+// each side of it as well), shorter while the grid has less than two rounds of
+// the two blocks that fit on an SM.
+int adv64_segments(const Grid& g) {
+  const long long cols = (long long)((g.nx + TILE_X - 1) / TILE_X) * ((g.ny + TILE_Y - 1) / TILE_Y);
+  int p = 8;
+  while (p > 1 && cols * ((g.nz + p - 1) / p) < 2 * 2 * 152) p /= 2;
+  return std::max(1, (g.nz + p - 1) / p);
+}
+
 cudaError_t launch_advection(const LBArgs& a, cudaStream_t s) {
+  const dim3 grid = lattice_grid32(a.g, a.advseg);
   switch (a.ph.K) {
     case 0: return cudaSuccess;
-    case 1: k_advect<1><<<lattice_grid(a.g), lattice_block(), 0, s>>>(a); break;
-    case 2: k_advect<2><<<lattice_grid(a.g), lattice_block(), 0, s>>>(a); break;
-    case 3: k_advect<3><<<lattice_grid(a.g), lattice_block(), 0, s>>>(a); break;
-    case 4: k_advect<4><<<lattice_grid(a.g), lattice_block(), 0, s>>>(a); break;
+#define EK_CASE(KK) \
+  case KK: k_advect<KK><<<grid, lattice_block(), sizeof(Adv64Smem<KK>), s>>>(a); break;
+    EK_CASE(1)
+    EK_CASE(2)
+    EK_CASE(3)
+    EK_CASE(4)
+#undef EK_CASE
     default: return cudaErrorInvalidValue;
   }
   return cudaGetLastError();
