@@ -751,19 +751,27 @@ __global__ void __launch_bounds__(FAST_T) k_fast_yz(PassArgs<float> a, int tx) {
 
 // Y (AXIS 1, forward or inverse) or Z (AXIS 2: forward, Green multiply,
 // inverse) pass for lines of NL = 16 N2 points (256, 512) as four-step
-// transforms on tiles of TX = 256 / N2 consecutive kx: x[N2 n1 + n2] ->
-// X[k1 + 16 k2].  Thread (c, n2) holds the 16 points n1 of its line in
+// transforms on tiles of 16 consecutive kx (128-byte rows): x[N2 n1 + n2] ->
+// X[k1 + 16 k2].  A thread (c, n2) holds the 16 points n1 of its line in
 // registers, transforms them, multiplies by the twiddle exp(-+2 pi i n2 k1 / NL)
-// and writes them to shared memory; after one barrier thread (c, k1) reads the
-// N2 points n2 and transforms them.  The Z pass keeps the result in
-// registers for the Green multiply and runs the inverse the same way back.
-// The shared layout c + TX (n2 + N2 k1) makes both the writes and the reads
-// of a warp contiguous.
+// and writes them to shared memory (512 points: for two n2, one after the
+// other); after one barrier thread (c, k1) reads the N2 points n2 and transforms
+// them.  The Z pass keeps the result in registers for the Green multiply and
+// runs the inverse the same way back.  The shared layout c + 16 (n2 + N2 k1)
+// makes both the writes and the reads of a warp contiguous.
+//
+// With tiles of 256 / N2 = 8 columns the 512-point passes moved 64-byte rows
+// and left half of the threads idle in the second transform: y 0.290 and z
+// 0.561 ms at 512^3 against 0.225 and 0.431 (S1 1.98 -> 1.72).
+template <int NL>
+constexpr size_t line4_smem() { return (size_t)(16 * NL + NL) * sizeof(float2); }
+
 template <int NL, int AXIS, bool INV>
 __global__ void __launch_bounds__(256) k_line4(PassArgs<float> a) {
-  constexpr int N1 = 16, N2 = NL / 16, TX = 256 / N2;
-  __shared__ __align__(16) float2 T[TX * NL];
-  __shared__ float2 tw[NL];
+  constexpr int N1 = 16, N2 = NL / 16, TX = 16, PER = TX * N2 / 256;
+  extern __shared__ __align__(16) unsigned char line4_raw[];
+  float2* const T = reinterpret_cast<float2*>(line4_raw);  // TX * NL
+  float2* const tw = T + TX * NL;
   const AxisPlan& P = AXIS == 1 ? a.ay : a.az;
   load_twiddles<NL>(tw, P);
   const int nxh = a.nxh;
@@ -774,28 +782,33 @@ __global__ void __launch_bounds__(256) k_line4(PassArgs<float> a) {
   const long long stride = AXIS == 1 ? (long long)nxh : (long long)nxh * a.ny;
   const long long base = (AXIS == 1 ? (long long)other * a.ny * nxh : (long long)other * nxh) + kx0;
   const int t = threadIdx.x;
-  const int c = t % TX;
+  const int c = t % TX, r = t / TX;
   const bool col = kx0 + c < nxh;
   constexpr bool FINV = AXIS == 1 && INV;  // direction of the first transform
   {
-    // thread (c, n2): the 16 points x[N2 n1 + n2]
-    const int n2 = t / TX;
-    float2 v[N1];
+    // (c, n2): the 16 points x[N2 n1 + n2]; all loads before the twiddles' barrier
+    float2 v[PER][N1];
 #pragma unroll
-    for (int n1 = 0; n1 < N1; ++n1)
-      v[n1] = col ? a.S[base + (long long)(N2 * n1 + n2) * stride + c] : make_float2(0.0f, 0.0f);
+    for (int q = 0; q < PER; ++q)
+#pragma unroll
+      for (int n1 = 0; n1 < N1; ++n1)
+        v[q][n1] = col ? a.S[base + (long long)(N2 * n1 + r + 16 * q) * stride + c] : make_float2(0.0f, 0.0f);
     __syncthreads();  // the twiddles
-    dft_reg<N1, FINV>(v);
 #pragma unroll
-    for (int k1 = 0; k1 < N1; ++k1) {
-      const float2 w = tw[n2 * k1];
-      T[c + TX * (n2 + N2 * k1)] = FINV ? cmulconj(v[k1], w) : cmul(v[k1], w);
+    for (int q = 0; q < PER; ++q) {
+      const int n2 = r + 16 * q;
+      dft_reg<N1, FINV>(v[q]);
+#pragma unroll
+      for (int k1 = 0; k1 < N1; ++k1) {
+        const float2 w = tw[n2 * k1];
+        T[c + TX * (n2 + N2 * k1)] = FINV ? cmulconj(v[q][k1], w) : cmul(v[q][k1], w);
+      }
     }
   }
   __syncthreads();
-  if (t < TX * N1) {
-    // thread (c, k1): the N2 points n2, giving X[k1 + 16 k2]
-    const int k1 = t / TX;
+  {
+    // (c, k1): the N2 points n2, giving X[k1 + 16 k2]
+    const int k1 = r;
     float2 z[N2];
 #pragma unroll
     for (int n2 = 0; n2 < N2; ++n2) z[n2] = T[c + TX * (n2 + N2 * k1)];
@@ -824,24 +837,35 @@ __global__ void __launch_bounds__(256) k_line4(PassArgs<float> a) {
   }
   if constexpr (AXIS == 2) {
     __syncthreads();
-    const int n2 = t / TX;
-    float2 v[N1];
 #pragma unroll
-    for (int k1 = 0; k1 < N1; ++k1) v[k1] = T[c + TX * (n2 + N2 * k1)];
-    dft_reg<N1, true>(v);
-    if (col) {
+    for (int q = 0; q < PER; ++q) {
+      const int n2 = r + 16 * q;
+      float2 v[N1];
 #pragma unroll
-      for (int n1 = 0; n1 < N1; ++n1) a.S[base + (long long)(N2 * n1 + n2) * stride + c] = v[n1];
+      for (int k1 = 0; k1 < N1; ++k1) v[k1] = T[c + TX * (n2 + N2 * k1)];
+      dft_reg<N1, true>(v);
+      if (col) {
+#pragma unroll
+        for (int n1 = 0; n1 < N1; ++n1) a.S[base + (long long)(N2 * n1 + n2) * stride + c] = v[n1];
+      }
     }
   }
 }
 
 template <int NL, int AXIS, bool INV>
 void launch_line4(PassArgs<float>& a, cudaStream_t s) {
-  constexpr int TX = 256 / (NL / 16);
-  const int ntile = (a.nxh + TX - 1) / TX;
+  const int ntile = (a.nxh + 15) / 16;
   const int nother = AXIS == 1 ? a.nz : a.ny;
-  k_line4<NL, AXIS, INV><<<(unsigned)(ntile * nother), 256, 0, s>>>(a);
+  k_line4<NL, AXIS, INV><<<(unsigned)(ntile * nother), 256, line4_smem<NL>(), s>>>(a);
+}
+template <int NL>
+cudaError_t line4_attr() {
+  cudaError_t e = cudaFuncSetAttribute(k_line4<NL, 1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)line4_smem<NL>());
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_line4<NL, 1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)line4_smem<NL>());
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_line4<NL, 2, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)line4_smem<NL>());
+  return e;
 }
 
 // X pass, inverse (complex-to-real), two rows per complex transform (as k_fft_x_inv).
@@ -1348,8 +1372,10 @@ cudaError_t poisson_plan_create(PoissonPlan& p, int nx, int ny, int nz, std::str
     if (e == cudaSuccess) e = plane_batch_attr_n<32>();
     if (e == cudaSuccess) e = plane_batch_attr_n<48>();
     if (e == cudaSuccess) e = plane_batch_attr_n<64>();
+    if (e == cudaSuccess) e = line4_attr<256>();
+    if (e == cudaSuccess) e = line4_attr<512>();
     if (e != cudaSuccess) {
-      err = "shared-memory size of the plane FFT kernels could not be set";
+      err = "shared-memory size of the FFT kernels could not be set";
       return e;
     }
   }
