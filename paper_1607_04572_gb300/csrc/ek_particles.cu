@@ -1170,6 +1170,11 @@ __global__ void __launch_bounds__(PT) k_claim(PartArgs a) { claim_body<FM>(a, gr
 // float, with the exact FP64 test of the octree where the float distance lies
 // within the margin of R^2 (see classify_f32).  A centre within the cell's u
 // extent (cells of spheres below R = 2) takes every plane's test.
+//
+// Bound by its instructions (780 000 cells at 512^3 with 1000 spheres of R = 6).
+// Where the centre lies beyond the cell along all three axes a column's far
+// line is the near line of a column further out, so one count on each of the
+// 17 x 17 lines replaces two on each of the 256 columns: 0.81 -> 0.71 ms there.
 constexpr int PSI_CTA = 256;  // threads per CTA of k_psi_surface
 
 struct PsiCell {
@@ -1266,10 +1271,46 @@ __device__ __noinline__ int psi_settle(const PsiCell* c, float S, float e0, int 
   return T;
 }
 
+// The same count for a cell whose v and w extents do not hold the centre either:
+// the column's corner lines run through the planes jv and lw, so the test is
+// that of a lattice point (the far corner of one column and the near face's
+// corner of the next have the same FP64 offsets).
+__device__ __noinline__ bool psi_exact_point(const PsiCell* c, int mu, int jv, int lw) {
+  double o[3];
+  o[c->u] = fabs(plane_off_d(*c, c->u, mu));
+  o[c->v] = fabs(plane_off_d(*c, c->v, jv));
+  o[c->w] = fabs(plane_off_d(*c, c->w, lw));
+  return dist2(o[0], o[1], o[2]) < c->R2;
+}
+__device__ __noinline__ int psi_settle_point(const PsiCell* c, float S, float e0, int near, int step, float bu,
+                                             float fu, int jv, int lw) {
+  const float A = c->R2f - S;
+  int T = 0;
+  if (A > 2.0f * c->margin) {
+    const float ra = rsqrtf(A);
+    T = min(max((int)ceilf((A * ra - e0) * 16.0f), 0), 17);
+  } else if (A > 0.0f) {
+    T = min(max((int)ceilf((sqrtf(A) - e0) * 16.0f), 0), 17);
+  }
+  auto off = [](float b, float f, int m) { return __fsub_rn(b + (0.0625f * (float)m - 0.5f), f); };
+  auto pin = [&](int t) {
+    const int m = near + step * t;
+    const float gu = fabsf(off(bu, fu, m));
+    const float d = gu * gu + S;
+    if (d < c->R2f - c->margin) return true;
+    if (d > c->R2f + c->margin) return false;
+    return psi_exact_point(c, m, jv, lw);
+  };
+  while (T > 0 && !pin(T - 1)) --T;
+  while (T < 17 && pin(T)) ++T;
+  return T;
+}
+
 template <class FM>
 __device__ __forceinline__ void psi_surface_body(const PartArgs& a, const Blk bk) {
-  // per warp: the squared far and near offsets of the 16 slabs along w
-  __shared__ float wslab[PSI_CTA / 32][2][16];
+  // per warp: the squared far and near offsets of the 16 slabs along w, or (the
+  // lattice form) the squared offsets of the 17 planes along w
+  __shared__ float wslab[PSI_CTA / 32][2][17];
   const int lane = threadIdx.x & 31;
   const int wib = threadIdx.x >> 5;
   const int warp = (bk.x * PSI_CTA + threadIdx.x) >> 5;
@@ -1295,18 +1336,21 @@ __device__ __forceinline__ void psi_surface_body(const PartArgs& a, const Blk bk
     }
     const int v = u == 0 ? 1 : 0;
     const int w = u == 2 ? 1 : 2;
-    // near end of the columns: the plane nearest the centre, when the centre
-    // lies beyond the cell along u.  Exact without FP64: the centre is
-    // ipos + frac with frac = fpos + fposlo (the residual's sign exact), so
-    // pos <= X - 1/2 iff m = X - ipos >= 2, or m = 1 and frac <= 1/2, and
-    // pos >= X + 1/2 iff m <= -1, or m = 0 and frac >= 1/2
-    const int mu_ = X[u] - P.ipos[u];
-    const float fh = P.fpos[u], fl = P.fposlo[u];
-    const bool le_half = fh < 0.5f || (fh == 0.5f && fl <= 0.0f);
-    const bool ge_half = fh > 0.5f || (fh == 0.5f && fl >= 0.0f);
-    const int near = (mu_ >= 2 || (mu_ == 1 && le_half)) ? 0
-                     : ((mu_ <= -1 || (mu_ == 0 && ge_half)) ? 16 : -1);
+    // near end of the cell along an axis: the plane (0 or 16) nearest the
+    // centre when the centre lies beyond the cell, else -1.  Exact without FP64:
+    // the centre is ipos + frac with frac = fpos + fposlo (the residual's sign
+    // exact), so pos <= X - 1/2 iff m = X - ipos >= 2, or m = 1 and frac <= 1/2,
+    // and pos >= X + 1/2 iff m <= -1, or m = 0 and frac >= 1/2
+    auto near_end = [&](int d) {
+      const int m = X[d] - P.ipos[d];
+      const float fh = P.fpos[d], fl = P.fposlo[d];
+      const bool le_half = fh < 0.5f || (fh == 0.5f && fl <= 0.0f);
+      const bool ge_half = fh > 0.5f || (fh == 0.5f && fl >= 0.0f);
+      return (m >= 2 || (m == 1 && le_half)) ? 0 : ((m <= -1 || (m == 0 && ge_half)) ? 16 : -1);
+    };
+    const int near = near_end(u);
     const int step = near == 0 ? 1 : -1;
+    const int nearv = near_end(v), nearw = near_end(w);
     // per-axis constants of the float offsets (registers, not indexed)
     const float bu = fb[u], bv = fb[v], bw = fb[w];
     const float fu = P.fpos[u], fv_ = P.fpos[v], fw_ = P.fpos[w];
@@ -1315,20 +1359,8 @@ __device__ __forceinline__ void psi_surface_body(const PartArgs& a, const Blk bk
     // lane's columns share one v slab (j = lane mod 16) and take their w slabs
     // (l) from the warp's table
     const int jl = lane & 15;
-    float FV2, NV2;
-    {
-      const float v0 = off(bv, fv_, jl), v1 = off(bv, fv_, jl + 1);
-      const float w0 = off(bw, fw_, jl), w1 = off(bw, fw_, jl + 1);
-      const float fv = slab_f(v0, v1, true), nv = slab_f(v0, v1, false);
-      const float fw = slab_f(w0, w1, true), nw = slab_f(w0, w1, false);
-      FV2 = fv * fv;
-      NV2 = nv * nv;
-      if (lane < 16) {
-        wslab[wib][0][jl] = fw * fw;
-        wslab[wib][1][jl] = nw * nw;
-      }
-    }
-    __syncwarp();
+    const float e0 = near >= 0 ? fabsf(off(bu, fu, near)) : 0.0f;
+    int units = 0;
     // the cell in the form the plane tests take (built where they run)
     auto cell = [&]() {
       PsiCell c;
@@ -1345,8 +1377,69 @@ __device__ __forceinline__ void psi_surface_body(const PartArgs& a, const Blk bk
       c.w = w;
       return c;
     };
-    int units = 0;
-    const float e0 = near >= 0 ? fabsf(off(bu, fu, near)) : 0.0f;
+    float FV2 = 0.0f, NV2 = 0.0f;
+    if (near >= 0 && nearv >= 0 && nearw >= 0) {
+      // The centre lies beyond the cell along every axis (all but the cells
+      // around the sphere's equators): with the planes numbered from the near
+      // ends, column (j, l) has its near line through the planes (j, l) and its
+      // far one through (j + 1, l + 1).  So T, the count of planes along u
+      // nearer than R on a line, is needed on the 17 x 17 lines only, and a line
+      // counts min(T, 16) near faces for the column beyond it (j, l < 16) and
+      // T - 1 inside cubes for the column before it (j, l >= 1).
+      const int stv = nearv == 0 ? 1 : -1, stw = nearw == 0 ? 1 : -1;
+      if (lane < 17) {
+        const float o = off(bw, fw_, nearw + stw * lane);
+        wslab[wib][0][lane] = o * o;
+      }
+      const float ov = off(bv, fv_, nearv + stv * jl), ov16 = off(bv, fv_, nearv + stv * 16);
+      const float V2 = ov * ov, V216 = ov16 * ov16;
+      __syncwarp();
+      // lines (jl, (lane >> 4) + 2 q), q < 8; then the edge lines (jl, 16) and
+      // (16, jl), and (16, 16) by lane 0
+      unsigned unsure = 0u;
+      auto line = [&](int q, int& jv, int& lw) {
+        jv = q < 8 ? jl : (q == 9 || lane >= 16 ? 16 : jl);
+        lw = q < 8 ? (lane >> 4) + 2 * q : (q == 9 || lane < 16 ? 16 : jl);
+      };
+      auto add = [&](int T, int jv, int lw) {
+        units += (jv < 16 && lw < 16 ? min(T, 16) : 0) + (jv >= 1 && lw >= 1 ? max(T - 1, 0) : 0);
+      };
+#pragma unroll
+      for (int q = 0; q < 9; ++q) {
+        int jv, lw;
+        line(q, jv, lw);
+        bool sure;
+        const float S = (q < 8 || lane < 16 ? V2 : V216) + wslab[wib][0][lw];
+        const int T = psi_count(S, R2f, margin, e0, 17, sure);
+        if (sure) add(T, jv, lw);
+        else unsure |= 1u << q;
+      }
+      if (lane == 0) unsure |= 1u << 9;
+      if (unsure) {
+        const PsiCell c = cell();
+        do {
+          const int q = __ffs(unsure) - 1;
+          unsure &= unsure - 1u;
+          int jv, lw;
+          line(q, jv, lw);
+          const float S = (jv == 16 ? V216 : V2) + wslab[wib][0][lw];
+          add(psi_settle_point(&c, S, e0, near, step, bu, fu, nearv + stv * jv, nearw + stw * lw), jv, lw);
+        } while (unsure);
+      }
+    } else {
+    {
+      const float v0 = off(bv, fv_, jl), v1 = off(bv, fv_, jl + 1);
+      const float w0 = off(bw, fw_, jl), w1 = off(bw, fw_, jl + 1);
+      const float fv = slab_f(v0, v1, true), nv = slab_f(v0, v1, false);
+      const float fw = slab_f(w0, w1, true), nw = slab_f(w0, w1, false);
+      FV2 = fv * fv;
+      NV2 = nv * nv;
+      if (lane < 16) {
+        wslab[wib][0][jl] = fw * fw;
+        wslab[wib][1][jl] = nw * nw;
+      }
+    }
+    __syncwarp();
     if (near >= 0) {
       // T: planes t = 0..16 from the near end whose far corner is inside
       // (T - 1 inside cubes); TN: cubes t = 0..15 whose near face is nearer
@@ -1396,6 +1489,7 @@ __device__ __forceinline__ void psi_surface_body(const PartArgs& a, const Blk bk
           if (psi_test(c, slab_f(a0, a1, false), near2, k, k + 1, j, l, false)) units += 1;
         }
       }
+    }
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) units += __shfl_xor_sync(0xffffffffu, units, o);
