@@ -46,3 +46,29 @@ def test_fp32_plans(gpu_lib, shape):
     got = s.get_fields(ek.FIELD_PHI).reshape(nz, ny, nx)
     # as for the specialised transforms: FP32 rounding of the spectrum
     assert np.max(np.abs(got - ref)) <= 2e-5 * np.max(np.abs(ref))
+
+
+@pytest.mark.parametrize("shape", [(256, 9, 9), (512, 9, 9), (256, 8, 8), (512, 18, 27), (256, 256, 9), (512, 64, 36),
+                                   (256, 36, 512)])
+@pytest.mark.parametrize("species", [(1,), (1, -1, 2)])
+def test_fp32_row_lines(gpu_lib, shape, species):
+    """The x passes of 256 and 512 points (two lines of two rows to a warp, four
+    warps to a block): odd and ragged numbers of rows, with a wall charge, one
+    and three species."""
+    ek = gpu_lib
+    nx, ny, nz = shape
+    K = len(species)
+    s = ek.EKSystem(shape, nu=1.0 / 6.0, rho0=1.0, bjerrum=0.7, valence=species, D=(0.3,) * K,
+                    bulk=(1e-3,) * K, flags=ek.EK_FP32)
+    q = 1e-3 * workloads.perturbation(nx * ny * nz, 0.5, 301)
+    s.set_field(ek.FIELD_WALL_CHARGE, q)
+    q = q.reshape(nz, ny, nx)
+    for k in range(K):
+        s.set_field(ek.FIELD_SPECIES, 1e-3 * (1.0 + workloads.perturbation(nx * ny * nz, 0.5, 302 + k)), component=k)
+        q = q + species[k] * s.get_fields(ek.FIELD_SPECIES, k).reshape(nz, ny, nx)
+    ref = O.poisson(q, 0.7)
+    s.run_stage(1)
+    got = s.get_fields(ek.FIELD_PHI).reshape(nz, ny, nx)
+    # as above: FP32 rounding of the spectrum
+    assert np.max(np.abs(got - ref)) <= 2e-5 * np.max(np.abs(ref))
+    s.close()
