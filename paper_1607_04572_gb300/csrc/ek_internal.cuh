@@ -434,6 +434,7 @@ struct PartArgs {
 // 32.6, 34.2; eight R = 4 48.8, 43.0, 44.8; 64 of R = 5 (256^3) 256 / 512: 167, 130.
 constexpr int FORCE_T = 128;
 constexpr int FORCE_CHUNK = 256;
+constexpr int FORCE_ROWS = 16 * FORCE_CHUNK / FORCE_T;  // most rows of a CTA
 // per particle: [0..5] Fh Th (momentum exchange), [6..11] Fs Ts (reaction of
 // the solute force), [12] sum w and [13..15] sum w (r - r_p) of the weights of
 // the particle's own charge (times the charge per unit weight, the field's force

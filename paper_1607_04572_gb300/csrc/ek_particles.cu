@@ -455,9 +455,8 @@ __device__ void column_sums(const double* tab, int nrow, int stride, int col0, d
 __device__ void integrate_all(const PartArgs& a);
 
 template <int NV, class Get>
-__device__ void block_sum_t(Get v, unsigned on, double* out) {
+__device__ void block_sum_t(Get v, double (*tr)[FORCE_T + 1], unsigned on, double* out) {
   constexpr int S = 16;
-  __shared__ double tr[NV][FORCE_T + 1];
   const int t = threadIdx.x;
 #pragma unroll
   for (int j = 0; j < NV; ++j)
@@ -495,7 +494,10 @@ __device__ void block_sum_t(Get v, unsigned on, double* out) {
 // weight, a division, is applied once per particle (integrate_all).
 // Block (p, b) takes the rows b, b + nb, b + 2 nb, ... of FORCE_T cells of the
 // widened box (nb blocks for this particle), so the cells next to the sphere
-// are spread over all blocks.
+// are spread over all blocks.  Bound by the latency of the loads, one row ahead.
+// The links are taken after the rows, from a list: a row of 32 cells holds few
+// nodes next to the sphere, and without the links' registers in the loop more
+// blocks are in flight (S4 1.35 -> 1.12 ms at 512^3 with 1000 particles).
 // ONE: a single particle, which claims every node of its widened box without
 // keys (1), several (0), or either (2: the batched launch; tested per cell it
 // costs 8% at 1000 particles).
@@ -604,8 +606,16 @@ __device__ __forceinline__ void particle_forces_body(const PartArgs& a, const Bl
     gate = 2.0 * P.radius + 4.0 <= (double)nmin;
     rlink = P.radius + 1.5;
   }
+  // the warp's fluid nodes next to the particle (at most one per cell), as box
+  // offsets of ten bits each: the links are taken after the loop, 32 nodes at a
+  // time.  The list takes the room of the block sums that follow it.
+  __shared__ double tr[FPART][FORCE_T + 1];
+  static_assert(sizeof(tr) >= FORCE_ROWS * FORCE_T * sizeof(unsigned), "one entry per cell");
+  unsigned* const list = reinterpret_cast<unsigned*>(tr) + (threadIdx.x >> 5) * (FORCE_ROWS * 32);
+  int nlist = 0;
   for (int k = 0; k < rows; ++k) {
-    if (!nvalid) break;
+    const bool valid = nvalid;
+    if (!__any_sync(0xffffffffu, valid)) break;
     const int X = nX, Y = nY, Z = nZ;
     const long long n = nn;
     const double mx = nmx, my = nmy, mz = nmz;
@@ -635,7 +645,7 @@ __device__ __forceinline__ void particle_forces_body(const PartArgs& a, const Bl
     }
     const bool in_box = X >= P.lo[0] && X < P.hi[0] && Y >= P.lo[1] && Y < P.hi[1] &&
                         Z >= P.lo[2] && Z < P.hi[2];
-    bool near = own == FLUID && in_box;
+    bool near = valid && own == FLUID && in_box;
     if (near && gate) {
       if (FM::fp32) {
         const float ex = __fsub_rn((float)(X - P.ipos[0]), P.fpos[0]);
@@ -647,82 +657,14 @@ __device__ __forceinline__ void particle_forces_body(const PartArgs& a, const Bl
         near = ex * ex + ey * ey + ez * ez < rlink * rlink;
       }
     }
+    const unsigned nl = __ballot_sync(0xffffffffu, near);
     if (near) {
-      // momentum exchange on every link from this fluid node into the particle
-      // (Eq. 11): the links first (all 18 owner loads in flight together), the
-      // FP64 arithmetic only at nodes next to the surface
-      const Nbr b = make_nbr(w3[0], w3[1], w3[2], g);
-      unsigned links = 0;
-#pragma unroll
-      for (int i = 1; i < Q; ++i) {
-        const long long m = node_index(g, nb_x(b, w3[0], dcx(i)), nb_y(b, w3[1], dcy(i)),
-                                       nb_z(b, w3[2], dcz(i)));
-        if (a.owner[m] == p) links |= 1u << i;
-      }
-      if (links && FM::fp32) {
-        // FP32 form, in float: the populations are stored as deviations
-        // g = f - w rho0, so f*_i + f_ibar = 2 g_ibar + 2 w rho0 + 6 w rho0 c.w;
-        // the deviation terms are small, and the rest-density term is summed
-        // as an exact integer count of 36 w_i c_i
-        const float d0x = __fsub_rn((float)(X - P.ipos[0]), P.fpos[0]);
-        const float d0y = __fsub_rn((float)(Y - P.ipos[1]), P.fpos[1]);
-        const float d0z = __fsub_rn((float)(Z - P.ipos[2]), P.fpos[2]);
-        const float wx = vxf + (qyf * d0z - qzf * d0y);
-        const float wy = vyf + (qzf * d0x - qxf * d0z);
-        const float wz = vzf + (qxf * d0y - qyf * d0x);
-        const float r0 = rho0f;
-        float fx = 0.0f, fy = 0.0f, fz = 0.0f;
-        int kx = 0, ky = 0, kz = 0;  // sum of 36 w_i c_i over the links
-#pragma unroll
-        for (int i = 1; i < Q; ++i) {
-          if (!(links & (1u << i))) continue;
-          const float gdev = ((const float*)a.f)[(long long)opp(i) * N + n];
-          float cw = 0.0f;
-          if (dcx(i)) cw = dcx(i) > 0 ? cw + wx : cw - wx;
-          if (dcy(i)) cw = dcy(i) > 0 ? cw + wy : cw - wy;
-          if (dcz(i)) cw = dcz(i) > 0 ? cw + wz : cw - wz;
-          const float mom = 2.0f * gdev + 6.0f * (float)wgt(i) * r0 * cw;
-          const int k36 = i < 7 ? 2 : 1;
-          if (dcx(i)) { fx = dcx(i) > 0 ? fx + mom : fx - mom; kx += dcx(i) * k36; }
-          if (dcy(i)) { fy = dcy(i) > 0 ? fy + mom : fy - mom; ky += dcy(i) * k36; }
-          if (dcz(i)) { fz = dcz(i) > 0 ? fz + mom : fz - mom; kz += dcz(i) * k36; }
-        }
-        const float cst = 2.0f * r0 / 36.0f;
-        fx += cst * (float)kx;
-        fy += cst * (float)ky;
-        fz += cst * (float)kz;
-        touched |= 1u;
-        macc[0] += fx;
-        macc[1] += fy;
-        macc[2] += fz;
-        macc[3] += d0y * fz - d0z * fy;
-        macc[4] += d0z * fx - d0x * fz;
-        macc[5] += d0x * fy - d0y * fx;
-      } else if (links) {
-        const double d0x = (double)X - P.pos[0], d0y = (double)Y - P.pos[1], d0z = (double)Z - P.pos[2];
-        const double wx = P.vel[0] + (P.omega[1] * d0z - P.omega[2] * d0y);
-        const double wy = P.vel[1] + (P.omega[2] * d0x - P.omega[0] * d0z);
-        const double wz = P.vel[2] + (P.omega[0] * d0y - P.omega[1] * d0x);
-        double fx = 0.0, fy = 0.0, fz = 0.0;
-#pragma unroll
-        for (int i = 1; i < Q; ++i) {
-          if (!(links & (1u << i))) continue;
-          const double refl = pop_abs<FM>(a.f, opp(i), N, n, rho0);
-          const double fs = refl + 6.0 * wgt(i) * rho0 * cdot(i, wx, wy, wz);  // the population that hit the wall
-          const double mom = fs + refl;
-          if (dcx(i)) fx = dcx(i) > 0 ? fx + mom : fx - mom;
-          if (dcy(i)) fy = dcy(i) > 0 ? fy + mom : fy - mom;
-          if (dcz(i)) fz = dcz(i) > 0 ? fz + mom : fz - mom;
-        }
-        touched |= 1u;
-        acc[0] += fx;
-        acc[1] += fy;
-        acc[2] += fz;
-        acc[3] += d0y * fz - d0z * fy;
-        acc[4] += d0z * fx - d0x * fz;
-        acc[5] += d0x * fy - d0y * fx;
-      }
+      // in_box: the box offsets are below 1024
+      list[nlist + __popc(nl & ((1u << (threadIdx.x & 31)) - 1u))] =
+          (unsigned)(X - P.lo[0]) | (unsigned)(Y - P.lo[1]) << 10 | (unsigned)(Z - P.lo[2]) << 20;
     }
+    nlist += __popc(nl);
+    if (!valid) continue;
     // reaction of the internal solute force on the fluid nodes this particle claims
     // the key of a node is cleared by the particle it names, right after
     // reading it: any other particle reading it meanwhile finds either that
@@ -792,6 +734,88 @@ __device__ __forceinline__ void particle_forces_body(const PartArgs& a, const Bl
       }
     }
   }
+  // the list, whole warps of neighbours of the surface (a row of the box has few)
+  __syncwarp();
+  for (int q = threadIdx.x & 31; q < nlist; q += 32) {
+    const unsigned at = list[q];
+    const int X = P.lo[0] + (int)(at & 1023u), Y = P.lo[1] + (int)(at >> 10 & 1023u), Z = P.lo[2] + (int)(at >> 20);
+    const int w3[3] = {wrap_box(X, g.nx), wrap_box(Y, g.ny), wrap_box(Z, g.nz)};
+    const long long n = (long long)(w3[0] + g.nx * (w3[1] + g.ny * w3[2]));
+    // momentum exchange on every link from this fluid node into the particle
+    // (Eq. 11): the links first (all 18 owner loads in flight together), the
+    // FP64 arithmetic only at nodes next to the surface
+    const Nbr b = make_nbr(w3[0], w3[1], w3[2], g);
+    unsigned links = 0;
+#pragma unroll
+    for (int i = 1; i < Q; ++i) {
+      const long long m = node_index(g, nb_x(b, w3[0], dcx(i)), nb_y(b, w3[1], dcy(i)),
+                                     nb_z(b, w3[2], dcz(i)));
+      if (a.owner[m] == p) links |= 1u << i;
+    }
+    if (links && FM::fp32) {
+      // FP32 form, in float: the populations are stored as deviations
+      // g = f - w rho0, so f*_i + f_ibar = 2 g_ibar + 2 w rho0 + 6 w rho0 c.w;
+      // the deviation terms are small, and the rest-density term is summed
+      // as an exact integer count of 36 w_i c_i
+      const float d0x = __fsub_rn((float)(X - P.ipos[0]), P.fpos[0]);
+      const float d0y = __fsub_rn((float)(Y - P.ipos[1]), P.fpos[1]);
+      const float d0z = __fsub_rn((float)(Z - P.ipos[2]), P.fpos[2]);
+      const float wx = vxf + (qyf * d0z - qzf * d0y);
+      const float wy = vyf + (qzf * d0x - qxf * d0z);
+      const float wz = vzf + (qxf * d0y - qyf * d0x);
+      const float r0 = rho0f;
+      float fx = 0.0f, fy = 0.0f, fz = 0.0f;
+      int kx = 0, ky = 0, kz = 0;  // sum of 36 w_i c_i over the links
+#pragma unroll
+      for (int i = 1; i < Q; ++i) {
+        if (!(links & (1u << i))) continue;
+        const float gdev = ((const float*)a.f)[(long long)opp(i) * N + n];
+        float cw = 0.0f;
+        if (dcx(i)) cw = dcx(i) > 0 ? cw + wx : cw - wx;
+        if (dcy(i)) cw = dcy(i) > 0 ? cw + wy : cw - wy;
+        if (dcz(i)) cw = dcz(i) > 0 ? cw + wz : cw - wz;
+        const float mom = 2.0f * gdev + 6.0f * (float)wgt(i) * r0 * cw;
+        const int k36 = i < 7 ? 2 : 1;
+        if (dcx(i)) { fx = dcx(i) > 0 ? fx + mom : fx - mom; kx += dcx(i) * k36; }
+        if (dcy(i)) { fy = dcy(i) > 0 ? fy + mom : fy - mom; ky += dcy(i) * k36; }
+        if (dcz(i)) { fz = dcz(i) > 0 ? fz + mom : fz - mom; kz += dcz(i) * k36; }
+      }
+      const float cst = 2.0f * r0 / 36.0f;
+      fx += cst * (float)kx;
+      fy += cst * (float)ky;
+      fz += cst * (float)kz;
+      touched |= 1u;
+      macc[0] += fx;
+      macc[1] += fy;
+      macc[2] += fz;
+      macc[3] += d0y * fz - d0z * fy;
+      macc[4] += d0z * fx - d0x * fz;
+      macc[5] += d0x * fy - d0y * fx;
+    } else if (links) {
+      const double d0x = (double)X - P.pos[0], d0y = (double)Y - P.pos[1], d0z = (double)Z - P.pos[2];
+      const double wx = P.vel[0] + (P.omega[1] * d0z - P.omega[2] * d0y);
+      const double wy = P.vel[1] + (P.omega[2] * d0x - P.omega[0] * d0z);
+      const double wz = P.vel[2] + (P.omega[0] * d0y - P.omega[1] * d0x);
+      double fx = 0.0, fy = 0.0, fz = 0.0;
+#pragma unroll
+      for (int i = 1; i < Q; ++i) {
+        if (!(links & (1u << i))) continue;
+        const double refl = pop_abs<FM>(a.f, opp(i), N, n, rho0);
+        const double fs = refl + 6.0 * wgt(i) * rho0 * cdot(i, wx, wy, wz);  // the population that hit the wall
+        const double mom = fs + refl;
+        if (dcx(i)) fx = dcx(i) > 0 ? fx + mom : fx - mom;
+        if (dcy(i)) fy = dcy(i) > 0 ? fy + mom : fy - mom;
+        if (dcz(i)) fz = dcz(i) > 0 ? fz + mom : fz - mom;
+      }
+      touched |= 1u;
+      acc[0] += fx;
+      acc[1] += fy;
+      acc[2] += fz;
+      acc[3] += d0y * fz - d0z * fy;
+      acc[4] += d0z * fx - d0x * fz;
+      acc[5] += d0x * fy - d0y * fx;
+    }
+  }
   float facc[FPART];
   if (FM::fp32) {
 #pragma unroll
@@ -831,9 +855,9 @@ __device__ __forceinline__ void particle_forces_body(const PartArgs& a, const Bl
   if (FM::fp32) {
     // each thread's float sums over its own few cells, widened to FP64 (the
     // lattice slice is FP64 already); everything above them in FP64
-    block_sum_t<FPART>([&](int j) { return (j >= 18 && j < 21) ? acc[j] : (double)facc[j]; }, on, out);
+    block_sum_t<FPART>([&](int j) { return (j >= 18 && j < 21) ? acc[j] : (double)facc[j]; }, tr, on, out);
   } else {
-    block_sum_t<FPART>([&](int j) { return acc[j]; }, on, out);
+    block_sum_t<FPART>([&](int j) { return acc[j]; }, tr, on, out);
   }
   // the particle's last block sums its rows; the last particle integrates
   __shared__ bool last;
@@ -861,11 +885,13 @@ __device__ __forceinline__ void particle_forces_body(const PartArgs& a, const Bl
   }
 }
 
-// four blocks per SM: with five (96 registers, spills in the cell loop) S4 takes
-// 1.50 ms instead of 1.35 at 512^3 with 1000 particles, 126 us instead of 121 at
-// 256^3 with 64, 33.4 instead of 29.5 with one at 128^3
+// Blocks per SM 4 / 5 / 6 (118, 96, 80 registers; the spills lie outside the cell
+// loop), S4 and the step's graph in ms: 512^3 with 1000 particles 1.184, 1.122,
+// 1.104 and 10.88, 10.84, 10.90 (the graph runs S4 beside S3); 256^3 with 64
+// particles 0.117, 0.111, 0.109 and 1.396, 1.396, 1.404; one particle at 128^3
+// 29.6, 30.4, 31.6 us.  The batched launch spills 134 bytes at five.
 template <class FM, int ONE>
-__global__ void __launch_bounds__(FORCE_T, 4) k_particle_forces(PartArgs a) {
+__global__ void __launch_bounds__(FORCE_T, FM::fp32 && ONE == 0 ? 5 : 4) k_particle_forces(PartArgs a) {
   particle_forces_body<FM, ONE>(a, grid_blk());
 }
 __device__ __forceinline__ void particle_forces_any(const PartArgs& a, const Blk bk) {
