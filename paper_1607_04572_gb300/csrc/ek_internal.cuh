@@ -2,6 +2,7 @@
 // layout, the D3Q19 velocity set and the kernel launchers of each stage.
 #pragma once
 
+#include <utility>
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -133,6 +134,45 @@ struct FormF32 {
   using real_t = float;
   static constexpr bool fp32 = true;
 };
+
+// Launches of a chain whose next kernel waits for the one before it on the same
+// stream.  A kernel launched by launch_next may be brought onto the SMs while its
+// predecessor still runs (programmatic dependent launch); it calls after_previous
+// before it touches anything the predecessor writes or reads, which returns once
+// that kernel has finished and its writes are visible.  A kernel calls
+// let_next_start to allow its successor's launch; without it, or with an ordinary
+// launch, the successor starts after its end.  Every kernel of such a chain calls
+// after_previous in all of its threads, so that its end implies the end of all
+// before it.
+//
+// These chains are bound by the launches where the kernels take a few us each:
+// the Poisson solve of a 48 x 32 x 72 box (FP64, five passes) 43.8 -> 38.9 us, 13
+// V-cycles at 128^3 4.33 -> 3.34 ms, the set-up of the conjugate gradients there
+// 0.2 ms less, stage 5 of a 32^3 box 44 -> 32 us.  Under
+// capture the launches stay ordinary: a graph starts its next kernel soon enough
+// by itself, and successors that wait on the SMs beside a forked branch hold it
+// up (a step's graph with and without: 32^3 65.9, 68.0 us; 128^3 209, 205;
+// 256^3 1422, 1398).
+__device__ __forceinline__ void after_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+inline bool early_launch(cudaStream_t s) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  return cudaStreamIsCapturing(s, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone;
+}
+template <class... P, class... A>
+void launch_next(void (*k)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A&&... args) {
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t c = {};
+  c.gridDim = grid;
+  c.blockDim = block;
+  c.dynamicSmemBytes = smem;
+  c.stream = s;
+  c.attrs = &at;
+  c.numAttrs = early_launch(s) ? 1 : 0;
+  cudaLaunchKernelEx(&c, k, std::forward<A>(args)...);  // errors: cudaGetLastError, as for <<<>>>
+}
 
 // Transition record: one solute transfer of S5 (target node, amount per species).
 struct Transfer {

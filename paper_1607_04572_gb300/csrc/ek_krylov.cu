@@ -267,6 +267,8 @@ __global__ void __launch_bounds__(CG_T) k_cg_prep(Box b, CGView v, double* D, co
 // block b takes items b, b + gridDim.x, ...: node coordinates come from the
 // item, with no division per node.
 __global__ void __launch_bounds__(CG_T) k_cg_apply(Box b, CGView v, int tx, int ty) {
+  let_next_start();
+  after_previous();
   const int N = (int)b.N, sy = b.nx, sz = b.nx * b.ny;
   const int items = tx * ty * b.nz;
   const double* __restrict__ cx = v.cf;
@@ -306,6 +308,8 @@ __global__ void __launch_bounds__(CG_T) k_cg_apply(Box b, CGView v, int tx, int 
 // r and D^-1 r; then beta = r.z(new) / r.z(old), r.r for the convergence test
 // and, with the projection (every node free), m = mean r and r.z, r.r of r - m
 __global__ void __launch_bounds__(CG_T) k_cg_update(Box b, CGView v, double* x, int neutral) {
+  let_next_start();
+  after_previous();
   const double alpha = v.sc[2];
   double rz = 0.0, rr = 0.0, s1 = 0.0, s2 = 0.0;
   for (long long n = blockIdx.x * (long long)CG_T + threadIdx.x; n < b.N; n += (long long)gridDim.x * CG_T) {
@@ -360,6 +364,8 @@ __global__ void __launch_bounds__(CG_T) k_cg_update(Box b, CGView v, double* x, 
 // r -= m (the projection; m = 0 with fixed nodes), p = D^-1 r + beta p on
 // the free nodes
 __global__ void __launch_bounds__(CG_T) k_cg_direction(Box b, CGView v, int neutral) {
+  let_next_start();
+  after_previous();
   const double beta = v.sc[3], m = v.sc[10];
   const unsigned n = blockIdx.x * CG_T + threadIdx.x;
   if (n >= (unsigned)b.N) return;
@@ -472,12 +478,16 @@ __device__ __forceinline__ void half_node(const MGLevel& L, unsigned j, int colo
   L.x[n] = L.dinv[n] * level_gather(L, L.x, n, x, y, z);
 }
 __global__ void __launch_bounds__(CG_T) k_mg_half(MGLevel L, int colour) {
+  let_next_start();
+  after_previous();
   const unsigned j = blockIdx.x * CG_T + threadIdx.x;
   if (j < (unsigned)L.n / 2) half_node(L, j, colour);
 }
 // the last half sweep (red) of the fine level, with b.x: a red node's
 // neighbour x ^ 1 in the row is black and final
 __global__ void __launch_bounds__(CG_T) k_mg_half_dot(MGLevel L, CGView v, int first) {
+  let_next_start();
+  after_previous();
   double t = 0.0;
   for (unsigned j = blockIdx.x * CG_T + threadIdx.x; j < (unsigned)L.n / 2; j += gridDim.x * CG_T) {
     int x, y, z;
@@ -501,11 +511,15 @@ __device__ __forceinline__ double jacobi_node(const MGLevel& L, const double* in
   return fma(MG_OMEGA * di, level_gather(L, in, n, x, y, z), (1.0 - MG_OMEGA) * in[n]);
 }
 __global__ void __launch_bounds__(CG_T) k_mg_jacobi(MGLevel L, const double* in, double* out) {
+  let_next_start();
+  after_previous();
   const unsigned n = blockIdx.x * CG_T + threadIdx.x;
   if (n < (unsigned)L.n) out[n] = jacobi_node(L, in, (int)n);
 }
 // the last sweep of the fine level, with b.x
 __global__ void __launch_bounds__(CG_T) k_mg_jacobi_dot(MGLevel L, const double* in, double* out, CGView v, int first) {
+  let_next_start();
+  after_previous();
   double t = 0.0;
   for (unsigned i = blockIdx.x * CG_T + threadIdx.x; i < (unsigned)L.n; i += gridDim.x * CG_T) {
     const int n = (int)i;
@@ -552,6 +566,8 @@ __device__ __forceinline__ void restrict_node(const MGLevel& F, const MGLevel& C
   if (C.rb && !((X + Y + Z) & 1)) C.x[n] = di * s;
 }
 __global__ void __launch_bounds__(CG_T) k_mg_restrict(MGLevel F, MGLevel C) {
+  let_next_start();
+  after_previous();
   const unsigned n = blockIdx.x * CG_T + threadIdx.x;
   if (n < (unsigned)C.n) restrict_node(F, C, (int)n);
 }
@@ -566,12 +582,16 @@ __device__ __forceinline__ void prolong_node(const MGLevel& F, const MGLevel& C,
     F.x[n] += C.x[(x >> (F.fx - 1)) + C.nx * ((y >> (F.fy - 1)) + C.ny * (z >> (F.fz - 1)))];
 }
 __global__ void __launch_bounds__(CG_T) k_mg_prolong(MGLevel F, MGLevel C) {
+  let_next_start();
+  after_previous();
   const unsigned j = blockIdx.x * CG_T + threadIdx.x;
   if (j < (unsigned)(F.rb ? F.n / 2 : F.n)) prolong_node(F, C, j);
 }
 
 // the coarse level's faces and fixed nodes from the fine level
 __global__ void __launch_bounds__(CG_T) k_mg_coarsen(MGLevel F, MGLevel C) {
+  let_next_start();
+  after_previous();
   const int n = (int)(blockIdx.x * CG_T + threadIdx.x);
   if ((unsigned)n >= (unsigned)C.n) return;
   int X, Y, Z;
@@ -597,6 +617,8 @@ __global__ void __launch_bounds__(CG_T) k_mg_coarsen(MGLevel F, MGLevel C) {
 }
 
 __global__ void __launch_bounds__(CG_T) k_mg_diag(MGLevel C) {
+  let_next_start();
+  after_previous();
   const int n = (int)(blockIdx.x * CG_T + threadIdx.x);
   if ((unsigned)n >= (unsigned)C.n) return;
   int x, y, z, m[6];
@@ -660,6 +682,8 @@ __device__ void coarse_solve(const MGLevel& C) {
   if (in) C.x[n] = xn;
 }
 __global__ void __launch_bounds__(MG_SMALL_T) k_mg_small(const __grid_constant__ MGSmall S) {
+  let_next_start();
+  after_previous();
   cg::cluster_group cl = cg::this_cluster();
   const unsigned first = blockIdx.x * MG_SMALL_T + threadIdx.x, step = gridDim.x * MG_SMALL_T;
   auto half = [&](const MGLevel& A, int colour) {
@@ -706,6 +730,8 @@ __global__ void __launch_bounds__(MG_SMALL_T) k_mg_small(const __grid_constant__
 // Without the projection the preconditioner's first half sweep from zero,
 // z = D^-1 r on the red nodes, comes along.
 __global__ void __launch_bounds__(CG_T) k_pcg_update(Box b, CGView v, double* x, MGLevel L, int neutral) {
+  let_next_start();
+  after_previous();
   const double alpha = v.sc[2];
   double rr = 0.0, s1 = 0.0;
   for (long long i = blockIdx.x * (long long)CG_T + threadIdx.x; i < b.N; i += (long long)gridDim.x * CG_T) {
@@ -744,6 +770,8 @@ __global__ void __launch_bounds__(CG_T) k_pcg_update(Box b, CGView v, double* x,
 // r -= its mean (only without fixed nodes; before the first cycle m = 0), and
 // the preconditioner's first half sweep from zero
 __global__ void __launch_bounds__(CG_T) k_pcg_project(Box b, CGView v, MGLevel L, int shift) {
+  let_next_start();
+  after_previous();
   const double m = shift ? v.sc[10] : 0.0;
   for (long long i = blockIdx.x * (long long)CG_T + threadIdx.x; i < b.N; i += (long long)gridDim.x * CG_T) {
     const int n = (int)i;
@@ -760,6 +788,8 @@ __global__ void __launch_bounds__(CG_T) k_pcg_project(Box b, CGView v, MGLevel L
 
 // p = z + beta p on the free nodes
 __global__ void __launch_bounds__(CG_T) k_pcg_direction(Box b, CGView v, const double* z) {
+  let_next_start();
+  after_previous();
   const double beta = v.sc[3];
   const unsigned n = blockIdx.x * CG_T + threadIdx.x;
   if (n < (unsigned)b.N && !is_zero(v.dinv[n])) v.p[n] = z[n] + beta * v.p[n];
@@ -835,13 +865,15 @@ cudaError_t launch_small(const MGLevel* lev, int L, cudaStream_t s) {
   cfg.gridDim = dim3(MG_SMALL_CTAS);
   cfg.blockDim = dim3(MG_SMALL_T);
   cfg.stream = s;
-  cudaLaunchAttribute at;
-  at.id = cudaLaunchAttributeClusterDimension;
-  at.val.clusterDim.x = MG_SMALL_CTAS;
-  at.val.clusterDim.y = 1;
-  at.val.clusterDim.z = 1;
-  cfg.attrs = &at;
-  cfg.numAttrs = 1;
+  cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = MG_SMALL_CTAS;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = early_launch(s) ? 2 : 1;
   return cudaLaunchKernelEx(&cfg, k_mg_small, S);
 }
 
@@ -854,31 +886,31 @@ cudaError_t vcycle(const MGLevel* lev, int L, const CGView& v, int first, cudaSt
   for (int l = 0; l < small; ++l) {
     const MGLevel& A = lev[l];
     if (A.rb) {
-      k_mg_half<<<nblocks(A.n / 2), CG_T, 0, s>>>(A, 1);
-      k_mg_half<<<nblocks(A.n / 2), CG_T, 0, s>>>(A, 0);
-      k_mg_half<<<nblocks(A.n / 2), CG_T, 0, s>>>(A, 1);
+      launch_next(k_mg_half, nblocks(A.n / 2), CG_T, 0, s, A, 1);
+      launch_next(k_mg_half, nblocks(A.n / 2), CG_T, 0, s, A, 0);
+      launch_next(k_mg_half, nblocks(A.n / 2), CG_T, 0, s, A, 1);
     } else {
-      k_mg_jacobi<<<nblocks(A.n), CG_T, 0, s>>>(A, nullptr, A.xt);
-      k_mg_jacobi<<<nblocks(A.n), CG_T, 0, s>>>(A, A.xt, A.x);
+      launch_next(k_mg_jacobi, nblocks(A.n), CG_T, 0, s, A, nullptr, A.xt);
+      launch_next(k_mg_jacobi, nblocks(A.n), CG_T, 0, s, A, A.xt, A.x);
     }
-    k_mg_restrict<<<nblocks(lev[l + 1].n), CG_T, 0, s>>>(A, lev[l + 1]);
+    launch_next(k_mg_restrict, nblocks(lev[l + 1].n), CG_T, 0, s, A, lev[l + 1]);
   }
   const cudaError_t e = launch_small(lev + small, L - small, s);
   if (e != cudaSuccess) return e;
   for (int l = small - 1; l >= 0; --l) {
     const MGLevel& A = lev[l];
     const unsigned nb = std::min<unsigned>(CG_BLOCKS, nblocks(A.rb ? A.n / 2 : A.n));
-    k_mg_prolong<<<nblocks(A.rb ? A.n / 2 : A.n), CG_T, 0, s>>>(A, lev[l + 1]);
+    launch_next(k_mg_prolong, nblocks(A.rb ? A.n / 2 : A.n), CG_T, 0, s, A, lev[l + 1]);
     if (A.rb) {
-      k_mg_half<<<nblocks(A.n / 2), CG_T, 0, s>>>(A, 1);
-      k_mg_half<<<nblocks(A.n / 2), CG_T, 0, s>>>(A, 0);
-      k_mg_half<<<nblocks(A.n / 2), CG_T, 0, s>>>(A, 1);
-      if (l > 0) k_mg_half<<<nblocks(A.n / 2), CG_T, 0, s>>>(A, 0);
-      else k_mg_half_dot<<<nb, CG_T, 0, s>>>(A, v, first);
+      launch_next(k_mg_half, nblocks(A.n / 2), CG_T, 0, s, A, 1);
+      launch_next(k_mg_half, nblocks(A.n / 2), CG_T, 0, s, A, 0);
+      launch_next(k_mg_half, nblocks(A.n / 2), CG_T, 0, s, A, 1);
+      if (l > 0) launch_next(k_mg_half, nblocks(A.n / 2), CG_T, 0, s, A, 0);
+      else launch_next(k_mg_half_dot, nb, CG_T, 0, s, A, v, first);
     } else {
-      k_mg_jacobi<<<nblocks(A.n), CG_T, 0, s>>>(A, A.x, A.xt);
-      if (l > 0) k_mg_jacobi<<<nblocks(A.n), CG_T, 0, s>>>(A, A.xt, A.x);
-      else k_mg_jacobi_dot<<<nb, CG_T, 0, s>>>(A, A.xt, A.x, v, first);
+      launch_next(k_mg_jacobi, nblocks(A.n), CG_T, 0, s, A, A.x, A.xt);
+      if (l > 0) launch_next(k_mg_jacobi, nblocks(A.n), CG_T, 0, s, A, A.xt, A.x);
+      else launch_next(k_mg_jacobi_dot, nb, CG_T, 0, s, A, A.xt, A.x, v, first);
     }
   }
   return cudaGetLastError();
@@ -927,28 +959,28 @@ cudaError_t poisson_solve_cg(const double* q, const double* eps, const unsigned 
   int it = 0;
   double rel = 0.0;
   auto iterate = [&]() {
-    k_cg_apply<<<na, CG_T, 0, s>>>(b, v, tx, ty);
+    launch_next(k_cg_apply, na, CG_T, 0, s, b, v, tx, ty);
     if (!mg) {
-      k_cg_update<<<nb, CG_T, 0, s>>>(b, v, phi, neutral);
-      k_cg_direction<<<nblocks((int)b.N), CG_T, 0, s>>>(b, v, neutral);
+      launch_next(k_cg_update, nb, CG_T, 0, s, b, v, phi, neutral);
+      launch_next(k_cg_direction, nblocks((int)b.N), CG_T, 0, s, b, v, neutral);
       return;
     }
-    k_pcg_update<<<nb, CG_T, 0, s>>>(b, v, phi, lev[0], neutral);
-    if (neutral) k_pcg_project<<<nb, CG_T, 0, s>>>(b, v, lev[0], 1);
+    launch_next(k_pcg_update, nb, CG_T, 0, s, b, v, phi, lev[0], neutral);
+    if (neutral) launch_next(k_pcg_project, nb, CG_T, 0, s, b, v, lev[0], 1);
     const cudaError_t ve = vcycle(lev, nlev, v, 0, s);
     if (e == cudaSuccess) e = ve;
-    k_pcg_direction<<<nblocks((int)b.N), CG_T, 0, s>>>(b, v, lev[0].x);
+    launch_next(k_pcg_direction, nblocks((int)b.N), CG_T, 0, s, b, v, lev[0].x);
   };
   if (mg && bnorm > 0.0) {
     // the coarse levels' operators, then p = z = M r and r.z
     for (int l = 1; l < nlev; ++l) {
-      k_mg_coarsen<<<nblocks(lev[l].n), CG_T, 0, s>>>(lev[l - 1], lev[l]);
-      k_mg_diag<<<nblocks(lev[l].n), CG_T, 0, s>>>(lev[l]);
+      launch_next(k_mg_coarsen, nblocks(lev[l].n), CG_T, 0, s, lev[l - 1], lev[l]);
+      launch_next(k_mg_diag, nblocks(lev[l].n), CG_T, 0, s, lev[l]);
     }
-    if (lev[0].rb) k_pcg_project<<<nb, CG_T, 0, s>>>(b, v, lev[0], 0);
+    if (lev[0].rb) launch_next(k_pcg_project, nb, CG_T, 0, s, b, v, lev[0], 0);
     e = vcycle(lev, nlev, v, 1, s);
     if (e != cudaSuccess) return e;
-    k_pcg_direction<<<nblocks((int)b.N), CG_T, 0, s>>>(b, v, lev[0].x);
+    launch_next(k_pcg_direction, nblocks((int)b.N), CG_T, 0, s, b, v, lev[0].x);
   }
   // the iterations between two residual reads as one graph (a caller stream
   // other than the legacy default stream can be captured); else the launches

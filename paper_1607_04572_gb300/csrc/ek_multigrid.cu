@@ -152,6 +152,8 @@ __global__ void __launch_bounds__(MG_T) k_mg_rhs(const double* q, double* phi, d
 
 // one colour of a red-black Gauss-Seidel sweep: phi = sum nb / 6 + b
 __global__ void __launch_bounds__(MG_T) k_mg_half(double* phi, const double* b, int nx, int ny, int nz, int colour) {
+  let_next_start();
+  after_previous();
   const unsigned j = blockIdx.x * MG_T + threadIdx.x;
   if (j >= (unsigned)nx / 2u * (unsigned)ny * (unsigned)nz) return;
   int x, y, z;
@@ -165,6 +167,8 @@ __global__ void __launch_bounds__(MG_T) k_mg_half(double* phi, const double* b, 
 template <bool MAX>
 __global__ void __launch_bounds__(MG_T) k_mg_resid(const double* phi, const double* b, double* r, int nx, int ny,
                                                    int nz, Scalars* sc) {
+  let_next_start();
+  after_previous();
   const unsigned j = blockIdx.x * MG_T + threadIdx.x;
   unsigned long long m = 0;
   if (j < (unsigned)nx / 2u * (unsigned)ny * (unsigned)nz) {
@@ -197,6 +201,8 @@ __global__ void __launch_bounds__(MG_T) k_mg_resid_max(const double* phi, const 
 // coarse level's first red half sweep from zero comes along.
 __global__ void __launch_bounds__(MG_T) k_mg_restrict(const double* rf, int nx, int ny, int nz, double* bc,
                                                       double* phic) {
+  let_next_start();
+  after_previous();
   const int cx = nx / 2, cy = ny / 2, cz = nz / 2;
   const unsigned i = blockIdx.x * MG_T + threadIdx.x;
   if (i >= (unsigned)cx * (unsigned)cy * (unsigned)cz) return;
@@ -218,6 +224,8 @@ __global__ void __launch_bounds__(MG_T) k_mg_restrict(const double* rf, int nx, 
 // one half way between (x - 1) / 2 and (x + 1) / 2 (periodic); a black node has
 // one odd axis or three
 __global__ void __launch_bounds__(MG_T) k_mg_prolong(const double* phic, int nx, int ny, int nz, double* phif) {
+  let_next_start();
+  after_previous();
   const int cx = nx / 2, cy = ny / 2, cz = nz / 2;
   const unsigned j = blockIdx.x * MG_T + threadIdx.x;
   if (j >= (unsigned)nx / 2u * (unsigned)ny * (unsigned)nz) return;
@@ -305,13 +313,13 @@ cudaError_t mean_of(const Solver& S, const double* x, long long n) {
 }
 
 void half(const Solver& S, const Level& l, int colour) {
-  k_mg_half<<<blocks(l.n / 2), MG_T, 0, S.s>>>(l.phi, l.b, l.nx, l.ny, l.nz, colour);
+  launch_next(k_mg_half, blocks(l.n / 2), MG_T, 0, S.s, l.phi, l.b, l.nx, l.ny, l.nz, colour);
 }
 void restrict_to(const Solver& S, const Level& l, const Level& c) {
-  k_mg_restrict<<<blocks(c.n), MG_T, 0, S.s>>>(l.r, l.nx, l.ny, l.nz, c.b, c.phi);
+  launch_next(k_mg_restrict, blocks(c.n), MG_T, 0, S.s, l.r, l.nx, l.ny, l.nz, c.b, c.phi);
 }
 void prolong_to(const Solver& S, const Level& l, const Level& c) {
-  k_mg_prolong<<<blocks(l.n / 2), MG_T, 0, S.s>>>(c.phi, l.nx, l.ny, l.nz, l.phi);
+  launch_next(k_mg_prolong, blocks(l.n / 2), MG_T, 0, S.s, c.phi, l.nx, l.ny, l.nz, l.phi);
 }
 
 // one V-cycle from level k >= 1 down, from zero; the red nodes have had their
@@ -329,7 +337,7 @@ cudaError_t vcycle(const Solver& S, size_t k) {
   half(S, l, 1);
   half(S, l, 0);
   half(S, l, 1);
-  k_mg_resid<false><<<blocks(l.n / 2), MG_T, 0, S.s>>>(l.phi, l.b, l.r, l.nx, l.ny, l.nz, S.sc);
+  launch_next(k_mg_resid<false>, blocks(l.n / 2), MG_T, 0, S.s, l.phi, l.b, l.r, l.nx, l.ny, l.nz, S.sc);
   restrict_to(S, l, S.lv[k + 1]);
   cudaError_t e = vcycle(S, k + 1);
   if (e != cudaSuccess) return e;

@@ -1100,7 +1100,10 @@ __device__ __forceinline__ void save_prev_body(const PartArgs& a, const Blk bk) 
   a.owner_prev[n] = a.owner[n];
 }
 
-__global__ void k_save_prev(PartArgs a) { save_prev_body(a, grid_blk()); }
+__global__ void k_save_prev(PartArgs a) {
+  let_next_start();
+  after_previous();
+  save_prev_body(a, grid_blk()); }
 
 template <class FM>
 __device__ __forceinline__ void clear_body(const PartArgs& a, const Blk bk) {
@@ -1118,7 +1121,10 @@ __device__ __forceinline__ void clear_body(const PartArgs& a, const Blk bk) {
 }
 
 template <class FM>
-__global__ void k_clear(PartArgs a) { clear_body<FM>(a, grid_blk()); }
+__global__ void k_clear(PartArgs a) {
+  let_next_start();
+  after_previous();
+  clear_body<FM>(a, grid_blk()); }
 
 template <class FM>
 __global__ void k_reset_all(PartArgs a) {
@@ -1172,7 +1178,10 @@ __device__ __forceinline__ void claim_body(const PartArgs& a, const Blk bk) {
 }
 
 template <class FM>
-__global__ void __launch_bounds__(PT) k_claim(PartArgs a) { claim_body<FM>(a, grid_blk()); }
+__global__ void __launch_bounds__(PT) k_claim(PartArgs a) {
+  let_next_start();
+  after_previous();
+  claim_body<FM>(a, grid_blk()); }
 
 // Psi_p of a surface cell (level 0 undecided) from the finest level alone.
 // In FP64 the octree's decisions are inherited: a cube decided inside at some
@@ -1535,6 +1544,8 @@ __device__ __forceinline__ void psi_surface_body(const PartArgs& a, const Blk bk
 
 template <class FM>
 __global__ void __launch_bounds__(PSI_CTA) k_psi_surface(PartArgs a) {
+  let_next_start();
+  after_previous();
   psi_surface_body<FM>(a, grid_blk());
 }
 
@@ -1567,7 +1578,10 @@ __device__ __forceinline__ void charge_scatter_body(const PartArgs& a, const Blk
 }
 
 template <class FM>
-__global__ void k_charge_scatter(PartArgs a) { charge_scatter_body<FM>(a, grid_blk()); }
+__global__ void k_charge_scatter(PartArgs a) {
+  let_next_start();
+  after_previous();
+  charge_scatter_body<FM>(a, grid_blk()); }
 
 __device__ __forceinline__ bool steady_fluid(const PartArgs& a, long long m) {
   return a.owner_prev[m] == FLUID && a.owner[m] == FLUID;
@@ -1792,7 +1806,10 @@ __device__ __forceinline__ void transitions_body(const PartArgs& a, const Blk bk
 }
 
 template <class FM>
-__global__ void __launch_bounds__(PT) k_transitions(PartArgs a) { transitions_body<FM>(a, grid_blk()); }
+__global__ void __launch_bounds__(PT) k_transitions(PartArgs a) {
+  let_next_start();
+  after_previous();
+  transitions_body<FM>(a, grid_blk()); }
 
 template <class FM>
 __device__ __forceinline__ void apply_transfers_body(const PartArgs& a, const Blk bk) {
@@ -1809,7 +1826,10 @@ __device__ __forceinline__ void apply_transfers_body(const PartArgs& a, const Bl
 }
 
 template <class FM>
-__global__ void k_apply_transfers(PartArgs a) { apply_transfers_body<FM>(a, grid_blk()); }
+__global__ void k_apply_transfers(PartArgs a) {
+  let_next_start();
+  after_previous();
+  apply_transfers_body<FM>(a, grid_blk()); }
 
 template <class FM>
 cudaError_t particle_forces_t(const PartArgs& a, cudaStream_t s, int parts) {
@@ -1835,7 +1855,7 @@ cudaError_t reflag_t(const PartArgs& a, bool transitions, cudaStream_t s, int pa
     if (a.P == 0 || !transitions) return cudaSuccess;
     // (k_save_prev of this step emptied the transfer list)
     k_transitions<FM><<<dim3(a.P, uchunks), PT, 0, s>>>(a);
-    k_apply_transfers<FM><<<152, 256, 0, s>>>(a);
+    launch_next(k_apply_transfers<FM>, 152, 256, 0, s, a);
     return cudaGetLastError();
   }
   if (!transitions) {
@@ -1847,15 +1867,15 @@ cudaError_t reflag_t(const PartArgs& a, bool transitions, cudaStream_t s, int pa
   const unsigned bchunks = (unsigned)((a.boxmax + PT - 1) / PT);
   if (transitions) {
     k_save_prev<<<dim3(a.P, uchunks), PT, 0, s>>>(a);
-    k_clear<FM><<<dim3(a.P, uchunks), PT, 0, s>>>(a);
+    launch_next(k_clear<FM>, dim3(a.P, uchunks), PT, 0, s, a);
   }
   if (!transitions) cudaMemsetAsync(a.surf_count, 0, sizeof(int), s);  // else k_clear resets it
-  k_claim<FM><<<dim3(a.P, bchunks), PT, 0, s>>>(a);
-  k_psi_surface<FM><<<8 * 152, PSI_CTA, 0, s>>>(a);
-  k_charge_scatter<FM><<<dim3(a.P, bchunks), PT, 0, s>>>(a);
+  launch_next(k_claim<FM>, dim3(a.P, bchunks), PT, 0, s, a);
+  launch_next(k_psi_surface<FM>, 8 * 152, PSI_CTA, 0, s, a);
+  launch_next(k_charge_scatter<FM>, dim3(a.P, bchunks), PT, 0, s, a);
   if (transitions && (parts & 2)) {
     k_transitions<FM><<<dim3(a.P, uchunks), PT, 0, s>>>(a);
-    k_apply_transfers<FM><<<152, 256, 0, s>>>(a);
+    launch_next(k_apply_transfers<FM>, 152, 256, 0, s, a);
   }
   return cudaGetLastError();
 }

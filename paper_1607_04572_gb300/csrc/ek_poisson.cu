@@ -386,6 +386,8 @@ __device__ __forceinline__ const C* line_twiddles(const AxisPlan& P, C* sm) {
 // function (a power of two: the same rounding).
 template <typename R>
 __global__ void __launch_bounds__(FFT_THREADS) k_fft_x_fwd(PassArgs<R> a, int pairs_per_cta) {
+  let_next_start();
+  after_previous();
   using C = typename CT<R>::type;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* smem = reinterpret_cast<C*>(smem_raw);
@@ -427,6 +429,8 @@ __global__ void __launch_bounds__(FFT_THREADS) k_fft_x_fwd(PassArgs<R> a, int pa
 // multiply and the inverse transform fused.
 template <typename R, int AXIS, bool INV>
 __global__ void __launch_bounds__(FFT_THREADS) k_fft_yz(PassArgs<R> a, int tx, unsigned mtx) {
+  let_next_start();
+  after_previous();
   using C = typename CT<R>::type;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* smem = reinterpret_cast<C*>(smem_raw);
@@ -477,6 +481,8 @@ __global__ void __launch_bounds__(FFT_THREADS) k_fft_yz(PassArgs<R> a, int tx, u
 // X pass, inverse (complex-to-real), two rows per complex transform.
 template <typename R>
 __global__ void __launch_bounds__(FFT_THREADS) k_fft_x_inv(PassArgs<R> a, int pairs_per_cta) {
+  let_next_start();
+  after_previous();
   using C = typename CT<R>::type;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* smem = reinterpret_cast<C*>(smem_raw);
@@ -687,6 +693,8 @@ __device__ __forceinline__ void fast_x_fwd_body(const PassArgs<float>& a, int bx
 
 template <int NX, bool KMAJOR, bool VEC>
 __global__ void __launch_bounds__(FAST_XT) k_fast_x_fwd(PassArgs<float> a) {
+  let_next_start();
+  after_previous();
   fast_x_fwd_body<NX, KMAJOR, VEC>(a, blockIdx.x);
 }
 
@@ -694,6 +702,8 @@ __global__ void __launch_bounds__(FAST_XT) k_fast_x_fwd(PassArgs<float> a) {
 // inverse) pass on tiles of tx consecutive kx (as k_fft_yz)
 template <int NL, int AXIS, bool INV>
 __global__ void __launch_bounds__(FAST_T) k_fast_yz(PassArgs<float> a, int tx) {
+  let_next_start();
+  after_previous();
   constexpr int LS = fpad(NL);
   __shared__ __align__(16) float2 buf[2][(FAST_ELEMS / NL) * LS];
   __shared__ float2 tw[NL];
@@ -768,6 +778,8 @@ constexpr size_t line4_smem() { return (size_t)(16 * NL + NL) * sizeof(float2); 
 
 template <int NL, int AXIS, bool INV>
 __global__ void __launch_bounds__(256) k_line4(PassArgs<float> a) {
+  let_next_start();
+  after_previous();
   constexpr int N1 = 16, N2 = NL / 16, TX = 16, PER = TX * N2 / 256;
   extern __shared__ __align__(16) unsigned char line4_raw[];
   float2* const T = reinterpret_cast<float2*>(line4_raw);  // TX * NL
@@ -856,7 +868,7 @@ template <int NL, int AXIS, bool INV>
 void launch_line4(PassArgs<float>& a, cudaStream_t s) {
   const int ntile = (a.nxh + 15) / 16;
   const int nother = AXIS == 1 ? a.nz : a.ny;
-  k_line4<NL, AXIS, INV><<<(unsigned)(ntile * nother), 256, line4_smem<NL>(), s>>>(a);
+  launch_next(k_line4<NL, AXIS, INV>, (unsigned)(ntile * nother), 256, line4_smem<NL>(), s, a);
 }
 template <int NL>
 cudaError_t line4_attr() {
@@ -926,6 +938,8 @@ __device__ __forceinline__ void fast_x_inv_body(const PassArgs<float>& a, int bx
 
 template <int NX, bool KMAJOR>
 __global__ void __launch_bounds__(FAST_IT) k_fast_x_inv(PassArgs<float> a) {
+  let_next_start();
+  after_previous();
   fast_x_inv_body<NX, KMAJOR>(a, blockIdx.x);
 }
 
@@ -985,6 +999,8 @@ __device__ __forceinline__ float2 shfl2(float2 v, int src) {
 
 template <int NX>
 __global__ void __launch_bounds__(32 * X4_WARPS, 4) k_line4_x_fwd(PassArgs<float> a) {
+  let_next_start();
+  after_previous();
   using L = X4<NX>;
   constexpr int N2 = L::N2, U = L::U;
   __shared__ __align__(16) L sm;
@@ -1052,6 +1068,8 @@ __global__ void __launch_bounds__(32 * X4_WARPS, 4) k_line4_x_fwd(PassArgs<float
 
 template <int NX>
 __global__ void __launch_bounds__(32 * X4_WARPS, 4) k_line4_x_inv(PassArgs<float> a) {
+  let_next_start();
+  after_previous();
   using L = X4<NX>;
   constexpr int N2 = L::N2, U = L::U;
   __shared__ __align__(16) L sm;
@@ -1116,7 +1134,7 @@ void launch_fast_x(PassArgs<float>& a, bool inverse, bool kmajor, cudaStream_t s
   if constexpr (FOUR) {
     if (!kmajor) {
       const unsigned g = (unsigned)((npairs + 2 * X4_WARPS - 1) / (2 * X4_WARPS));
-      if (inverse) k_line4_x_inv<NX><<<g, 32 * X4_WARPS, 0, s>>>(a);
+      if (inverse) launch_next(k_line4_x_inv<NX>, g, 32 * X4_WARPS, 0, s, a);
       else k_line4_x_fwd<NX><<<g, 32 * X4_WARPS, 0, s>>>(a);
       return;
     }
@@ -1124,8 +1142,8 @@ void launch_fast_x(PassArgs<float>& a, bool inverse, bool kmajor, cudaStream_t s
   if (inverse) {
     constexpr int ppc = FAST_IELEMS / NX > 0 ? FAST_IELEMS / NX : 1;
     const unsigned g = (unsigned)((npairs + ppc - 1) / ppc);
-    if (kmajor) k_fast_x_inv<NX, true><<<g, FAST_IT, 0, s>>>(a);
-    else if constexpr (!FOUR) k_fast_x_inv<NX, false><<<g, FAST_IT, 0, s>>>(a);
+    if (kmajor) launch_next(k_fast_x_inv<NX, true>, g, FAST_IT, 0, s, a);
+    else if constexpr (!FOUR) launch_next(k_fast_x_inv<NX, false>, g, FAST_IT, 0, s, a);
   } else {
     constexpr int ppc = FAST_XELEMS / NX > 0 ? FAST_XELEMS / NX : 1;
     const unsigned g = (unsigned)((npairs + ppc - 1) / ppc);
@@ -1149,7 +1167,7 @@ void launch_fast_yz_n(PassArgs<float>& a, cudaStream_t s) {
   const int ntile = (a.nxh + txmax - 1) / txmax;
   const int tx = (a.nxh + ntile - 1) / ntile;
   const int nother = AXIS == 1 ? a.nz : a.ny;
-  k_fast_yz<NL, AXIS, INV><<<(unsigned)(ntile * nother), FAST_T, 0, s>>>(a, tx);
+  launch_next(k_fast_yz<NL, AXIS, INV>, (unsigned)(ntile * nother), FAST_T, 0, s, a, tx);
 }
 
 template <int AXIS, bool INV>
@@ -1356,6 +1374,8 @@ __device__ __forceinline__ void fast_yzplane2_body(const PassArgs<float>& a, int
 template <int NY, int NZ>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PLANE2_T, 1)
     k_fast_yzplane2(PassArgs<float> a) {
+  let_next_start();
+  after_previous();
   fast_yzplane2_body<NY, NZ>(a, blockIdx.x);
 }
 
@@ -1369,7 +1389,7 @@ inline bool plane_edge(int n) { return n == 32 || n == 48 || n == 64 || n == 128
 
 template <int NY, int NZ>
 cudaError_t launch_plane_nn(PassArgs<float>& a, cudaStream_t s) {
-  k_fast_yzplane2<NY, NZ><<<2 * (unsigned)a.nxh, PLANE2_T, plane2_smem_bytes<NY, NZ>(), s>>>(a);
+  launch_next(k_fast_yzplane2<NY, NZ>, 2 * (unsigned)a.nxh, PLANE2_T, plane2_smem_bytes<NY, NZ>(), s, a);
   return cudaGetLastError();
 }
 
@@ -1656,19 +1676,19 @@ cudaError_t run_passes(const PoissonPlan& p, PassArgs<R>& a, double bjerrum, cud
     if (fx) launch_fast_x_any(a, false, false, s);
     if (!fx) k_fft_x_fwd<R><<<gx, nx_t, smem(ppc, p.nx), s>>>(a, ppc);
     if (fy) launch_fast_yz<1, false>(a, p.ny, s);
-    if (!fy) k_fft_yz<R, 1, false><<<gy, ny_t, smem(txy, p.ny), s>>>(a, txy, div_magic(txy));
+    if (!fy) launch_next(k_fft_yz<R, 1, false>, gy, ny_t, smem(txy, p.ny), s, a, txy, div_magic(txy));
     if (fz) launch_fast_yz<2, false>(a, p.nz, s);
-    if (!fz) k_fft_yz<R, 2, false><<<gz, nz_t, smem(txz, p.nz), s>>>(a, txz, div_magic(txz));
+    if (!fz) launch_next(k_fft_yz<R, 2, false>, gz, nz_t, smem(txz, p.nz), s, a, txz, div_magic(txz));
     if (fy) launch_fast_yz<1, true>(a, p.ny, s);
-    if (!fy) k_fft_yz<R, 1, true><<<gy, ny_t, smem(txy, p.ny), s>>>(a, txy, div_magic(txy));
+    if (!fy) launch_next(k_fft_yz<R, 1, true>, gy, ny_t, smem(txy, p.ny), s, a, txy, div_magic(txy));
     if (fx) launch_fast_x_any(a, true, false, s);
-    if (!fx) k_fft_x_inv<R><<<gx, nx_t, smem(ppc, p.nx), s>>>(a, ppc);
+    if (!fx) launch_next(k_fft_x_inv<R>, gx, nx_t, smem(ppc, p.nx), s, a, ppc);
   } else {
     k_fft_x_fwd<R><<<gx, nx_t, smem(ppc, p.nx), s>>>(a, ppc);
-    k_fft_yz<R, 1, false><<<gy, ny_t, smem(txy, p.ny), s>>>(a, txy, div_magic(txy));
-    k_fft_yz<R, 2, false><<<gz, nz_t, smem(txz, p.nz), s>>>(a, txz, div_magic(txz));
-    k_fft_yz<R, 1, true><<<gy, ny_t, smem(txy, p.ny), s>>>(a, txy, div_magic(txy));
-    k_fft_x_inv<R><<<gx, nx_t, smem(ppc, p.nx), s>>>(a, ppc);
+    launch_next(k_fft_yz<R, 1, false>, gy, ny_t, smem(txy, p.ny), s, a, txy, div_magic(txy));
+    launch_next(k_fft_yz<R, 2, false>, gz, nz_t, smem(txz, p.nz), s, a, txz, div_magic(txz));
+    launch_next(k_fft_yz<R, 1, true>, gy, ny_t, smem(txy, p.ny), s, a, txy, div_magic(txy));
+    launch_next(k_fft_x_inv<R>, gx, nx_t, smem(ppc, p.nx), s, a, ppc);
   }
   return cudaGetLastError();
 }
