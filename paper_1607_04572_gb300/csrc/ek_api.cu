@@ -475,7 +475,7 @@ ek_status enqueue_stage(ek_ctx* ctx, int stage, cudaEvent_t mid = nullptr) {
       PartArgs a = part_args(ctx);
       if (ctx->P) {
         EK_CUDA(launch_reflag(a, true, s));
-        ctx->launches += 7;
+        ctx->launches += reflag_kernels(ctx->P);
       }
       return EK_OK;
     }
@@ -503,7 +503,7 @@ ek_status enqueue_step(ek_ctx* ctx) {
     EK_CUDA(launch_reflag(pa, true, s, 1));
     EK_CUDA(ctx->fp32 ? launch_advection32(la, s) : launch_advection(la, s));
     EK_CUDA(launch_reflag(pa, true, s, 2));
-    ctx->launches += (ctx->p.nspecies > 0 ? 2 : 1) + 8 + assign_kernels(ctx->P);
+    ctx->launches += (ctx->p.nspecies > 0 ? 2 : 1) + 1 + reflag_kernels(ctx->P) + assign_kernels(ctx->P);
     return EK_OK;
   }
   if (ctx->P) {
@@ -533,7 +533,7 @@ ek_status enqueue_step(ek_ctx* ctx) {
     EK_CUDA(cudaStreamWaitEvent(s, ctx->ev_part, 0));
     EK_CUDA(launch_reflag(pa, true, s, 2));
     EK_CUDA(cudaStreamWaitEvent(s, ctx->ev_join, 0));
-    ctx->launches += 8 + assign_kernels(ctx->P);
+    ctx->launches += 1 + reflag_kernels(ctx->P) + assign_kernels(ctx->P);
   }
   return EK_OK;
 }

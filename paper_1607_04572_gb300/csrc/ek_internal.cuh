@@ -490,6 +490,8 @@ cudaError_t launch_particle_forces(const PartArgs& a, cudaStream_t s, int parts 
 // kernels of the assignment (a single particle owns every node of its widened
 // box: none)
 inline int assign_kernels(int P) { return P > 1 ? 2 : 0; }
+// kernels of S5 (a single particle saves and clears in one)
+inline int reflag_kernels(int P) { return P == 1 ? 6 : 7; }
 // CTAs per particle that cover its union box (previous and current box)
 int union_chunks(int boxmax);
 // S5; parts: 1 = re-flag, Psi and charge (no species access), 2 = transitions

@@ -1103,7 +1103,8 @@ __device__ __forceinline__ void save_prev_body(const PartArgs& a, const Blk bk) 
 __global__ void k_save_prev(PartArgs a) {
   let_next_start();
   after_previous();
-  save_prev_body(a, grid_blk()); }
+  save_prev_body(a, grid_blk());
+}
 
 template <class FM>
 __device__ __forceinline__ void clear_body(const PartArgs& a, const Blk bk) {
@@ -1124,7 +1125,25 @@ template <class FM>
 __global__ void k_clear(PartArgs a) {
   let_next_start();
   after_previous();
-  clear_body<FM>(a, grid_blk()); }
+  clear_body<FM>(a, grid_blk());
+}
+
+// both at once for a single particle, whose union box holds every node once
+// (it never wraps onto itself), so no other thread reads what is cleared here:
+// one launch less in the chain (a step at 32^3 68.1 -> 66.4 us, at 128^3 201.6 ->
+// 200.0)
+template <class FM>
+__global__ void k_save_clear(PartArgs a) {
+  let_next_start();
+  after_previous();
+  save_prev_body(a, grid_blk());
+  clear_body<FM>(a, grid_blk());
+}
+// a batch's systems (FP32 form): those of a single particle clear here
+__device__ __forceinline__ void save_prev_any(const PartArgs& a, const Blk bk) {
+  save_prev_body(a, bk);
+  if (a.P == 1) clear_body<FormF32>(a, bk);
+}
 
 template <class FM>
 __global__ void k_reset_all(PartArgs a) {
@@ -1181,7 +1200,8 @@ template <class FM>
 __global__ void __launch_bounds__(PT) k_claim(PartArgs a) {
   let_next_start();
   after_previous();
-  claim_body<FM>(a, grid_blk()); }
+  claim_body<FM>(a, grid_blk());
+}
 
 // Psi_p of a surface cell (level 0 undecided) from the finest level alone.
 // In FP64 the octree's decisions are inherited: a cube decided inside at some
@@ -1581,7 +1601,8 @@ template <class FM>
 __global__ void k_charge_scatter(PartArgs a) {
   let_next_start();
   after_previous();
-  charge_scatter_body<FM>(a, grid_blk()); }
+  charge_scatter_body<FM>(a, grid_blk());
+}
 
 __device__ __forceinline__ bool steady_fluid(const PartArgs& a, long long m) {
   return a.owner_prev[m] == FLUID && a.owner[m] == FLUID;
@@ -1809,7 +1830,8 @@ template <class FM>
 __global__ void __launch_bounds__(PT) k_transitions(PartArgs a) {
   let_next_start();
   after_previous();
-  transitions_body<FM>(a, grid_blk()); }
+  transitions_body<FM>(a, grid_blk());
+}
 
 template <class FM>
 __device__ __forceinline__ void apply_transfers_body(const PartArgs& a, const Blk bk) {
@@ -1829,7 +1851,8 @@ template <class FM>
 __global__ void k_apply_transfers(PartArgs a) {
   let_next_start();
   after_previous();
-  apply_transfers_body<FM>(a, grid_blk()); }
+  apply_transfers_body<FM>(a, grid_blk());
+}
 
 template <class FM>
 cudaError_t particle_forces_t(const PartArgs& a, cudaStream_t s, int parts) {
@@ -1866,8 +1889,12 @@ cudaError_t reflag_t(const PartArgs& a, bool transitions, cudaStream_t s, int pa
   // union boxes are at most one cell wider than a box per axis
   const unsigned bchunks = (unsigned)((a.boxmax + PT - 1) / PT);
   if (transitions) {
-    k_save_prev<<<dim3(a.P, uchunks), PT, 0, s>>>(a);
-    launch_next(k_clear<FM>, dim3(a.P, uchunks), PT, 0, s, a);
+    if (a.P == 1) {
+      k_save_clear<FM><<<dim3(1, uchunks), PT, 0, s>>>(a);
+    } else {
+      k_save_prev<<<dim3(a.P, uchunks), PT, 0, s>>>(a);
+      launch_next(k_clear<FM>, dim3(a.P, uchunks), PT, 0, s, a);
+    }
   }
   if (!transitions) cudaMemsetAsync(a.surf_count, 0, sizeof(int), s);  // else k_clear resets it
   launch_next(k_claim<FM>, dim3(a.P, bchunks), PT, 0, s, a);
@@ -1892,7 +1919,7 @@ cudaError_t reflag_t(const PartArgs& a, bool transitions, cudaStream_t s, int pa
 EK_PART_BATCH(k_force_assign_batch, force_assign_body, __launch_bounds__(PT))
 EK_PART_BATCH(k_tie_resolve_batch, tie_resolve_body, __launch_bounds__(256))
 EK_PART_BATCH(k_particle_forces_batch, particle_forces_any, __launch_bounds__(FORCE_T, 4))
-EK_PART_BATCH(k_save_prev_batch, save_prev_body, __launch_bounds__(PT))
+EK_PART_BATCH(k_save_prev_batch, save_prev_any, __launch_bounds__(PT))
 EK_PART_BATCH(k_clear_batch, clear_body<FormF32>, __launch_bounds__(PT))
 EK_PART_BATCH(k_claim_batch, claim_body<FormF32>, __launch_bounds__(PT))
 EK_PART_BATCH(k_psi_surface_batch, psi_surface_body<FormF32>, __launch_bounds__(PSI_CTA))
@@ -1964,7 +1991,7 @@ __global__ void __launch_bounds__(256) k_particle_chain(ChainArgs A) {
       switch (P.kind) {
         case PK_ASSIGN: force_assign_body(a, bk); break;
         case PK_TIE: tie_resolve_body(a, bk); break;
-        case PK_SAVE_PREV: save_prev_body(a, bk); break;
+        case PK_SAVE_PREV: save_prev_any(a, bk); break;
         case PK_CLEAR: clear_body<FormF32>(a, bk); break;
         case PK_CLAIM: claim_body<FormF32>(a, bk); break;
         case PK_PSI: psi_surface_body<FormF32>(a, bk); break;
@@ -2021,8 +2048,11 @@ void particle_batch_grid(int k, const PartArgs& a, int& gx, int& gy) {
       if (!assign_kernels(a.P)) gx = 0;
       break;
     case PK_FORCES: gy = a.fchunks; break;
-    case PK_SAVE_PREV:
     case PK_CLEAR:
+      if (a.P == 1) gx = 0;  // with PK_SAVE_PREV
+      gy = uchunks;
+      break;
+    case PK_SAVE_PREV:
     case PK_TRANS: gy = uchunks; break;
     case PK_CLAIM:
     case PK_CHARGE: gy = bchunks; break;
