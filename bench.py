@@ -72,7 +72,9 @@ def lb_bytes_per_node(fp32, K):
     return 2 * 19 * 8 + 2 * K * 8 + 9 + 8            # 353 for K = 2
 
 
-LB_FP64_FLOP_PER_NODE = 950
+# additions, multiplications and FMAs (two each) per node, from the kernel's
+# operation counters at 128^3
+LB_FP64_FLOP_PER_NODE = 425
 
 
 # Algorithmic bytes per node of a whole step (S1-S5), the state read once and
@@ -103,8 +105,8 @@ FP64_PEAK_TFLOPS = 152 * 2.07e9 * 4 / 1e12
 # DRAM traffic (dram__bytes_read.sum + dram__bytes_write.sum) per lattice node
 # of one launch of the kernel, from an ncu capture, valid only for the kernel
 # source it was taken on (otherwise the traffic is reported as null).
-TRAFFIC = {"k_lb32": {"bytes_per_node": (202409472 + 178517504) / 128 ** 3,
-                      "source_sha": "b124e8565c46b3fd", "file": "ek_lattice32.cu"}}
+TRAFFIC = {"k_lb32": {"bytes_per_node": (205391104 + 178442496) / 128 ** 3,
+                      "source_sha": "9a3cc8989bf3c12e", "file": "ek_lattice32.cu"}}
 
 
 def src_sha(name: str) -> str:
@@ -564,10 +566,10 @@ def main():
 
 # Multigrid V-cycle traffic at the finest level, per node (an estimate of the
 # bytes that must cross HBM, intermediates in L2 not subtracted): 8 red-black
-# half-sweeps (read phi and the colour's b, write the colour's phi: 16 B),
-# residual 24, restriction 8, prolongation 17, the residual and its norm
-# after the cycle 32; the coarser levels add an eighth per level.
-MG_BYTES_PER_NODE_CYCLE = round((8 * 16 + 24 + 8 + 17 + 32) * 8 / 7)   # 239
+# half-sweeps (read phi and the colour's b, write the colour's phi: 16 B), the
+# red nodes' residual with its maximum 16, restriction 6, prolongation onto the
+# black nodes 9; the coarser levels add an eighth per level.
+MG_BYTES_PER_NODE_CYCLE = round((8 * 16 + 16 + 6 + 9) * 8 / 7)   # 182
 
 
 def measure_poisson_mg(ek, torch, shape=(128, 128, 128), reps=3):
