@@ -148,11 +148,11 @@ struct FormF32 {
 // These chains are bound by the launches where the kernels take a few us each:
 // the Poisson solve of a 48 x 32 x 72 box (FP64, five passes) 43.8 -> 38.9 us, 13
 // V-cycles at 128^3 4.33 -> 3.34 ms, the set-up of the conjugate gradients there
-// 0.2 ms less, stage 5 of a 32^3 box 44 -> 32 us.  Under
-// capture the launches stay ordinary: a graph starts its next kernel soon enough
-// by itself, and successors that wait on the SMs beside a forked branch hold it
-// up (a step's graph with and without: 32^3 65.9, 68.0 us; 128^3 209, 205;
-// 256^3 1422, 1398).
+// 0.2 ms less, stage 5 of a 32^3 box 44 -> 32 us.  (Index arithmetic before the
+// wait changed none of them.)  Under capture the launches stay ordinary: a graph
+// starts its next kernel soon enough by itself, and successors that wait on the
+// SMs beside a forked branch hold it up (a step's graph with and without: 32^3
+// 65.9, 68.0 us; 128^3 209, 205; 256^3 1422, 1398).
 __device__ __forceinline__ void after_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 inline bool early_launch(cudaStream_t s) {
