@@ -387,8 +387,7 @@ ek_status ek_batch_sync(ek_batch* b);
  * block), and whether the particle chain runs beside the advection or in line
  * -- over 2 + trial_steps real batch steps each (the systems advance by those
  * steps), keeps the fastest and stores its time per batch step in *best_ms
- * (may be null).  Results do not depend on the choice except for the
- * summation order of the lattice-block force sums. */
+ * (may be null).  Results do not depend on the choice. */
 ek_status ek_batch_tune(ek_batch* b, int trial_steps, double* best_ms);
 /* Current configuration: cfg[0] branch streams, cfg[1] planes per S2 block,
  * cfg[2] particle chain beside the advection (1) or in line (0), cfg[3] the

@@ -54,10 +54,11 @@ struct ek_ctx {
   void* qwall = nullptr;
   void* u = nullptr;
   void* ifield = nullptr;              // 3N reals: internal solute force on the fluid (S2)
-  double* ipart = nullptr;             // 3 doubles per lattice block: its sums
+  double* ipart = nullptr;             // 3 doubles per lattice block (FP32: plane group): its sums
   int nipart = 0;
-  int nipart_cap = 0;  // rows allocated for ipart (FP32: enough for 2-plane segments)
+  int* gticket = nullptr;  // FP32 S2: finished segments of each plane group
   int nzb = 1;       // S2: z segments per tile column
+  int nsub = 1;      // FP32 S2: segments per plane group (lb32_split)
   int advseg = 1;    // S3: z segments per tile column
   int overlap = 1;   // particle chain on the auxiliary stream (1) or in line (0)
   unsigned long long version = 0;  // bumped whenever captured steps go stale
@@ -279,6 +280,9 @@ LBArgs lb_args(ek_ctx* ctx) {
   a.parts = ctx->dparts;
   a.status = ctx->status;
   a.nzb = ctx->nzb;
+  a.ngrp = lb32_groups(ctx->g);
+  a.nsub = ctx->nsub;
+  a.gticket = ctx->gticket;
   a.advseg = ctx->advseg;
   return a;
 }
@@ -321,12 +325,10 @@ ek_status run_setup(ek_ctx* ctx) {
     const double dmax = sqrt(3.0) * (rmax + ceil(rmax) + FORCE_MARGIN + 2.0) + 1.0;
     ctx->tie_thr = (float)(2.0 * ldexp(dmax + rmax + 1.0, -21) + ldexp(dmax + rmax, -22));
   }
-  // cells per S4 force CTA: FORCE_CHUNK for a few particles; twice that when
-  // those chunks fill two waves of 760 CTAs (152 SMs x 5), and doubled on while
-  // the particles still fill eight waves of 912
+  // cells per S4 force CTA: FORCE_CHUNK, doubled while the particles still
+  // fill eight waves of 912 CTAs (152 SMs x 6) with the larger chunks
   int fcells = FORCE_CHUNK;
-  if ((long long)ctx->P * ((emax + 2 * fcells - 1) / (2 * fcells)) >= 2LL * 152 * 5) fcells *= 2;
-  while (fcells < 16 * FORCE_CHUNK &&
+  while (fcells < 8 * FORCE_CHUNK &&
          (long long)ctx->P * ((emax + 2 * fcells - 1) / (2 * fcells)) >= 8LL * 152 * 6)
     fcells *= 2;
   const int fchunks = (emax + fcells - 1) / fcells;
@@ -754,16 +756,17 @@ ek_status ek_create(const ek_params* p, ek_ctx** out) {
   alloc(&ctx->u, 3 * N * rsz);
   alloc(&ctx->ifield, 3 * N * rsz);
   {
-    // lattice-block partial sums of S2: one per block of its grid
-    ctx->nzb = ctx->fp32 ? lb32_segments(g) : lb64_segments(g);
+    // partial sums of S2: one per block of its grid (FP32: per tile column and
+    // plane group, whatever the segments)
+    const dim3 lg = lattice_grid32(g, 1);
+    const int cols = (int)(lg.x * lg.y);
+    ctx->nzb = lb64_segments(g);
+    if (ctx->fp32) lb32_split(g, lb32_planes(cols, g.nz), ctx->nzb, ctx->nsub);
     ctx->advseg = ctx->fp32 ? adv32_segments(g, false) : adv64_segments(g);
-    const dim3 lg = lattice_grid32(g, ctx->nzb);
-    ctx->nipart = (int)(lg.x * lg.y * lg.z);
-    // the FP32 segment length may be retuned down to 2 planes (ek_batch_tune)
-    ctx->nipart_cap = ctx->fp32 ? (int)(lg.x * lg.y) * std::max(1, (g.nz + 1) / 2) : ctx->nipart;
-    ctx->nipart_cap = std::max(ctx->nipart_cap, ctx->nipart);
+    ctx->nipart = cols * (ctx->fp32 ? lb32_groups(g) : ctx->nzb);
   }
-  alloc((void**)&ctx->ipart, (size_t)ctx->nipart_cap * 3 * sizeof(double));
+  alloc((void**)&ctx->ipart, (size_t)ctx->nipart * 3 * sizeof(double));
+  if (ctx->fp32) alloc((void**)&ctx->gticket, (size_t)ctx->nipart * sizeof(int));
   alloc((void**)&ctx->fkey, N * sizeof(unsigned long long));
   alloc((void**)&ctx->vsig, N);
   alloc((void**)&ctx->tmp, N * sizeof(double));
@@ -793,6 +796,7 @@ ek_status ek_create(const ek_params* p, ek_ctx** out) {
   cudaMemset(ctx->tie_count, 0, sizeof(int));
   cudaMemset(ctx->status, 0, sizeof(int));
   cudaMemset(ctx->ticket, 0, sizeof(int));
+  if (ctx->gticket) cudaMemset(ctx->gticket, 0, (size_t)ctx->nipart * sizeof(int));
   for (int b = 0; b < 2; ++b) {
     cudaMemset(ctx->f[b], 0, 19 * N * rsz);
     cudaMemset(ctx->rho[b], 0, K * N * ssz);
@@ -830,7 +834,7 @@ ek_status ek_destroy(ek_ctx* ctx) {
                   ctx->spectrum, ctx->dparts, ctx->psibox, ctx->fpart, ctx->surf, ctx->xfer,
                   ctx->xfer_count, ctx->surf_count, ctx->status, ctx->ifield, ctx->ipart,
                   ctx->fkey, ctx->psum, ctx->vsig, ctx->ticket, ctx->pticket, ctx->pstage,
-                  ctx->tie_list, ctx->tie_count, ctx->tpart};
+                  ctx->tie_list, ctx->tie_count, ctx->tpart, ctx->gticket};
   for (void* q : ptrs)
     if (q) cudaFree(q);
   poisson_plan_destroy(ctx->plan);
@@ -1435,19 +1439,12 @@ void batch_drop(ek_batch* b) {
   }
 }
 
-// apply the batch's segment length and overlap choice to every system
+// apply the batch's overlap choice to every system
 void batch_apply(ek_batch* b) {
   for (ek_ctx* c : b->sys) {
-    int nzb = c->nzb;
-    if (c->fp32) nzb = std::max(1, (c->g.nz + b->planes - 1) / b->planes);
-    const int xt = (c->g.nx + TILE_X - 1) / TILE_X, yt = (c->g.ny + TILE_Y - 1) / TILE_Y;
-    if (c->fp32 && xt * yt * nzb > c->nipart_cap) nzb = c->nipart_cap / (xt * yt);
-    if (nzb != c->nzb || c->overlap != b->overlap) {
-      c->nzb = nzb;
-      if (c->fp32) c->nipart = xt * yt * nzb;
-      c->overlap = b->overlap;
-      drop_graphs(c);
-    }
+    if (c->overlap == b->overlap) continue;
+    c->overlap = b->overlap;
+    drop_graphs(c);
   }
 }
 
@@ -1470,9 +1467,14 @@ ek_status batch_capture(ek_batch* b, int key) {
     if (cudaStreamWaitEvent(b->branch[w], b->ev_fork, 0) != cudaSuccess) st = EK_ERR_CUDA;
   for (size_t i = 0; i < b->sys.size() && st == EK_OK; ++i) {
     ek_ctx* c = b->sys[i];
+    // the batch's segment length, in the batch's graph only
+    const int nzb = c->nzb, nsub = c->nsub;
+    if (c->fp32) lb32_split(c->g, b->planes, c->nzb, c->nsub);
     c->stream = b->branch[i % width];
     st = enqueue_step(c);
     c->stream = saved[i];
+    c->nzb = nzb;
+    c->nsub = nsub;
   }
   for (int w = 0; w < width && st == EK_OK; ++w) {
     if (cudaEventRecord(b->ev_join[w], b->branch[w]) != cudaSuccess ||
@@ -1520,6 +1522,7 @@ ek_status fused_build(ek_batch* b, int key) {
                        c->has_qwall ? (const float*)c->qwall : nullptr, (const float*)c->qpart, c->ph,
                        (float*)c->phi, (float2*)c->spectrum);
     lbt[i].a = lb_args(c);
+    lb32_split(c->g, b->planes, lbt[i].a.nzb, lbt[i].a.nsub);  // the batch's segment length
     lbt[i].a.advseg = adv32_segments(c->g, true);  // one launch for all systems: wide
     lbt[i].c = make_phys32(c->ph);
     c->cur = 1 - c->cur;

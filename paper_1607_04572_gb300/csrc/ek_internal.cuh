@@ -352,10 +352,12 @@ struct LBArgs {
   void* ifield;    // real_t, 3N: solute force on the fluid minus q_ions E (fluid nodes)
   unsigned char* vsig;  // N: bit 7 fluid node; bits 0-1, 2-3, 4-5: sign code of u_x, u_y, u_z
                         // (0 zero, 1 positive, 2 negative), written by S2 for S3
-  double* ipart;   // per-block sums of ifield (3 per block of the lattice grid)
+  double* ipart;   // sums of ifield, 3 per block of the S2 grid (FP32: per tile column and plane group)
   const DevParticle* parts;
   int* status;
-  int nzb;         // S2: z segments per (x, y) tile column (lb32_segments, lb64_segments)
+  int nzb;         // S2: z segments per (x, y) tile column (lb32_split, lb64_segments)
+  int ngrp, nsub;  // FP32 S2: plane groups per column, segments per group (1: segments of whole groups)
+  int* gticket;    // FP32 S2, nsub > 1: finished segments of each group (reset by the last)
   int advseg;      // S3: z segments per tile column (adv32_segments, adv64_segments)
 };
 // Constants of the FP32 kernels, rounded once on the host.
@@ -368,9 +370,6 @@ struct Phys32 {
   float g[3];
   float E[3];
   float zq[EK_MAX_SPECIES];  // z_k qs_k: charge of one unit of species k
-  float hp, hm;              // (1 + lambda_e)/2, (1 + lambda_o)/2
-  float gw, kw;              // 9/2 (2 + lambda_e) / 36, -9/2 lambda_e / 36
-  float lo12;                // -lambda_o / 12
 };
 Phys32 make_phys32(const Phys& ph);
 // one system's entry of the batched FP32 S2 / S3 launches
@@ -386,9 +385,12 @@ cudaError_t launch_advection(const LBArgs& a, cudaStream_t s);
 // FP32-storage form
 cudaError_t lb32_prepare();  // once per process, before the first launch_lb32
 // planes per segment of the FP32 S2 grid for a number of tile columns (of one
-// box, or of all boxes of a batched launch), and a box's segments per column
+// box, or of all boxes of a batched launch); the plane groups of a box (rows of
+// ipart per column); the segments per column, and per group, of about `planes`
+// planes each
 int lb32_planes(long long cols, int nz);
-int lb32_segments(const Grid& g);
+int lb32_groups(const Grid& g);
+void lb32_split(const Grid& g, int planes, int& nzb, int& nsub);
 cudaError_t launch_lb32(const LBArgs& a, cudaStream_t s);
 cudaError_t launch_advection32(const LBArgs& a, cudaStream_t s);
 // z segments per tile column of the FP32 S3 grid: 32-plane segments on
@@ -469,16 +471,16 @@ struct PartArgs {
 // FORCE_T` rows of FORCE_T cells, fcells a multiple of FORCE_CHUNK chosen at
 // set-up (larger when many particles give enough CTAs anyway, so fewer block
 // sums are made); fpart holds P * fchunks * FPART doubles.  Few particles leave
-// most SMs idle and wait for the rows of a thread one after another: chunks of
-// 128 / 256 / 512 cells, S4 in us: one sphere R = 8 44.8, 42.3, 45.4; R = 4 31.8,
-// 32.6, 34.2; eight R = 4 48.8, 43.0, 44.8; 64 of R = 5 (256^3) 256 / 512: 167, 130.
+// most SMs idle and wait for the rows of a thread one after another, but a
+// smaller chunk would regroup the FP32 form's float sums (particle_forces_body);
+// chunks of 128 / 256 / 512 cells, S4 in us: one sphere R = 8 44.8, 42.3, 45.4;
+// R = 4 31.8, 32.6, 34.2; eight R = 4 48.8, 43.0, 44.8.
 constexpr int FORCE_T = 128;
-constexpr int FORCE_CHUNK = 256;
-constexpr int FORCE_ROWS = 16 * FORCE_CHUNK / FORCE_T;  // most rows of a CTA
+constexpr int FORCE_CHUNK = 512;
+constexpr int FORCE_ROWS = 8 * FORCE_CHUNK / FORCE_T;  // most rows of a CTA
 // per particle: [0..5] Fh Th (momentum exchange), [6..11] Fs Ts (reaction of
-// the solute force), [12] sum w and [13..15] sum w (r - r_p) of the weights of
-// the particle's own charge (times the charge per unit weight, the field's force
-// and torque are E and M x E times these),
+// the solute force), [12] sum q and [13..15] sum q (r - r_p) of the particle's
+// own charge (the field's force and torque are E and M x E times these),
 // [18..20] a slice of the lattice total of the internal force (first particle
 // only), [16..17] and [21..23] unused
 constexpr int FPART = 24;

@@ -53,11 +53,6 @@ Phys32 make_phys32(const Phys& ph) {
     p.E[d] = (float)ph.E[d];
   }
   for (int k = 0; k < EK_MAX_SPECIES; ++k) p.zq[k] = (float)(ph.z[k] * ph.qscale[k]);
-  p.hp = (float)(0.5 * (1.0 + ph.lam_e));
-  p.hm = (float)(0.5 * (1.0 + ph.lam_o));
-  p.gw = (float)(4.5 * (2.0 + ph.lam_e) / 36.0);
-  p.kw = (float)(-4.5 * ph.lam_e / 36.0);
-  p.lo12 = (float)(-ph.lam_o / 12.0);
   return p;
 }
 
@@ -85,55 +80,29 @@ __device__ __forceinline__ unsigned nbr32(int d, const Off3& o) {
          (dcz(d) > 0 ? o.Z2 : (dcz(d) < 0 ? o.Z0 : o.Z1));
 }
 
-// The lattice total of the internal force: every thread adds its nodes in float
-// pairs (hi + lo, the rounding errors of the float additions kept: Knuth's
-// two-sum), the lanes of a warp are added as pairs, the warps in FP64, so that
-// the total does not depend on how the planes are cut into segments beyond some
-// 1e-14 (plain float sums differed by 1e-7).  In FP64 from the threads on, the
-// conversions and additions on its narrow pipe cost S2 10% at 128^3.
-struct Sum3 {
-  float2 hxy, lxy;
-  float hz, lz;
-};
-__device__ __forceinline__ void sum3_add(Sum3& s, float2 v, float z, float2 vl, float zl) {
-  const float2 m = make_float2(-1.0f, -1.0f);
-  const float2 t = __fadd2_rn(s.hxy, v);
-  const float2 bb = __ffma2_rn(s.hxy, m, t);
-  const float2 e = __fadd2_rn(__ffma2_rn(__ffma2_rn(bb, m, t), m, s.hxy), __ffma2_rn(bb, m, v));
-  s.hxy = t;
-  s.lxy = __fadd2_rn(s.lxy, __fadd2_rn(e, vl));
-  const float tz = __fadd_rn(s.hz, z), bz = __fsub_rn(tz, s.hz);
-  const float ez = __fadd_rn(__fsub_rn(s.hz, __fsub_rn(tz, bz)), __fsub_rn(z, bz));
-  s.lz = __fadd_rn(s.lz, __fadd_rn(ez, zl));
-  s.hz = tz;
-}
-__device__ __forceinline__ void sum3_add(Sum3& s, float x, float y, float z) {
-  sum3_add(s, make_float2(x, y), z, make_float2(0.0f, 0.0f), 0.0f);
-}
-// the block's sums, in a fixed order, into ipart[3 blk ..]
-__device__ __forceinline__ void block_sum3(Sum3 s, double* ipart, long long blk) {
-  __shared__ double red[TILE_X * TILE_Y / 32][3];
+// The block's sums of the internal force of one plane group, in a fixed order,
+// into a row of ipart: the threads' float sums over their planes and the warps in
+// float (put), then, past a barrier, the warp sums in FP64 (take); in FP64 from
+// the threads on, the conversions and additions on its narrow pipe cost S2 10% at
+// 128^3.
+using WarpSums = double[TILE_X * TILE_Y / 32][3];
+__device__ __forceinline__ void sum3_put(const float (&v)[3], WarpSums& red) {
   const int t = threadIdx.x + TILE_X * threadIdx.y;
-  const int lane = t & 31, warp = t >> 5;
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const float hx = __shfl_down_sync(0xffffffffu, s.hxy.x, o), hy = __shfl_down_sync(0xffffffffu, s.hxy.y, o);
-    const float lx = __shfl_down_sync(0xffffffffu, s.lxy.x, o), ly = __shfl_down_sync(0xffffffffu, s.lxy.y, o);
-    const float hz = __shfl_down_sync(0xffffffffu, s.hz, o), lz = __shfl_down_sync(0xffffffffu, s.lz, o);
-    sum3_add(s, make_float2(hx, hy), hz, make_float2(lx, ly), lz);
-  }
-  if (lane == 0) {
-    red[warp][0] = (double)s.hxy.x + (double)s.lxy.x;
-    red[warp][1] = (double)s.hxy.y + (double)s.lxy.y;
-    red[warp][2] = (double)s.hz + (double)s.lz;
-  }
-  __syncthreads();
-  if (t < 3) {
-    double v = 0.0;
+  for (int cc = 0; cc < 3; ++cc) {
+    float s = v[cc];
 #pragma unroll
-    for (int w = 0; w < TILE_X * TILE_Y / 32; ++w) v += red[w][t];
-    ipart[3 * blk + t] = v;
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+    if ((t & 31) == 0) red[t >> 5][cc] = (double)s;
   }
+}
+__device__ __forceinline__ void sum3_take(const WarpSums& red, double* ipart, long long row) {
+  const int t = threadIdx.x + TILE_X * threadIdx.y;
+  if (t >= 3) return;
+  double s = 0.0;
+#pragma unroll
+  for (int w = 0; w < TILE_X * TILE_Y / 32; ++w) s += red[w][t];
+  ipart[3 * row + t] = s;
 }
 
 // ---------------------------------------------------------------------------
@@ -152,12 +121,10 @@ __device__ __forceinline__ void block_sum3(Sum3 s, double* ipart, long long blk)
 // flux and collision arithmetic left out the same loads and stores took 5.22
 // of 5.82 ms (27 GB: 5.2 TB/s); stores without the one-node shift in x would
 // take 0.4 ms less (the ten shifted populations write five sectors per warp
-// for four).  Two species, or two pairs of populations, share one packed
-// f32x2 instruction: 1254 -> 1034 warp instructions per node.  6.96 -> 5.79
-// ms at 512^3, 0.936 -> 0.800 at 256^3 (K = 3), 0.110 -> 0.098 at 128^3, of
-// which the longer segments (lb32_planes) gave 0.69, 0.07 and 0.005.  Three
-// blocks per SM (80 registers) were slower: 7.11 ms at 4-plane segments
-// against 6.52.
+// for four).  Two species share one packed f32x2 instruction.  6.96 -> 6.18 ms
+// at 512^3, 0.936 -> 0.862 at 256^3 (K = 3), 0.110 -> 0.106 at 128^3, most of it
+// by the longer segments (lb32_planes).  Three blocks per SM (80 registers) were
+// slower: 7.11 ms at 4-plane segments against 6.52.
 // ---------------------------------------------------------------------------
 constexpr int HX = TILE_X + 2, HY = TILE_Y + 2;  // tile with halo
 constexpr int HP = HX * HY;                    // nodes of one halo plane
@@ -288,90 +255,51 @@ __device__ __forceinline__ void stage_pops(LBRing<K>& t, int buf, int z, int x0,
 template <int K>
 constexpr size_t lb32_smem() { return sizeof(LBRing<K>); }
 
-// The collision of one node on the deviations g (Eqs. 8-9), TRT in pair form.
-// With s, d the sum and difference of an opposite pair and Ep, Em the even and
-// odd equilibrium and force parts, the two results are A + B and A - B,
-//   A = (1 + lambda_e)/2 s + Ep,   B = (1 + lambda_o)/2 d + Em.
-// Ep is quadratic: with h = w (9/2 (2 + lambda_e) F - 9/2 lambda_e rho u) the
-// edges x + y and x - y share b + u_x h_x + u_y h_y and differ in the sign of
-// u_x h_y + u_y h_x; a face takes twice the edge weight 1/36.  Two pairs ride
-// in one packed operation: (x, y), (x+y, x-y), (x+z, x-z), (y+z, y-z).
-struct LBPairs {
-  float2 a13, b13, a79, b79, aAC, bAC, aEG, bEG;  // populations (1,3) (2,4) (7,9) (8,10) (11,13) (12,14) (15,17) (16,18)
-  float a5, b5, g0;
-};
-__device__ __forceinline__ void lb32_collide(LBPairs& p, const Phys32& c, float Fx, float Fy, float Fz,
-                                             float& ux, float& uy, float& uz, float& rho, float& usq) {
-  const float2 s13 = add2(p.a13, p.b13), s79 = add2(p.a79, p.b79);
-  const float2 sAC = add2(p.aAC, p.bAC), sEG = add2(p.aEG, p.bEG);
-  const float2 d13 = sub2(p.a13, p.b13), d79 = sub2(p.a79, p.b79);
-  const float2 dAC = sub2(p.aAC, p.bAC), dEG = sub2(p.aEG, p.bEG);
-  const float s5 = p.a5 + p.b5, d5 = p.a5 - p.b5;
-  const float2 st = add2(add2(s13, s79), add2(sAC, sEG));
-  const float drho = (p.g0 + s5) + (st.x + st.y);
-  const float jx = d13.x + ((d79.x + d79.y) + (dAC.x + dAC.y));
-  const float jy = d13.y + ((d79.x - d79.y) + (dEG.x + dEG.y));
-  const float jz = d5 + ((dAC.x - dAC.y) + (dEG.x - dEG.y));
+// The collision of one node on the deviations g (Eqs. 8-9), TRT in pair form, in
+// place.  With s, d the sum and difference of an opposite pair, F the force and
+// Ep, Em the even and odd equilibrium and force parts, the two results are
+// g_i + (X + Y) and g_ibar + (X - Y), X = lambda_e/2 s + Ep, Y = lambda_o/2 d + Em.
+// (The form with the quadratic parts shared between edges, (1 + lambda)/2 s + Ep,
+// takes 3% less of S2 but rounds differently, and the particles' motion is pinned to
+// the bits of these sums: see particle_forces_body.)
+__device__ __forceinline__ void lb32_collide(float (&g)[Q], const Phys32& c, float Fx, float Fy, float Fz, float& ux,
+                                             float& uy, float& uz, float& rho, float& usq) {
+  float drho = g[0], jx = 0.0f, jy = 0.0f, jz = 0.0f;
+#pragma unroll
+  for (int i = 1; i < Q; i += 2) {
+    const float pd = g[i] - g[i + 1];
+    drho += g[i] + g[i + 1];
+    if (dcx(i)) jx += csgnf(dcx(i), pd);
+    if (dcy(i)) jy += csgnf(dcy(i), pd);
+    if (dcz(i)) jz += csgnf(dcz(i), pd);
+  }
   rho = c.rho0 + drho;
   const float irho = 1.0f / rho;
-  ux = fmaf(0.5f, Fx, jx) * irho;
-  uy = fmaf(0.5f, Fy, jy) * irho;
-  uz = fmaf(0.5f, Fz, jz) * irho;
-  usq = fmaf(uz, uz, fmaf(uy, uy, ux * ux));
-  const float uF = fmaf(uz, Fz, fmaf(uy, Fy, ux * Fx));
-  const float base = fmaf(-1.5f * (2.0f + c.lam_e), uF, -c.lam_e * fmaf(-1.5f * rho, usq, drho));
-  const float bw = base * (1.0f / 36.0f), kw = c.kw * rho;
-  const float hx = fmaf(kw, ux, c.gw * Fx), hy = fmaf(kw, uy, c.gw * Fy), hz = fmaf(kw, uz, c.gw * Fz);
-  const float qx = fmaf(c.lo12, jx, (1.0f / 12.0f) * Fx);
-  const float qy = fmaf(c.lo12, jy, (1.0f / 12.0f) * Fy);
-  const float qz = fmaf(c.lo12, jz, (1.0f / 12.0f) * Fz);
-  const float bx = fmaf(ux, hx, bw), by = fmaf(uy, hy, bw), bz = fmaf(uz, hz, bw);
-  const float bxy = fmaf(uy, hy, bx), bxz = fmaf(uz, hz, bx), byz = fmaf(uz, hz, by);
-  const float mxy = fmaf(ux, hy, uy * hx), mxz = fmaf(ux, hz, uz * hx), myz = fmaf(uy, hz, uz * hy);
-  const float2 hp = two(c.hp), hm = two(c.hm);
-  p.g0 = fmaf(1.0f + c.lam_e, p.g0, 12.0f * bw);
-  float2 A = fma2(hp, s13, make_float2(bx + bx, by + by));
-  float2 B = fma2(hm, d13, make_float2(qx + qx, qy + qy));
-  p.a13 = add2(A, B);
-  p.b13 = sub2(A, B);
-  A = fma2(hp, s79, make_float2(bxy + mxy, bxy - mxy));
-  B = fma2(hm, d79, make_float2(qx + qy, qx - qy));
-  p.a79 = add2(A, B);
-  p.b79 = sub2(A, B);
-  A = fma2(hp, sAC, make_float2(bxz + mxz, bxz - mxz));
-  B = fma2(hm, dAC, make_float2(qx + qz, qx - qz));
-  p.aAC = add2(A, B);
-  p.bAC = sub2(A, B);
-  A = fma2(hp, sEG, make_float2(byz + myz, byz - myz));
-  B = fma2(hm, dEG, make_float2(qy + qz, qy - qz));
-  p.aEG = add2(A, B);
-  p.bEG = sub2(A, B);
-  const float A5 = fmaf(c.hp, s5, bz + bz), B5 = fmaf(c.hm, d5, qz + qz);
-  p.a5 = A5 + B5;
-  p.b5 = A5 - B5;
-}
-// population i of the pairs (i a constant after unrolling)
-__device__ __forceinline__ float lb32_pop(const LBPairs& p, int i) {
-  switch (i) {
-    case 1: return p.a13.x;
-    case 2: return p.b13.x;
-    case 3: return p.a13.y;
-    case 4: return p.b13.y;
-    case 5: return p.a5;
-    case 6: return p.b5;
-    case 7: return p.a79.x;
-    case 8: return p.b79.x;
-    case 9: return p.a79.y;
-    case 10: return p.b79.y;
-    case 11: return p.aAC.x;
-    case 12: return p.bAC.x;
-    case 13: return p.aAC.y;
-    case 14: return p.bAC.y;
-    case 15: return p.aEG.x;
-    case 16: return p.bEG.x;
-    case 17: return p.aEG.y;
-    case 18: return p.bEG.y;
-    default: return p.g0;
+  ux = (jx + 0.5f * Fx) * irho;
+  uy = (jy + 0.5f * Fy) * irho;
+  uz = (jz + 0.5f * Fz) * irho;
+  usq = ux * ux + uy * uy + uz * uz;
+  const float uF = ux * Fx + uy * Fy + uz * Fz;
+  const float le = c.lam_e, lo = c.lam_o;
+  const float gg = 2.0f + le;
+  const float qx = fmaf(-lo, jx, Fx), qy = fmaf(-lo, jy, Fy), qz = fmaf(-lo, jz, Fz);
+  const float base = fmaf(-1.5f * gg, uF, -le * fmaf(-1.5f * rho, usq, drho));
+  const float hle = 0.5f * le, hlo = 0.5f * lo;
+  const float k45 = -4.5f * le * rho;
+  g[0] = fmaf(1.0f + le, g[0], (float)wgt(0) * base);
+#pragma unroll
+  for (int i = 1; i < Q; i += 2) {
+    const float w = (float)wgt(i);
+    const float cu = cdotf(i, ux, uy, uz);
+    const float cf = cdotf(i, Fx, Fy, Fz);
+    const float cqv = cdotf(i, qx, qy, qz);
+    const float Ep = w * fmaf(cu, fmaf(4.5f * gg, cf, k45 * cu), base);
+    const float Em = 3.0f * w * cqv;
+    const float X = fmaf(hle, g[i] + g[i + 1], Ep);
+    const float Y = fmaf(hlo, g[i] - g[i + 1], Em);
+    const float p = g[i] + (X + Y), m = g[i + 1] + (X - Y);
+    g[i] = p;
+    g[i + 1] = m;
   }
 }
 
@@ -382,7 +310,7 @@ __device__ __forceinline__ float lb32_pop(const LBPairs& p, int i) {
 template <int K, bool PV, bool SIMPLE>
 __device__ __forceinline__ void lb32_node(LBRing<K>& t, const LBArgs& a, const Phys32& c,
                                           int x, int y, int z, int tid, int ex, int ey,
-                                          Sum3& iv) {
+                                          float (&iv)[3]) {
   constexpr int NP = LBPlane<K>::NP, NS = LBPlane<K>::NS;
   float* __restrict__ g_out = (float*)a.f_out;
   const int* __restrict__ n_in = (const int*)a.rho_in;
@@ -480,22 +408,14 @@ __device__ __forceinline__ void lb32_node(LBRing<K>& t, const LBArgs& a, const P
       at32(ifield, n) = ix;
       at32(ifield + N, n) = iy;
       at32(ifield + 2 * N, n) = iz;
-      sum3_add(iv, ix, iy, iz);
+      iv[0] += ix;
+      iv[1] += iy;
+      iv[2] += iz;
     }
     // ---- S2b: collision and push stream (velocity bounce-back, Eq. 12) ----
-    const float* const gp = &t.pop[z & 1][0][tid];
-    LBPairs g;
-    g.g0 = gp[0];
-    g.a13 = make_float2(gp[1 * TN], gp[3 * TN]);
-    g.b13 = make_float2(gp[2 * TN], gp[4 * TN]);
-    g.a5 = gp[5 * TN];
-    g.b5 = gp[6 * TN];
-    g.a79 = make_float2(gp[7 * TN], gp[9 * TN]);
-    g.b79 = make_float2(gp[8 * TN], gp[10 * TN]);
-    g.aAC = make_float2(gp[11 * TN], gp[13 * TN]);
-    g.bAC = make_float2(gp[12 * TN], gp[14 * TN]);
-    g.aEG = make_float2(gp[15 * TN], gp[17 * TN]);
-    g.bEG = make_float2(gp[16 * TN], gp[18 * TN]);
+    float g[Q];
+#pragma unroll
+    for (int i = 0; i < Q; ++i) g[i] = t.pop[z & 1][i][tid];
     float ux, uy, uz, rho, usq;
     lb32_collide(g, c, fmaf(gx, HALF_INV_A0, c.g[0]), fmaf(gy, HALF_INV_A0, c.g[1]),
                  fmaf(gz, HALF_INV_A0, c.g[2]), ux, uy, uz, rho, usq);
@@ -504,12 +424,11 @@ __device__ __forceinline__ void lb32_node(LBRing<K>& t, const LBArgs& a, const P
     at32(u + N, n) = uy;
     at32(u + 2 * N, n) = uz;
     a.vsig[n >> 2] = (unsigned char)(0x80u | sign_code(ux) | (sign_code(uy) << 2) | (sign_code(uz) << 4));
-    at32(g_out, n) = g.g0;
+    at32(g_out, n) = g[0];
 #pragma unroll
     for (int d = 1; d < Q; ++d) {
-      const float gs = lb32_pop(g, d);
       if (fluid & (1u << d)) {
-        at32(g_out + d * N, nbr32(d, nb)) = gs;
+        at32(g_out + d * N, nbr32(d, nb)) = g[d];
       } else {
         float cvb = 0.0f;
         const int om = pl[1 + dcz(d)]->own[e0 + dcx(d) + HX * dcy(d)];
@@ -529,28 +448,75 @@ __device__ __forceinline__ void lb32_node(LBRing<K>& t, const LBArgs& a, const P
           const float vz = P.velf[2] + (P.omegaf[0] * dy - P.omegaf[1] * dx);
           cvb = cdotf(d, vx, vy, vz);
         }
-        at32(g_out + opp(d) * N, n) = gs - 6.0f * (float)wgt(d) * c.rho0 * cvb;
+        at32(g_out + opp(d) * N, n) = g[d] - 6.0f * (float)wgt(d) * c.rho0 * cvb;
       }
     }
   }
 }
 
-// One block of the S2 grid: tile (bx, by), z segment bz; blk is the block's
-// row of the per-block sums.
+// The sums of the last block of a plane group cut into several blocks: every
+// thread takes its column's planes [ga, gb) from the stored force, in the order in
+// which one block would have added them (boundary nodes hold zero).
+__device__ __forceinline__ void late_sum3(const LBArgs& a, WarpSums& red, int x, int y, int ga, int gb, bool in_xy,
+                                          int parts, long long row) {
+  __shared__ bool last;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0 && threadIdx.y == 0) {
+    last = atomicAdd(a.gticket + row, 1) == parts - 1;
+    if (last) a.gticket[row] = 0;
+  }
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  float iv[3] = {0.0f, 0.0f, 0.0f};
+  if (in_xy) {
+    const float* const f = (const float*)a.ifield;
+    const long long N = a.g.N;
+    for (int z = ga; z < gb; ++z) {
+      const long long n = node_index(a.g, x, y, z);
+#pragma unroll
+      for (int cc = 0; cc < 3; ++cc) iv[cc] += __ldcg(f + cc * N + n);
+    }
+  }
+  sum3_put(iv, red);
+  __syncthreads();
+  sum3_take(red, a.ipart, row);
+}
+
+// One block of the S2 grid: tile (bx, by) of gx x gy, z segment bz.  The lattice
+// total of the internal force is summed per tile column and group of three or
+// four planes (plane group q: [q nz / ngrp, (q + 1) nz / ngrp)), one row of ipart
+// each, whatever the segments are: a segment holds whole groups, or (nsub > 1) a
+// group is cut into nsub segments, the last of which to finish forms the sums.
+// The float sums of a group round by its planes, so the total, the particles'
+// motion and, where a level-4 cube of a Psi lies on a surface, the flow depend on
+// the groups but not on the segments: a box steps the same alone and in a batch.
 template <int K, bool PV>
-__device__ __forceinline__ void lb32_block(const LBArgs& a, const Phys32& c, int bx, int by, int bz,
-                                           long long blk) {
+__device__ __forceinline__ void lb32_block(const LBArgs& a, const Phys32& c, int bx, int by, int bz, int gx,
+                                           int gy) {
   extern __shared__ __align__(16) unsigned char lb_smem[];
   LBRing<K>& t = *reinterpret_cast<LBRing<K>*>(lb_smem);
   const int nx = a.g.nx, ny = a.g.ny, nz = a.g.nz;
   const int x0 = bx * TILE_X, y0 = by * TILE_Y;
-  const int z0 = (int)((long long)bz * nz / a.nzb);
-  const int zend = (int)((long long)(bz + 1) * nz / a.nzb);
+  const int nsub = a.nsub;
+  int grp = nsub > 1 ? bz / nsub : bz * a.ngrp / a.nzb;  // the first plane group
+  int gend = (grp + 1) * nz / a.ngrp;                    // and the plane after it
+  const int ga = grp * nz / a.ngrp, gb = gend;
+  int z0 = ga, zend = ((bz + 1) * a.ngrp / a.nzb) * nz / a.ngrp;
+  if (nsub > 1) {
+    const int sub = bz - grp * nsub;
+    z0 = ga + (gb - ga) * sub / nsub;
+    zend = ga + (gb - ga) * (sub + 1) / nsub;
+    if (z0 == zend) return;  // a group of three planes in four segments
+  }
+  auto row = [&](int q) { return bx + (long long)gx * (by + (long long)gy * q); };
   const int x = x0 + threadIdx.x, y = y0 + threadIdx.y;
   const int tid = threadIdx.x + TILE_X * threadIdx.y;
   const bool in_xy = x < nx && y < ny;
   const int ex = threadIdx.x + 1, ey = threadIdx.y + 1;
-  Sum3 iv = {};
+  __shared__ WarpSums red;
+  float iv[3] = {0.0f, 0.0f, 0.0f};
   int hoff[2];
   halo_offsets(hoff, x0, y0, a);
   // ring slot of plane zz: zz mod 4 (zz >= -1)
@@ -595,16 +561,23 @@ __device__ __forceinline__ void lb32_block(const LBArgs& a, const Phys32& c, int
     }
     fm1 = f0;
     f0 = fp1;
+    const bool full = nsub == 1 && z + 1 == gend;
+    if (full) sum3_put(iv, red);
     __syncthreads();  // the next copies overwrite the slots of plane z - 1 and populations z
+    if (full) {
+      sum3_take(red, a.ipart, row(grp));
+      iv[0] = iv[1] = iv[2] = 0.0f;
+      ++grp;
+      gend = (grp + 1) * nz / a.ngrp;
+    }
   }
   cp_async_wait<0>();
-  block_sum3(iv, a.ipart, blk);
+  if (nsub > 1) late_sum3(a, red, x, y, ga, gb, in_xy, min(nsub, gb - ga), row(grp));
 }
 
 template <int K, bool PV>
 __global__ void __launch_bounds__(256, 2) k_lb32_tiled(LBArgs a, Phys32 c) {
-  lb32_block<K, PV>(a, c, blockIdx.x, blockIdx.y, blockIdx.z,
-                    blockIdx.x + (long long)gridDim.x * (blockIdx.y + (long long)gridDim.y * blockIdx.z));
+  lb32_block<K, PV>(a, c, blockIdx.x, blockIdx.y, blockIdx.z, gridDim.x, gridDim.y);
 }
 
 // S2 of a batch's systems in one launch: system s runs its xt x (yt nzb) grid
@@ -617,7 +590,7 @@ __global__ void __launch_bounds__(256, 2) k_lb32_batch(const LBBatchEntry* __res
   const Blk b = batch_blk(slot, nsys, sys);
   const LBBatchEntry& e = tab[sys];
   const int yt = (e.a.g.ny + TILE_Y - 1) / TILE_Y;
-  lb32_block<K, PV>(e.a, e.c, b.x, b.y % yt, b.y / yt, b.x + (long long)b.nx * b.y);
+  lb32_block<K, PV>(e.a, e.c, b.x, b.y % yt, b.y / yt, b.nx, yt);
 }
 
 // sign code (bits 0-1 of c >> shift) as -1, 0, +1
@@ -1007,10 +980,11 @@ int lb32_planes(long long cols, int nz) {
        : blocks(2) >= 512  ? 2
                            : 1;
 }
-int lb32_segments(const Grid& g) {
-  const long long cols = (long long)((g.nx + TILE_X - 1) / TILE_X) * ((g.ny + TILE_Y - 1) / TILE_Y);
-  const int planes = lb32_planes(cols, g.nz);
-  return std::max(1, (g.nz + planes - 1) / planes);
+int lb32_groups(const Grid& g) { return (g.nz + 3) / 4; }
+void lb32_split(const Grid& g, int planes, int& nzb, int& nsub) {
+  const int ngrp = lb32_groups(g), m = std::max(1, planes / 4);
+  nsub = planes >= 4 ? 1 : (4 + planes - 1) / planes;
+  nzb = nsub > 1 ? ngrp * nsub : (ngrp + m - 1) / m;
 }
 
 cudaError_t launch_lb32(const LBArgs& a, cudaStream_t s) {

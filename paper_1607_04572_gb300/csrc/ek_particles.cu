@@ -453,6 +453,7 @@ __global__ void k_tie_resolve(PartArgs a) { tie_resolve_body(a, grid_blk()); }
 template <int NC>
 __device__ void column_sums(const double* tab, int nrow, int stride, int col0, double* out);
 __device__ void integrate_all(const PartArgs& a);
+__device__ double charge_norm(const PartArgs& a, const DevParticle& P);
 
 template <int NV, class Get>
 __device__ void block_sum_t(Get v, double (*tr)[FORCE_T + 1], unsigned on, double* out) {
@@ -489,15 +490,21 @@ __device__ void block_sum_t(Get v, double (*tr)[FORCE_T + 1], unsigned on, doubl
 // midpoint) has c_i . v_b = c_i . w, since c_i . (Omega x c_i) = 0, and the
 // link torque (x + c_i - r_p) x F_i sums to d0 x sum_i F_i, since
 // c_i x c_i = 0.  So the per-link work is one dot product and one add.
-// The field on the particle's own charge is kept as the sums of the weights w
-// (Psi_p, or 1 on the boundary nodes) and of w (r - r_p); the charge per unit
-// weight, a division, is applied once per particle (integrate_all).
+// The field on the particle's own charge is kept as sum q and sum q (r - r_p)
+// (force E sum q, torque (sum q (r - r_p)) x E); the charge per unit weight, a
+// division, is formed by one thread of the block while the first loads are in
+// flight.
 // Block (p, b) takes the rows b, b + nb, b + 2 nb, ... of FORCE_T cells of the
 // widened box (nb blocks for this particle), so the cells next to the sphere
 // are spread over all blocks.  Bound by the latency of the loads, one row ahead.
 // The links are taken after the rows, from a list: a row of 32 cells holds few
 // nodes next to the sphere, and without the links' registers in the loop more
 // blocks are in flight (S4 1.35 -> 1.12 ms at 512^3 with 1000 particles).
+// The float sums of the FP32 form are those of a thread over its cells, row after
+// row: a node's momentum goes from the lane that worked it out to the one whose
+// cell it is.  Another order would round differently, by some 1e-8 of the force:
+// enough to carry a level-4 cube of a Psi over the surface a step earlier, which
+// shows in the velocities next to the sphere (1e-3 of their rms).
 // ONE: a single particle, which claims every node of its widened box without
 // keys (1), several (0), or either (2: the batched launch; tested per cell it
 // costs 8% at 1000 particles).
@@ -567,6 +574,7 @@ __device__ __forceinline__ void particle_forces_body(const PartArgs& a, const Bl
   // widened box are the particle's own), so no load waits on the key
   float nif[3] = {0.0f, 0.0f, 0.0f};
   const float* const ifl = (const float*)a.ifield;
+  __shared__ double s_qn;
   const bool only = ONE == 2 ? a.P == 1 : ONE == 1;
   auto fetch = [&]() {
     nown = a.owner[nn];
@@ -588,6 +596,10 @@ __device__ __forceinline__ void particle_forces_body(const PartArgs& a, const Bl
     nfirst = locate(cnext, nX, nY, nZ, nn, nw3, nmx, nmy, nmz);
     fetch();
   }
+  if (threadIdx.x == 0) s_qn = charge_norm(a, P);
+  __syncthreads();
+  const double qnorm = s_qn;
+  const float qnormf = (float)qnorm;
   // Links into the sphere start at fluid nodes within R + sqrt(2) of the
   // centre (a covered node lies within R); the test below takes R + 1.5.  The
   // box offsets X - r_p it measures are the minimum-image ones for every
@@ -608,11 +620,21 @@ __device__ __forceinline__ void particle_forces_body(const PartArgs& a, const Bl
   }
   // the warp's fluid nodes next to the particle (at most one per cell), as box
   // offsets of ten bits each: the links are taken after the loop, 32 nodes at a
-  // time.  The list takes the room of the block sums that follow it.
+  // time.  FP32 form: also the entries of each row (its lanes, the first's place),
+  // and the momentum of 32 nodes.  All of it takes the room of the block sums that
+  // follow.
   __shared__ double tr[FPART][FORCE_T + 1];
-  static_assert(sizeof(tr) >= FORCE_ROWS * FORCE_T * sizeof(unsigned), "one entry per cell");
-  unsigned* const list = reinterpret_cast<unsigned*>(tr) + (threadIdx.x >> 5) * (FORCE_ROWS * 32);
+  struct WarpList {
+    unsigned at[FORCE_ROWS * 32];
+    uint2 row[FORCE_ROWS];
+    float mom[32][6];
+  };
+  static_assert(sizeof(tr) >= FORCE_T / 32 * sizeof(WarpList) && alignof(double) >= alignof(WarpList), "room");
+  WarpList& wl = reinterpret_cast<WarpList*>(tr)[threadIdx.x >> 5];
+  unsigned* const list = wl.at;
+  const int lane = threadIdx.x & 31;
   int nlist = 0;
+  unsigned my_rows = 0;  // the rows whose cell of this lane is listed
   for (int k = 0; k < rows; ++k) {
     const bool valid = nvalid;
     if (!__any_sync(0xffffffffu, valid)) break;
@@ -660,9 +682,11 @@ __device__ __forceinline__ void particle_forces_body(const PartArgs& a, const Bl
     const unsigned nl = __ballot_sync(0xffffffffu, near);
     if (near) {
       // in_box: the box offsets are below 1024
-      list[nlist + __popc(nl & ((1u << (threadIdx.x & 31)) - 1u))] =
+      list[nlist + __popc(nl & ((1u << lane) - 1u))] =
           (unsigned)(X - P.lo[0]) | (unsigned)(Y - P.lo[1]) << 10 | (unsigned)(Z - P.lo[2]) << 20;
+      my_rows |= 1u << k;
     }
+    if (FM::fp32 && lane == 0) wl.row[k] = make_uint2(nl, (unsigned)nlist);
     nlist += __popc(nl);
     if (!valid) continue;
     // reaction of the internal solute force on the fluid nodes this particle claims
@@ -704,40 +728,49 @@ __device__ __forceinline__ void particle_forces_body(const PartArgs& a, const Bl
     }
     // the particle's own charge in this cell
     if (in_box) {
-      double ps = 0.0;
+      double qq = 0.0;
       float psf = 0.0f;
       bool has_q = false;
       if (pv) {
         const int bx = P.hi[0] - P.lo[0], by = P.hi[1] - P.lo[1];
         const int cb = (X - P.lo[0]) + bx * ((Y - P.lo[1]) + by * (Z - P.lo[2]));
-        ps = a.psibox[(long long)p * a.boxmax + cb];
-        has_q = (__double_as_longlong(ps) << 1) != 0;
-        if (FM::fp32) psf = psibox_float((unsigned long long)__double_as_longlong(ps));
+        const double ps = a.psibox[(long long)p * a.boxmax + cb];
+        if (FM::fp32) {
+          // the weight itself is applied in float below
+          psf = psibox_float((unsigned long long)__double_as_longlong(ps));
+          has_q = psf != 0.0f;
+        } else {
+          qq = qnorm * ps;
+          has_q = qq != 0.0;
+        }
       } else if (own == p) {
-        ps = 1.0;
+        qq = qnorm;
         psf = 1.0f;
-        has_q = true;
+        has_q = (__double_as_longlong(qnorm) << 1) != 0;
       }
       if (has_q) {
         touched |= 4u;
         if (FM::fp32) {
-          macc[6] += psf;
-          macc[7] += psf * __fsub_rn((float)(X - P.ipos[0]), P.fpos[0]);
-          macc[8] += psf * __fsub_rn((float)(Y - P.ipos[1]), P.fpos[1]);
-          macc[9] += psf * __fsub_rn((float)(Z - P.ipos[2]), P.fpos[2]);
+          const float qf = qnormf * psf;
+          macc[6] += qf;
+          macc[7] += qf * __fsub_rn((float)(X - P.ipos[0]), P.fpos[0]);
+          macc[8] += qf * __fsub_rn((float)(Y - P.ipos[1]), P.fpos[1]);
+          macc[9] += qf * __fsub_rn((float)(Z - P.ipos[2]), P.fpos[2]);
         } else {
-          acc[12] += ps;
-          acc[13] += ps * ((double)X - P.pos[0]);
-          acc[14] += ps * ((double)Y - P.pos[1]);
-          acc[15] += ps * ((double)Z - P.pos[2]);
+          acc[12] += qq;
+          acc[13] += qq * ((double)X - P.pos[0]);
+          acc[14] += qq * ((double)Y - P.pos[1]);
+          acc[15] += qq * ((double)Z - P.pos[2]);
         }
       }
     }
   }
   // the list, whole warps of neighbours of the surface (a row of the box has few)
   __syncwarp();
-  for (int q = threadIdx.x & 31; q < nlist; q += 32) {
-    const unsigned at = list[q];
+  for (int q0 = 0; q0 < nlist; q0 += 32) {
+    const bool listed = q0 + lane < nlist;
+    const unsigned at = listed ? list[q0 + lane] : 0u;
+    float m[6] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};  // FP32 form: the node's force and torque
     const int X = P.lo[0] + (int)(at & 1023u), Y = P.lo[1] + (int)(at >> 10 & 1023u), Z = P.lo[2] + (int)(at >> 20);
     const int w3[3] = {wrap_box(X, g.nx), wrap_box(Y, g.ny), wrap_box(Z, g.nz)};
     const long long n = (long long)(w3[0] + g.nx * (w3[1] + g.ny * w3[2]));
@@ -746,11 +779,13 @@ __device__ __forceinline__ void particle_forces_body(const PartArgs& a, const Bl
     // FP64 arithmetic only at nodes next to the surface
     const Nbr b = make_nbr(w3[0], w3[1], w3[2], g);
     unsigned links = 0;
+    if (listed) {
 #pragma unroll
-    for (int i = 1; i < Q; ++i) {
-      const long long m = node_index(g, nb_x(b, w3[0], dcx(i)), nb_y(b, w3[1], dcy(i)),
-                                     nb_z(b, w3[2], dcz(i)));
-      if (a.owner[m] == p) links |= 1u << i;
+      for (int i = 1; i < Q; ++i) {
+        const long long nb = node_index(g, nb_x(b, w3[0], dcx(i)), nb_y(b, w3[1], dcy(i)),
+                                        nb_z(b, w3[2], dcz(i)));
+        if (a.owner[nb] == p) links |= 1u << i;
+      }
     }
     if (links && FM::fp32) {
       // FP32 form, in float: the populations are stored as deviations
@@ -785,12 +820,12 @@ __device__ __forceinline__ void particle_forces_body(const PartArgs& a, const Bl
       fy += cst * (float)ky;
       fz += cst * (float)kz;
       touched |= 1u;
-      macc[0] += fx;
-      macc[1] += fy;
-      macc[2] += fz;
-      macc[3] += d0y * fz - d0z * fy;
-      macc[4] += d0z * fx - d0x * fz;
-      macc[5] += d0x * fy - d0y * fx;
+      m[0] = fx;
+      m[1] = fy;
+      m[2] = fz;
+      m[3] = d0y * fz - d0z * fy;
+      m[4] = d0z * fx - d0x * fz;
+      m[5] = d0x * fy - d0y * fx;
     } else if (links) {
       const double d0x = (double)X - P.pos[0], d0y = (double)Y - P.pos[1], d0z = (double)Z - P.pos[2];
       const double wx = P.vel[0] + (P.omega[1] * d0z - P.omega[2] * d0y);
@@ -814,6 +849,20 @@ __device__ __forceinline__ void particle_forces_body(const PartArgs& a, const Bl
       acc[3] += d0y * fz - d0z * fy;
       acc[4] += d0z * fx - d0x * fz;
       acc[5] += d0x * fy - d0y * fx;
+    }
+    if (FM::fp32) {
+#pragma unroll
+      for (int j = 0; j < 6; ++j) wl.mom[lane][j] = m[j];
+      __syncwarp();
+      while (my_rows) {
+        const uint2 r = wl.row[__ffs(my_rows) - 1];
+        const int e = (int)r.y + __popc(r.x & ((1u << lane) - 1u)) - q0;
+        if (e >= 32) break;
+        my_rows &= my_rows - 1u;
+#pragma unroll
+        for (int j = 0; j < 6; ++j) macc[j] += wl.mom[e][j];
+      }
+      __syncwarp();
     }
   }
   float facc[FPART];
@@ -1021,11 +1070,9 @@ __device__ void integrate_all(const PartArgs& a) {
       for (int d = d0; d < 3; d += dstep) {
         const int d1 = d == 2 ? 0 : d + 1, d2 = d == 0 ? 2 : d - 1;  // (d, d1, d2) cyclic
         const int nn = d == 0 ? a.g.nx : (d == 1 ? a.g.ny : a.g.nz);
-        // field on the own charge: E sum q, (sum q (r - r_p)) x E, with q the
-        // summed weights times the charge per unit weight
-        const double qn = charge_norm(a, *Pp);
-        const double Tq = qn * (__ldcg(acc + 13 + d1) * E[d2] - __ldcg(acc + 13 + d2) * E[d1]);
-        const double F = __ldcg(acc + d) + __ldcg(acc + 6 + d) + qn * __ldcg(acc + 12) * E[d] - rem[d] +
+        // field on the own charge: E sum q, (sum q (r - r_p)) x E
+        const double Tq = __ldcg(acc + 13 + d1) * E[d2] - __ldcg(acc + 13 + d2) * E[d1];
+        const double F = __ldcg(acc + d) + __ldcg(acc + 6 + d) + __ldcg(acc + 12) * E[d] - rem[d] +
                          Pp->ftrans[d];
         const double T = __ldcg(acc + 3 + d) + __ldcg(acc + 9 + d) + Tq;
         double pos = Pp->pos[d], vel = Pp->vel[d], omega = Pp->omega[d];
