@@ -17,8 +17,10 @@
 // What bounds it: the FP64 pipe on the finest level, launches below.  So the
 // right-hand side is kept as b / (6 c) (a half sweep is 5 additions and one FMA
 // a node), residuals are formed on the red nodes only (those of the black ones,
-// updated last, are zero to rounding; the residual that is returned is taken
-// over all nodes), the restriction weighs the 13 red nodes of its 27, and the
+// updated last, are zero to rounding, once that last half sweep divides by 6
+// with both parts of 1/6: by the rounded 1/6 alone every black node kept a residual of
+// 6 2^-54 phi, of one sign, which the cycles did not see; the residual that is
+// returned is taken over all nodes), the restriction weighs the 13 red nodes of its 27, and the
 // correction goes to the black nodes only (the red half sweep that follows does
 // not read the others).  The coarse levels run while the host waits for the
 // residual.  128^3 to 1e-12 (GB300): 13 cycles of 0.51 ms -> 13 of 0.36 ms.  Of
@@ -96,6 +98,9 @@ __global__ void k_mg_sum(const double* x, long long n, double* part, Scalars* ou
   }
 }
 
+// 1/6 as a sum of two doubles
+constexpr double SIXTH = 1.0 / 6.0, SIXTH_LO = 0x1.5555555555555p-57;
+
 // the bits of |v| (they order as the values do); 0 for a NaN
 __device__ __forceinline__ unsigned long long abs_bits(double v) {
   const unsigned long long b = (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffULL;
@@ -142,15 +147,17 @@ __global__ void __launch_bounds__(MG_T) k_mg_rhs(const double* q, double* phi, d
     const unsigned row = i / (unsigned)nx;
     const int x = (int)(i - row * (unsigned)nx), y = (int)(row % (unsigned)ny), z = (int)(row / (unsigned)ny);
     const double v = s * (q[i] - sc->mean);  // read before phi, which may alias q, is written
-    constexpr double SIXTH = 1.0 / 6.0;
-    b[i] = v * SIXTH;
-    phi[i] = ((x + y + z) & 1) ? 0.0 : v * SIXTH;
+    const double v6 = fma(v, SIXTH, v * SIXTH_LO);
+    b[i] = v6;
+    phi[i] = ((x + y + z) & 1) ? 0.0 : v6;
     m = abs_bits(v);
   }
   grid_max(m, sc);
 }
 
-// one colour of a red-black Gauss-Seidel sweep: phi = sum nb / 6 + b
+// one colour of a red-black Gauss-Seidel sweep: phi = sum nb / 6 + b (FULL: both
+// parts of 1/6)
+template <bool FULL>
 __global__ void __launch_bounds__(MG_T) k_mg_half(double* phi, const double* b, int nx, int ny, int nz, int colour) {
   let_next_start();
   after_previous();
@@ -158,8 +165,8 @@ __global__ void __launch_bounds__(MG_T) k_mg_half(double* phi, const double* b, 
   if (j >= (unsigned)nx / 2u * (unsigned)ny * (unsigned)nz) return;
   int x, y, z;
   const int i = colour_node(j, nx, ny, colour, x, y, z);
-  constexpr double SIXTH = 1.0 / 6.0;
-  phi[i] = fma(nb_sum(phi, i, x, y, z, nx, ny, nz), SIXTH, b[i]);
+  const double s = nb_sum(phi, i, x, y, z, nx, ny, nz);
+  phi[i] = fma(s, SIXTH, FULL ? fma(s, SIXTH_LO, b[i]) : b[i]);
 }
 
 // residual over 4^-l on the red nodes, r = sum nb - 6 (phi - b); with MAX the
@@ -312,8 +319,9 @@ cudaError_t mean_of(const Solver& S, const double* x, long long n) {
   return cudaGetLastError();
 }
 
-void half(const Solver& S, const Level& l, int colour) {
-  launch_next(k_mg_half, blocks(l.n / 2), MG_T, 0, S.s, l.phi, l.b, l.nx, l.ny, l.nz, colour);
+void half(const Solver& S, const Level& l, int colour, bool full = false) {
+  launch_next(full ? k_mg_half<true> : k_mg_half<false>, blocks(l.n / 2), MG_T, 0, S.s, l.phi, l.b, l.nx, l.ny, l.nz,
+              colour);
 }
 void restrict_to(const Solver& S, const Level& l, const Level& c) {
   launch_next(k_mg_restrict, blocks(c.n), MG_T, 0, S.s, l.r, l.nx, l.ny, l.nz, c.b, c.phi);
@@ -437,7 +445,7 @@ cudaError_t poisson_solve_mg(const PoissonPlan& coarse_plan, const double* q, do
       if (rmax <= tol * bmax) break;
     }
   } else if (bmax > 0.0) {
-    half(S, f, 1);  // the first sweep's black half
+    half(S, f, 1, true);  // the first sweep's black half
     for (;;) {
       e = clear_max();
       if (e != cudaSuccess) return e;
@@ -464,7 +472,7 @@ cudaError_t poisson_solve_mg(const PoissonPlan& coarse_plan, const double* q, do
       prolong_to(S, f, S.lv[1]);
       for (int sweep = 0; sweep < 4; ++sweep) {
         half(S, f, 0);
-        half(S, f, 1);
+        half(S, f, 1, sweep == 3);
       }
       ++done;
     }
