@@ -20,13 +20,15 @@
 // no bit reversal pass is needed.
 //
 // The FP64 passes are bound by the FP64 pipe (2 lanes per clock per SM), so
-// their butterflies are written as chains of FMAs that take the twiddles along
-// (Linzer and Feig, IEEE Trans. Signal Processing 41, 1993; Goedecker, SIAM J.
-// Sci. Comput. 18, 1997): 24 instructions for a radix-4 butterfly with its three
-// twiddles, against 28 with separate products, and 256^3 in 2.27 ms against 2.65
-// (2.93 before, with divisions in the index arithmetic as well); 48 x 32 x 72,
-// where CTAs of 1024 elements left most SMs idle, 84 -> 47 us.  The errors are
-// those of the separate products (eigenvalue tables: 3e-15 to 1e-14).
+// their butterflies take twiddles along in FMAs (Linzer and Feig, IEEE Trans.
+// Signal Processing 41, 1993; Goedecker, SIAM J. Sci. Comput. 18, 1997): 24
+// instructions for a radix-4 butterfly with its three twiddles, against 28 with
+// separate products, and 256^3 in 2.32 ms against 2.65 (2.93 before, with
+// divisions in the index arithmetic as well); 48 x 32 x 72, where CTAs of 1024
+// elements left most SMs idle, 82 -> 37 us.  The transforms' own errors are within
+// 1% of the separate products' (64^3 9.89e-16 and 9.85e-16, 128 x 128 x 64
+// 1.139e-15 and 1.129e-15, against long double transforms with the same tables);
+// the eigenvalue tables' are larger (3e-15 to 1e-14).
 #include <math.h>
 #include <cstdint>
 #include <cstring>
@@ -176,12 +178,6 @@ template <typename C> __device__ __forceinline__ C twice_minus(C a, C t) {
   using R = decltype(C().x);
   return mkc(fma(R(2), a.x, -t.x), fma(R(2), a.y, -t.y));
 }
-// t - i w u and t + i w u (forward; inverse: conjugate twiddle, signs changed)
-template <bool INV, typename C> __device__ __forceinline__ C fma_tw_rot(C w, C u, C t) {
-  return INV ? mkc(fma(-w.x, u.y, fma(w.y, u.x, t.x)), fma(w.x, u.x, fma(w.y, u.y, t.y)))
-             : mkc(fma(w.x, u.y, fma(w.y, u.x, t.x)), fma(-w.x, u.x, fma(w.y, u.y, t.y)));
-}
-
 // padding of a line in shared memory: one element every 16
 __device__ __host__ __forceinline__ int gpad(int i) { return i + (i >> 4); }
 
@@ -226,14 +222,16 @@ __device__ __forceinline__ void gen_stage(const C* a, C* b, int nl, int n, int N
         o[1] = cadd(d02, d13);
         o[3] = csub(d02, d13);
       } else {
-        // w^3 = w w^2: both inner pairs take the twiddle w^2, the outer ones w
-        const C w1 = tw[k * ts], w2 = tw[2 * k * ts];
+        // every twiddle from the table (w^3 taken as w w^2, in one instruction chain
+        // with the butterfly, rounds it twice: errors 2 to 5% larger)
+        const C w1 = tw[k * ts], w2 = tw[2 * k * ts], w3 = tw[3 * k * ts];
+        const C t1 = INV ? cmulconj(v[1], w1) : cmul(v[1], w1);
         const C s02 = fma_tw<INV>(w2, v[2], v[0]), d02 = twice_minus(v[0], s02);
-        const C s13 = fma_tw<INV>(w2, v[3], v[1]), d13 = twice_minus(v[1], s13);
-        o[0] = fma_tw<INV>(w1, s13, s02);
-        o[2] = twice_minus(s02, o[0]);
-        o[1] = fma_tw_rot<INV>(w1, d13, d02);
-        o[3] = twice_minus(d02, o[1]);
+        const C s13 = fma_tw<INV>(w3, v[3], t1), d13 = rot(twice_minus(t1, s13), INV);
+        o[0] = cadd(s02, s13);
+        o[2] = csub(s02, s13);
+        o[1] = cadd(d02, d13);
+        o[3] = csub(d02, d13);
       }
     } else {  // 8, 9 (FP32)
       if (!FIRST) {
