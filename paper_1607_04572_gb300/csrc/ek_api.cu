@@ -1,5 +1,6 @@
 // Host side of the C ABI declared in include/ek.h: context, device memory,
 // the time-step driver and field / particle exchange.
+#include <cuda.h>
 #include <math.h>
 #include <string.h>
 
@@ -578,6 +579,38 @@ ek_status ready(ek_ctx* ctx) {
   return run_setup(ctx);
 }
 
+// A kernel of the context's GPU may store doubles to [p, p + bytes): aligned memory
+// of that very device, inside one allocation.  Memory of another GPU (which a copy
+// reaches without peer access), host or managed memory, and what no single
+// allocation holds are left to a copy, which reaches or refuses them.
+bool device_may_store(const ek_ctx* ctx, const void* p, size_t bytes) {
+  if (((uintptr_t)p & (sizeof(double) - 1)) != 0) return false;
+  // cuPointerGetAttributes (one call of about 1 us), without a link to the driver
+  // library
+  using AttributesOf = decltype(&cuPointerGetAttributes);
+  static const AttributesOf attributes_of = [] {
+    void* f = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPointByVersion("cuPointerGetAttributes", &f, 12000, cudaEnableDefault, &q) != cudaSuccess) {
+      cudaGetLastError();
+      f = nullptr;
+    }
+    return reinterpret_cast<AttributesOf>(f);
+  }();
+  unsigned type = 0, managed = 1;
+  int device = -1;
+  CUdeviceptr base = 0;
+  size_t size = 0;
+  CUpointer_attribute which[] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_IS_MANAGED,
+                                 CU_POINTER_ATTRIBUTE_DEVICE_ORDINAL, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR,
+                                 CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+  void* out[] = {&type, &managed, &device, &base, &size};
+  const CUdeviceptr at = (CUdeviceptr)(uintptr_t)p;
+  if (!attributes_of || attributes_of(5, which, out, at) != CUDA_SUCCESS) return false;
+  if (type != CU_MEMORYTYPE_DEVICE || managed || device != ctx->device || base > at) return false;
+  return at - base <= size && bytes <= size - (at - base);
+}
+
 size_t field_size(const ek_ctx* ctx, ek_field w) {
   const size_t N = (size_t)ctx->g.N;
   switch (w) {
@@ -1002,10 +1035,9 @@ ek_status ek_get_fields(ek_ctx* ctx, ek_field which, int component, double* dst,
   const Grid& g = ctx->g;
   cudaStream_t s = ctx->stream;
   const bool f32 = ctx->fp32 != 0;
-  // A converted field goes straight to a device destination (a copy of its own
-  // would move every value twice more), to a host one, or one that no double
-  // may be stored to, through tmp.
-  const bool direct = dst_on_device && ((uintptr_t)dst & (sizeof(double) - 1)) == 0;
+  // A converted field goes straight to a destination on this device (a copy of
+  // its own would move every value twice more), to any other through tmp.
+  const bool direct = dst_on_device && device_may_store(ctx, dst, count * sizeof(double));
   double* const conv = direct ? dst : ctx->tmp;
   // copy one converted N-element block (tmp) to dst + offset
   auto out_block = [&](size_t offset) -> cudaError_t {
