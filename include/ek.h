@@ -404,6 +404,10 @@ ek_status ek_batch_set_config(ek_batch* b, const int cfg[4]);
  * were out of memory, so that ek_create frees what it allocated and returns
  * EK_ERR_NOMEM; n <= 0 clears the hook.  Process-wide; for tests. */
 void ek_debug_fail_alloc(int n);
+/* Test hook: the ek_poisson_solve_cg calls that follow behave as on a device
+ * that places no cluster of more than n thread blocks (they take a smaller
+ * one, with the same result); n <= 0 clears it.  Process-wide; for tests. */
+void ek_debug_cluster_limit(int n);
 /* Failure-detection test hook for form 2: in the steps captured from now on,
  * CTA leave_cta of each persistent particle-chain launch returns before the
  * first grid barrier (-1: none), and a wait at a barrier gives up after

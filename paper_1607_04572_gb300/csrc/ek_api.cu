@@ -858,6 +858,8 @@ ek_status ek_create(const ek_params* p, ek_ctx** out) {
 
 void ek_debug_fail_alloc(int n) { g_alloc_fault.store(n > 0 ? n : 0); }
 
+void ek_debug_cluster_limit(int n) { poisson_cg_cluster_limit(n); }
+
 ek_status ek_destroy(ek_ctx* ctx) {
   if (!ctx) return EK_ERR_ARG;
   cudaSetDevice(ctx->device);

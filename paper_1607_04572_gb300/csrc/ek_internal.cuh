@@ -319,6 +319,7 @@ cudaError_t charge_density(const Grid& g, const Phys& ph, const void* rho, const
 // by multigrid-preconditioned conjugate gradients (ek_krylov.cu); *bad_eps is set
 // (and nothing solved) when a permittivity is not positive and finite
 size_t poisson_cg_scratch_bytes(int nx, int ny, int nz);
+void poisson_cg_cluster_limit(int n);  // ek_debug_cluster_limit
 cudaError_t poisson_solve_cg(const double* q, const double* eps, const unsigned char* fixed,
                              const double* phi_fixed, double* phi, int nx, int ny, int nz, double bjerrum,
                              double tol, int max_iter, void* scratch, cudaStream_t s, int* iters,

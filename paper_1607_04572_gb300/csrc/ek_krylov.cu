@@ -35,6 +35,7 @@
 #include <math.h>
 
 #include <algorithm>
+#include <atomic>
 
 #include <cooperative_groups.h>
 
@@ -634,7 +635,8 @@ __global__ void __launch_bounds__(CG_T) k_mg_diag(MGLevel C) {
 // of one cluster, whose CTAs meet at cluster barriers between the half sweeps.
 // Each of these phases is short: as launches of their own (nine per level) they
 // took 3 to 4 us each, most of an iteration at 64^3.  The FP64 pipes of 16 SMs
-// hold up to 32^3 nodes (15 us).  The coarsest level (every edge below 8: at
+// hold up to 32^3 nodes (15 us); a part of a GPU that cannot place a cluster of 16
+// (above the portable size) takes a smaller one, with the same result.  The coarsest level (every edge below 8: at
 // most 343 nodes) is done by the first CTA, a node per thread with its faces in
 // registers and x in shared memory.
 constexpr int MG_COARSE_MAX = 343;
@@ -854,33 +856,54 @@ size_t full_layout(int nx, int ny, int nz, CGView* v, void* base, MGLevel* lev, 
 
 unsigned nblocks(int n) { return ((unsigned)n + CG_T - 1) / CG_T; }
 
-// a cluster of MG_SMALL_CTAS CTAs is above the portable size
-cudaError_t launch_small(const MGLevel* lev, int L, cudaStream_t s) {
+// the small launch's configuration for a cluster of n CTAs
+struct SmallLaunch {
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute at[2];
+  SmallLaunch(int n, cudaStream_t s, bool early) {
+    cfg.gridDim = dim3(n);
+    cfg.blockDim = dim3(MG_SMALL_T);
+    cfg.stream = s;
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = n;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = early ? 2 : 1;
+  }
+};
+
+std::atomic<int> g_cluster_limit{0};  // ek_debug_cluster_limit
+
+// CTAs of the small launch: the largest cluster that the device can place
+cudaError_t small_ctas(cudaStream_t s, int& n) {
   cudaError_t e = cudaFuncSetAttribute(k_mg_small, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   if (e != cudaSuccess) return e;
+  const int limit = g_cluster_limit.load();
+  for (n = MG_SMALL_CTAS; n > 1; n /= 2) {
+    if (limit > 0 && n > limit) continue;
+    SmallLaunch c(n, s, false);
+    int fit = 0;
+    if (cudaOccupancyMaxActiveClusters(&fit, k_mg_small, &c.cfg) == cudaSuccess && fit > 0) break;
+    cudaGetLastError();
+  }
+  return cudaSuccess;
+}
+
+cudaError_t launch_small(const MGLevel* lev, int L, int ctas, cudaStream_t s) {
   MGSmall S;
   S.n = L;
   std::copy(lev, lev + L, S.lev);
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(MG_SMALL_CTAS);
-  cfg.blockDim = dim3(MG_SMALL_T);
-  cfg.stream = s;
-  cudaLaunchAttribute at[2];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = MG_SMALL_CTAS;
-  at[0].val.clusterDim.y = 1;
-  at[0].val.clusterDim.z = 1;
-  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[1].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = early_launch(s) ? 2 : 1;
-  return cudaLaunchKernelEx(&cfg, k_mg_small, S);
+  const SmallLaunch c(ctas, s, early_launch(s));
+  return cudaLaunchKernelEx(&c.cfg, k_mg_small, S);
 }
 
 // z = M r: one V-cycle over the levels, then r.z and beta.  The first half
 // sweep of a red-black level has been made where its right-hand side was.  The
 // fine level is never in the small launch: its last sweep forms r.z.
-cudaError_t vcycle(const MGLevel* lev, int L, const CGView& v, int first, cudaStream_t s) {
+cudaError_t vcycle(const MGLevel* lev, int L, int ctas, const CGView& v, int first, cudaStream_t s) {
   int small = 1;
   while (small < L - 1 && lev[small].n > MG_SMALL) ++small;
   for (int l = 0; l < small; ++l) {
@@ -895,7 +918,7 @@ cudaError_t vcycle(const MGLevel* lev, int L, const CGView& v, int first, cudaSt
     }
     launch_next(k_mg_restrict, nblocks(lev[l + 1].n), CG_T, 0, s, A, lev[l + 1]);
   }
-  const cudaError_t e = launch_small(lev + small, L - small, s);
+  const cudaError_t e = launch_small(lev + small, L - small, ctas, s);
   if (e != cudaSuccess) return e;
   for (int l = small - 1; l >= 0; --l) {
     const MGLevel& A = lev[l];
@@ -918,6 +941,8 @@ cudaError_t vcycle(const MGLevel* lev, int L, const CGView& v, int first, cudaSt
 
 }  // namespace
 
+void poisson_cg_cluster_limit(int n) { g_cluster_limit.store(n > 0 ? n : 0); }
+
 size_t poisson_cg_scratch_bytes(int nx, int ny, int nz) {
   return full_layout(nx, ny, nz, nullptr, nullptr, nullptr, nullptr);
 }
@@ -932,12 +957,14 @@ cudaError_t poisson_solve_cg(const double* q, const double* eps, const unsigned 
   int nlev = 1;
   full_layout(nx, ny, nz, &v, scratch, lev, &nlev);
   const bool mg = nlev >= 2;
+  int ctas = 1;  // of the cycle's small launch
   const int nb = (int)std::min<long long>(CG_BLOCKS, (b.N + CG_T - 1) / CG_T);
   const int tx = (nx + 31) / 32, ty = (ny + 7) / 8;
   const int na = (int)std::min<long long>(CG_BLOCKS, (long long)tx * ty * nz);  // operator blocks
   double h[16];
   *bad_eps = false;
   cudaError_t e = cudaMemsetAsync(v.sc, 0, 16 * sizeof(double), s);
+  if (e == cudaSuccess && mg) e = small_ctas(s, ctas);
   if (e != cudaSuccess) return e;
   k_cg_faces<<<nb, CG_T, 0, s>>>(b, v, q, eps, fixed);
   // the invalid permittivities are counted before phi is written
@@ -967,7 +994,7 @@ cudaError_t poisson_solve_cg(const double* q, const double* eps, const unsigned 
     }
     launch_next(k_pcg_update, nb, CG_T, 0, s, b, v, phi, lev[0], neutral);
     if (neutral) launch_next(k_pcg_project, nb, CG_T, 0, s, b, v, lev[0], 1);
-    const cudaError_t ve = vcycle(lev, nlev, v, 0, s);
+    const cudaError_t ve = vcycle(lev, nlev, ctas, v, 0, s);
     if (e == cudaSuccess) e = ve;
     launch_next(k_pcg_direction, nblocks((int)b.N), CG_T, 0, s, b, v, lev[0].x);
   };
@@ -978,7 +1005,7 @@ cudaError_t poisson_solve_cg(const double* q, const double* eps, const unsigned 
       launch_next(k_mg_diag, nblocks(lev[l].n), CG_T, 0, s, lev[l]);
     }
     if (lev[0].rb) launch_next(k_pcg_project, nb, CG_T, 0, s, b, v, lev[0], 0);
-    e = vcycle(lev, nlev, v, 1, s);
+    e = vcycle(lev, nlev, ctas, v, 1, s);
     if (e != cudaSuccess) return e;
     launch_next(k_pcg_direction, nblocks((int)b.N), CG_T, 0, s, b, v, lev[0].x);
   }

@@ -52,7 +52,7 @@ EXPORTS = ["ek_create", "ek_destroy", "ek_add_particle", "ek_set_field", "ek_get
            "ek_poisson_solve_mg", "ek_poisson_cg_scratch_bytes", "ek_poisson_solve_cg",
            "ek_batch_create", "ek_batch_destroy", "ek_batch_set_stream", "ek_batch_step_async",
            "ek_batch_step", "ek_batch_sync", "ek_batch_tune", "ek_batch_config", "ek_batch_set_config",
-           "ek_batch_wait_test", "ek_batch_size", "ek_debug_fail_alloc",
+           "ek_batch_wait_test", "ek_batch_size", "ek_debug_fail_alloc", "ek_debug_cluster_limit",
            "ek_batch_last_error"]
 
 
@@ -141,6 +141,8 @@ def load_library(path: str | None = None) -> ctypes.CDLL:
     lib.ek_batch_wait_test.argtypes = [vp, ip, dp]
     lib.ek_debug_fail_alloc.argtypes = [ip]
     lib.ek_debug_fail_alloc.restype = None
+    lib.ek_debug_cluster_limit.argtypes = [ip]
+    lib.ek_debug_cluster_limit.restype = None
     lib.ek_batch_size.argtypes = [vp]
     lib.ek_batch_size.restype = ip
     lib.ek_batch_last_error.argtypes = [vp]
@@ -148,7 +150,7 @@ def load_library(path: str | None = None) -> ctypes.CDLL:
     for name in EXPORTS:
         if name not in ("ek_num_particles", "ek_last_error", "ek_lattice_dirs",
                         "ek_poisson_scratch_bytes", "ek_kernel_launches", "ek_batch_size",
-                        "ek_poisson_mg_scratch_bytes", "ek_debug_fail_alloc",
+                        "ek_poisson_mg_scratch_bytes", "ek_debug_fail_alloc", "ek_debug_cluster_limit",
                         "ek_poisson_cg_scratch_bytes",
                         "ek_batch_last_error"):
             getattr(lib, name).restype = ip
@@ -160,6 +162,12 @@ def debug_fail_alloc(n: int) -> None:
     """Test hook: the n-th field allocation of ek_create from now on fails (see
     ek_debug_fail_alloc in include/ek.h); n <= 0 clears it."""
     load_library().ek_debug_fail_alloc(int(n))
+
+
+def debug_cluster_limit(n: int) -> None:
+    """Test hook: conjugate-gradient solves from now on take clusters of at most n
+    blocks (see ek_debug_cluster_limit in include/ek.h); n <= 0 clears it."""
+    load_library().ek_debug_cluster_limit(int(n))
 
 
 def lattice_dirs() -> np.ndarray:
