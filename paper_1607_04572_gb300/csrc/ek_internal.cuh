@@ -145,14 +145,20 @@ struct FormF32 {
 // after_previous in all of its threads, so that its end implies the end of all
 // before it.
 //
+// Where let_next_start stands: kernels of a node or two per thread call it first, the
+// FP64 and generic line transforms before their last stores.  Called first, the
+// blocks of a whole chain of small grids come onto the SMs together, are spread
+// unevenly and stay where they are: a 54^3 solve (FP64, five passes) took 115 us so,
+// 107 with ordinary launches of the earlier passes, 56 with the call at the end.
+//
 // These chains are bound by the launches where the kernels take a few us each:
-// the Poisson solve of a 48 x 32 x 72 box (FP64, five passes) 43.8 -> 38.9 us, 13
+// the Poisson solve of a 48 x 32 x 72 box (FP64, five passes) 44.6 -> 36.9 us, 13
 // V-cycles at 128^3 4.33 -> 3.34 ms, the set-up of the conjugate gradients there
 // 0.2 ms less, stage 5 of a 32^3 box 44 -> 32 us.  (Index arithmetic before the
 // wait changed none of them.)  Under capture the launches stay ordinary: a graph
 // starts its next kernel soon enough by itself, and successors that wait on the
-// SMs beside a forked branch hold it up (a step's graph with and without: 32^3
-// 65.9, 68.0 us; 128^3 209, 205; 256^3 1422, 1398).
+// SMs beside a forked branch hold it up in all but the smallest boxes (a step's
+// graph with and without: 32^3 65.9, 68.0 us; 128^3 209, 205; 256^3 1422, 1398).
 __device__ __forceinline__ void after_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 inline bool early_launch(cudaStream_t s) {

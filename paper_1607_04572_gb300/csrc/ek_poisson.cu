@@ -384,7 +384,6 @@ __device__ __forceinline__ const C* line_twiddles(const AxisPlan& P, C* sm) {
 // function (a power of two: the same rounding).
 template <typename R>
 __global__ void __launch_bounds__(FFT_THREADS) k_fft_x_fwd(PassArgs<R> a, int pairs_per_cta) {
-  let_next_start();
   after_previous();
   using C = typename CT<R>::type;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -406,6 +405,7 @@ __global__ void __launch_bounds__(FFT_THREADS) k_fft_x_fwd(PassArgs<R> a, int pa
   }
   __syncthreads();
   const C* res = fft_lines<false>(b0, b1, pairs_per_cta, a.ax, tw);
+  let_next_start();
   const int nxh = a.nxh;
   constexpr R h = sizeof(R) == sizeof(double) ? R(1) : R(0.5);
   for (int t = threadIdx.x; t < pairs_per_cta * nxh; t += blockDim.x) {
@@ -427,7 +427,6 @@ __global__ void __launch_bounds__(FFT_THREADS) k_fft_x_fwd(PassArgs<R> a, int pa
 // multiply and the inverse transform fused.
 template <typename R, int AXIS, bool INV>
 __global__ void __launch_bounds__(FFT_THREADS) k_fft_yz(PassArgs<R> a, int tx, unsigned mtx) {
-  let_next_start();
   after_previous();
   using C = typename CT<R>::type;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -470,6 +469,7 @@ __global__ void __launch_bounds__(FFT_THREADS) k_fft_yz(PassArgs<R> a, int tx, u
     __syncthreads();
     res = fft_lines<true>(res, res == b0 ? b1 : b0, nc, P, tw);
   }
+  let_next_start();
   for (int t = threadIdx.x; t < tx * n; t += blockDim.x) {
     const int j = div_by(t, mtx), c = t - j * tx;
     if (c < nc) S[j * stride + c] = res[c * LS + gpad(j)];
@@ -479,7 +479,6 @@ __global__ void __launch_bounds__(FFT_THREADS) k_fft_yz(PassArgs<R> a, int tx, u
 // X pass, inverse (complex-to-real), two rows per complex transform.
 template <typename R>
 __global__ void __launch_bounds__(FFT_THREADS) k_fft_x_inv(PassArgs<R> a, int pairs_per_cta) {
-  let_next_start();
   after_previous();
   using C = typename CT<R>::type;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -504,6 +503,7 @@ __global__ void __launch_bounds__(FFT_THREADS) k_fft_x_inv(PassArgs<R> a, int pa
   }
   __syncthreads();
   const C* res = fft_lines<true>(b0, b1, pairs_per_cta, a.ax, tw);
+  let_next_start();
   for (int t = threadIdx.x; t < pairs_per_cta * n; t += blockDim.x) {
     const int l = div_by(t, a.mnx), x = t - l * n;
     const int r0 = 2 * (p0 + l), r1 = r0 + 1;
