@@ -276,7 +276,7 @@ LBArgs lb_args(ek_ctx* ctx) {
   a.owner = ctx->owner;
   a.u = ctx->u;
   a.ifield = ctx->ifield;
-  a.ipart = ctx->ipart;
+  a.ipart = ctx->P || !ctx->fp32 ? ctx->ipart : nullptr;
   a.vsig = ctx->vsig;
   a.parts = ctx->dparts;
   a.status = ctx->status;

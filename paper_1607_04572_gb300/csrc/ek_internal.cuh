@@ -359,7 +359,8 @@ struct LBArgs {
   void* ifield;    // real_t, 3N: solute force on the fluid minus q_ions E (fluid nodes)
   unsigned char* vsig;  // N: bit 7 fluid node; bits 0-1, 2-3, 4-5: sign code of u_x, u_y, u_z
                         // (0 zero, 1 positive, 2 negative), written by S2 for S3
-  double* ipart;   // sums of ifield, 3 per block of the S2 grid (FP32: per tile column and plane group)
+  double* ipart;   // sums of ifield, 3 per block of the S2 grid (FP32: per tile column and plane group;
+                   // null without particles, which alone read them)
   const DevParticle* parts;
   int* status;
   int nzb;         // S2: z segments per (x, y) tile column (lb32_split, lb64_segments)

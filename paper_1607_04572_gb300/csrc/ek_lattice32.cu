@@ -561,7 +561,7 @@ __device__ __forceinline__ void lb32_block(const LBArgs& a, const Phys32& c, int
     }
     fm1 = f0;
     f0 = fp1;
-    const bool full = nsub == 1 && z + 1 == gend;
+    const bool full = a.ipart && nsub == 1 && z + 1 == gend;
     if (full) sum3_put(iv, red);
     __syncthreads();  // the next copies overwrite the slots of plane z - 1 and populations z
     if (full) {
@@ -572,7 +572,7 @@ __device__ __forceinline__ void lb32_block(const LBArgs& a, const Phys32& c, int
     }
   }
   cp_async_wait<0>();
-  if (nsub > 1) late_sum3(a, red, x, y, ga, gb, in_xy, min(nsub, gb - ga), row(grp));
+  if (a.ipart && nsub > 1) late_sum3(a, red, x, y, ga, gb, in_xy, min(nsub, gb - ga), row(grp));
 }
 
 template <int K, bool PV>
@@ -966,17 +966,20 @@ cudaError_t lb32_prepare() {
 // stages the plane on each side of it as well and starts with an empty
 // pipeline, so long segments waste less; short ones give the block scheduler
 // enough blocks (two resident per SM) to even out the SMs, and a small box
-// enough to fill them at all.  Measured on GB300 (ms per launch at 1 / 2 / 4 / 8
-// planes): 32^3 0.0142, 0.0187, 0.0290, 0.0492; 48 x 64 x 32 0.0167, 0.0212,
-// 0.0294, 0.0492; 64^3 0.0264, 0.0235, 0.0344, 0.0474; 96^3 0.0738, 0.0614,
-// 0.0634, 0.0751; 192 x 108 x 72 0.116, 0.0863, 0.0777, 0.0787; at 4 / 8 / 16 /
-// 32 planes: 128^3 0.103, 0.098, 0.102, 0.129; 256^3 (K = 3) 0.872, 0.816,
-// 0.800, 0.830; 512^3 6.48, 6.01, 5.79, 5.81.
+// enough to fill them at all (blocks next to a particle take longer, so boxes
+// with one want more of them than boxes without); segments below a plane group
+// pay for joining its sums.  Measured on GB300, a step's graph in us at 1 / 2 / 4 /
+// 8 / 16 planes with one particle and without, K = 2: 32^3 68, 72, 82, 95, 111 and
+// 26, 27, 31, 37, 53; 64^3 82, 78, 88, 96, 113 and 41, 41, 40, 41, 57; 96 x 64 x 48
+// 87, 84, 88, 99, 130 and 45, 42, 41, 43, 59; 64 x 64 x 128 120, 110, 106, 118, 128
+// and 72, 65, 65, 62, 70; 96^3 162, 145, 137, 144, 157 and 115, 103, 97, 98, 104;
+// 192 x 108 x 72 226, 197, 175, 186, 192 and 168, 147, 139, 143, 157; 128^3 263, 224,
+// 197, 197, 200; 192^3 810, 678, 576, 561, 560.
 int lb32_planes(long long cols, int nz) {
   auto blocks = [&](int p) { return cols * ((nz + p - 1) / p); };
   return blocks(16) >= 4096 ? 16
        : blocks(8) >= 1024 ? 8
-       : blocks(4) >= 1024 ? 4
+       : blocks(4) >= 512  ? 4
        : blocks(2) >= 512  ? 2
                            : 1;
 }
