@@ -286,7 +286,8 @@ ek_status ek_poisson_solve_mg(const double* q, double* phi, int nx, int ny, int 
  * the fine faces it covers, summed, over the halving along its axis; two
  * red-black Gauss-Seidel sweeps before and after, damped Jacobi ones on levels
  * with an odd edge; a few Jacobi sweeps on the coarsest level) when an edge can
- * be halved, else the diagonal (Jacobi); the residual is checked
+ * be halved, else the diagonal (Jacobi), as for rods (one edge of 8 or more,
+ * which is 64 or more or has another edge of 1 beside it); the residual is checked
  * every 2 (multigrid) or 10 (Jacobi) iterations.  Every inner product is a
  * fixed-order sum, so a solve is bit-reproducible.
  *

@@ -797,8 +797,13 @@ __global__ void __launch_bounds__(CG_T) k_pcg_direction(Box b, CGView v, const d
   if (n < (unsigned)b.N && !is_zero(v.dinv[n])) v.p[n] = z[n] + beta * v.p[n];
 }
 
-// the multigrid levels of a box (one: no edge to halve, the diagonal is the
-// preconditioner): the edges of each, and the halving towards the next
+// the multigrid levels of a box (one: the diagonal is the preconditioner): the
+// edges of each, and the halving towards the next.  A rod, whose one long edge would
+// be halved alone level after level, keeps the diagonal from 64 nodes on, or when
+// another edge is 1: the coupling across it comes to outweigh the one along it, and
+// the point sweeps no longer damp what the coarse level cannot hold (ms to 1e-10,
+// diagonal and V-cycle, without fixed nodes: 1 x 1 x 100 1.3, 3.0; 7 x 7 x 64 2.2,
+// 2.5; 7 x 7 x 32 1.5, 1.4; 6 x 6 x 64 2.2, 1.9; 9 x 9 x 64 2.5, 1.9).
 int mg_levels(int nx, int ny, int nz, int (*dims)[6]) {
   int L = 0;
   int d[3] = {nx, ny, nz};
@@ -813,6 +818,8 @@ int mg_levels(int nx, int ny, int nz, int (*dims)[6]) {
     if (!more) break;
     for (int k = 0; k < 3; ++k) d[k] = d[k] >= 8 ? (d[k] + 1) / 2 : d[k];
   }
+  const int longest = std::max(nx, std::max(ny, nz)), shortest = std::min(nx, std::min(ny, nz));
+  if ((nx >= 8) + (ny >= 8) + (nz >= 8) == 1 && (longest >= 64 || shortest == 1)) return 1;
   const int* c = dims[L - 1];
   return c[0] * c[1] * c[2] <= MG_COARSE_MAX ? L : 1;
 }
