@@ -1129,16 +1129,19 @@ __global__ void k_box_update(PartArgs a) {
   P.nb = 0;
 }
 
+// the counts that k_claim and k_psi_surface sum afresh; with the first particle's,
+// the transfer list: the last step's transitions have been applied, this step's
+// append to an empty one (a kernel of the chain instead of a memset node after the
+// transfers)
+__device__ __forceinline__ void reset_counts(const PartArgs& a, DevParticle& P, bool first) {
+  for (int j = 0; j < 8; ++j) P.psiunits[j] = 0;
+  P.nb = 0;
+  if (first) *a.xfer_count = 0;
+}
+
 __device__ __forceinline__ void save_prev_body(const PartArgs& a, const Blk bk) {
   DevParticle& P = a.parts[bk.x];
-  if (bk.y == 0 && threadIdx.x == 0) {  // k_claim and k_psi_surface sum these afresh
-    for (int j = 0; j < 8; ++j) P.psiunits[j] = 0;
-    P.nb = 0;
-    // the transfer list of the last step's transitions has been applied;
-    // this step's transitions append to an empty one (a kernel of the chain
-    // instead of a memset node after the transfers)
-    if (bk.x == 0) *a.xfer_count = 0;
-  }
+  if (bk.y == 0 && threadIdx.x == 0) reset_counts(a, P, bk.x == 0);
   const int c = bk.y * blockDim.x + threadIdx.x;
   if (c >= box_cells(P.ulo, P.uhi)) return;
   int X, Y, Z;
@@ -1175,21 +1178,40 @@ __global__ void k_clear(PartArgs a) {
   clear_body<FM>(a, grid_blk());
 }
 
-// both at once for a single particle, whose union box holds every node once
-// (it never wraps onto itself), so no other thread reads what is cleared here:
-// one launch less in the chain (a step at 32^3 68.1 -> 66.4 us, at 128^3 201.6 ->
-// 200.0)
+// both at once for a single particle: one launch less in the chain (a step at 32^3
+// 68.1 -> 66.4 us, at 128^3 201.6 -> 200.0).  A union box wider than the lattice (a
+// sphere of 2 R + 6 = the edge that moves three cells or more in a step) holds some
+// nodes twice; their first cell alone saves and clears them, so that none is saved
+// after it has been cleared.
+template <class FM>
+__device__ __forceinline__ void save_clear_body(const PartArgs& a, const Blk bk) {
+  DevParticle& P = a.parts[0];
+  if (bk.y == 0 && threadIdx.x == 0) {
+    reset_counts(a, P, true);
+    *a.surf_count = 0;
+  }
+  const int c = bk.y * blockDim.x + threadIdx.x;
+  if (c >= box_cells(P.ulo, P.uhi)) return;
+  int X, Y, Z;
+  box_coord(c, P.ulo, P.uhi, X, Y, Z);
+  if (X - P.ulo[0] >= a.g.nx || Y - P.ulo[1] >= a.g.ny || Z - P.ulo[2] >= a.g.nz) return;
+  const long long n = node_of(X, Y, Z, a.g);
+  const int own = a.owner[n];
+  a.owner_prev[n] = own;
+  if (own >= 0) a.owner[n] = FLUID;
+  real_set<FM>(a.psi, n, 0.0);
+  real_set<FM>(a.qpart, n, 0.0);
+}
 template <class FM>
 __global__ void k_save_clear(PartArgs a) {
   let_next_start();
   after_previous();
-  save_prev_body(a, grid_blk());
-  clear_body<FM>(a, grid_blk());
+  save_clear_body<FM>(a, grid_blk());
 }
 // a batch's systems (FP32 form): those of a single particle clear here
 __device__ __forceinline__ void save_prev_any(const PartArgs& a, const Blk bk) {
-  save_prev_body(a, bk);
-  if (a.P == 1) clear_body<FormF32>(a, bk);
+  if (a.P == 1) save_clear_body<FormF32>(a, bk);
+  else save_prev_body(a, bk);
 }
 
 template <class FM>
