@@ -36,3 +36,15 @@ def test_the_longest_wave_has_no_bias(gpu_lib, shape, axis):
     lam = 2 - 2 * np.cos(2 * np.arccos(long(-1)) / n)
     want = 4 * np.arccos(long(-1)) * long(LB) * (q.astype(long) * w).sum() / lam
     assert abs((phi.astype(long) * w).sum() / want - 1) < 1e-14
+
+
+@pytest.mark.parametrize("shape", [(54, 54, 54), (162, 27, 32)])
+def test_a_box_that_cannot_be_coarsened_takes_one_cycle(gpu_lib, shape):
+    """Also below the residual that rounding leaves, eps 12 max|phi| / max|b| and more:
+    the FFT solves the whole problem, and again would give the same."""
+    q = np.random.default_rng(9).standard_normal(shape[::-1])
+    first, cycles, res = solve(gpu_lib, q, shape, tol=1e-9, max_cycles=50)
+    assert cycles == 1 and res < 1e-9
+    again, cycles, res = solve(gpu_lib, q, shape, tol=1e-17, max_cycles=50)
+    assert cycles == 1 and 1e-17 < res < 1e-9
+    assert np.array_equal(first, again)
