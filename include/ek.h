@@ -382,13 +382,13 @@ ek_status ek_batch_step(ek_batch* b, int nsteps);
 /* Wait for the batch stream and read every system's device status word; the
  * first failing system's status is returned (ek_batch_last_error names it). */
 ek_status ek_batch_sync(ek_batch* b);
-/* Autotuner: times every candidate configuration -- the fused forms (where
- * the batch allows them) or branches with 8, 16, 32, 64 or one branch stream
- * per system (at most 64), FP32 S2 segment length (2, 4 or 8 planes per
- * block), and whether the particle chain runs beside the advection or in line
- * -- over 2 + trial_steps real batch steps each (the systems advance by those
- * steps), keeps the fastest and stores its time per batch step in *best_ms
- * (may be null).  Results do not depend on the choice. */
+/* Autotuner: times every candidate configuration -- the one in use, then the
+ * fused forms (where the batch allows them) or branches with 8, 16, 32, 64 or
+ * one branch stream per system (at most 64), FP32 S2 segment length (2, 4 or 8
+ * planes per block), and whether the particle chain runs beside the advection
+ * or in line -- over 2 + trial_steps real batch steps each (the systems advance
+ * by those steps), keeps the fastest and stores its time per batch step in
+ * *best_ms (may be null).  Results do not depend on the choice. */
 ek_status ek_batch_tune(ek_batch* b, int trial_steps, double* best_ms);
 /* Current configuration: cfg[0] branch streams, cfg[1] planes per S2 block,
  * cfg[2] particle chain beside the advection (1) or in line (0), cfg[3] the

@@ -1870,16 +1870,18 @@ ek_status ek_batch_create(ek_ctx* const* systems, int nsys, ek_batch** out) {
     b->fusable = b->fusable && c->fp32 && c->ph.K == b->sys[0]->ph.K && c->ph.pv == b->sys[0]->ph.pv;
   b->fuse = b->fusable ? 1 : 0;
   {
-    // one S2 launch holds every system's tile columns: the segment length
-    // goes by their total (64 boxes of edges 32-64 at 4 and 8 planes: 0.469
-    // and 0.397 ms)
+    // the SMs hold the tile columns of every FP32 system at once, in one launch
+    // or in launches side by side: the segment length goes by their total (64
+    // boxes of edges 32-64 at 4 and 8 planes: 0.469 and 0.397 ms), from the
+    // shortest that the tuner tries
     long long cols = 0, nodes = 0;
     for (ek_ctx* c : b->sys) {
+      if (!c->fp32) continue;
       const dim3 lg = lattice_grid32(c->g, 1);
       cols += (long long)lg.x * lg.y;
       nodes += (long long)lg.x * lg.y * c->g.nz;
     }
-    if (b->fuse) b->planes = lb32_planes(cols, (int)(nodes / cols));
+    if (cols) b->planes = std::max(2, lb32_planes(cols, (int)(nodes / cols)));
   }
   if (!ok) {
     ek_batch_destroy(b);
@@ -1990,8 +1992,8 @@ ek_status ek_batch_wait_test(ek_batch* b, int leave_cta, double limit_ms) {
   return EK_OK;
 }
 
-// Autotuner: every candidate (branch width x S2 segment length x overlap of
-// the particle chain) is captured and timed over `trial_steps` real steps of
+// Autotuner: every candidate (the configuration in use, then form x branch width x
+// S2 segment length x overlap of the particle chain) is captured and timed over `trial_steps` real steps of
 // the whole batch (CUDA events on the batch stream, after one untimed step
 // that uploads the graph); the fastest is kept.
 ek_status ek_batch_tune(ek_batch* b, int trial_steps, double* best_ms) {
@@ -2003,8 +2005,10 @@ ek_status ek_batch_tune(ek_batch* b, int trial_steps, double* best_ms) {
     if (w < nbranch) widths.push_back(w);
   widths.push_back(nbranch);
   // candidates (fuse, branch width, planes per S2 block, overlap); the fused
-  // step has no branches
+  // step has no branches.  The configuration it comes with is the first, so the
+  // one it leaves is no slower.
   std::vector<std::tuple<int, int, int, int>> cands;
+  cands.emplace_back(b->fusable ? b->fuse : 0, b->width, b->planes, b->overlap);
   for (int pl : {2, 4, 8})
     for (int ov = 0; ov <= 1; ++ov) {
       if (b->fusable) {
@@ -2013,6 +2017,7 @@ ek_status ek_batch_tune(ek_batch* b, int trial_steps, double* best_ms) {
       }
       for (int w : widths) cands.emplace_back(0, w, pl, ov);
     }
+  cands.erase(std::remove(cands.begin() + 1, cands.end(), cands[0]), cands.end());  // once
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess)
     return bfail(b, EK_ERR_CUDA, "event creation failed");

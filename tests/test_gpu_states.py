@@ -121,3 +121,22 @@ def test_the_segments_of_s2_do_not_change_a_step(gpu_lib, fused):
         b.close()
         for s in sys_:
             s.close()
+
+
+@pytest.mark.parametrize("fp64_too", [False, True])
+def test_a_batch_starts_from_a_configuration_the_tuner_tries(gpu_lib, fp64_too):
+    """Its segment length is one of the tuner's, in both forms, and the tuner also
+    tries the configuration in use: it cannot leave the batch slower."""
+    ek = gpu_lib
+    ws = workloads.batch_ensemble(3, seed=2025, edges=(32,))
+    sys_ = [make(ek, w) for w in ws]
+    if fp64_too:  # no fused form
+        w = ws[0]
+        sys_.append(ek.EKSystem(w["shape"], valence=w["valence"], D=w["D"], bulk=w["bulk"], flags=ek.EK_PV))
+    b = ek.EKBatch(sys_)
+    assert b.config()["fused"] == (0 if fp64_too else 1)
+    assert b.config()["planes_per_block"] == 2  # 12 tile columns: the shortest it tries
+    b.set_config(planes_per_block=5)
+    cfg, _ = b.tune(2)
+    assert cfg["planes_per_block"] in (2, 4, 5, 8)
+    b.close()
