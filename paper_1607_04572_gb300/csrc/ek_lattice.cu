@@ -45,8 +45,8 @@ __device__ __forceinline__ void boundary_velocity(const DevParticle& P, int xb, 
 // work and shared memory are free beside them.  Each link flux is computed
 // once, by the end whose link points up in z (or, in the plane, along (1,0),
 // (0,1), (1,1), (1,-1)): the values of the nine links go to shared memory, from
-// where the other end takes them with the opposite sign.  A link value is the
-// same number for both ends, so what leaves one node enters the other exactly.
+// where the other end takes them with the opposite sign: what leaves one node
+// enters the other up to the rounding of the sums.
 // Where no node of the three planes is a boundary or partly covered (SIMPLE)
 // the partial-volume factors drop out.  The collision is the pair form of
 // lb32_collide.
