@@ -105,8 +105,8 @@ FP64_PEAK_TFLOPS = 152 * 2.07e9 * 4 / 1e12
 # DRAM traffic (dram__bytes_read.sum + dram__bytes_write.sum) per lattice node
 # of one launch of the kernel, from an ncu capture, valid only for the kernel
 # source it was taken on (otherwise the traffic is reported as null).
-TRAFFIC = {"k_lb32": {"bytes_per_node": (205391104 + 178442496) / 128 ** 3,
-                      "source_sha": "9a3cc8989bf3c12e", "file": "ek_lattice32.cu"}}
+TRAFFIC = {"k_lb32": {"bytes_per_node": (205370368 + 178822144) / 128 ** 3,
+                      "source_sha": "60e75247ae4e17aa", "file": "ek_lattice32.cu"}}
 
 
 def src_sha(name: str) -> str:

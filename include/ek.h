@@ -396,7 +396,8 @@ ek_status ek_batch_tune(ek_batch* b, int trial_steps, double* best_ms);
  * forces as three persistent launches whose phases meet at grid barriers. */
 ek_status ek_batch_config(const ek_batch* b, int cfg[4]);
 /* Set the configuration (cfg as ek_batch_config gives it: branch streams 1 ..
- * min(nsys, 64), planes per S2 block 1 .. 64, overlap 0 or 1, form 0, 1 or 2);
+ * min(nsys, 64), planes per S2 block 1 .. 64 (about: from 4 on a block holds
+ * whole groups of three or four planes), overlap 0 or 1, form 0, 1 or 2);
  * waits for the batch's earlier work.  EK_ERR_ARG for a value out of range or
  * a fused form on a batch that does not allow it. */
 ek_status ek_batch_set_config(ek_batch* b, const int cfg[4]);

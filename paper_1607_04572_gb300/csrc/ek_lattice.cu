@@ -48,13 +48,13 @@ __device__ __forceinline__ void boundary_velocity(const DevParticle& P, int xb, 
 // where the other end takes them with the opposite sign: what leaves one node
 // enters the other up to the rounding of the sums.
 // Where no node of the three planes is a boundary or partly covered (SIMPLE)
-// the partial-volume factors drop out.  The collision is the pair form of
-// lb32_collide.
+// the partial-volume factors drop out.  The collision is a pair form
+// (lb64_collide).
 //
 // One thread per node with all 18 links evaluated at both ends took 900 FP64
 // instructions per node, the pipe 87% busy: 3.30 ms at 128^3, 0.433 ms at 64^3.
-// This form takes 365: 1.50 and 0.244 ms, the pipe 79% busy (barriers and the
-// latency of the FP64 chains between them are the rest).
+// This form takes 350: 1.49 and 0.243 ms, the pipe 84% busy at 128^3 (barriers and
+// the latency of the FP64 chains between them are the rest).
 // ---------------------------------------------------------------------------
 constexpr int HX = TILE_X + 2, HY = TILE_Y + 2, HP = HX * HY, TN = TILE_X * TILE_Y;
 

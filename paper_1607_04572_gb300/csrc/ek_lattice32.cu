@@ -121,9 +121,9 @@ __device__ __forceinline__ void sum3_take(const WarpSums& red, double* ipart, lo
 // flux and collision arithmetic left out the same loads and stores took 5.22
 // of 5.82 ms (27 GB: 5.2 TB/s); stores without the one-node shift in x would
 // take 0.4 ms less (the ten shifted populations write five sectors per warp
-// for four).  Two species share one packed f32x2 instruction.  6.96 -> 6.18 ms
-// at 512^3, 0.936 -> 0.862 at 256^3 (K = 3), 0.110 -> 0.106 at 128^3, most of it
-// by the longer segments (lb32_planes).  Three blocks per SM (80 registers) were
+// for four).  Two species share one packed f32x2 instruction: 1254 -> 1085 warp
+// instructions per node.  6.96 -> 6.2 ms at 512^3, 0.936 -> 0.865 at 256^3 (K = 3),
+// 0.110 -> 0.106 at 128^3, most of it by the longer segments (lb32_planes).  Three blocks per SM (80 registers) were
 // slower: 7.11 ms at 4-plane segments against 6.52.
 // ---------------------------------------------------------------------------
 constexpr int HX = TILE_X + 2, HY = TILE_Y + 2;  // tile with halo

@@ -23,7 +23,7 @@
 // returned is taken over all nodes), the restriction weighs the 13 red nodes of its 27, and the
 // correction goes to the black nodes only (the red half sweep that follows does
 // not read the others).  The coarse levels run while the host waits for the
-// residual.  128^3 to 1e-12 (GB300): 13 cycles of 0.51 ms -> 13 of 0.36 ms.  Of
+// residual.  128^3 to 1e-12 (GB300): 13 cycles of 0.51 ms -> 13 of 0.26 ms.  Of
 // a cycle (launches one by one, cold L2) the finest level's half sweeps take 8 x
 // 15 us (FP64 pipe: 10 us), its residual, restriction and prolongation 41 us,
 // 64^3 48 us, 32^3 35 us and the FFT of 16^3 50 us.
